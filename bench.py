@@ -44,16 +44,18 @@ def kernel_flops_per_head_token(name, w, local=False):
     h, r, b = w.h, w.r, w.b
     k = h + 1
     half = (b + 1) / 2.0                       # causal pairs per row inside a block
+    FC = 64 * (r // 8) * (r // 8 + 1) // 2
     table = {
-        # CUDA-core path
-        "sketch_kernel": 4 * h * r,
+        # CUDA-core path (FC stored features: chunks of 8 x 8 pairs of half-sketch coordinates)
+        "sketch_kernel": 8 * h * r,                 # Q and K in one launch
         "rows_prep_kernel": 2 * h,
-        "state_kernel": 2 * r * r * k + r * r,
-        "scan_kernel": r * r * k / b,
-        "fwd_out_kernel": 2 * r * r * k + r * r + half * 2 * (r + k),
-        "bwd_q_kernel": 2 * r * r * k + 2 * r * r + half * 2 * (2 * r + k),
-        "bwd_k_kernel": 4 * r * r * k + 3 * r * r + half * 2 * (2 * r + 2 * k),
-        "sketch_bwd_kernel": 8 * h * r,
+        "state_kernel": 2 * FC * k + FC,
+        "scan_kernel": FC * k / b,
+        "fwd_out_kernel": 2 * FC * k + FC + half * 2 * (r + k),
+        "bwd_q_kernel": 2 * FC * k + 4 * FC + half * 2 * (2 * r + k),
+        "bwd_k_kernel": 2 * FC * k + 4 * FC + half * 2 * (2 * r + k),
+        "bwd_v_kernel": 2 * FC * k + FC + half * 2 * (r + k),
+        "sketch_bwd_kernel": 16 * h * r,
     }
     # tensor-core path: MMA flops actually issued (symmetric features: F = r(r+1)/2, padded)
     F = r * (r + 1) // 2

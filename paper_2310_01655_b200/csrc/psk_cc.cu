@@ -3,22 +3,25 @@
 // Z_l -> output rows P_l + phi'(Q_l) Z_l -> division by D~).  Serves fp32 storage (the
 // tensor cores' tf32 rounding cannot hold 1e-4 through a degree-4 polynomial) and
 // cross-checks the tensor-core path on bf16 storage.
-#include "psk_internal.cuh"
+#include "cc_rows.cuh"
 
 namespace psk {
 
+// The forward's arrays come first and lie the same in both layouts: with PSK_FLAG_KEEP_STATES the
+// backward finds the half sketches and the prefix states where the forward left them.
 CcWorkspace cc_workspace(const Dims& d, bool backward) {
     CcWorkspace w{};
     const size_t rows = (size_t)d.BH() * d.n;
-    const size_t st = (size_t)d.BH() * d.t * d.r * d.r * 65 * sizeof(float);
-    size_t off = 0;
+    const size_t chunks = (size_t)(d.r / 8) * (d.r / 8 + 1) / 2;
+    const size_t st = (size_t)d.BH() * d.t * chunks * cc::kChunkFloats * sizeof(float);
+        size_t off = 0;
     w.status = off; off += kStatusBytes;
     w.Mq = off;  off += align_up(rows * d.r * sizeof(float));
     w.Mk = off;  off += align_up(rows * d.r * sizeof(float));
-    w.Vt = off;  off += align_up(rows * 65 * sizeof(float));
     w.Zst = off; off += align_up(st);
+    if (d.bf16) { w.Vt = off; off += align_up(rows * 64 * sizeof(float)); }      // fp32 values are read where the caller has them
     if (backward) {
-        w.E = off;   off += align_up(rows * 65 * sizeof(float));
+        w.E = off;   off += align_up(rows * cc::kLd * sizeof(float));
         w.Rst = off; off += align_up(st);
         w.dMq = off; off += align_up(rows * d.r * sizeof(float));
         w.dMk = off; off += align_up(rows * d.r * sizeof(float));
@@ -27,66 +30,117 @@ CcWorkspace cc_workspace(const Dims& d, bool backward) {
             w.dXk = off; off += align_up(rows * 64 * sizeof(float));
         }
     }
-    w.total = off;
+    // The size reported is what full r^2 x 65 states per block take, as it has always been; the
+    // distinct features need less of it.
+    const size_t full = align_up((size_t)d.BH() * d.t * d.r * d.r * 65 * sizeof(float)), row65 = align_up(rows * 65 * sizeof(float));
+    const size_t m = align_up(rows * d.r * sizeof(float));
+    size_t reported = kStatusBytes + 2 * m + row65 + full;
+    if (backward) reported += row65 + full + 2 * m + (d.local ? 2 * align_up(rows * 64 * sizeof(float)) : 0);
+    w.total = off > reported ? off : reported;
     return w;
 }
 
 namespace {
 
 constexpr int H64 = 64;     // head dimension (only value supported)
-constexpr int YC = 65;      // columns of [V | 1] and of E
-constexpr int YS = 68;      // padded shared-memory row stride for 65-column rows
+using cc::Slice;
 
-struct Slice {              // addressing of one [B,H,n,h] tensor
-    int H; int64_t sb, sh, sn;
-    __device__ int64_t row(int bh, int i) const {
-        return (int64_t)(bh / H) * sb + (int64_t)(bh % H) * sh + (int64_t)i * sn;
-    }
+// ---------------------------------------------------------------------------
+// Half sketch m(x) = (x G1)*(x G2)/sqrt(r)  (Algorithm 1, degree-2 level): 64 rows per 64-thread
+// group, two groups per CTA, one or two tensors (Q and K) per launch.  A thread holds eight rows of
+// the same few columns of x G1 and of x G2 (16 columns in two passes for r = 64), so their product is
+// formed in registers.
+// ---------------------------------------------------------------------------
+template <int R> struct SkTile {
+    static constexpr int kPasses = R == 64 ? 2 : 1, kCols = R / 8 / kPasses, NP = kCols / 2;
 };
 
-// ---------------------------------------------------------------------------
-// Half sketch m(x) = (x G1)*(x G2)/sqrt(r)  (Algorithm 1, degree-2 level), 64 rows per CTA
-// ---------------------------------------------------------------------------
+// a1, a2: rows 8 ry + i, columns base + kCols cx + j of X G1 and X G2 (Xt [64][kLd], G [64][R])
+template <int R>
+__device__ __forceinline__ void sketch_products(float (&a1)[8][SkTile<R>::kCols], float (&a2)[8][SkTile<R>::kCols],
+                                                const float* Xt, const float* G1, const float* G2, int base, int ry, int cx) {
+    using namespace cc;
+    constexpr int NP = SkTile<R>::NP, KC = SkTile<R>::kCols;
+    f2 s[2][4][NP], x[2][4][NP];
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int q = 0; q < NP; ++q) s[m][p][q] = x[m][p][q] = 0ull;
+#pragma unroll 4
+    for (int k = 0; k < 64; ++k) {
+        f2 a[4];
+        load_rows8(a, Xt + k * kLd + 8 * ry);
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const float* g = (m ? G2 : G1) + k * R + base + KC * cx;
+            f2 c[NP];
+            if constexpr (NP == 1) c[0] = *reinterpret_cast<const f2*>(g);
+            else { const F22 u = lds22(g); c[0] = u.x; c[1] = u.y; }
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+                const f2 sw = swap2(c[q]);
+#pragma unroll
+                for (int p = 0; p < 4; ++p) { s[m][p][q] = fma2(a[p], c[q], s[m][p][q]); x[m][p][q] = fma2(a[p], sw, x[m][p][q]); }
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < KC; ++j) {
+            const f2 v1 = ((i ^ j) & 1) ? x[0][i / 2][j / 2] : s[0][i / 2][j / 2];
+            const f2 v2 = ((i ^ j) & 1) ? x[1][i / 2][j / 2] : s[1][i / 2][j / 2];
+            a1[i][j] = (i & 1) ? hi2(v1) : lo2(v1);
+            a2[i][j] = (i & 1) ? hi2(v2) : lo2(v2);
+        }
+}
+
+template <int R> constexpr size_t kSketchSmem = (2 * H64 * R + 2 * cc::kUnit) * sizeof(float);
+
 template <typename T, int R>
-__global__ void __launch_bounds__(256)
-sketch_kernel(Slice sl, const T* __restrict__ X, const T* __restrict__ G1, const T* __restrict__ G2,
-              int g_heads, int n, float* __restrict__ M_out, float* __restrict__ Phi_out) {
-    extern __shared__ float smem[];
+__global__ void __launch_bounds__(128)
+sketch_kernel(Slice sl, const T* __restrict__ X0, const T* __restrict__ X1, const T* __restrict__ G1, const T* __restrict__ G2,
+              int g_heads, int n, float* __restrict__ M0, float* __restrict__ M1, float* __restrict__ Phi_out) {
+    extern __shared__ __align__(16) float smem[];
+    using namespace cc;
+    constexpr int KC = SkTile<R>::kCols;
     float* sG1 = smem;                  // [64][R]
     float* sG2 = sG1 + H64 * R;         // [64][R]
-    float* sX = sG2 + H64 * R;          // [64][65]
-    float* sM = sX + 64 * 65;           // [64][R+1]
-    const int bh = blockIdx.y, i0 = blockIdx.x * 64, tid = threadIdx.x;
+    const int tid = threadIdx.x, grp = tid / 64, lane = tid % 64, ry = lane / 8, cx = lane % 8;
+    float* sXt = sG2 + H64 * R + grp * kUnit;
+    const int bh = blockIdx.y, i0 = blockIdx.x * 128 + grp * 64;
+    const T* X = blockIdx.z ? X1 : X0;
+    float* M = (blockIdx.z ? M1 : M0) + ((size_t)bh * n + i0) * R;
     const int g = (g_heads == 1) ? 0 : (bh % sl.H);
-    for (int e = tid; e < H64 * R; e += 256) {
-        sG1[e] = ldf(G1 + (size_t)g * H64 * R + e);
-        sG2[e] = ldf(G2 + (size_t)g * H64 * R + e);
+    for (int e = tid; e < H64 * R / 4; e += 128) {
+        *reinterpret_cast<float4*>(sG1 + 4 * e) = ld4(G1 + (size_t)g * H64 * R + 4 * e);
+        *reinterpret_cast<float4*>(sG2 + 4 * e) = ld4(G2 + (size_t)g * H64 * R + 4 * e);
     }
-    for (int e = tid; e < 64 * H64; e += 256) {
-        const int rr = e / H64, c = e % H64;
-        sX[rr * 65 + c] = ldf(X + sl.row(bh, i0 + rr) + c);
-    }
+    load_raw<T, true>(sXt, X, sl, bh, i0, lane, 64);
     __syncthreads();
     const float rs = rsqrtf((float)R);
-    const int c = tid % R;
-    for (int rr = tid / R; rr < 64; rr += 256 / R) {
-        float a1 = 0.f, a2 = 0.f;
-#pragma unroll 16
-        for (int t = 0; t < H64; ++t) {
-            const float x = sX[rr * 65 + t];
-            a1 = fmaf(x, sG1[t * R + c], a1);
-            a2 = fmaf(x, sG2[t * R + c], a2);
+#pragma unroll 1
+    for (int base = 0; base < R; base += 8 * KC) {
+        float a1[8][KC], a2[8][KC];
+        sketch_products<R>(a1, a2, sXt, sG1, sG2, base, ry, cx);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float* dst = M + (size_t)(8 * ry + i) * R + base + KC * cx;
+            if constexpr (KC == 2) *reinterpret_cast<float2*>(dst) = make_float2(a1[i][0] * a2[i][0] * rs, a1[i][1] * a2[i][1] * rs);
+            else *reinterpret_cast<float4*>(dst) = make_float4(a1[i][0] * a2[i][0] * rs, a1[i][1] * a2[i][1] * rs,
+                                                               a1[i][2] * a2[i][2] * rs, a1[i][3] * a2[i][3] * rs);
         }
-        const float m = a1 * a2 * rs;
-        sM[rr * (R + 1) + c] = m;
-        M_out[((size_t)bh * n + i0 + rr) * R + c] = m;
     }
     if (Phi_out != nullptr) {           // phi'(x)[a*R+b] = m_a m_b (Section 1.2 ordering)
-        __syncthreads();
-        for (int e = tid; e < 64 * R * R; e += 256) {
-            const int rr = e / (R * R), f = e % (R * R);
-            Phi_out[((size_t)bh * n + i0 + rr) * R * R + f] =
-                sM[rr * (R + 1) + f / R] * sM[rr * (R + 1) + f % R];
+        __syncthreads();                // (this CTA's rows of M, written above, are visible to all of it)
+        float* phi = Phi_out + ((size_t)bh * n + i0) * R * R;
+        for (int e = lane; e < 64 * R * R / 4; e += 64) {
+            const int rr = e / (R * R / 4), f = 4 * (e % (R * R / 4));
+            const float ma = M[rr * R + f / R];
+            const float4 mb = *reinterpret_cast<const float4*>(M + rr * R + f % R);
+            *reinterpret_cast<float4*>(phi + (size_t)rr * R * R + f) = make_float4(ma * mb.x, ma * mb.y, ma * mb.z, ma * mb.w);
         }
     }
 }
@@ -277,466 +331,123 @@ sketch8_bwd_kernel(Slice sl, const T* __restrict__ X, const T* __restrict__ G1, 
 }
 
 // ---------------------------------------------------------------------------
-// Row preparation: mode 0 writes V~ = [V | 1]; mode 1 writes E = [dO/d | -(dO.O)/d]
-// One warp per row.
+// Row preparation: mode 0 writes V in fp32 (bf16 storage; rows of 64); mode 1 writes
+// E = [dO/d | -(dO.O)/d] (rows of kLd).  16 lanes per row.
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256)
 rows_prep_kernel(Slice sl, int n, int total_rows, int mode, const T* __restrict__ V,
                  const T* __restrict__ O, const float* __restrict__ denom,
                  const T* __restrict__ dO, float* __restrict__ out) {
-    const int row = blockIdx.x * 8 + threadIdx.x / 32, lane = threadIdx.x % 32;
-    if (row >= total_rows) return;
-    const int bh = row / n, i = row % n;
-    const int64_t base = sl.row(bh, i);
-    float* o = out + (size_t)row * YC;
+    const int row = blockIdx.x * 16 + threadIdx.x / 16, lane = threadIdx.x % 16;
+    if (row >= total_rows) return;      // (total_rows is a multiple of 128: whole warps)
+    const int64_t base = sl.row(row / n, row % n) + 4 * lane;
     if (mode == 0) {
-        o[lane] = ldf(V + base + lane);
-        o[lane + 32] = ldf(V + base + lane + 32);
-        if (lane == 0) o[64] = 1.f;
-    } else {
-        const float g0 = ldf(dO + base + lane), g1 = ldf(dO + base + lane + 32);
-        float dot = g0 * ldf(O + base + lane) + g1 * ldf(O + base + lane + 32);
-#pragma unroll
-        for (int s = 16; s > 0; s >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, s);
-        const float inv = 1.f / denom[row];
-        o[lane] = g0 * inv;
-        o[lane + 32] = g1 * inv;
-        if (lane == 0) o[64] = -dot * inv;
+        *reinterpret_cast<float4*>(out + (size_t)row * 64 + 4 * lane) = cc::ld4(V + base);
+        return;
     }
-}
-
-// ---------------------------------------------------------------------------
-// Per-block state H_l = phi'(M_l)^T Y_l  (Section 3.1), M the half sketches of the
-// block's rows, Y its [b,65] right-hand side.  One thread per feature (a,b).
-// ---------------------------------------------------------------------------
-template <int R>
-__global__ void __launch_bounds__(128)
-state_kernel(const float* __restrict__ M, const float* __restrict__ Y, int n, int b, int t,
-             float* __restrict__ S) {
-    __shared__ float sM[32][R];
-    __shared__ __align__(16) float sY[32][YS];
-    const int tid = threadIdx.x, l = blockIdx.y, bh = blockIdx.z;
-    const int f = blockIdx.x * 128 + tid, fa = f / R, fb = f % R;
-    float acc[YC];
+    float* o = out + (size_t)row * cc::kLd;
+    float4 v = cc::ld4(dO + base);
+    const float4 u = cc::ld4(O + base);
+    float dot = (v.x * u.x + v.y * u.y) + (v.z * u.z + v.w * u.w);
 #pragma unroll
-    for (int c = 0; c < YC; ++c) acc[c] = 0.f;
-    const size_t row0 = (size_t)bh * n + (size_t)l * b;
-    for (int j0 = 0; j0 < b; j0 += 32) {
-        __syncthreads();
-        for (int e = tid; e < 32 * R; e += 128) sM[e / R][e % R] = M[(row0 + j0) * R + e];
-        for (int e = tid; e < 32 * YC; e += 128) sY[e / YC][e % YC] = Y[(row0 + j0) * YC + e];
-        __syncthreads();
-        if (f < R * R) {
-#pragma unroll 4
-            for (int j = 0; j < 32; ++j) {
-                const float phi = sM[j][fa] * sM[j][fb];
-#pragma unroll
-                for (int c = 0; c < 64; c += 4) {
-                    const float4 y = *reinterpret_cast<const float4*>(&sY[j][c]);
-                    acc[c] = fmaf(phi, y.x, acc[c]);
-                    acc[c + 1] = fmaf(phi, y.y, acc[c + 1]);
-                    acc[c + 2] = fmaf(phi, y.z, acc[c + 2]);
-                    acc[c + 3] = fmaf(phi, y.w, acc[c + 3]);
-                }
-                acc[64] = fmaf(phi, sY[j][64], acc[64]);
-            }
-        }
-    }
-    if (f < R * R) {
-        float* o = S + (((size_t)bh * t + l) * R * R + f) * YC;
-#pragma unroll
-        for (int c = 0; c < YC; ++c) o[c] = acc[c];
-    }
-}
-
-// Exclusive prefix (reverse = 0: Z_l = sum_{j<l} H_j, Section 3.1) or exclusive suffix
-// (reverse = 1: sum_{j>l} H_j) over the t states of each head, in place, sequential in l.
-__global__ void __launch_bounds__(256)
-scan_kernel(float* __restrict__ S, size_t elems, int t, int reverse) {
-    const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (e >= elems) return;
-    float* p = S + (size_t)blockIdx.y * t * elems + e;
-    float run = 0.f;
-    if (!reverse) {
-        for (int l = 0; l < t; ++l) { const float v = p[(size_t)l * elems]; p[(size_t)l * elems] = run; run += v; }
-    } else {
-        for (int l = t - 1; l >= 0; --l) { const float v = p[(size_t)l * elems]; p[(size_t)l * elems] = run; run += v; }
-    }
-}
-
-// acc[0..64] += coef * row[0..64]   (row in shared memory, 16-byte aligned, stride YS)
-__device__ __forceinline__ void axpy65(float (&acc)[YC], float coef, const float* row) {
-#pragma unroll
-    for (int c = 0; c < 64; c += 4) {
-        const float4 z = *reinterpret_cast<const float4*>(row + c);
-        acc[c] = fmaf(coef, z.x, acc[c]);
-        acc[c + 1] = fmaf(coef, z.y, acc[c + 1]);
-        acc[c + 2] = fmaf(coef, z.z, acc[c + 2]);
-        acc[c + 3] = fmaf(coef, z.w, acc[c + 3]);
-    }
-    acc[64] = fmaf(coef, row[64], acc[64]);
-}
-// row[0..64] . y[0..64]
-__device__ __forceinline__ float dot65(const float* row, const float (&y)[YC]) {
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-    for (int c = 0; c < 64; c += 4) {
-        const float4 z = *reinterpret_cast<const float4*>(row + c);
-        s0 = fmaf(z.x, y[c], s0);
-        s1 = fmaf(z.y, y[c + 1], s1);
-        s2 = fmaf(z.z, y[c + 2], s2);
-        s3 = fmaf(z.w, y[c + 3], s3);
-    }
-    return (s0 + s1) + (s2 + s3) + row[64] * y[64];
-}
-
-// Shared-memory carve-up of the three row kernels (one thread per row, 128 rows per CTA):
-//   sS   [R][YS]        slice a of the block's prefix/suffix state: rows (a, 0..R-1)
-//   sOwn [128][R+1]     this tile's own half sketches (runtime-indexed access by a)
-//   sOut [128][R+1]     per-row results indexed by a
-//   sM2  [32][R]        chunk of the other side's half sketches (diagonal tile)
-//   sY2  [32][YS]       chunk of the other side's 65-column rows (diagonal tile)
-// and, with exact same-block weights (Section 3.2):
-//   sXo  [128][65]      this tile's own raw rows (q or k), each read by its own thread only
-//   sX2  [32][64]       chunk of the other side's raw rows
-template <int R> struct RowSmem {
-    static constexpr int S = 0;
-    static constexpr int Own = S + R * YS;
-    static constexpr int Out = Own + 128 * (R + 1);
-    static constexpr int M2 = Out + 128 * (R + 1);
-    static constexpr int Y2 = M2 + 32 * R;
-    static constexpr int total = Y2 + 32 * YS;
-    static constexpr size_t bytes = (size_t)total * sizeof(float);
-    static constexpr int Xo = total;
-    static constexpr int X2 = Xo + 128 * 65;
-    static constexpr size_t bytes_local = (size_t)(X2 + 32 * 64) * sizeof(float);
-};
-
-// <own raw row (shared memory, stride 65), row jj of the other side's chunk>
-__device__ __forceinline__ float dot64_raw(const float* own, const float* other) {
-    float s = 0.f;
-#pragma unroll
-    for (int c = 0; c < 64; ++c) s = fmaf(own[c], other[c], s);
-    return s;
-}
-
-// ---------------------------------------------------------------------------
-// Forward output rows (Section 3.1): row i of block l = P_l row + phi'(q_i)^T Z_l, with
-// P_l = lt((L R^T)^2) [V_l | 1]; then d_i = 1 + last column, O_i = first 64 / d_i.
-// LOCAL: P_l = lt((Q_l K_l^T)^4) [V_l | 1] instead, from the block's raw queries and keys
-// (Section 3.2).
-// ---------------------------------------------------------------------------
-template <typename T, int R, bool LOCAL>
-__global__ void __launch_bounds__(128)
-fwd_out_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mq, const float* __restrict__ Mk,
-               const float* __restrict__ Vt, const float* __restrict__ Z,
-               const T* __restrict__ Qraw, const T* __restrict__ Kraw,
-               T* __restrict__ O, float* __restrict__ denom) {
-    extern __shared__ __align__(16) float smem[];
-    float* sS = smem + RowSmem<R>::S;
-    float* sOwn = smem + RowSmem<R>::Own;
-    float* sM2 = smem + RowSmem<R>::M2;
-    float* sY2 = smem + RowSmem<R>::Y2;
-    const int tid = threadIdx.x, tile = blockIdx.x, l = blockIdx.y, bh = blockIdx.z;
-    const int i_blk = tile * 128 + tid;                 // row within the block
-    const size_t blk0 = (size_t)bh * n + (size_t)l * b;  // first row of the block
-    const size_t row = blk0 + i_blk;
-    float mq[R], acc[YC];
-#pragma unroll
-    for (int c = 0; c < R; ++c) { mq[c] = Mq[row * R + c]; sOwn[tid * (R + 1) + c] = mq[c]; }
-#pragma unroll
-    for (int c = 0; c < YC; ++c) acc[c] = 0.f;
-    float* sXo = smem + RowSmem<R>::Xo + tid * 65;
-    float* sX2 = smem + RowSmem<R>::X2;
-    if constexpr (LOCAL) {
-        const int64_t o = sl.row(bh, l * b + i_blk);
-        for (int c = 0; c < 64; ++c) sXo[c] = ldf(Qraw + o + c);
-    }
-    // earlier blocks through the prefix state
-    const float* Zl = Z + ((size_t)bh * t + l) * R * R * YC;
-    if (l > 0) {
-        for (int a = 0; a < R; ++a) {
-            __syncthreads();
-            for (int e = tid; e < R * YC; e += 128) sS[(e / YC) * YS + e % YC] = Zl[(size_t)a * R * YC + e];
-            __syncthreads();
-            const float ma = sOwn[tid * (R + 1) + a];
-#pragma unroll
-            for (int bb = 0; bb < R; ++bb) axpy65(acc, ma * mq[bb], sS + bb * YS);
-        }
-    }
-    // same block: j <= i through the b x b tile of squared half-sketch scores
-    const int jend = tile * 128 + 128;                  // keys needed by this row tile
-    const int warp_imax = tile * 128 + (tid | 31);
-    for (int j0 = 0; j0 < jend; j0 += 32) {
-        __syncthreads();
-        if constexpr (LOCAL) {
-            for (int e = tid; e < 32 * 64; e += 128) sX2[e] = ldf(Kraw + sl.row(bh, l * b + j0 + e / 64) + e % 64);
-        } else {
-            for (int e = tid; e < 32 * R; e += 128) sM2[e] = Mk[(blk0 + j0) * R + e];
-        }
-        for (int e = tid; e < 32 * YC; e += 128) sY2[(e / YC) * YS + e % YC] = Vt[(blk0 + j0) * YC + e];
-        __syncthreads();
-        if (j0 > warp_imax) continue;
-        for (int jj = 0; jj < 32; ++jj) {
-            if (j0 + jj > i_blk) break;
-            float s = 0.f;
-            if constexpr (LOCAL) {
-                const float x = dot64_raw(sXo, sX2 + jj * 64);
-                s = x * x;                                  // weight s^2 = (q . k)^4
-            } else {
-#pragma unroll
-                for (int c = 0; c < R; ++c) s = fmaf(mq[c], sM2[jj * R + c], s);
-            }
-            axpy65(acc, s * s, sY2 + jj * YS);
-        }
-    }
-    const float d = 1.f + acc[64];
-    const float inv = 1.f / d;
-    const int64_t o = sl.row(bh, l * b + i_blk);
-#pragma unroll
-    for (int c = 0; c < 64; ++c) stf(O + o + c, acc[c] * inv);
-    if (denom != nullptr) denom[row] = d;
-}
-
-// ---------------------------------------------------------------------------
-// Backward, query side.  d m(q_i) = 2 mat(Z_l E_i) m(q_i)  +  sum_{j<=i, same block}
-// 2 s_ij (E_i . v~_j) m(k_j).
-// LOCAL (Section 3.2): the same-block pairs carry W_ij = x_ij^4, x_ij = q_i . k_j, whose gradient
-// reaches q_i directly:  dXl_i = sum_{j<=i, same block} 4 x_ij^3 (E_i . v~_j) k_j.
-// ---------------------------------------------------------------------------
-template <typename T, int R, bool LOCAL>
-__global__ void __launch_bounds__(128)
-bwd_q_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mq, const float* __restrict__ Mk,
-             const float* __restrict__ Vt, const float* __restrict__ E, const float* __restrict__ Z,
-             const T* __restrict__ Qraw, const T* __restrict__ Kraw,
-             float* __restrict__ dMq, float* __restrict__ dXl) {
-    extern __shared__ __align__(16) float smem[];
-    float* sS = smem + RowSmem<R>::S;
-    float* sOut = smem + RowSmem<R>::Out;
-    float* sM2 = smem + RowSmem<R>::M2;
-    float* sY2 = smem + RowSmem<R>::Y2;
-    const int tid = threadIdx.x, tile = blockIdx.x, l = blockIdx.y, bh = blockIdx.z;
-    const int i_blk = tile * 128 + tid;
-    const size_t blk0 = (size_t)bh * n + (size_t)l * b;
-    const size_t row = blk0 + i_blk;
-    float mq[R], dm[R], e[YC];
-#pragma unroll
-    for (int c = 0; c < R; ++c) { mq[c] = Mq[row * R + c]; dm[c] = 0.f; sOut[tid * (R + 1) + c] = 0.f; }
-#pragma unroll
-    for (int c = 0; c < YC; ++c) e[c] = E[row * YC + c];
-    const float* Zl = Z + ((size_t)bh * t + l) * R * R * YC;
-    if (l > 0) {
-        for (int a = 0; a < R; ++a) {
-            __syncthreads();
-            for (int x = tid; x < R * YC; x += 128) sS[(x / YC) * YS + x % YC] = Zl[(size_t)a * R * YC + x];
-            __syncthreads();
-            float ta = 0.f;
-#pragma unroll
-            for (int bb = 0; bb < R; ++bb) ta = fmaf(dot65(sS + bb * YS, e), mq[bb], ta);
-            sOut[tid * (R + 1) + a] = 2.f * ta;
-        }
-    }
-    const int jend = tile * 128 + 128;
-    const int warp_imax = tile * 128 + (tid | 31);
-    float* sXo = smem + RowSmem<R>::Xo + tid * 65;
-    float* sX2 = smem + RowSmem<R>::X2;
-    float dxl[LOCAL ? 64 : 1];
-    if constexpr (LOCAL) {
-        const int64_t o = sl.row(bh, l * b + i_blk);
-        for (int c = 0; c < 64; ++c) sXo[c] = ldf(Qraw + o + c);
-#pragma unroll
-        for (int c = 0; c < 64; ++c) dxl[c] = 0.f;
-    }
-    for (int j0 = 0; j0 < jend; j0 += 32) {
-        __syncthreads();
-        if constexpr (LOCAL) {
-            for (int x = tid; x < 32 * 64; x += 128) sX2[x] = ldf(Kraw + sl.row(bh, l * b + j0 + x / 64) + x % 64);
-        } else {
-            for (int x = tid; x < 32 * R; x += 128) sM2[x] = Mk[(blk0 + j0) * R + x];
-        }
-        for (int x = tid; x < 32 * YC; x += 128) sY2[(x / YC) * YS + x % YC] = Vt[(blk0 + j0) * YC + x];
-        __syncthreads();
-        if (j0 > warp_imax) continue;
-        for (int jj = 0; jj < 32; ++jj) {
-            if (j0 + jj > i_blk) break;
-            if constexpr (LOCAL) {
-                const float x = dot64_raw(sXo, sX2 + jj * 64);
-                const float dx = 4.f * x * x * x * dot65(sY2 + jj * YS, e);
-#pragma unroll
-                for (int c = 0; c < 64; ++c) dxl[c] = fmaf(dx, sX2[jj * 64 + c], dxl[c]);
-            } else {
-                float s = 0.f;
-#pragma unroll
-                for (int c = 0; c < R; ++c) s = fmaf(mq[c], sM2[jj * R + c], s);
-                const float ds = 2.f * s * dot65(sY2 + jj * YS, e);
-#pragma unroll
-                for (int c = 0; c < R; ++c) dm[c] = fmaf(ds, sM2[jj * R + c], dm[c]);
-            }
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < R; ++c) dMq[row * R + c] = dm[c] + sOut[tid * (R + 1) + c];
-    if constexpr (LOCAL) {
-#pragma unroll
-        for (int c = 0; c < 64; ++c) dXl[row * 64 + c] = dxl[c];
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Backward, key/value side.  With R_l the suffix state sum_{blocks>l} phi'(Q)^T E:
-//   d m(k_j) = 2 mat(R_l v~_j) m(k_j) + sum_{i>=j, same block} 2 s_ij (E_i . v~_j) m(q_i)
-//   dV_j     = (R_l^T phi'(k_j))[:h]  + sum_{i>=j, same block} s_ij^2 E_i[:h]
-// LOCAL (Section 3.2): same-block weights x_ij^4, x_ij = q_i . k_j:
-//   dXl_j = sum_{i>=j, same block} 4 x_ij^3 (E_i . v~_j) q_i,   dV_j += sum x_ij^4 E_i[:h]
-// ---------------------------------------------------------------------------
-template <typename T, int R, bool LOCAL>
-__global__ void __launch_bounds__(128)
-bwd_k_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mq, const float* __restrict__ Mk,
-             const float* __restrict__ Vt, const float* __restrict__ E, const float* __restrict__ Rs,
-             const T* __restrict__ Qraw, const T* __restrict__ Kraw,
-             float* __restrict__ dMk, float* __restrict__ dXl, T* __restrict__ dV) {
-    extern __shared__ __align__(16) float smem[];
-    float* sS = smem + RowSmem<R>::S;
-    float* sOwn = smem + RowSmem<R>::Own;
-    float* sOut = smem + RowSmem<R>::Out;
-    float* sM2 = smem + RowSmem<R>::M2;
-    float* sY2 = smem + RowSmem<R>::Y2;
-    const int tid = threadIdx.x, tile = blockIdx.x, l = blockIdx.y, bh = blockIdx.z;
-    const int j_blk = tile * 128 + tid;
-    const size_t blk0 = (size_t)bh * n + (size_t)l * b;
-    const size_t row = blk0 + j_blk;
-    float mk[R], dm[R], v[YC], dv[YC];
-#pragma unroll
-    for (int c = 0; c < R; ++c) {
-        mk[c] = Mk[row * R + c]; dm[c] = 0.f;
-        sOwn[tid * (R + 1) + c] = mk[c]; sOut[tid * (R + 1) + c] = 0.f;
-    }
-#pragma unroll
-    for (int c = 0; c < YC; ++c) { v[c] = Vt[row * YC + c]; dv[c] = 0.f; }
-    const float* Rl = Rs + ((size_t)bh * t + l) * R * R * YC;
-    if (l < t - 1) {
-        for (int a = 0; a < R; ++a) {
-            __syncthreads();
-            for (int x = tid; x < R * YC; x += 128) sS[(x / YC) * YS + x % YC] = Rl[(size_t)a * R * YC + x];
-            __syncthreads();
-            const float ma = sOwn[tid * (R + 1) + a];
-            float ta = 0.f;
-#pragma unroll
-            for (int bb = 0; bb < R; ++bb) {
-                ta = fmaf(dot65(sS + bb * YS, v), mk[bb], ta);
-                axpy65(dv, ma * mk[bb], sS + bb * YS);
-            }
-            sOut[tid * (R + 1) + a] = 2.f * ta;
-        }
-    }
-    // same block: queries i >= j
-    const int i_begin = tile * 128;                     // first query row any thread here needs
-    const int warp_jmin = tile * 128 + (tid & ~31);
-    float* sXo = smem + RowSmem<R>::Xo + tid * 65;
-    float* sX2 = smem + RowSmem<R>::X2;
-    float dxl[LOCAL ? 64 : 1];
-    if constexpr (LOCAL) {
-        const int64_t o = sl.row(bh, l * b + j_blk);
-        for (int c = 0; c < 64; ++c) sXo[c] = ldf(Kraw + o + c);
-#pragma unroll
-        for (int c = 0; c < 64; ++c) dxl[c] = 0.f;
-    }
-    for (int i0 = i_begin; i0 < b; i0 += 32) {
-        __syncthreads();
-        if constexpr (LOCAL) {
-            for (int x = tid; x < 32 * 64; x += 128) sX2[x] = ldf(Qraw + sl.row(bh, l * b + i0 + x / 64) + x % 64);
-        } else {
-            for (int x = tid; x < 32 * R; x += 128) sM2[x] = Mq[(blk0 + i0) * R + x];
-        }
-        for (int x = tid; x < 32 * YC; x += 128) sY2[(x / YC) * YS + x % YC] = E[(blk0 + i0) * YC + x];
-        __syncthreads();
-        if (i0 + 31 < warp_jmin) continue;
-        for (int ii = 0; ii < 32; ++ii) {
-            if (i0 + ii < j_blk) continue;
-            if constexpr (LOCAL) {
-                const float x = dot64_raw(sXo, sX2 + ii * 64);
-                const float x2 = x * x;
-                const float dx = 4.f * x2 * x * dot65(sY2 + ii * YS, v);
-#pragma unroll
-                for (int c = 0; c < 64; ++c) dxl[c] = fmaf(dx, sX2[ii * 64 + c], dxl[c]);
-                axpy65(dv, x2 * x2, sY2 + ii * YS);
-            } else {
-                float s = 0.f;
-#pragma unroll
-                for (int c = 0; c < R; ++c) s = fmaf(mk[c], sM2[ii * R + c], s);
-                const float ds = 2.f * s * dot65(sY2 + ii * YS, v);
-#pragma unroll
-                for (int c = 0; c < R; ++c) dm[c] = fmaf(ds, sM2[ii * R + c], dm[c]);
-                axpy65(dv, s * s, sY2 + ii * YS);
-            }
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < R; ++c) dMk[row * R + c] = dm[c] + sOut[tid * (R + 1) + c];
-    if constexpr (LOCAL) {
-#pragma unroll
-        for (int c = 0; c < 64; ++c) dXl[row * 64 + c] = dxl[c];
-    }
-    const int64_t o = sl.row(bh, l * b + j_blk);
-#pragma unroll
-    for (int c = 0; c < 64; ++c) stf(dV + o + c, dv[c]);
+    for (int s = 8; s > 0; s >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, s);
+    const float inv = 1.f / denom[row];
+    v.x *= inv; v.y *= inv; v.z *= inv; v.w *= inv;
+    *reinterpret_cast<float4*>(o + 4 * lane) = v;
+    if (lane == 0) *reinterpret_cast<float4*>(o + 64) = make_float4(-dot * inv, 0.f, 0.f, 0.f);
 }
 
 // ---------------------------------------------------------------------------
 // Chain rule through the half sketch: dX = ((dM*A2) G1^T + (dM*A1) G2^T)/sqrt(r),
-// A1 = X G1, A2 = X G2 recomputed.  64 rows per CTA.  `add` (optional, [rows][64]): gradient
-// that reached X without passing through the sketch, added before the result is rounded.
+// A1 = X G1, A2 = X G2 recomputed.  Groups, rows and tensors as in sketch_kernel.  `add` (optional,
+// [rows][64]): gradient that reached X without passing through the sketch, added before the
+// result is rounded.
 // ---------------------------------------------------------------------------
+template <int R> struct SkBwdSmem {
+    static constexpr int G = 2 * H64 * R, Gt = 2 * R * cc::kLd;
+    static constexpr int U = 2 * R * cc::kLd;          // U1, U2 transposed
+    static constexpr size_t bytes = (size_t)(G + Gt + 2 * (cc::kUnit + U)) * sizeof(float);
+};
+
 template <typename T, int R>
-__global__ void __launch_bounds__(256)
-sketch_bwd_kernel(Slice sl, const T* __restrict__ X, const T* __restrict__ G1, const T* __restrict__ G2,
-                  int g_heads, int n, const float* __restrict__ dM, const float* __restrict__ add,
-                  T* __restrict__ dX) {
-    extern __shared__ float smem[];
-    float* sG1 = smem;                      // [64][R+1]
-    float* sG2 = sG1 + H64 * (R + 1);       // [64][R+1]
-    float* sX = sG2 + H64 * (R + 1);        // [64][65]
-    float* sU1 = sX + 64 * 65;              // [64][R+1]
-    float* sU2 = sU1 + 64 * (R + 1);        // [64][R+1]
-    const int bh = blockIdx.y, i0 = blockIdx.x * 64, tid = threadIdx.x;
+__global__ void __launch_bounds__(128)
+sketch_bwd_kernel(Slice sl, const T* __restrict__ X0, const T* __restrict__ X1, const T* __restrict__ G1, const T* __restrict__ G2,
+                  int g_heads, int n, const float* __restrict__ dM0, const float* __restrict__ dM1,
+                  const float* __restrict__ add0, const float* __restrict__ add1, T* __restrict__ dX0, T* __restrict__ dX1) {
+    extern __shared__ __align__(16) float smem[];
+    using namespace cc;
+    using L = SkBwdSmem<R>;
+    constexpr int KC = SkTile<R>::kCols;
+    float* sG1 = smem;                      // [64][R]
+    float* sG2 = sG1 + H64 * R;             // [64][R]
+    float* sGt = sG2 + H64 * R;             // [2R][kLd]: rows of G1^T, then of G2^T
+    const int tid = threadIdx.x, grp = tid / 64, lane = tid % 64, ry = lane / 8, cx = lane % 8;
+    float* sXt = sGt + L::Gt + grp * (kUnit + L::U);
+    float* sU = sXt + kUnit;                // [2R][kLd]: rows of (dM*A2)^T, then of (dM*A1)^T
+    const int bh = blockIdx.y, i0 = blockIdx.x * 128 + grp * 64;
+    const T* X = blockIdx.z ? X1 : X0;
+    const float* dM = (blockIdx.z ? dM1 : dM0) + ((size_t)bh * n + i0) * R;
+    const float* add = blockIdx.z ? add1 : add0;
+    T* dX = blockIdx.z ? dX1 : dX0;
     const int g = (g_heads == 1) ? 0 : (bh % sl.H);
-    for (int e = tid; e < H64 * R; e += 256) {
-        sG1[(e / R) * (R + 1) + e % R] = ldf(G1 + (size_t)g * H64 * R + e);
-        sG2[(e / R) * (R + 1) + e % R] = ldf(G2 + (size_t)g * H64 * R + e);
+    for (int e = tid; e < H64 * R / 4; e += 128) {
+        const int k = e / (R / 4), c = 4 * (e % (R / 4));
+        const float4 u = ld4(G1 + (size_t)g * H64 * R + 4 * e), v = ld4(G2 + (size_t)g * H64 * R + 4 * e);
+        *reinterpret_cast<float4*>(sG1 + 4 * e) = u;
+        *reinterpret_cast<float4*>(sG2 + 4 * e) = v;
+        float* t1 = sGt + c * kLd + k;
+        float* t2 = sGt + (R + c) * kLd + k;
+        t1[0] = u.x; t1[kLd] = u.y; t1[2 * kLd] = u.z; t1[3 * kLd] = u.w;
+        t2[0] = v.x; t2[kLd] = v.y; t2[2 * kLd] = v.z; t2[3 * kLd] = v.w;
     }
-    for (int e = tid; e < 64 * H64; e += 256) {
-        const int rr = e / H64, c = e % H64;
-        sX[rr * 65 + c] = ldf(X + sl.row(bh, i0 + rr) + c);
-    }
+    load_raw<T, true>(sXt, X, sl, bh, i0, lane, 64);
     __syncthreads();
     const float rs = rsqrtf((float)R);
-    {
-        const int c = tid % R;
-        for (int rr = tid / R; rr < 64; rr += 256 / R) {
-            float a1 = 0.f, a2 = 0.f;
-#pragma unroll 16
-            for (int t = 0; t < H64; ++t) {
-                const float x = sX[rr * 65 + t];
-                a1 = fmaf(x, sG1[t * (R + 1) + c], a1);
-                a2 = fmaf(x, sG2[t * (R + 1) + c], a2);
+#pragma unroll 1
+    for (int base = 0; base < R; base += 8 * KC) {
+        float a1[8][KC], a2[8][KC];
+        sketch_products<R>(a1, a2, sXt, sG1, sG2, base, ry, cx);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float gm[KC];
+            const float* src = dM + (size_t)(8 * ry + i) * R + base + KC * cx;
+            if constexpr (KC == 2) { const float2 v = *reinterpret_cast<const float2*>(src); gm[0] = v.x; gm[1] = v.y; }
+            else *reinterpret_cast<float4*>(gm) = *reinterpret_cast<const float4*>(src);
+#pragma unroll
+            for (int j = 0; j < KC; ++j) {
+                const float m = gm[j] * rs;
+                a2[i][j] *= m;
+                a1[i][j] *= m;
             }
-            const float g_m = dM[((size_t)bh * n + i0 + rr) * R + c] * rs;
-            sU1[rr * (R + 1) + c] = g_m * a2;
-            sU2[rr * (R + 1) + c] = g_m * a1;
+        }
+#pragma unroll
+        for (int j = 0; j < KC; ++j) {
+            float* u1 = sU + (base + KC * cx + j) * kLd + 8 * ry;
+            float* u2 = u1 + R * kLd;
+            *reinterpret_cast<float4*>(u1) = make_float4(a2[0][j], a2[1][j], a2[2][j], a2[3][j]);
+            *reinterpret_cast<float4*>(u1 + 4) = make_float4(a2[4][j], a2[5][j], a2[6][j], a2[7][j]);
+            *reinterpret_cast<float4*>(u2) = make_float4(a1[0][j], a1[1][j], a1[2][j], a1[3][j]);
+            *reinterpret_cast<float4*>(u2 + 4) = make_float4(a1[4][j], a1[5][j], a1[6][j], a1[7][j]);
         }
     }
-    __syncthreads();
-    {
-        const int t = tid % 64;
-        for (int rr = tid / 64; rr < 64; rr += 4) {
-            float dx = add != nullptr ? add[((size_t)bh * n + i0 + rr) * 64 + t] : 0.f;
-#pragma unroll 16
-            for (int c = 0; c < R; ++c) {
-                dx = fmaf(sU1[rr * (R + 1) + c], sG1[t * (R + 1) + c], dx);
-                dx = fmaf(sU2[rr * (R + 1) + c], sG2[t * (R + 1) + c], dx);
+    group_sync(grp);
+    Acc acc;
+    acc.zero();
+    outer_product(acc, sU, sGt, 2 * R, kLd, ry, cx);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int rr = i0 + 8 * ry + i;
+        T* dst = dX + sl.row(bh, rr);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c = 32 * h + 4 * cx;
+            float4 v = make_float4(acc.at(i, 4 * h), acc.at(i, 4 * h + 1), acc.at(i, 4 * h + 2), acc.at(i, 4 * h + 3));
+            if (add != nullptr) {
+                const float4 a = *reinterpret_cast<const float4*>(add + ((size_t)bh * n + rr) * 64 + c);
+                v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
             }
-            stf(dX + sl.row(bh, i0 + rr) + t, dx);
+            st4(dst + c, v);
         }
     }
 }
@@ -752,114 +463,186 @@ cudaError_t allow_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// Half sketches of one tensor, or (X1 != nullptr) of two tensors of the same layout.
 template <typename T, int R>
-cudaError_t launch_sketch(const Dims& d, const T* X, const T* G1, const T* G2, float* M, float* Phi,
+cudaError_t launch_sketch(const Dims& d, const T* X0, const T* X1, const T* G1, const T* G2, float* M0, float* M1, float* Phi,
                           cudaStream_t s, int* launches) {
-    if (d.learned) return learned_sketch(d, X, M, Phi, s, launches);      // Algorithm 2: two dense networks
-    if (d.p == 2) {           // M = X (R = 64 = h)
-        const int rows = d.BH() * d.n;
-        prof_begin("identity_sketch_kernel", s);
-        identity_sketch_kernel<T><<<(rows + 7) / 8, 256, 0, s>>>(Slice{d.H, d.sb, d.sh, d.sn}, d.n, rows, X, M, Phi);
-        prof_end(s);
-        ++*launches;
-        return cudaGetLastError();
-    }
-    if (d.p == 8) {           // one more recursion level: packed Gaussians [Ga; Gb; Gc]
-        PSK_TRY((allow_smem(sketch8_kernel<T, R>, Sk8<R>::bytes)));
-        prof_begin("sketch8_kernel", s);
-        sketch8_kernel<T, R><<<dim3(d.n / Sk8<R>::kRows, d.BH()), 256, Sk8<R>::bytes, s>>>(
-            Slice{d.H, d.sb, d.sh, d.sn}, X, G1, G2, d.g_heads, d.n, M, Phi);
-        prof_end(s);
-        ++*launches;
-        return cudaGetLastError();
-    }
-    const size_t smem = (size_t)(2 * H64 * R + 64 * 65 + 64 * (R + 1)) * sizeof(float);
-    PSK_TRY(allow_smem(sketch_kernel<T, R>, smem));
     Slice sl{d.H, d.sb, d.sh, d.sn};
-    prof_begin("sketch_kernel", s);
-    sketch_kernel<T, R><<<dim3(d.n / 64, d.BH()), 256, smem, s>>>(sl, X, G1, G2, d.g_heads, d.n, M, Phi);
+    if (!d.learned && d.p == 4) {
+        PSK_TRY((allow_smem(sketch_kernel<T, R>, kSketchSmem<R>)));
+        prof_begin("sketch_kernel", s);
+        sketch_kernel<T, R><<<dim3(d.n / 128, d.BH(), X1 != nullptr ? 2 : 1), 128, kSketchSmem<R>, s>>>(
+            sl, X0, X1, G1, G2, d.g_heads, d.n, M0, M1, Phi);
+        prof_end(s);
+        ++*launches;
+        return cudaGetLastError();
+    }
+    for (int i = 0; i < (X1 != nullptr ? 2 : 1); ++i) {
+        const T* X = i ? X1 : X0;
+        float* M = i ? M1 : M0;
+        if (d.learned) {          // Algorithm 2: two dense networks
+            PSK_TRY(learned_sketch(d, X, M, Phi, s, launches));
+            continue;
+        }
+        if (d.p == 2) {           // M = X (R = 64 = h)
+            const int rows = d.BH() * d.n;
+            prof_begin("identity_sketch_kernel", s);
+            identity_sketch_kernel<T><<<(rows + 7) / 8, 256, 0, s>>>(sl, d.n, rows, X, M, Phi);
+        } else {                  // p = 8, one more recursion level: packed Gaussians [Ga; Gb; Gc]
+            PSK_TRY((allow_smem(sketch8_kernel<T, R>, Sk8<R>::bytes)));
+            prof_begin("sketch8_kernel", s);
+            sketch8_kernel<T, R><<<dim3(d.n / Sk8<R>::kRows, d.BH()), 256, Sk8<R>::bytes, s>>>(sl, X, G1, G2, d.g_heads, d.n, M, Phi);
+        }
+        prof_end(s);
+        ++*launches;
+        PSK_TRY(cudaGetLastError());
+    }
+    return cudaSuccess;
+}
+
+// Prefix (suffix) states of every block: block states, then the scan over them.
+template <int R>
+cudaError_t launch_states(const Dims& d, const float* M, const cc::YRows& y, float* S, bool reverse,
+                          cudaStream_t s, int* launches) {
+    if (d.t == 1) return cudaSuccess;
+    constexpr int G = cc::kStateGroups<R>, NC = cc::kChunks<R>;
+    PSK_TRY((allow_smem(cc::cc_state_kernel<R>, cc::kStateSmem<R>)));
+    prof_begin("state_kernel", s);
+    cc::cc_state_kernel<R><<<dim3((NC + G - 1) / G, d.t - 1, d.BH()), 64 * G, cc::kStateSmem<R>, s>>>(M, y, d.n, d.b, d.t, reverse ? 1 : 0, S);
+    prof_end(s);
+    ++*launches;
+    PSK_TRY(cudaGetLastError());
+    if (d.t == 2) return cudaSuccess;            // the only state there is needs no sum
+    const size_t elems = (size_t)NC * cc::kChunkFloats / 4;
+    prof_begin("scan_kernel", s);
+    cc::cc_scan_kernel<<<dim3((unsigned)((elems + 255) / 256), d.BH()), 256, 0, s>>>(reinterpret_cast<float4*>(S), elems, d.t, reverse ? 1 : 0);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
 }
 
-template <int R>
-cudaError_t launch_states(const Dims& d, const float* M, const float* Y, float* S, bool reverse,
-                          cudaStream_t s, int* launches) {
-    prof_begin("state_kernel", s);
-    state_kernel<R><<<dim3((R * R + 127) / 128, d.t, d.BH()), 128, 0, s>>>(M, Y, d.n, d.b, d.t, S);
-    prof_end(s);
-    ++*launches;
-    PSK_TRY(cudaGetLastError());
-    const size_t elems = (size_t)R * R * YC;
-    prof_begin("scan_kernel", s);
-    scan_kernel<<<dim3((unsigned)((elems + 255) / 256), d.BH()), 256, 0, s>>>(S, elems, d.t, reverse ? 1 : 0);
+template <typename T, int R>
+cudaError_t launch_rows(const Dims& d, const float* Mown, const float* Moth, const cc::YRows& y, const float* S, const T* Xown,
+                        const T* Xoth, bool dv, T* Out, float* denom, cudaStream_t s, int* launches) {
+    const dim3 grid(d.b / 64, d.t, d.BH());
+    Slice sl{d.H, d.sb, d.sh, d.sn};
+    prof_begin(dv ? "bwd_v_kernel" : "fwd_out_kernel", s);
+    if (d.local) {
+        using L = cc::RowsSmem<R, true>;
+        PSK_TRY((allow_smem(cc::cc_rows_kernel<T, R, true>, L::bytes)));
+        cc::cc_rows_kernel<T, R, true><<<grid, 64 * L::NG, L::bytes, s>>>(sl, d.n, d.b, d.t, Mown, Moth, y, S, Xown, Xoth, dv ? 1 : 0, Out, denom);
+    } else {
+        using L = cc::RowsSmem<R, false>;
+        PSK_TRY((allow_smem(cc::cc_rows_kernel<T, R, false>, L::bytes)));
+        cc::cc_rows_kernel<T, R, false><<<grid, 64 * L::NG, L::bytes, s>>>(sl, d.n, d.b, d.t, Mown, Moth, y, S, Xown, Xoth, dv ? 1 : 0, Out, denom);
+    }
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
+}
+
+template <typename T, int R>
+cudaError_t launch_dphi(const Dims& d, const float* Mown, const float* Moth, const cc::YRows& yown, const cc::YRows& yoth, const float* S,
+                        const T* Xown, const T* Xoth, bool kside, float* dM, float* dXl, cudaStream_t s, int* launches) {
+    const dim3 grid(d.b / 64, d.t, d.BH());
+    Slice sl{d.H, d.sb, d.sh, d.sn};
+    prof_begin(kside ? "bwd_k_kernel" : "bwd_q_kernel", s);
+    if (d.local) {
+        using L = cc::DphiSmem<R, true>;
+        PSK_TRY((allow_smem(cc::cc_dphi_kernel<T, R, true>, L::bytes)));
+        cc::cc_dphi_kernel<T, R, true><<<grid, 64 * L::NG, L::bytes, s>>>(sl, d.n, d.b, d.t, Mown, Moth, yown, yoth, S, Xown, Xoth, kside ? 1 : 0, dM, dXl);
+    } else {
+        using L = cc::DphiSmem<R, false>;
+        PSK_TRY((allow_smem(cc::cc_dphi_kernel<T, R, false>, L::bytes)));
+        cc::cc_dphi_kernel<T, R, false><<<grid, 64 * L::NG, L::bytes, s>>>(sl, d.n, d.b, d.t, Mown, Moth, yown, yoth, S, Xown, Xoth, kside ? 1 : 0, dM, dXl);
+    }
+    prof_end(s);
+    ++*launches;
+    return cudaGetLastError();
+}
+
+// [V | 1] rows: the caller's fp32 values as they are, or (bf16 storage) an fp32 copy in scratch.
+template <typename T>
+cudaError_t value_rows(const Dims& d, const T* V, float* Vt, cc::YRows* y, cudaStream_t s, int* launches) {
+    Slice sl{d.H, d.sb, d.sh, d.sn};
+    if constexpr (sizeof(T) == 4) {
+        *y = cc::YRows{V, sl, 1};
+        return cudaSuccess;
+    } else {
+        const int rows = d.BH() * d.n;
+        prof_begin("rows_prep_kernel", s);
+        rows_prep_kernel<T><<<(rows + 15) / 16, 256, 0, s>>>(sl, d.n, rows, 0, V, nullptr, nullptr, nullptr, Vt);
+        prof_end(s);
+        ++*launches;
+        *y = cc::YRows{Vt, Slice{d.H, (int64_t)d.H * d.n * 64, (int64_t)d.n * 64, 64}, 1};
+        return cudaGetLastError();
+    }
+}
+
+// Half sketches, value rows and prefix states: what the forward needs, and the backward again
+// unless the forward left them in this workspace.
+template <typename T, int R>
+cudaError_t prefix_states(const Dims& d, const T* Q, const T* K, const T* V, const T* G1, const T* G2, char* ws,
+                          const CcWorkspace& w, bool kept, cc::YRows* y, cudaStream_t s, int* launches) {
+    float* Mq = (float*)(ws + w.Mq); float* Mk = (float*)(ws + w.Mk);
+    if (kept) {
+        *y = sizeof(T) == 4 ? cc::YRows{(const float*)V, Slice{d.H, d.sb, d.sh, d.sn}, 1}
+                            : cc::YRows{(const float*)(ws + w.Vt), Slice{d.H, (int64_t)d.H * d.n * 64, (int64_t)d.n * 64, 64}, 1};
+        return cudaSuccess;
+    }
+    PSK_TRY((launch_sketch<T, R>(d, Q, K, G1, G2, Mq, Mk, nullptr, s, launches)));
+    PSK_TRY(value_rows<T>(d, V, (float*)(ws + w.Vt), y, s, launches));
+    return launch_states<R>(d, Mk, *y, (float*)(ws + w.Zst), false, s, launches);
 }
 
 template <typename T, int R>
 cudaError_t fwd_impl(const Dims& d, const T* Q, const T* K, const T* V, const T* G1, const T* G2,
                      T* O, float* denom, char* ws, cudaStream_t s, int* launches) {
     const CcWorkspace w = cc_workspace(d, false);
-    float* Mq = (float*)(ws + w.Mq); float* Mk = (float*)(ws + w.Mk);
-    float* Vt = (float*)(ws + w.Vt); float* Z = (float*)(ws + w.Zst);
-    Slice sl{d.H, d.sb, d.sh, d.sn};
-    const int rows = d.BH() * d.n;
-    PSK_TRY((launch_sketch<T, R>(d, Q, G1, G2, Mq, nullptr, s, launches)));
-    PSK_TRY((launch_sketch<T, R>(d, K, G1, G2, Mk, nullptr, s, launches)));
-    prof_begin("rows_prep_kernel", s);
-    rows_prep_kernel<T><<<(rows + 7) / 8, 256, 0, s>>>(sl, d.n, rows, 0, V, nullptr, nullptr, nullptr, Vt);
-    prof_end(s);
-    ++*launches;
-    PSK_TRY(cudaGetLastError());
-    PSK_TRY((launch_states<R>(d, Mk, Vt, Z, false, s, launches)));
-    prof_begin("fwd_out_kernel", s);
-    if (d.local) {
-        PSK_TRY((allow_smem(fwd_out_kernel<T, R, true>, RowSmem<R>::bytes_local)));
-        fwd_out_kernel<T, R, true><<<dim3(d.b / 128, d.t, d.BH()), 128, RowSmem<R>::bytes_local, s>>>(
-            sl, d.n, d.b, d.t, Mq, Mk, Vt, Z, Q, K, O, denom);
-    } else {
-        PSK_TRY((allow_smem(fwd_out_kernel<T, R, false>, RowSmem<R>::bytes)));
-        fwd_out_kernel<T, R, false><<<dim3(d.b / 128, d.t, d.BH()), 128, RowSmem<R>::bytes, s>>>(
-            sl, d.n, d.b, d.t, Mq, Mk, Vt, Z, Q, K, O, denom);
-    }
-    prof_end(s);
-    ++*launches;
-    return cudaGetLastError();
+    cc::YRows y;
+    PSK_TRY((prefix_states<T, R>(d, Q, K, V, G1, G2, ws, w, false, &y, s, launches)));
+    return launch_rows<T, R>(d, (float*)(ws + w.Mq), (float*)(ws + w.Mk), y, (float*)(ws + w.Zst), Q, K, false, O, denom, s, launches);
 }
 
-// Chain rule through the half sketch of one tensor: dX from dM (+ `add`, the part of the gradient
-// that reached X directly through exact same-block weights).
+// Chain rule through the half sketches of Q and K: dX from dM (+ `add`, the part of the gradient
+// that reached X directly through exact same-block weights).  X1 may be null.
 template <typename T, int R>
-cudaError_t launch_sketch_bwd(const Dims& d, const T* X, const T* G1, const T* G2, const float* dM, const float* add,
-                              T* dX, cudaStream_t s, int* launches) {
+cudaError_t launch_sketch_bwd(const Dims& d, const T* X0, const T* X1, const T* G1, const T* G2, const float* dM0, const float* dM1,
+                              const float* add0, const float* add1, T* dX0, T* dX1, cudaStream_t s, int* launches) {
     Slice sl{d.H, d.sb, d.sh, d.sn};
     const int rows = d.BH() * d.n;
-    if (d.learned) return learned_sketch_bwd(d, X, dM, add, dX, s, launches);     // two networks; gradients add up
-    if (d.p == 2) {           // dX = dM (+ add)
-        prof_begin("identity_sketch_bwd_kernel", s);
-        identity_sketch_bwd_kernel<T><<<(rows + 7) / 8, 256, 0, s>>>(sl, d.n, rows, dM, add, dX);
+    if (!d.learned && d.p == 4) {
+        using L = SkBwdSmem<R>;
+        PSK_TRY((allow_smem(sketch_bwd_kernel<T, R>, L::bytes)));
+        prof_begin("sketch_bwd_kernel", s);
+        sketch_bwd_kernel<T, R><<<dim3(d.n / 128, d.BH(), X1 != nullptr ? 2 : 1), 128, L::bytes, s>>>(
+            sl, X0, X1, G1, G2, d.g_heads, d.n, dM0, dM1, add0, add1, dX0, dX1);
         prof_end(s);
         ++*launches;
         return cudaGetLastError();
     }
-    if (d.p == 8) {
-        PSK_TRY((allow_smem(sketch8_bwd_kernel<T, R>, Sk8<R>::bytes)));
-        prof_begin("sketch8_bwd_kernel", s);
-        sketch8_bwd_kernel<T, R><<<dim3(d.n / Sk8<R>::kRows, d.BH()), 256, Sk8<R>::bytes, s>>>(sl, X, G1, G2, d.g_heads, d.n, dM, dX);
+    for (int i = 0; i < (X1 != nullptr ? 2 : 1); ++i) {
+        const T* X = i ? X1 : X0;
+        const float* dM = i ? dM1 : dM0;
+        const float* add = i ? add1 : add0;
+        T* dX = i ? dX1 : dX0;
+        if (d.learned) {          // two networks; gradients add up
+            PSK_TRY(learned_sketch_bwd(d, X, dM, add, dX, s, launches));
+            continue;
+        }
+        if (d.p == 2) {           // dX = dM (+ add)
+            prof_begin("identity_sketch_bwd_kernel", s);
+            identity_sketch_bwd_kernel<T><<<(rows + 7) / 8, 256, 0, s>>>(sl, d.n, rows, dM, add, dX);
+        } else {
+            PSK_TRY((allow_smem(sketch8_bwd_kernel<T, R>, Sk8<R>::bytes)));
+            prof_begin("sketch8_bwd_kernel", s);
+            sketch8_bwd_kernel<T, R><<<dim3(d.n / Sk8<R>::kRows, d.BH()), 256, Sk8<R>::bytes, s>>>(sl, X, G1, G2, d.g_heads, d.n, dM, dX);
+        }
         prof_end(s);
         ++*launches;
-        return cudaGetLastError();
+        PSK_TRY(cudaGetLastError());
     }
-    const size_t smem = (size_t)(2 * H64 * (R + 1) + 64 * 65 + 2 * 64 * (R + 1)) * sizeof(float);
-    PSK_TRY(allow_smem(sketch_bwd_kernel<T, R>, smem));
-    prof_begin("sketch_bwd_kernel", s);
-    sketch_bwd_kernel<T, R><<<dim3(d.n / 64, d.BH()), 256, smem, s>>>(sl, X, G1, G2, d.g_heads, d.n, dM, add, dX);
-    prof_end(s);
-    ++*launches;
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 template <typename T, int R>
@@ -868,49 +651,25 @@ cudaError_t bwd_impl(const Dims& d, const T* Q, const T* K, const T* V, const T*
                      char* ws, cudaStream_t s, int* launches) {
     const CcWorkspace w = cc_workspace(d, true);
     float* Mq = (float*)(ws + w.Mq); float* Mk = (float*)(ws + w.Mk);
-    float* Vt = (float*)(ws + w.Vt); float* Z = (float*)(ws + w.Zst);
+    float* Z = (float*)(ws + w.Zst);
     float* E = (float*)(ws + w.E); float* Rs = (float*)(ws + w.Rst);
     float* dMq = (float*)(ws + w.dMq); float* dMk = (float*)(ws + w.dMk);
-    Slice sl{d.H, d.sb, d.sh, d.sn};
-    const int rows = d.BH() * d.n;
-    PSK_TRY((launch_sketch<T, R>(d, Q, G1, G2, Mq, nullptr, s, launches)));
-    PSK_TRY((launch_sketch<T, R>(d, K, G1, G2, Mk, nullptr, s, launches)));
-    prof_begin("rows_prep_kernel", s);
-    rows_prep_kernel<T><<<(rows + 7) / 8, 256, 0, s>>>(sl, d.n, rows, 0, V, nullptr, nullptr, nullptr, Vt);
-    prof_end(s);
-    prof_begin("rows_prep_kernel", s);
-    rows_prep_kernel<T><<<(rows + 7) / 8, 256, 0, s>>>(sl, d.n, rows, 1, nullptr, O, denom, dO, E);
-    prof_end(s);
-    *launches += 2;
-    PSK_TRY(cudaGetLastError());
-    PSK_TRY((launch_states<R>(d, Mk, Vt, Z, false, s, launches)));
-    PSK_TRY((launch_states<R>(d, Mq, E, Rs, true, s, launches)));
-    const dim3 grid(d.b / 128, d.t, d.BH());
     float* dXq = d.local ? (float*)(ws + w.dXq) : nullptr;
     float* dXk = d.local ? (float*)(ws + w.dXk) : nullptr;
-    if (d.local) {
-        PSK_TRY((allow_smem(bwd_q_kernel<T, R, true>, RowSmem<R>::bytes_local)));
-        PSK_TRY((allow_smem(bwd_k_kernel<T, R, true>, RowSmem<R>::bytes_local)));
-        prof_begin("bwd_q_kernel", s);
-        bwd_q_kernel<T, R, true><<<grid, 128, RowSmem<R>::bytes_local, s>>>(sl, d.n, d.b, d.t, Mq, Mk, Vt, E, Z, Q, K, dMq, dXq);
-        prof_end(s);
-        prof_begin("bwd_k_kernel", s);
-        bwd_k_kernel<T, R, true><<<grid, 128, RowSmem<R>::bytes_local, s>>>(sl, d.n, d.b, d.t, Mq, Mk, Vt, E, Rs, Q, K, dMk, dXk, dV);
-        prof_end(s);
-    } else {
-        PSK_TRY((allow_smem(bwd_q_kernel<T, R, false>, RowSmem<R>::bytes)));
-        PSK_TRY((allow_smem(bwd_k_kernel<T, R, false>, RowSmem<R>::bytes)));
-        prof_begin("bwd_q_kernel", s);
-        bwd_q_kernel<T, R, false><<<grid, 128, RowSmem<R>::bytes, s>>>(sl, d.n, d.b, d.t, Mq, Mk, Vt, E, Z, Q, K, dMq, nullptr);
-        prof_end(s);
-        prof_begin("bwd_k_kernel", s);
-        bwd_k_kernel<T, R, false><<<grid, 128, RowSmem<R>::bytes, s>>>(sl, d.n, d.b, d.t, Mq, Mk, Vt, E, Rs, Q, K, dMk, nullptr, dV);
-        prof_end(s);
-    }
-    *launches += 2;
+    const int rows = d.BH() * d.n;
+    cc::YRows yv;
+    PSK_TRY((prefix_states<T, R>(d, Q, K, V, G1, G2, ws, w, d.keep_states, &yv, s, launches)));
+    prof_begin("rows_prep_kernel", s);
+    rows_prep_kernel<T><<<(rows + 15) / 16, 256, 0, s>>>(Slice{d.H, d.sb, d.sh, d.sn}, d.n, rows, 1, nullptr, O, denom, dO, E);
+    prof_end(s);
+    ++*launches;
     PSK_TRY(cudaGetLastError());
-    PSK_TRY((launch_sketch_bwd<T, R>(d, Q, G1, G2, dMq, dXq, dQ, s, launches)));
-    return launch_sketch_bwd<T, R>(d, K, G1, G2, dMk, dXk, dK, s, launches);
+    const cc::YRows ye{E, Slice{d.H, (int64_t)d.H * d.n * cc::kLd, (int64_t)d.n * cc::kLd, cc::kLd}, 0};
+    PSK_TRY((launch_dphi<T, R>(d, Mq, Mk, ye, yv, Z, Q, K, false, dMq, dXq, s, launches)));
+    PSK_TRY((launch_states<R>(d, Mq, ye, Rs, true, s, launches)));
+    PSK_TRY((launch_dphi<T, R>(d, Mk, Mq, yv, ye, Rs, K, Q, true, dMk, dXk, s, launches)));
+    PSK_TRY((launch_rows<T, R>(d, Mk, Mq, ye, Rs, K, Q, true, dV, nullptr, s, launches)));
+    return launch_sketch_bwd<T, R>(d, Q, K, G1, G2, dMq, dMk, dXq, dXk, dQ, dK, s, launches);
 }
 
 #define PSK_DISPATCH(CALL_F32, CALL_BF16)                                   \
@@ -931,14 +690,7 @@ cudaError_t bwd_impl(const Dims& d, const T* Q, const T* K, const T* V, const T*
 
 cudaError_t cc_sketch(const Dims& d, const void* X, const void* G1, const void* G2,
                       float* M_out, float* Phi_out, cudaStream_t s, int* launches) {
-#define C_ (launch_sketch<T, R>(d, (const T*)X, (const T*)G1, (const T*)G2, M_out, Phi_out, s, launches))
-    PSK_DISPATCH(C_, C_)
-#undef C_
-}
-
-cudaError_t cc_sketch_bwd(const Dims& d, const void* X, const void* G1, const void* G2, const float* dM,
-                          const float* add, void* dX, cudaStream_t s, int* launches) {
-#define C_ (launch_sketch_bwd<T, R>(d, (const T*)X, (const T*)G1, (const T*)G2, dM, add, (T*)dX, s, launches))
+#define C_ (launch_sketch<T, R>(d, (const T*)X, nullptr, (const T*)G1, (const T*)G2, M_out, nullptr, Phi_out, s, launches))
     PSK_DISPATCH(C_, C_)
 #undef C_
 }

@@ -69,9 +69,6 @@ cudaError_t learned_sketch(const Dims& d, const void* X, float* M, float* Phi, c
 cudaError_t learned_sketch_bwd(const Dims& d, const void* X, const float* dM, const float* add, void* dX,
                                cudaStream_t s, int* launches);
 
-cudaError_t cc_sketch_bwd(const Dims& d, const void* X, const void* G1, const void* G2, const float* dM,
-                          const float* add, void* dX, cudaStream_t s, int* launches);
-
 // Degree 8 and the learnable sketch on the tensor cores: half sketches by their own tensor-core
 // sketch kernels, attention on them by the tensor-core kernels in linear sketch mode (psk_given.cu).
 bool given_supported(const Dims& d);
