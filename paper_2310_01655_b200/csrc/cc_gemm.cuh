@@ -132,6 +132,31 @@ __device__ __forceinline__ void dot_half(f2 (&d)[4][8], const float* A, const fl
         }
     }
 }
+// all eight rows at once: two thirds of the shared-memory loads per product, for 128 accumulator registers
+template <int LDA, int LDB>
+__device__ __forceinline__ void dot_full(f2 (&d)[8][8], const float* A, const float* B, int K4, int ry, int cx) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) d[i][j] = 0ull;
+    const float* a0 = A + ry * LDA;
+    const float* b0 = B + cx * LDB;
+#pragma unroll 1
+    for (int k = 0; k < 4 * K4; k += 4) {
+        F22 b[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) b[j] = lds22(b0 + 8 * j * LDB + k);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const F22 a = lds22(a0 + 8 * i * LDA + k);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                d[i][j] = fma2(a.x, b[j].x, d[i][j]);
+                d[i][j] = fma2(a.y, b[j].y, d[i][j]);
+            }
+        }
+    }
+}
 __device__ __forceinline__ float sum2(f2 v) { return lo2(v) + hi2(v); }
 
 }  // namespace cc

@@ -55,14 +55,14 @@ __device__ __forceinline__ void load_y_rows(float* dst, const YRows& y, int bh, 
 // grid (ceil(chunks / G), t - 1, BH).  Bound by the FMA pipe: per token and thread 32 packed FMAs
 // beside 4 multiplies, 8 moves and 5 loads.
 // ---------------------------------------------------------------------------
-template <int R> constexpr int kStateGroups = R == 16 ? 3 : (R == 32 ? 5 : 4);
-template <int R> constexpr size_t kStateSmem = 2 * (64 * R + kUnit) * sizeof(float);
+template <int R> constexpr int kStateGroups = R == 16 ? 3 : (R == 32 ? 2 : 4);     // divides the chunk count
+template <int R> constexpr size_t kStateSmem = 2 * (64 * (R + 4) + kUnit) * sizeof(float);
 
 template <int R>
-__global__ void __launch_bounds__(64 * kStateGroups<R>)
+__global__ void __launch_bounds__(64 * kStateGroups<R>, R == 64 ? 2 : (R == 32 ? 4 : 2))
 cc_state_kernel(const float* __restrict__ M, YRows y, int n, int b, int t, int reverse, float* __restrict__ S) {
     extern __shared__ __align__(16) float smem[];
-    constexpr int G = kStateGroups<R>, NT = 64 * G, kBuf = 64 * R + kUnit;
+    constexpr int G = kStateGroups<R>, NT = 64 * G, LD = R + 4, kBuf = 64 * LD + kUnit;
     const int tid = threadIdx.x, grp = tid / 64, lane = tid % 64, ry = lane / 8, cx = lane % 8;
     const int l = blockIdx.y + (reverse ? 1 : 0), bh = blockIdx.z;
     const int chunk = blockIdx.x * G + grp;
@@ -72,13 +72,13 @@ cc_state_kernel(const float* __restrict__ M, YRows y, int n, int b, int t, int r
     auto load = [&](int k) {
         float* dst = smem + (k & 1) * kBuf;
         const float* src = M + ((size_t)bh * n + (size_t)l * b + k * 64) * R;
-        for (int e = tid; e < 64 * R / 4; e += NT) cp16(dst + 4 * e, src + 4 * e);
-        load_y_rows(dst + 64 * R, y, bh, l * b + k * 64, tid, NT);
+        for (int e = tid; e < 64 * R / 4; e += NT) cp16(dst + (e / (R / 4)) * LD + 4 * (e % (R / 4)), src + 4 * e);
+        load_y_rows(dst + 64 * LD, y, bh, l * b + k * 64, tid, NT);
         cp_commit();
     };
     load(0);
     if (y.ones)
-        for (int e = tid; e < 128; e += NT) smem[(e / 64) * kBuf + 64 * R + (e % 64) * kLd + 64] = 1.f;
+        for (int e = tid; e < 128; e += NT) smem[(e / 64) * kBuf + 64 * LD + (e % 64) * kLd + 64] = 1.f;
     Acc acc;
     acc.zero();
     f2 ext[4] = {0ull, 0ull, 0ull, 0ull};
@@ -88,15 +88,15 @@ cc_state_kernel(const float* __restrict__ M, YRows y, int n, int b, int t, int r
         __syncthreads();
         if (live) {
             const float* sM = smem + (k & 1) * kBuf;
-            const float* sY = sM + 64 * R;
+            const float* sY = sM + 64 * LD;
             const float* pa = sM + 8 * ab + ry;
             const float* pb = sM + 8 * bb;
 #pragma unroll 4
             for (int j = 0; j < 64; ++j) {
-                const float ma = pa[j * R];
+                const float ma = pa[j * LD];
                 const f2 ma2 = pack2(ma, ma);
                 f2 phi[4];
-                load_rows8(phi, pb + j * R);
+                load_rows8(phi, pb + j * LD);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) phi[i] = mul2(phi[i], ma2);
                 acc.step(phi, lds22(sY + j * kLd + 4 * cx), lds22(sY + j * kLd + 32 + 4 * cx));
@@ -104,10 +104,10 @@ cc_state_kernel(const float* __restrict__ M, YRows y, int n, int b, int t, int r
             // the last column: the eight threads of a feature share the tokens
 #pragma unroll 2
             for (int j = cx; j < 64; j += 8) {
-                const float my = pa[j * R] * sY[j * kLd + 64];
+                const float my = pa[j * LD] * sY[j * kLd + 64];
                 const f2 my2 = pack2(my, my);
                 f2 mb[4];
-                load_rows8(mb, pb + j * R);
+                load_rows8(mb, pb + j * LD);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) ext[i] = fma2(mb[i], my2, ext[i]);
             }
@@ -156,6 +156,7 @@ cc_scan_kernel(float4* __restrict__ S, size_t elems, int t, int reverse) {
 // rows [64][C] of fp32 scratch -> shared memory transposed, dst[c][kLd] (row index contiguous)
 template <int C>
 __device__ __forceinline__ void load_transposed(float* dst, const float* src, int tid, int nthr) {
+#pragma unroll 8
     for (int e = tid; e < 64 * C / 4; e += nthr) {
         const int rr = e % 64, c = (e / 64) * 4;
         const float4 v = *reinterpret_cast<const float4*>(src + (size_t)rr * C + c);
@@ -177,6 +178,7 @@ __device__ __forceinline__ void st4(__nv_bfloat16* p, float4 v) {
 // 64 raw rows of a caller's tensor, as they are (dst[row][kLd]) or transposed (dst[c][kLd])
 template <typename T, bool TRANSPOSE>
 __device__ __forceinline__ void load_raw(float* dst, const T* X, const Slice& sl, int bh, int i0, int tid, int nthr) {
+#pragma unroll 8
     for (int e = tid; e < 64 * 16; e += nthr) {
         const int rr = TRANSPOSE ? e % 64 : e / 16, c = 4 * (TRANSPOSE ? e / 64 : e % 16);
         const float4 v = ld4(X + sl.row(bh, i0 + rr) + c);
@@ -199,7 +201,7 @@ __device__ __forceinline__ void load_raw(float* dst, const T* X, const Slice& sl
 // added at the end: even one head's few rows keep every SM's warps busy.
 // grid (b / 64, t, BH).  Bound by the FMA pipe (72 of its clocks per 64 FMAs of a warp's thread).
 // ---------------------------------------------------------------------------
-template <int R, bool LOCAL>
+template <int R, bool LOCAL, int NG>
 struct RowsSmem {
     static constexpr int own = R * kLd + (LOCAL ? kUnit : 0);
     // other side's half sketches (or raw rows), its Y tile, the weights; the two chunk buffers alias
@@ -207,19 +209,18 @@ struct RowsSmem {
     static constexpr bool kAlias = LOCAL || R == 64;
     static constexpr int oth = kAlias ? kUnit : R * kLd;
     static constexpr int grp = kAlias ? 2 * kUnit : oth + 2 * kUnit;
-    static constexpr int NG = 4;
     static constexpr size_t bytes = (size_t)(own + NG * grp) * sizeof(float);
     static_assert(bytes <= 232448, "shared memory");
 };
 
-template <typename T, int R, bool LOCAL>
-__global__ void __launch_bounds__(64 * RowsSmem<R, LOCAL>::NG)
+template <typename T, int R, bool LOCAL, int NG>
+__global__ void __launch_bounds__(64 * NG)
 cc_rows_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mown, const float* __restrict__ Moth, YRows y,
                const float* __restrict__ S, const T* __restrict__ Xown, const T* __restrict__ Xoth, int dv,
                T* __restrict__ Out, float* __restrict__ denom) {
     extern __shared__ __align__(16) float smem[];
-    using L = RowsSmem<R, LOCAL>;
-    constexpr int NG = L::NG, NT = 64 * NG, NC = kChunks<R>;
+    using L = RowsSmem<R, LOCAL, NG>;
+    constexpr int NT = 64 * NG, NC = kChunks<R>;
     const int tid = threadIdx.x, grp = tid / 64, lane = tid % 64, ry = lane / 8, cx = lane % 8;
     const int tile = blockIdx.x, l = blockIdx.y, bh = blockIdx.z;
     float* sMt = smem;
@@ -369,7 +370,7 @@ cc_rows_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mown, co
 // Work items and groups as in cc_rows_kernel; the products are in dot form, because both the
 // states' rows and Y's rows are contiguous along the 65 columns that are summed over.
 // ---------------------------------------------------------------------------
-template <int R, bool LOCAL>
+template <int R, bool LOCAL, int NG>
 struct DphiSmem {
     static constexpr int ldm = R + 4;
     static constexpr int own_m = 0, own_y = 64 * ldm, own_x = own_y + kUnit;
@@ -377,19 +378,18 @@ struct DphiSmem {
     // per group: two chunk buffers = the other side's half sketches (raw rows) and Y tile / ds;
     // then the gradient accumulator
     static constexpr int dm = 2 * kUnit, grp = dm + 64 * ldm;
-    static constexpr int NG = R == 64 ? 3 : 4;
     static constexpr size_t bytes = (size_t)(own + NG * grp) * sizeof(float);
     static_assert(bytes <= 232448, "shared memory");
 };
 
-template <typename T, int R, bool LOCAL>
-__global__ void __launch_bounds__(64 * DphiSmem<R, LOCAL>::NG)
+template <typename T, int R, bool LOCAL, int NG>
+__global__ void __launch_bounds__(64 * NG)
 cc_dphi_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mown, const float* __restrict__ Moth, YRows yown,
                YRows yoth, const float* __restrict__ S, const T* __restrict__ Xown, const T* __restrict__ Xoth, int kside,
                float* __restrict__ dM, float* __restrict__ dXl) {
     extern __shared__ __align__(16) float smem[];
-    using L = DphiSmem<R, LOCAL>;
-    constexpr int NG = L::NG, NT = 64 * NG, NC = kChunks<R>, LDM = L::ldm;
+    using L = DphiSmem<R, LOCAL, NG>;
+    constexpr int NT = 64 * NG, NC = kChunks<R>, LDM = L::ldm;
     constexpr int LDS_ = LOCAL ? kLd : LDM;             // leading dimension of the rows a score is made of
     constexpr int NCOL = LOCAL ? 8 : R / 8;             // columns of the same-block gradient per thread
     const int tid = threadIdx.x, grp = tid / 64, lane = tid % 64, ry = lane / 8, cx = lane % 8;
@@ -429,16 +429,15 @@ cc_dphi_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mown, co
             int ab, bb;
             chunk_pair<R>(item, ab, bb);
             const float* z = sG + buf * kUnit;
-#pragma unroll 1
-            for (int half = 0; half < 2; ++half) {
-                f2 d[4][8];
-                dot_half<kLd, kLd>(d, sYo, z, 16, half, ry, cx);
+            {
+                f2 d[8][8];
+                dot_full<kLd, kLd>(d, sYo, z, 16, ry, cx);
                 float zl[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) zl[j] = z[(cx + 8 * j) * kLd + 64];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int rr = ry + 32 * half + 8 * i;
+                for (int i = 0; i < 8; ++i) {
+                    const int rr = ry + 8 * i;
                     const float yl = sYo[rr * kLd + 64];
                     const float* mr = sM + rr * LDM;
                     const float ma = mr[8 * ab + cx];

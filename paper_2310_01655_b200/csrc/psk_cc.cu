@@ -47,57 +47,70 @@ using cc::Slice;
 
 // ---------------------------------------------------------------------------
 // Half sketch m(x) = (x G1)*(x G2)/sqrt(r)  (Algorithm 1, degree-2 level): 64 rows per 64-thread
-// group, two groups per CTA, one or two tensors (Q and K) per launch.  A thread holds eight rows of
-// the same few columns of x G1 and of x G2 (16 columns in two passes for r = 64), so their product is
-// formed in registers.
+// group, two groups per CTA, one or two tensors (Q and K) per launch.  Dot form (cc_gemm.cuh): the rows
+// lie in shared memory as they are in memory, only [G1 | G2] is transposed, once per CTA, which then
+// walks several row tiles (the next one in flight).  A thread holds eight rows of the same columns of
+// x G1 and of x G2 (two passes of 32 + 32 columns for r = 64), so their product is formed in registers.
 // ---------------------------------------------------------------------------
 template <int R> struct SkTile {
-    static constexpr int kPasses = R == 64 ? 2 : 1, kCols = R / 8 / kPasses, NP = kCols / 2;
+    static constexpr int kPasses = R == 64 ? 2 : 1, kCols = R / 8 / kPasses;       // columns per thread, matrix and pass
+    static constexpr int Gt = 2 * R * cc::kLd;                                     // [2R][kLd]: rows of G1^T, then of G2^T
+    static constexpr size_t bytes = (size_t)(Gt + 4 * cc::kUnit) * sizeof(float);  // two row buffers per group
 };
 
-// a1, a2: rows 8 ry + i, columns base + kCols cx + j of X G1 and X G2 (Xt [64][kLd], G [64][R])
+template <typename T, int R>
+__device__ __forceinline__ void load_g_transposed(float* sGt, const T* G1, const T* G2, int g, int tid, int nthr) {
+#pragma unroll 4
+    for (int e = tid; e < 2 * 64 * (R / 4); e += nthr) {
+        const int k = e % 64, c = 4 * ((e / 64) % (R / 4)), m = e / (64 * (R / 4));
+        const float4 v = cc::ld4((m ? G2 : G1) + (size_t)g * H64 * R + k * R + c);
+        float* t = sGt + (m * R + c) * cc::kLd + k;
+        t[0] = v.x; t[cc::kLd] = v.y; t[2 * cc::kLd] = v.z; t[3 * cc::kLd] = v.w;
+    }
+}
+// 64 rows of a caller's tensor: asynchronous copies for fp32, converted for bf16
+template <typename T>
+__device__ __forceinline__ void load_x_rows(float* dst, const T* X, const Slice& sl, int bh, int i0, int lane) {
+    if constexpr (sizeof(T) == 4) {
+        for (int e = lane; e < 64 * 16; e += 64) cc::cp16(dst + (e / 16) * cc::kLd + 4 * (e % 16), X + sl.row(bh, i0 + e / 16) + 4 * (e % 16));
+    } else {
+        cc::load_raw<T, false>(dst, X, sl, bh, i0, lane, 64);
+    }
+    cc::cp_commit();
+}
+// a1, a2: rows ry + 8 i, columns base + cx + 8 j of X G1 and X G2
 template <int R>
 __device__ __forceinline__ void sketch_products(float (&a1)[8][SkTile<R>::kCols], float (&a2)[8][SkTile<R>::kCols],
-                                                const float* Xt, const float* G1, const float* G2, int base, int ry, int cx) {
+                                                const float* X, const float* Gt, int base, int ry, int cx) {
     using namespace cc;
-    constexpr int NP = SkTile<R>::NP, KC = SkTile<R>::kCols;
-    f2 s[2][4][NP], x[2][4][NP];
+    constexpr int KC = SkTile<R>::kCols;
+    f2 d[8][2 * KC];
 #pragma unroll
-    for (int m = 0; m < 2; ++m)
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int p = 0; p < 4; ++p)
+        for (int j = 0; j < 2 * KC; ++j) d[i][j] = 0ull;
+    const float* x0 = X + ry * kLd;
+    const float* g0 = Gt + (base + cx) * kLd;
+#pragma unroll 1
+    for (int k = 0; k < 64; k += 4) {
+        F22 b[2 * KC];
 #pragma unroll
-            for (int q = 0; q < NP; ++q) s[m][p][q] = x[m][p][q] = 0ull;
-#pragma unroll 4
-    for (int k = 0; k < 64; ++k) {
-        f2 a[4];
-        load_rows8(a, Xt + k * kLd + 8 * ry);
+        for (int j = 0; j < 2 * KC; ++j) b[j] = lds22(g0 + ((j / KC) * R + 8 * (j % KC)) * kLd + k);
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
-            const float* g = (m ? G2 : G1) + k * R + base + KC * cx;
-            f2 c[NP];
-            if constexpr (NP == 1) c[0] = *reinterpret_cast<const f2*>(g);
-            else { const F22 u = lds22(g); c[0] = u.x; c[1] = u.y; }
+        for (int i = 0; i < 8; ++i) {
+            const F22 a = lds22(x0 + 8 * i * kLd + k);
 #pragma unroll
-            for (int q = 0; q < NP; ++q) {
-                const f2 sw = swap2(c[q]);
-#pragma unroll
-                for (int p = 0; p < 4; ++p) { s[m][p][q] = fma2(a[p], c[q], s[m][p][q]); x[m][p][q] = fma2(a[p], sw, x[m][p][q]); }
+            for (int j = 0; j < 2 * KC; ++j) {
+                d[i][j] = fma2(a.x, b[j].x, d[i][j]);
+                d[i][j] = fma2(a.y, b[j].y, d[i][j]);
             }
         }
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < KC; ++j) {
-            const f2 v1 = ((i ^ j) & 1) ? x[0][i / 2][j / 2] : s[0][i / 2][j / 2];
-            const f2 v2 = ((i ^ j) & 1) ? x[1][i / 2][j / 2] : s[1][i / 2][j / 2];
-            a1[i][j] = (i & 1) ? hi2(v1) : lo2(v1);
-            a2[i][j] = (i & 1) ? hi2(v2) : lo2(v2);
-        }
+        for (int j = 0; j < KC; ++j) { a1[i][j] = sum2(d[i][j]); a2[i][j] = sum2(d[i][KC + j]); }
 }
-
-template <int R> constexpr size_t kSketchSmem = (2 * H64 * R + 2 * cc::kUnit) * sizeof(float);
 
 template <typename T, int R>
 __global__ void __launch_bounds__(128)
@@ -106,41 +119,39 @@ sketch_kernel(Slice sl, const T* __restrict__ X0, const T* __restrict__ X1, cons
     extern __shared__ __align__(16) float smem[];
     using namespace cc;
     constexpr int KC = SkTile<R>::kCols;
-    float* sG1 = smem;                  // [64][R]
-    float* sG2 = sG1 + H64 * R;         // [64][R]
     const int tid = threadIdx.x, grp = tid / 64, lane = tid % 64, ry = lane / 8, cx = lane % 8;
-    float* sXt = sG2 + H64 * R + grp * kUnit;
-    const int bh = blockIdx.y, i0 = blockIdx.x * 128 + grp * 64;
+    float* sX = smem + SkTile<R>::Gt + grp * 2 * kUnit;
+    const int bh = blockIdx.y, nt = n / 128;
     const T* X = blockIdx.z ? X1 : X0;
-    float* M = (blockIdx.z ? M1 : M0) + ((size_t)bh * n + i0) * R;
-    const int g = (g_heads == 1) ? 0 : (bh % sl.H);
-    for (int e = tid; e < H64 * R / 4; e += 128) {
-        *reinterpret_cast<float4*>(sG1 + 4 * e) = ld4(G1 + (size_t)g * H64 * R + 4 * e);
-        *reinterpret_cast<float4*>(sG2 + 4 * e) = ld4(G2 + (size_t)g * H64 * R + 4 * e);
-    }
-    load_raw<T, true>(sXt, X, sl, bh, i0, lane, 64);
+    float* Mbh = (blockIdx.z ? M1 : M0) + (size_t)bh * n * R;
+    load_x_rows<T>(sX, X, sl, bh, blockIdx.x * 128 + grp * 64, lane);
+    load_g_transposed<T, R>(smem, G1, G2, g_heads == 1 ? 0 : bh % sl.H, tid, 128);
     __syncthreads();
     const float rs = rsqrtf((float)R);
+    int buf = 0;
+    for (int tile = blockIdx.x; tile < nt; tile += gridDim.x, buf ^= 1) {
+        if (tile + gridDim.x < nt) { load_x_rows<T>(sX + (buf ^ 1) * kUnit, X, sl, bh, (tile + gridDim.x) * 128 + grp * 64, lane); cp_wait<1>(); }
+        else cp_wait<0>();
+        group_sync(grp);
+        float* M = Mbh + (size_t)(tile * 128 + grp * 64) * R;
 #pragma unroll 1
-    for (int base = 0; base < R; base += 8 * KC) {
-        float a1[8][KC], a2[8][KC];
-        sketch_products<R>(a1, a2, sXt, sG1, sG2, base, ry, cx);
+        for (int base = 0; base < R; base += 8 * KC) {
+            float a1[8][KC], a2[8][KC];
+            sketch_products<R>(a1, a2, sX + buf * kUnit, smem, base, ry, cx);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            float* dst = M + (size_t)(8 * ry + i) * R + base + KC * cx;
-            if constexpr (KC == 2) *reinterpret_cast<float2*>(dst) = make_float2(a1[i][0] * a2[i][0] * rs, a1[i][1] * a2[i][1] * rs);
-            else *reinterpret_cast<float4*>(dst) = make_float4(a1[i][0] * a2[i][0] * rs, a1[i][1] * a2[i][1] * rs,
-                                                               a1[i][2] * a2[i][2] * rs, a1[i][3] * a2[i][3] * rs);
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < KC; ++j) M[(ry + 8 * i) * R + base + cx + 8 * j] = a1[i][j] * a2[i][j] * rs;
         }
-    }
-    if (Phi_out != nullptr) {           // phi'(x)[a*R+b] = m_a m_b (Section 1.2 ordering)
-        __syncthreads();                // (this CTA's rows of M, written above, are visible to all of it)
-        float* phi = Phi_out + ((size_t)bh * n + i0) * R * R;
-        for (int e = lane; e < 64 * R * R / 4; e += 64) {
-            const int rr = e / (R * R / 4), f = 4 * (e % (R * R / 4));
-            const float ma = M[rr * R + f / R];
-            const float4 mb = *reinterpret_cast<const float4*>(M + rr * R + f % R);
-            *reinterpret_cast<float4*>(phi + (size_t)rr * R * R + f) = make_float4(ma * mb.x, ma * mb.y, ma * mb.z, ma * mb.w);
+        group_sync(grp);
+        if (Phi_out != nullptr) {           // phi'(x)[a*R+b] = m_a m_b (Section 1.2 ordering)
+            float* phi = Phi_out + ((size_t)bh * n + tile * 128 + grp * 64) * R * R;      // (the group's rows of M are written)
+            for (int e = lane; e < 64 * R * R / 4; e += 64) {
+                const int rr = e / (R * R / 4), f = 4 * (e % (R * R / 4));
+                const float ma = M[rr * R + f / R];
+                const float4 mb = *reinterpret_cast<const float4*>(M + rr * R + f % R);
+                *reinterpret_cast<float4*>(phi + (size_t)rr * R * R + f) = make_float4(ma * mb.x, ma * mb.y, ma * mb.z, ma * mb.w);
+            }
         }
     }
 }
@@ -360,14 +371,16 @@ rows_prep_kernel(Slice sl, int n, int total_rows, int mode, const T* __restrict_
 
 // ---------------------------------------------------------------------------
 // Chain rule through the half sketch: dX = ((dM*A2) G1^T + (dM*A1) G2^T)/sqrt(r),
-// A1 = X G1, A2 = X G2 recomputed.  Groups, rows and tensors as in sketch_kernel.  `add` (optional,
-// [rows][64]): gradient that reached X without passing through the sketch, added before the
-// result is rounded.
+// A1 = X G1, A2 = X G2 recomputed.  Groups, tiles and tensors as in sketch_kernel; the second product
+// contracts over the 2r sketch columns, [G1 | G2] as it lies in memory.  `add` (optional, [rows][64]):
+// gradient that reached X without passing through the sketch, added before the result is rounded.
 // ---------------------------------------------------------------------------
 template <int R> struct SkBwdSmem {
-    static constexpr int G = 2 * H64 * R, Gt = 2 * R * cc::kLd;
-    static constexpr int U = 2 * R * cc::kLd;          // U1, U2 transposed
-    static constexpr size_t bytes = (size_t)(G + Gt + 2 * (cc::kUnit + U)) * sizeof(float);
+    static constexpr int ldu = 2 * R + 4;
+    static constexpr int Gt = 2 * R * cc::kLd, Gc = 64 * ldu;       // [G1 | G2]^T, and [64][G1 | G2]
+    // per group: the rows, and U = [dM*A2 | dM*A1]
+    static constexpr int X = cc::kUnit, U = 64 * ldu;
+    static constexpr size_t bytes = (size_t)(Gt + Gc + 2 * (X + U)) * sizeof(float);
 };
 
 template <typename T, int R>
@@ -378,77 +391,60 @@ sketch_bwd_kernel(Slice sl, const T* __restrict__ X0, const T* __restrict__ X1, 
     extern __shared__ __align__(16) float smem[];
     using namespace cc;
     using L = SkBwdSmem<R>;
-    constexpr int KC = SkTile<R>::kCols;
-    float* sG1 = smem;                      // [64][R]
-    float* sG2 = sG1 + H64 * R;             // [64][R]
-    float* sGt = sG2 + H64 * R;             // [2R][kLd]: rows of G1^T, then of G2^T
+    constexpr int KC = SkTile<R>::kCols, LDU = L::ldu;
     const int tid = threadIdx.x, grp = tid / 64, lane = tid % 64, ry = lane / 8, cx = lane % 8;
-    float* sXt = sGt + L::Gt + grp * (kUnit + L::U);
-    float* sU = sXt + kUnit;                // [2R][kLd]: rows of (dM*A2)^T, then of (dM*A1)^T
-    const int bh = blockIdx.y, i0 = blockIdx.x * 128 + grp * 64;
+    float* sGc = smem + L::Gt;
+    float* sX = sGc + L::Gc + grp * (L::X + L::U);
+    float* sU = sX + L::X;
+    const int bh = blockIdx.y, nt = n / 128;
     const T* X = blockIdx.z ? X1 : X0;
-    const float* dM = (blockIdx.z ? dM1 : dM0) + ((size_t)bh * n + i0) * R;
+    const float* dM = (blockIdx.z ? dM1 : dM0) + (size_t)bh * n * R;
     const float* add = blockIdx.z ? add1 : add0;
     T* dX = blockIdx.z ? dX1 : dX0;
     const int g = (g_heads == 1) ? 0 : (bh % sl.H);
-    for (int e = tid; e < H64 * R / 4; e += 128) {
-        const int k = e / (R / 4), c = 4 * (e % (R / 4));
-        const float4 u = ld4(G1 + (size_t)g * H64 * R + 4 * e), v = ld4(G2 + (size_t)g * H64 * R + 4 * e);
-        *reinterpret_cast<float4*>(sG1 + 4 * e) = u;
-        *reinterpret_cast<float4*>(sG2 + 4 * e) = v;
-        float* t1 = sGt + c * kLd + k;
-        float* t2 = sGt + (R + c) * kLd + k;
-        t1[0] = u.x; t1[kLd] = u.y; t1[2 * kLd] = u.z; t1[3 * kLd] = u.w;
-        t2[0] = v.x; t2[kLd] = v.y; t2[2 * kLd] = v.z; t2[3 * kLd] = v.w;
+    load_x_rows<T>(sX, X, sl, bh, blockIdx.x * 128 + grp * 64, lane);
+    load_g_transposed<T, R>(smem, G1, G2, g, tid, 128);
+    for (int e = tid; e < 2 * 64 * (R / 4); e += 128) {
+        const int k = (e / (R / 4)) % 64, c = 4 * (e % (R / 4)), m = e / (64 * (R / 4));
+        *reinterpret_cast<float4*>(sGc + k * LDU + m * R + c) = ld4((m ? G2 : G1) + (size_t)g * H64 * R + k * R + c);
     }
-    load_raw<T, true>(sXt, X, sl, bh, i0, lane, 64);
     __syncthreads();
     const float rs = rsqrtf((float)R);
+    for (int tile = blockIdx.x; tile < nt; tile += gridDim.x) {
+        cp_wait<0>();
+        group_sync(grp);
+        const int i0 = tile * 128 + grp * 64;
 #pragma unroll 1
-    for (int base = 0; base < R; base += 8 * KC) {
-        float a1[8][KC], a2[8][KC];
-        sketch_products<R>(a1, a2, sXt, sG1, sG2, base, ry, cx);
+        for (int base = 0; base < R; base += 8 * KC) {
+            float a1[8][KC], a2[8][KC];
+            sketch_products<R>(a1, a2, sX, smem, base, ry, cx);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < KC; ++j) {
+                    const int c = base + cx + 8 * j;
+                    const float m = dM[(size_t)(i0 + ry + 8 * i) * R + c] * rs;
+                    sU[(ry + 8 * i) * LDU + c] = m * a2[i][j];
+                    sU[(ry + 8 * i) * LDU + R + c] = m * a1[i][j];
+                }
+        }
+        group_sync(grp);
+        // the rows have been read: the next tile's may arrive while the second product runs
+        if (tile + gridDim.x < nt) load_x_rows<T>(sX, X, sl, bh, (tile + gridDim.x) * 128 + grp * 64, lane);
+        f2 d[8][8];
+        dot_full<LDU, LDU>(d, sU, sGc, R / 2, ry, cx);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            float gm[KC];
-            const float* src = dM + (size_t)(8 * ry + i) * R + base + KC * cx;
-            if constexpr (KC == 2) { const float2 v = *reinterpret_cast<const float2*>(src); gm[0] = v.x; gm[1] = v.y; }
-            else *reinterpret_cast<float4*>(gm) = *reinterpret_cast<const float4*>(src);
+            const int rr = i0 + ry + 8 * i;
+            T* dst = dX + sl.row(bh, rr) + cx;
 #pragma unroll
-            for (int j = 0; j < KC; ++j) {
-                const float m = gm[j] * rs;
-                a2[i][j] *= m;
-                a1[i][j] *= m;
+            for (int j = 0; j < 8; ++j) {
+                float v = sum2(d[i][j]);
+                if (add != nullptr) v += add[((size_t)bh * n + rr) * 64 + cx + 8 * j];
+                stf(dst + 8 * j, v);
             }
         }
-#pragma unroll
-        for (int j = 0; j < KC; ++j) {
-            float* u1 = sU + (base + KC * cx + j) * kLd + 8 * ry;
-            float* u2 = u1 + R * kLd;
-            *reinterpret_cast<float4*>(u1) = make_float4(a2[0][j], a2[1][j], a2[2][j], a2[3][j]);
-            *reinterpret_cast<float4*>(u1 + 4) = make_float4(a2[4][j], a2[5][j], a2[6][j], a2[7][j]);
-            *reinterpret_cast<float4*>(u2) = make_float4(a1[0][j], a1[1][j], a1[2][j], a1[3][j]);
-            *reinterpret_cast<float4*>(u2 + 4) = make_float4(a1[4][j], a1[5][j], a1[6][j], a1[7][j]);
-        }
-    }
-    group_sync(grp);
-    Acc acc;
-    acc.zero();
-    outer_product(acc, sU, sGt, 2 * R, kLd, ry, cx);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int rr = i0 + 8 * ry + i;
-        T* dst = dX + sl.row(bh, rr);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int c = 32 * h + 4 * cx;
-            float4 v = make_float4(acc.at(i, 4 * h), acc.at(i, 4 * h + 1), acc.at(i, 4 * h + 2), acc.at(i, 4 * h + 3));
-            if (add != nullptr) {
-                const float4 a = *reinterpret_cast<const float4*>(add + ((size_t)bh * n + rr) * 64 + c);
-                v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
-            }
-            st4(dst + c, v);
-        }
+        group_sync(grp);
     }
 }
 
@@ -463,16 +459,25 @@ cudaError_t allow_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// CTAs along a head's 128-row tiles: about eight per SM in all, so that a CTA transposes the sketch matrices
+// once for several tiles when there are many, and every tile has a CTA of its own when there are few.
+inline unsigned sketch_grid(const Dims& d, int tensors) {
+    const int nt = d.n / 128;
+    const long want = 148L * 8 / ((long)d.BH() * tensors);
+    const long per = want >= nt ? 1 : want < 1 ? nt : (nt + want - 1) / want;      // tiles per CTA, the same for all but the last
+    return (unsigned)((nt + per - 1) / per);
+}
+
 // Half sketches of one tensor, or (X1 != nullptr) of two tensors of the same layout.
 template <typename T, int R>
 cudaError_t launch_sketch(const Dims& d, const T* X0, const T* X1, const T* G1, const T* G2, float* M0, float* M1, float* Phi,
                           cudaStream_t s, int* launches) {
     Slice sl{d.H, d.sb, d.sh, d.sn};
     if (!d.learned && d.p == 4) {
-        PSK_TRY((allow_smem(sketch_kernel<T, R>, kSketchSmem<R>)));
+        PSK_TRY((allow_smem(sketch_kernel<T, R>, SkTile<R>::bytes)));
+        const int nx = X1 != nullptr ? 2 : 1;
         prof_begin("sketch_kernel", s);
-        sketch_kernel<T, R><<<dim3(d.n / 128, d.BH(), X1 != nullptr ? 2 : 1), 128, kSketchSmem<R>, s>>>(
-            sl, X0, X1, G1, G2, d.g_heads, d.n, M0, M1, Phi);
+        sketch_kernel<T, R><<<dim3(sketch_grid(d, nx), d.BH(), nx), 128, SkTile<R>::bytes, s>>>(sl, X0, X1, G1, G2, d.g_heads, d.n, M0, M1, Phi);
         prof_end(s);
         ++*launches;
         return cudaGetLastError();
@@ -521,21 +526,42 @@ cudaError_t launch_states(const Dims& d, const float* M, const cc::YRows& y, flo
     return cudaGetLastError();
 }
 
+// Groups of 64 threads per CTA of the row kernels: two, so that two CTAs share an SM and one's
+// loads and final sums overlap the other's products, wherever their shared memory allows it (r <= 32,
+// sketched weights) and there are CTAs enough for every SM; else as many as fit one CTA, which also
+// spreads a few rows' work over the most warps.
+inline bool two_per_sm(const Dims& d) { return (long)d.BH() * (d.n / 64) >= 2 * 148; }
+
+template <typename T, int R, bool LOCAL, int NG>
+cudaError_t launch_rows_ng(const Dims& d, const float* Mown, const float* Moth, const cc::YRows& y, const float* S, const T* Xown,
+                           const T* Xoth, bool dv, T* Out, float* denom, cudaStream_t s, int* launches) {
+    using L = cc::RowsSmem<R, LOCAL, NG>;
+    PSK_TRY((allow_smem(cc::cc_rows_kernel<T, R, LOCAL, NG>, L::bytes)));
+    prof_begin(dv ? "bwd_v_kernel" : "fwd_out_kernel", s);
+    cc::cc_rows_kernel<T, R, LOCAL, NG><<<dim3(d.b / 64, d.t, d.BH()), 64 * NG, L::bytes, s>>>(
+        Slice{d.H, d.sb, d.sh, d.sn}, d.n, d.b, d.t, Mown, Moth, y, S, Xown, Xoth, dv ? 1 : 0, Out, denom);
+    prof_end(s);
+    ++*launches;
+    return cudaGetLastError();
+}
+
 template <typename T, int R>
 cudaError_t launch_rows(const Dims& d, const float* Mown, const float* Moth, const cc::YRows& y, const float* S, const T* Xown,
                         const T* Xoth, bool dv, T* Out, float* denom, cudaStream_t s, int* launches) {
-    const dim3 grid(d.b / 64, d.t, d.BH());
-    Slice sl{d.H, d.sb, d.sh, d.sn};
-    prof_begin(dv ? "bwd_v_kernel" : "fwd_out_kernel", s);
-    if (d.local) {
-        using L = cc::RowsSmem<R, true>;
-        PSK_TRY((allow_smem(cc::cc_rows_kernel<T, R, true>, L::bytes)));
-        cc::cc_rows_kernel<T, R, true><<<grid, 64 * L::NG, L::bytes, s>>>(sl, d.n, d.b, d.t, Mown, Moth, y, S, Xown, Xoth, dv ? 1 : 0, Out, denom);
-    } else {
-        using L = cc::RowsSmem<R, false>;
-        PSK_TRY((allow_smem(cc::cc_rows_kernel<T, R, false>, L::bytes)));
-        cc::cc_rows_kernel<T, R, false><<<grid, 64 * L::NG, L::bytes, s>>>(sl, d.n, d.b, d.t, Mown, Moth, y, S, Xown, Xoth, dv ? 1 : 0, Out, denom);
-    }
+    if (d.local) return launch_rows_ng<T, R, true, 4>(d, Mown, Moth, y, S, Xown, Xoth, dv, Out, denom, s, launches);
+    if constexpr (R <= 32)
+        if (two_per_sm(d)) return launch_rows_ng<T, R, false, 2>(d, Mown, Moth, y, S, Xown, Xoth, dv, Out, denom, s, launches);
+    return launch_rows_ng<T, R, false, 4>(d, Mown, Moth, y, S, Xown, Xoth, dv, Out, denom, s, launches);
+}
+
+template <typename T, int R, bool LOCAL, int NG>
+cudaError_t launch_dphi_ng(const Dims& d, const float* Mown, const float* Moth, const cc::YRows& yown, const cc::YRows& yoth, const float* S,
+                           const T* Xown, const T* Xoth, bool kside, float* dM, float* dXl, cudaStream_t s, int* launches) {
+    using L = cc::DphiSmem<R, LOCAL, NG>;
+    PSK_TRY((allow_smem(cc::cc_dphi_kernel<T, R, LOCAL, NG>, L::bytes)));
+    prof_begin(kside ? "bwd_k_kernel" : "bwd_q_kernel", s);
+    cc::cc_dphi_kernel<T, R, LOCAL, NG><<<dim3(d.b / 64, d.t, d.BH()), 64 * NG, L::bytes, s>>>(
+        Slice{d.H, d.sb, d.sh, d.sn}, d.n, d.b, d.t, Mown, Moth, yown, yoth, S, Xown, Xoth, kside ? 1 : 0, dM, dXl);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
@@ -544,21 +570,11 @@ cudaError_t launch_rows(const Dims& d, const float* Mown, const float* Moth, con
 template <typename T, int R>
 cudaError_t launch_dphi(const Dims& d, const float* Mown, const float* Moth, const cc::YRows& yown, const cc::YRows& yoth, const float* S,
                         const T* Xown, const T* Xoth, bool kside, float* dM, float* dXl, cudaStream_t s, int* launches) {
-    const dim3 grid(d.b / 64, d.t, d.BH());
-    Slice sl{d.H, d.sb, d.sh, d.sn};
-    prof_begin(kside ? "bwd_k_kernel" : "bwd_q_kernel", s);
-    if (d.local) {
-        using L = cc::DphiSmem<R, true>;
-        PSK_TRY((allow_smem(cc::cc_dphi_kernel<T, R, true>, L::bytes)));
-        cc::cc_dphi_kernel<T, R, true><<<grid, 64 * L::NG, L::bytes, s>>>(sl, d.n, d.b, d.t, Mown, Moth, yown, yoth, S, Xown, Xoth, kside ? 1 : 0, dM, dXl);
-    } else {
-        using L = cc::DphiSmem<R, false>;
-        PSK_TRY((allow_smem(cc::cc_dphi_kernel<T, R, false>, L::bytes)));
-        cc::cc_dphi_kernel<T, R, false><<<grid, 64 * L::NG, L::bytes, s>>>(sl, d.n, d.b, d.t, Mown, Moth, yown, yoth, S, Xown, Xoth, kside ? 1 : 0, dM, dXl);
-    }
-    prof_end(s);
-    ++*launches;
-    return cudaGetLastError();
+    constexpr int NG = R == 64 ? 3 : 4;
+    if (d.local) return launch_dphi_ng<T, R, true, NG>(d, Mown, Moth, yown, yoth, S, Xown, Xoth, kside, dM, dXl, s, launches);
+    if constexpr (R <= 32)
+        if (two_per_sm(d)) return launch_dphi_ng<T, R, false, 2>(d, Mown, Moth, yown, yoth, S, Xown, Xoth, kside, dM, dXl, s, launches);
+    return launch_dphi_ng<T, R, false, NG>(d, Mown, Moth, yown, yoth, S, Xown, Xoth, kside, dM, dXl, s, launches);
 }
 
 // [V | 1] rows: the caller's fp32 values as they are, or (bf16 storage) an fp32 copy in scratch.
@@ -615,7 +631,8 @@ cudaError_t launch_sketch_bwd(const Dims& d, const T* X0, const T* X1, const T* 
         using L = SkBwdSmem<R>;
         PSK_TRY((allow_smem(sketch_bwd_kernel<T, R>, L::bytes)));
         prof_begin("sketch_bwd_kernel", s);
-        sketch_bwd_kernel<T, R><<<dim3(d.n / 128, d.BH(), X1 != nullptr ? 2 : 1), 128, L::bytes, s>>>(
+        const int nx = X1 != nullptr ? 2 : 1;
+        sketch_bwd_kernel<T, R><<<dim3(sketch_grid(d, nx), d.BH(), nx), 128, L::bytes, s>>>(
             sl, X0, X1, G1, G2, d.g_heads, d.n, dM0, dM1, add0, add1, dX0, dX1);
         prof_end(s);
         ++*launches;
