@@ -30,6 +30,10 @@ class Shape(Structure):
 
 
 _lib = None
+_fast = None          # the native marshalling module (csrc/psk_binding.cpp), bound to _lib's entry points
+_FAST_ENTRIES = ("psk_workspace_bytes", "psk_causal_attn_fwd", "psk_causal_attn_bwd", "psk_lt_multiply_workspace_bytes",
+                 "psk_lt_multiply", "psk_lt_multiply_bf16_workspace_bytes", "psk_lt_multiply_bf16", "psk_decode_step",
+                 "psk_learned_workspace_bytes", "psk_learned_attn_fwd", "psk_learned_attn_bwd")
 
 
 def library_path() -> str:
@@ -98,6 +102,28 @@ def lib():
     L.psk_profile_get.argtypes = [c_int, ctypes.c_char_p, c_size_t, POINTER(ctypes.c_float)]
     _lib = L
     return L
+
+
+def _native():
+    """The native marshalling module: it takes a call's arguments, allocates what the call returns and calls
+    the C ABI; for arguments that need a closer look it returns None, and the checks below run."""
+    global _fast
+    if _fast is None:
+        L = lib()
+        try:
+            from . import _psk_native
+        except ImportError as e:
+            raise RuntimeError("_psk_native.so is not built: run `python -m paper_2310_01655_b200.build`") from e
+        _psk_native.init(*(ctypes.cast(getattr(L, name), c_void_p).value for name in _FAST_ENTRIES))
+        _fast = _psk_native
+    return _fast
+
+
+def _result(res, where):
+    """What a native call returned: its results, or the library's status."""
+    if type(res) is int:
+        raise PskError(res, where)
+    return res
 
 
 def status_string(code: int) -> str:
@@ -194,6 +220,9 @@ def sketch(X, G1, G2, r=None, b=128, want_phi=False, path=PATH_AUTO):
 def causal_attn_fwd(Q, K, V, G1, G2, b, p=4, path=PATH_AUTO, workspace=None, out=None, denom=None, flags=0,
                     seq_segments=0):
     """psk_causal_attn_fwd: returns (O, denom)."""
+    res = (_fast or _native()).attn_fwd(Q, K, V, G1, G2, b, p, path, workspace, out, denom, flags, seq_segments)
+    if res is not None:
+        return _result(res, "psk_causal_attn_fwd")
     _require_cuda(Q, K, V, G1, G2)
     _check_sketch_matrices(G1, G2)
     _check_keep_states(flags, workspace)
@@ -238,6 +267,9 @@ def causal_attn_fwd_static(Q, K, V, G1, G2, b, p=4, out=None, denom=None):
 def causal_attn_bwd(Q, K, V, G1, G2, O, denom, dO, b, p=4, path=PATH_AUTO, workspace=None, out=None, flags=0,
                     seq_segments=0):
     """psk_causal_attn_bwd: returns (dQ, dK, dV)."""
+    res = (_fast or _native()).attn_bwd(Q, K, V, G1, G2, O, denom, dO, b, p, path, workspace, out, flags, seq_segments)
+    if res is not None:
+        return _result(res, "psk_causal_attn_bwd")
     _require_cuda(Q, K, V, G1, G2, O, denom, dO)
     _check_sketch_matrices(G1, G2)
     _check_keep_states(flags, workspace)
@@ -309,6 +341,9 @@ def feature_table(r: int):
 
 def lt_multiply(A, B, C, b, workspace=None):
     """psk_lt_multiply: lt(A B^T) C for fp32 CUDA tensors A, B [batch, n, m] and C [batch, n, k]."""
+    res = (_fast or _native()).lt_multiply(A, B, C, b, workspace, False)
+    if res is not None:
+        return _result(res, "psk_lt_multiply")
     _require_cuda(A, B, C)
     for t in (A, B, C):
         if t.dtype != torch.float32 or t.dim() != 3 or not t.is_contiguous():
@@ -331,6 +366,9 @@ def lt_multiply(A, B, C, b, workspace=None):
 def lt_multiply_bf16(A, B, C, b, workspace=None):
     """psk_lt_multiply_bf16: lt(A B^T) C on the tensor cores for bf16 CUDA tensors A, B [batch, n, m] and
     C [batch, n, 64]; returns (Out fp32 [batch, n, 64], workspace) - pass the workspace to check()."""
+    res = (_fast or _native()).lt_multiply(A, B, C, b, workspace, True)
+    if res is not None:
+        return _result(res, "psk_lt_multiply_bf16")
     _require_cuda(A, B, C)
     for t in (A, B, C):
         if t.dtype != torch.bfloat16 or t.dim() != 3 or not t.is_contiguous():
@@ -413,6 +451,9 @@ def learned_workspace_bytes(Q, r, b, flags=0, for_backward=True, path=PATH_AUTO)
 
 def learned_attn_fwd(Q, K, V, params, r, b, flags=0, workspace=None, path=PATH_AUTO):
     """psk_learned_attn_fwd: returns (O, denom)."""
+    res = (_fast or _native()).learned_fwd(Q, K, V, params, r, b, flags, workspace, path)
+    if res is not None:
+        return _result(res, "psk_learned_attn_fwd")
     _require_cuda(Q, K, V, params)
     _same_layout(Q, K, V)
     shp = _learned_shape(Q, r, b, flags, path)
@@ -430,6 +471,9 @@ def learned_attn_fwd(Q, K, V, params, r, b, flags=0, workspace=None, path=PATH_A
 
 def learned_attn_bwd(Q, K, V, params, O, denom, dO, r, b, flags=0, workspace=None, path=PATH_AUTO):
     """psk_learned_attn_bwd: returns (dQ, dK, dV, dparams [2, count] fp32)."""
+    res = (_fast or _native()).learned_bwd(Q, K, V, params, O, denom, dO, r, b, flags, workspace, path)
+    if res is not None:
+        return _result(res, "psk_learned_attn_bwd")
     _require_cuda(Q, K, V, params, O, denom, dO)
     _same_layout(Q, K, V, O, dO)
     shp = _learned_shape(Q, r, b, flags, path)
@@ -452,6 +496,9 @@ def decode_state(B, H, r, device="cuda"):
 
 def decode_step(q, k, v, G1, G2, state):
     """psk_decode_step: q, k, v [B, H, h]; updates `state` in place; returns (o [B, H, h], denom [B, H])."""
+    res = (_fast or _native()).decode_step(q, k, v, G1, G2, state)
+    if res is not None:
+        return _result(res, "psk_decode_step")
     _require_cuda(q, k, v, G1, G2, state)
     B, H, h = q.shape
     r = G1.shape[-1]

@@ -1,4 +1,5 @@
-"""Builds libpsk.so (the C-ABI library) in-tree with nvcc for sm_100a.
+"""Builds libpsk.so (the C-ABI library) in-tree with nvcc for sm_100a, and _psk_native.so (the Python binding's
+argument marshalling, host code only) with g++.
 
     python -m paper_2310_01655_b200.build [--force] [--verbose]
 """
@@ -13,6 +14,7 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libpsk.so")
+NATIVE = os.path.join(PKG, "_psk_native.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -31,8 +33,27 @@ def _stale(obj, deps):
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_native(force=False):
+    """Compile csrc/psk_binding.cpp against torch's headers; returns the running compiler or None."""
+    src = os.path.join(CSRC, "psk_binding.cpp")
+    if not (force or _stale(NATIVE, [src, os.path.join(ROOT, "include", "psk.h"), __file__])):
+        return None
+    import sysconfig
+    import torch
+    troot = os.path.dirname(torch.__file__)
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+           "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], "-I", os.path.join(troot, "include"),
+           "-I", os.path.join(troot, "include", "torch", "csrc", "api", "include"),
+           "-I", os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include"),
+           src, "-o", NATIVE, "-L", os.path.join(troot, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-ltorch",
+           "-lc10_cuda", "-lc10"]
+    return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+
+
 def build(force=False, verbose=False):
-    """Compile every .cu under csrc/ and link libpsk.so; returns its path."""
+    """Compile every .cu under csrc/ and link libpsk.so, and the binding's native part; returns libpsk.so's path."""
+    native = build_native(force)
     hdrs = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h")) + [__file__]
     objdir = os.path.join(PKG, "build")
     os.makedirs(objdir, exist_ok=True)
@@ -49,6 +70,11 @@ def build(force=False, verbose=False):
         if p.returncode != 0 or verbose:
             sys.stderr.write("== %s\n%s\n" % (os.path.basename(src), out))
         failed |= p.returncode != 0
+    if native is not None:
+        out, _ = native.communicate()
+        if native.returncode != 0 or verbose:
+            sys.stderr.write("== psk_binding.cpp\n%s\n" % out)
+        failed |= native.returncode != 0
     if failed:
         raise RuntimeError("nvcc failed")
     if force or procs or _stale(LIB, objs):
