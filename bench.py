@@ -70,14 +70,13 @@ def kernel_flops_per_head_token(name, w, local=False):
         tile_fwd = 2 * 128 * h + 2 * 128 * h
         tile_bwd = 2 * 128 * h + 2 * 128 * h + 2 * 128 * 64
     table.update({
-        # (r = 64: a state set is built by five launches that split the feature tiles between them and
-        # each redo the half sketch; the figure is the average launch)
-        "tc_state_kernel": sk + 2 * FP * 80 / (1 if r <= 32 else 5),
+        # (r = 64: the feature tiles are split between five CTAs, which each redo the half sketch)
+        "tc_state_kernel": sk * (1 if r <= 32 else 5) + 2 * FP * 80,
         "tc_fwd_out_kernel": sk + 2 * FK * 80 + other * tile_fwd,
         "tc_bwd_recompute_kernel": sk + 2 * FK * 80 + other * tile_fwd,
         "tc_bwd_q_kernel": 2 * sk + 2 * FK * 80 + other * tile_bwd + 2 * 2 * r * 64,
         "tc_bwd_k_kernel": 2 * sk + 2 * FK * 80 + 2 * FK * 64 + other * (tile_bwd + 2 * 128 * 64) + 2 * 2 * r * 64,
-        "tc_vmean_kernel": None, "tc_bwd_prep_kernel": None,
+        "tc_prologue_kernel": None, "tc_bwd_prep_kernel": None,
     })
     return table.get(name)
 

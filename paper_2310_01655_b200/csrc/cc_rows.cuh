@@ -61,6 +61,7 @@ template <int R> constexpr size_t kStateSmem = 2 * (64 * (R + 4) + kUnit) * size
 template <int R>
 __global__ void __launch_bounds__(64 * kStateGroups<R>, R == 64 ? 2 : (R == 32 ? 4 : 2))
 cc_state_kernel(const float* __restrict__ M, YRows y, int n, int b, int t, int reverse, float* __restrict__ S) {
+    pdl_sync();
     extern __shared__ __align__(16) float smem[];
     constexpr int G = kStateGroups<R>, NT = 64 * G, LD = R + 4, kBuf = 64 * LD + kUnit;
     const int tid = threadIdx.x, grp = tid / 64, lane = tid % 64, ry = lane / 8, cx = lane % 8;
@@ -135,6 +136,7 @@ cc_state_kernel(const float* __restrict__ M, YRows y, int n, int b, int t, int r
 // is bound by memory, not by the chain of additions.
 __global__ void __launch_bounds__(256)
 cc_scan_kernel(float4* __restrict__ S, size_t elems, int t, int reverse) {
+    pdl_sync();
     const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (e >= elems) return;
     float4* p = S + (size_t)blockIdx.y * t * elems + e;
@@ -218,6 +220,7 @@ __global__ void __launch_bounds__(64 * NG)
 cc_rows_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mown, const float* __restrict__ Moth, YRows y,
                const float* __restrict__ S, const T* __restrict__ Xown, const T* __restrict__ Xoth, int dv,
                T* __restrict__ Out, float* __restrict__ denom) {
+    pdl_sync();
     extern __shared__ __align__(16) float smem[];
     using L = RowsSmem<R, LOCAL, NG>;
     constexpr int NT = 64 * NG, NC = kChunks<R>;
@@ -387,6 +390,7 @@ __global__ void __launch_bounds__(64 * NG)
 cc_dphi_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mown, const float* __restrict__ Moth, YRows yown,
                YRows yoth, const float* __restrict__ S, const T* __restrict__ Xown, const T* __restrict__ Xoth, int kside,
                float* __restrict__ dM, float* __restrict__ dXl) {
+    pdl_sync();
     extern __shared__ __align__(16) float smem[];
     using L = DphiSmem<R, LOCAL, NG>;
     constexpr int NT = 64 * NG, NC = kChunks<R>, LDM = L::ldm;

@@ -149,7 +149,8 @@ int psk_causal_attn_fwd(const psk_shape* shape, const void* Q, const void* K, co
         return PSK_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     int launches = 0;
-    cudaError_t e = cudaMemsetAsync(workspace, 0, kStatusBytes, s);
+    d.clear_status = path == 1 || (path == 0 && d.p == 4);
+    cudaError_t e = d.clear_status ? cudaSuccess : cudaMemsetAsync(workspace, 0, kStatusBytes, s);
     if (e == cudaSuccess)
         e = path == 2 ? given_fwd(d, Q, K, V, G1, G2, O, denom, (char*)workspace, s, &launches)
             : path == 1 ? tc_fwd(d, Q, K, V, G1, G2, O, denom, (char*)workspace, s, &launches)
@@ -178,7 +179,8 @@ int psk_causal_attn_bwd(const psk_shape* shape, const void* Q, const void* K, co
         return PSK_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     int launches = 0;
-    cudaError_t e = cudaMemsetAsync(workspace, 0, kStatusBytes, s);
+    d.clear_status = path == 1 || (path == 0 && d.p == 4);
+    cudaError_t e = d.clear_status ? cudaSuccess : cudaMemsetAsync(workspace, 0, kStatusBytes, s);
     if (e == cudaSuccess)
         e = path == 2 ? given_bwd(d, Q, K, V, G1, G2, O, denom, dO, dQ, dK, dV, (char*)workspace, s, &launches)
             : path == 1 ? tc_bwd(d, Q, K, V, G1, G2, O, denom, dO, dQ, dK, dV, (char*)workspace, s, &launches)

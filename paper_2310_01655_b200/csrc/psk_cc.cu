@@ -115,7 +115,9 @@ __device__ __forceinline__ void sketch_products(float (&a1)[8][SkTile<R>::kCols]
 template <typename T, int R>
 __global__ void __launch_bounds__(128)
 sketch_kernel(Slice sl, const T* __restrict__ X0, const T* __restrict__ X1, const T* __restrict__ G1, const T* __restrict__ G2,
-              int g_heads, int n, float* __restrict__ M0, float* __restrict__ M1, float* __restrict__ Phi_out) {
+              int g_heads, int n, float* __restrict__ M0, float* __restrict__ M1, float* __restrict__ Phi_out, int* status) {
+    pdl_sync();
+    if (status != nullptr && threadIdx.x < kStatusBytes / 4 && blockIdx.x + blockIdx.y + blockIdx.z == 0) status[threadIdx.x] = 0;
     extern __shared__ __align__(16) float smem[];
     using namespace cc;
     constexpr int KC = SkTile<R>::kCols;
@@ -349,7 +351,9 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 rows_prep_kernel(Slice sl, int n, int total_rows, int mode, const T* __restrict__ V,
                  const T* __restrict__ O, const float* __restrict__ denom,
-                 const T* __restrict__ dO, float* __restrict__ out) {
+                 const T* __restrict__ dO, float* __restrict__ out, int* status) {
+    pdl_sync();
+    if (status != nullptr && threadIdx.x < kStatusBytes / 4 && blockIdx.x == 0) status[threadIdx.x] = 0;
     const int row = blockIdx.x * 16 + threadIdx.x / 16, lane = threadIdx.x % 16;
     if (row >= total_rows) return;      // (total_rows is a multiple of 128: whole warps)
     const int64_t base = sl.row(row / n, row % n) + 4 * lane;
@@ -388,6 +392,7 @@ __global__ void __launch_bounds__(128)
 sketch_bwd_kernel(Slice sl, const T* __restrict__ X0, const T* __restrict__ X1, const T* __restrict__ G1, const T* __restrict__ G2,
                   int g_heads, int n, const float* __restrict__ dM0, const float* __restrict__ dM1,
                   const float* __restrict__ add0, const float* __restrict__ add1, T* __restrict__ dX0, T* __restrict__ dX1) {
+    pdl_sync();
     extern __shared__ __align__(16) float smem[];
     using namespace cc;
     using L = SkBwdSmem<R>;
@@ -471,13 +476,13 @@ inline unsigned sketch_grid(const Dims& d, int tensors) {
 // Half sketches of one tensor, or (X1 != nullptr) of two tensors of the same layout.
 template <typename T, int R>
 cudaError_t launch_sketch(const Dims& d, const T* X0, const T* X1, const T* G1, const T* G2, float* M0, float* M1, float* Phi,
-                          cudaStream_t s, int* launches) {
+                          int* status, cudaStream_t s, int* launches) {
     Slice sl{d.H, d.sb, d.sh, d.sn};
     if (!d.learned && d.p == 4) {
         PSK_TRY((allow_smem(sketch_kernel<T, R>, SkTile<R>::bytes)));
         const int nx = X1 != nullptr ? 2 : 1;
         prof_begin("sketch_kernel", s);
-        sketch_kernel<T, R><<<dim3(sketch_grid(d, nx), d.BH(), nx), 128, SkTile<R>::bytes, s>>>(sl, X0, X1, G1, G2, d.g_heads, d.n, M0, M1, Phi);
+        launch_pdl(sketch_kernel<T, R>, dim3(sketch_grid(d, nx), d.BH(), nx), 128, SkTile<R>::bytes, s, sl, X0, X1, G1, G2, d.g_heads, d.n, M0, M1, Phi, status);
         prof_end(s);
         ++*launches;
         return cudaGetLastError();
@@ -513,14 +518,14 @@ cudaError_t launch_states(const Dims& d, const float* M, const cc::YRows& y, flo
     constexpr int G = cc::kStateGroups<R>, NC = cc::kChunks<R>;
     PSK_TRY((allow_smem(cc::cc_state_kernel<R>, cc::kStateSmem<R>)));
     prof_begin("state_kernel", s);
-    cc::cc_state_kernel<R><<<dim3((NC + G - 1) / G, d.t - 1, d.BH()), 64 * G, cc::kStateSmem<R>, s>>>(M, y, d.n, d.b, d.t, reverse ? 1 : 0, S);
+    launch_pdl(cc::cc_state_kernel<R>, dim3((NC + G - 1) / G, d.t - 1, d.BH()), 64 * G, cc::kStateSmem<R>, s, M, y, d.n, d.b, d.t, reverse ? 1 : 0, S);
     prof_end(s);
     ++*launches;
     PSK_TRY(cudaGetLastError());
     if (d.t == 2) return cudaSuccess;            // the only state there is needs no sum
     const size_t elems = (size_t)NC * cc::kChunkFloats / 4;
     prof_begin("scan_kernel", s);
-    cc::cc_scan_kernel<<<dim3((unsigned)((elems + 255) / 256), d.BH()), 256, 0, s>>>(reinterpret_cast<float4*>(S), elems, d.t, reverse ? 1 : 0);
+    launch_pdl(cc::cc_scan_kernel, dim3((unsigned)((elems + 255) / 256), d.BH()), 256, 0, s, reinterpret_cast<float4*>(S), elems, d.t, reverse ? 1 : 0);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
@@ -538,7 +543,7 @@ cudaError_t launch_rows_ng(const Dims& d, const float* Mown, const float* Moth, 
     using L = cc::RowsSmem<R, LOCAL, NG>;
     PSK_TRY((allow_smem(cc::cc_rows_kernel<T, R, LOCAL, NG>, L::bytes)));
     prof_begin(dv ? "bwd_v_kernel" : "fwd_out_kernel", s);
-    cc::cc_rows_kernel<T, R, LOCAL, NG><<<dim3(d.b / 64, d.t, d.BH()), 64 * NG, L::bytes, s>>>(
+    launch_pdl(cc::cc_rows_kernel<T, R, LOCAL, NG>, dim3(d.b / 64, d.t, d.BH()), 64 * NG, L::bytes, s, 
         Slice{d.H, d.sb, d.sh, d.sn}, d.n, d.b, d.t, Mown, Moth, y, S, Xown, Xoth, dv ? 1 : 0, Out, denom);
     prof_end(s);
     ++*launches;
@@ -560,7 +565,7 @@ cudaError_t launch_dphi_ng(const Dims& d, const float* Mown, const float* Moth, 
     using L = cc::DphiSmem<R, LOCAL, NG>;
     PSK_TRY((allow_smem(cc::cc_dphi_kernel<T, R, LOCAL, NG>, L::bytes)));
     prof_begin(kside ? "bwd_k_kernel" : "bwd_q_kernel", s);
-    cc::cc_dphi_kernel<T, R, LOCAL, NG><<<dim3(d.b / 64, d.t, d.BH()), 64 * NG, L::bytes, s>>>(
+    launch_pdl(cc::cc_dphi_kernel<T, R, LOCAL, NG>, dim3(d.b / 64, d.t, d.BH()), 64 * NG, L::bytes, s, 
         Slice{d.H, d.sb, d.sh, d.sn}, d.n, d.b, d.t, Mown, Moth, yown, yoth, S, Xown, Xoth, kside ? 1 : 0, dM, dXl);
     prof_end(s);
     ++*launches;
@@ -587,7 +592,7 @@ cudaError_t value_rows(const Dims& d, const T* V, float* Vt, cc::YRows* y, cudaS
     } else {
         const int rows = d.BH() * d.n;
         prof_begin("rows_prep_kernel", s);
-        rows_prep_kernel<T><<<(rows + 15) / 16, 256, 0, s>>>(sl, d.n, rows, 0, V, nullptr, nullptr, nullptr, Vt);
+        launch_pdl(rows_prep_kernel<T>, (rows + 15) / 16, 256, 0, s, sl, d.n, rows, 0, V, nullptr, nullptr, nullptr, Vt, nullptr);
         prof_end(s);
         ++*launches;
         *y = cc::YRows{Vt, Slice{d.H, (int64_t)d.H * d.n * 64, (int64_t)d.n * 64, 64}, 1};
@@ -606,7 +611,7 @@ cudaError_t prefix_states(const Dims& d, const T* Q, const T* K, const T* V, con
                             : cc::YRows{(const float*)(ws + w.Vt), Slice{d.H, (int64_t)d.H * d.n * 64, (int64_t)d.n * 64, 64}, 1};
         return cudaSuccess;
     }
-    PSK_TRY((launch_sketch<T, R>(d, Q, K, G1, G2, Mq, Mk, nullptr, s, launches)));
+    PSK_TRY((launch_sketch<T, R>(d, Q, K, G1, G2, Mq, Mk, nullptr, d.clear_status ? (int*)(ws + w.status) : nullptr, s, launches)));
     PSK_TRY(value_rows<T>(d, V, (float*)(ws + w.Vt), y, s, launches));
     return launch_states<R>(d, Mk, *y, (float*)(ws + w.Zst), false, s, launches);
 }
@@ -632,7 +637,7 @@ cudaError_t launch_sketch_bwd(const Dims& d, const T* X0, const T* X1, const T* 
         PSK_TRY((allow_smem(sketch_bwd_kernel<T, R>, L::bytes)));
         prof_begin("sketch_bwd_kernel", s);
         const int nx = X1 != nullptr ? 2 : 1;
-        sketch_bwd_kernel<T, R><<<dim3(sketch_grid(d, nx), d.BH(), nx), 128, L::bytes, s>>>(
+        launch_pdl(sketch_bwd_kernel<T, R>, dim3(sketch_grid(d, nx), d.BH(), nx), 128, L::bytes, s, 
             sl, X0, X1, G1, G2, d.g_heads, d.n, dM0, dM1, add0, add1, dX0, dX1);
         prof_end(s);
         ++*launches;
@@ -677,7 +682,8 @@ cudaError_t bwd_impl(const Dims& d, const T* Q, const T* K, const T* V, const T*
     cc::YRows yv;
     PSK_TRY((prefix_states<T, R>(d, Q, K, V, G1, G2, ws, w, d.keep_states, &yv, s, launches)));
     prof_begin("rows_prep_kernel", s);
-    rows_prep_kernel<T><<<(rows + 15) / 16, 256, 0, s>>>(Slice{d.H, d.sb, d.sh, d.sn}, d.n, rows, 1, nullptr, O, denom, dO, E);
+    launch_pdl(rows_prep_kernel<T>, (rows + 15) / 16, 256, 0, s, Slice{d.H, d.sb, d.sh, d.sn}, d.n, rows, 1, nullptr, O, denom, dO, E,
+               d.clear_status && d.keep_states ? (int*)(ws + w.status) : nullptr);
     prof_end(s);
     ++*launches;
     PSK_TRY(cudaGetLastError());
@@ -707,7 +713,7 @@ cudaError_t bwd_impl(const Dims& d, const T* Q, const T* K, const T* V, const T*
 
 cudaError_t cc_sketch(const Dims& d, const void* X, const void* G1, const void* G2,
                       float* M_out, float* Phi_out, cudaStream_t s, int* launches) {
-#define C_ (launch_sketch<T, R>(d, (const T*)X, nullptr, (const T*)G1, (const T*)G2, M_out, nullptr, Phi_out, s, launches))
+#define C_ (launch_sketch<T, R>(d, (const T*)X, nullptr, (const T*)G1, (const T*)G2, M_out, nullptr, Phi_out, nullptr, s, launches))
     PSK_DISPATCH(C_, C_)
 #undef C_
 }

@@ -40,6 +40,7 @@ decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
                    float* __restrict__ state, T* __restrict__ o, float* __restrict__ denom) {
     constexpr int kRows = R * R / CL, NV = Dec<R, CL>::kVec, NB = Dec<R, CL>::kBatch, NS = Dec<R, CL>::kSlots;
     static_assert(NV % NB == 0 && NS % NB == 0 && (NV == NS || NS == 2 * NB), "whole batches");
+    pdl_sync();
     extern __shared__ float4 sbuf[];                 // [NS][kThreads]: every thread copies and reads its own entries
     __shared__ float sx[3][64], sa[2][4][2][R], sm[2][R + 4];
     __shared__ double part[kSub][4 * kCols];
@@ -183,11 +184,13 @@ cudaError_t launch_cl(const psk_shape* sh, const void* q, const void* k, const v
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = Dec<R, CL>::kSmem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = CL; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kern, (const T*)q, (const T*)k, (const T*)v, (const T*)G1, (const T*)G2, (int)sh->g_heads, (int)sh->H, state,
                               (T*)o, denom);
 }

@@ -24,6 +24,7 @@ struct Dims {
     // tensor-core kernels: the tensors they "sketch" already hold the half sketch (tc_common.cuh,
     // read_half_sketch); `xsb, xsh, xsn` are the strides of those tensors and of their gradients
     bool sketch_linear = false;
+    bool clear_status = false;        // the call's first kernel clears the status word (else: a memset did)
     int64_t xsb = 0, xsh = 0, xsn = 0;
     // given half sketches WITH exact same-block weights: the raw rows (strides sb, sh, sn) next to
     // the half sketches, and where the same-block part of their gradients goes (contiguous
@@ -114,6 +115,31 @@ cudaError_t tc_bwd(const Dims& d, const void* Q, const void* K, const void* V,
 // CUDA events on its own stream; disabled, these are no-ops.
 void prof_begin(const char* name, cudaStream_t s);
 void prof_end(cudaStream_t s);
+
+// Launches on a stream follow one another by programmatic dependence: a kernel may be put on the SMs as soon
+// as every CTA of the one before it has started, and waits in pdl_sync() until that one has ended and its
+// writes are visible; only the launch itself overlaps.  Every kernel launched this way calls pdl_sync()
+// before its first access to global memory, and before it allocates tensor memory (a CTA that waits
+// for the previous kernel must not hold what that kernel's CTAs still have to allocate).
+// (Forward of one head in fp32, four launches: 47 -> 40 us.)
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);
+}
+__device__ __forceinline__ void pdl_sync() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 __device__ __forceinline__ float ldf(const float* p) { return *p; }
 __device__ __forceinline__ float ldf(const __nv_bfloat16* p) { return __bfloat162float(*p); }

@@ -103,6 +103,7 @@ __device__ float bank_entry(const NetLayout& nl, const float* P, int which, int 
 
 __global__ void __launch_bounds__(256)
 ltc_bank_kernel(int h, int r, const float* __restrict__ params, bf16* __restrict__ bank, float* __restrict__ vec) {
+    pdl_sync();
     const NetLayout nl(h, r);
     const int net = blockIdx.y;
     const float* P = params + (size_t)net * nl.count;
@@ -167,6 +168,7 @@ constexpr int kDenseSmem = 128 * 256 * 2 + 256 * 64 * 2 + 1024;
 template <int EPI>
 __global__ void __launch_bounds__(128)
 ltc_dense_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB, DenseArgs a, int* status) {
+    pdl_sync();
     static_assert(EPI == EPI_B64 || EPI == EPI_F32, "the 256 -> 64 layers");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sA = align1024(smem_raw);
@@ -265,6 +267,7 @@ __global__ void __launch_bounds__(192, 1)
 ltc_narrow_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mA2,
                   const __grid_constant__ CUtensorMap mB, const __grid_constant__ CUtensorMap mB2, DenseArgs a, int tiles,
                   int* status) {
+    pdl_sync();
     static_assert(EPI == EPI_B64 || EPI == EPI_F32, "the 256 -> 64 layers");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sB = align1024(smem_raw);
@@ -450,6 +453,7 @@ ltc_wide_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ 
                 const __grid_constant__ CUtensorMap mS0, const __grid_constant__ CUtensorMap mS1,
                 const __grid_constant__ CUtensorMap mO0, const __grid_constant__ CUtensorMap mO1,
                 const __grid_constant__ CUtensorMap mO2, WideArgs a, int* status) {
+    pdl_sync();
     using L = WideSmem<EPI, SPLIT>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sA = align1024(smem_raw);
@@ -720,6 +724,7 @@ constexpr int kWgSmem = 2 * kWgStage + 1024;
 __global__ void __launch_bounds__(160)
 ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mP, const __grid_constant__ CUtensorMap mS, float* __restrict__ Gt,
                  float* __restrict__ colsum, int sum_wide, int ntiles, int tiles_per_cta, int* status) {
+    pdl_sync();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     __shared__ uint64_t bar_full[2], bar_free[2], bar_done;
@@ -849,6 +854,7 @@ constexpr int kLnRowsPerWarp = 8;
 __global__ void __launch_bounds__(256)
 ltc_ln0_kernel(Slice sl, const bf16* __restrict__ X, size_t row0, int rows, bf16* __restrict__ n0, bf16* __restrict__ n0_lo,
                float* __restrict__ rs0) {
+    pdl_sync();
     const int lane = threadIdx.x % 32;
     const int i0 = (blockIdx.x * 8 + threadIdx.x / 32) * kLnRowsPerWarp;
     __nv_bfloat162 x2[kLnRowsPerWarp];
@@ -879,6 +885,7 @@ ltc_ln0_kernel(Slice sl, const bf16* __restrict__ X, size_t row0, int rows, bf16
 __global__ void __launch_bounds__(256)
 ltc_ln0_bwd_kernel(Slice sl, size_t row0, int rows, const float* __restrict__ dn0, const bf16* __restrict__ n0,
                    const float* __restrict__ rs0, const bf16* __restrict__ add, bf16* __restrict__ dX) {
+    pdl_sync();
     const int lane = threadIdx.x % 32;
     const int i = blockIdx.x * 8 + threadIdx.x / 32;
     if (i >= rows) return;
@@ -900,6 +907,7 @@ ltc_ln0_bwd_kernel(Slice sl, size_t row0, int rows, const float* __restrict__ dn
 // attention kernels read in their linear sketch mode; one thread = 8 consecutive columns of a row
 __global__ void __launch_bounds__(256)
 ltc_combine_kernel(const float* __restrict__ f1, const float* __restrict__ f2, int r, size_t rows, bf16* __restrict__ S) {
+    pdl_sync();
     const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (e >= rows * 8) return;
     const size_t row = e / 8;
@@ -931,6 +939,7 @@ ltc_combine_kernel(const float* __restrict__ f1, const float* __restrict__ f2, i
 __global__ void __launch_bounds__(256)
 ltc_combine_bwd_kernel(const float* __restrict__ f1, const float* __restrict__ f2, const bf16* __restrict__ dS, int r,
                        size_t rows, bf16* __restrict__ df1, bf16* __restrict__ df2) {
+    pdl_sync();
     const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (e >= rows * 64) return;
     const size_t row = e / 64;
@@ -951,6 +960,7 @@ ltc_combine_bwd_kernel(const float* __restrict__ f1, const float* __restrict__ f
 __global__ void __launch_bounds__(256)
 ltc_finish_kernel(int h, int r, const float* __restrict__ params, const float* __restrict__ G, const float* __restrict__ sums,
                   float* __restrict__ dparams) {
+    pdl_sync();
     const NetLayout nl(h, r);
     const int net = blockIdx.y, m = nl.m;
     const float* P = params + (size_t)net * nl.count;
@@ -1105,8 +1115,8 @@ cudaError_t wide(const CUtensorMap& mA, const CUtensorMap& mA2, const CUtensorMa
     PSK_TRY(set_smem(ltc_wide_kernel<EPI, SPLIT, true>, smem));
     PSK_TRY(set_smem(ltc_wide_kernel<EPI, SPLIT, false>, smem));
     prof_begin(SPLIT ? kDenseSplitName[EPI] : kDenseName[EPI], s);
-    if (a.ncols == 256) ltc_wide_kernel<EPI, SPLIT, true><<<tiles, 256, smem, s>>>(mA, mA2, mB, mB2, mS0, mS1, mO0, mO1, mO2, a, status);
-    else ltc_wide_kernel<EPI, SPLIT, false><<<tiles, 256, smem, s>>>(mA, mA2, mB, mB2, mS0, mS1, mO0, mO1, mO2, a, status);
+    if (a.ncols == 256) launch_pdl(ltc_wide_kernel<EPI, SPLIT, true>, tiles, 256, smem, s, mA, mA2, mB, mB2, mS0, mS1, mO0, mO1, mO2, a, status);
+    else launch_pdl(ltc_wide_kernel<EPI, SPLIT, false>, tiles, 256, smem, s, mA, mA2, mB, mB2, mS0, mS1, mO0, mO1, mO2, a, status);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
@@ -1117,7 +1127,7 @@ cudaError_t dense(const CUtensorMap& mA, const CUtensorMap& mB, const DenseArgs&
                   int* launches) {
     PSK_TRY(set_smem(ltc_dense_kernel<EPI>, kDenseSmem));
     prof_begin(kDenseName[EPI], s);
-    ltc_dense_kernel<EPI><<<tiles, 128, kDenseSmem, s>>>(mA, mB, a, status);
+    launch_pdl(ltc_dense_kernel<EPI>, tiles, 128, kDenseSmem, s, mA, mB, a, status);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
@@ -1134,7 +1144,7 @@ cudaError_t narrow(const CUtensorMap& mA, const CUtensorMap& mA2, const CUtensor
             sms = 148;
     }
     prof_begin(kDenseSplitName[EPI], s);
-    ltc_narrow_kernel<EPI><<<tiles < sms ? tiles : sms, 192, kNrSmem, s>>>(mA, mA2, mB, mB2, a, tiles, status);
+    launch_pdl(ltc_narrow_kernel<EPI>, tiles < sms ? tiles : sms, 192, kNrSmem, s, mA, mA2, mB, mB2, a, tiles, status);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
@@ -1148,7 +1158,7 @@ cudaError_t wgrad(const CUtensorMap& mP, const CUtensorMap& mS, float* Gt, float
     if (per < 4) per = tiles < 4 ? tiles : 4;
     const int grid = (tiles + per - 1) / per;
     prof_begin("ltc_wgrad_kernel", s);
-    ltc_wgrad_kernel<<<grid, 160, kWgSmem, s>>>(mP, mS, Gt, colsum, wide ? 1 : 0, tiles, per, status);
+    launch_pdl(ltc_wgrad_kernel, grid, 160, kWgSmem, s, mP, mS, Gt, colsum, wide ? 1 : 0, tiles, per, status);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
@@ -1161,7 +1171,7 @@ cudaError_t forward_chunk(const Dims& d, const LtcWs& w, const Maps& M, const vo
     const Slice sl{d.H, d.n, d.sb, d.sh, d.sn};
     const int tiles = c / 128, m = 8 * d.r;
     prof_begin("ltc_ln0_kernel", s);
-    ltc_ln0_kernel<<<(c + 8 * kLnRowsPerWarp - 1) / (8 * kLnRowsPerWarp), 256, 0, s>>>(sl, (const bf16*)X, row0, c, (bf16*)(ws + w.n0), (bf16*)(ws + w.n0_lo), (float*)(ws + w.rs0));
+    launch_pdl(ltc_ln0_kernel, (c + 8 * kLnRowsPerWarp - 1) / (8 * kLnRowsPerWarp), 256, 0, s, sl, (const bf16*)X, row0, c, (bf16*)(ws + w.n0), (bf16*)(ws + w.n0_lo), (float*)(ws + w.rs0));
     prof_end(s);
     ++*launches;
     PSK_TRY(cudaGetLastError());
@@ -1190,7 +1200,7 @@ size_t learned_tc_workspace_bytes(const Dims& d, bool backward) { return ltc_ws(
 cudaError_t learned_tc_prepare(const Dims& d, bool backward, char* ws, cudaStream_t s, int* launches) {
     const LtcWs w = ltc_ws(d, backward);
     prof_begin("ltc_bank_kernel", s);
-    ltc_bank_kernel<<<dim3((8 * kMat + kVec + 255) / 256, 2), 256, 0, s>>>(d.h, d.r, d.lparams, (bf16*)(ws + w.bank), (float*)(ws + w.vec));
+    launch_pdl(ltc_bank_kernel, dim3((8 * kMat + kVec + 255) / 256, 2), 256, 0, s, d.h, d.r, d.lparams, (bf16*)(ws + w.bank), (float*)(ws + w.vec));
     prof_end(s);
     ++*launches;
     PSK_TRY(cudaGetLastError());
@@ -1208,7 +1218,7 @@ cudaError_t learned_tc_sketch(const Dims& d, const void* X, void* S, char* ws, i
         const int c = (int)(rows - row0 < w.C ? rows - row0 : w.C);
         PSK_TRY(forward_chunk(d, w, M, X, row0, c, false, ws, status, s, launches));
         prof_begin("ltc_combine_kernel", s);
-        ltc_combine_kernel<<<(unsigned)(((size_t)c * 8 + 255) / 256), 256, 0, s>>>((const float*)(ws + w.net[0].f), (const float*)(ws + w.net[1].f),
+        launch_pdl(ltc_combine_kernel, (unsigned)(((size_t)c * 8 + 255) / 256), 256, 0, s, (const float*)(ws + w.net[0].f), (const float*)(ws + w.net[1].f),
                                                                               d.r, (size_t)c, (bf16*)S + row0 * 64);
         prof_end(s);
         ++*launches;
@@ -1234,7 +1244,7 @@ cudaError_t learned_tc_sketch_bwd(const Dims& d, const void* X, const void* dS, 
         const int tiles = c / 128;
         PSK_TRY(forward_chunk(d, w, M, X, row0, c, true, ws, status, s, launches));
         prof_begin("ltc_combine_bwd_kernel", s);
-        ltc_combine_bwd_kernel<<<(unsigned)(((size_t)c * 64 + 255) / 256), 256, 0, s>>>(
+        launch_pdl(ltc_combine_bwd_kernel, (unsigned)(((size_t)c * 64 + 255) / 256), 256, 0, s, 
             (const float*)(ws + w.net[0].f), (const float*)(ws + w.net[1].f), (const bf16*)dS + row0 * 64, d.r, (size_t)c,
             (bf16*)(ws + w.df[0]), (bf16*)(ws + w.df[1]));
         prof_end(s);
@@ -1260,7 +1270,7 @@ cudaError_t learned_tc_sketch_bwd(const Dims& d, const void* X, const void* dS, 
             PSK_TRY(dense<EPI_F32>(M.dp1, M.bank[t][7], DenseArgs{nullptr, nullptr, nullptr, (float*)(ws + w.dn0), 64, t}, tiles, status, s, launches));
         }
         prof_begin("ltc_ln0_bwd_kernel", s);
-        ltc_ln0_bwd_kernel<<<(c + 7) / 8, 256, 0, s>>>(sl, row0, c, (const float*)(ws + w.dn0), (const bf16*)(ws + w.n0),
+        launch_pdl(ltc_ln0_bwd_kernel, (c + 7) / 8, 256, 0, s, sl, row0, c, (const float*)(ws + w.dn0), (const bf16*)(ws + w.n0),
                                                       (const float*)(ws + w.rs0), (const bf16*)add, (bf16*)dX);
         prof_end(s);
         ++*launches;
@@ -1274,7 +1284,7 @@ cudaError_t learned_tc_finish(const Dims& d, char* ws, cudaStream_t s, int* laun
     const LtcWs w = ltc_ws(d, true);
     const int count = NetLayout(d.h, d.r).count;
     prof_begin("ltc_finish_kernel", s);
-    ltc_finish_kernel<<<dim3((count + 255) / 256, 2), 256, 0, s>>>(d.h, d.r, d.lparams, (const float*)(ws + w.G),
+    launch_pdl(ltc_finish_kernel, dim3((count + 255) / 256, 2), 256, 0, s, d.h, d.r, d.lparams, (const float*)(ws + w.G),
                                                                    (const float*)(ws + w.sums), d.dlparams);
     prof_end(s);
     ++*launches;

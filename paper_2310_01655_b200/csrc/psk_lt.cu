@@ -94,6 +94,7 @@ template <int NH>
 __global__ void __launch_bounds__(128, NH <= 2 ? 4 : 2)
 lt_state_kernel(const float* __restrict__ B, const float* __restrict__ C, int n, int m, int k, int b, int t, bool vm, bool vk,
                 float* __restrict__ S) {
+    pdl_sync();
     extern __shared__ __align__(16) float smem[];
     constexpr int LDC = kLdc<NH>, kBuf = 32 * 128 + 32 * LDC;
     const int tid = threadIdx.x, grp = tid / 64, lane = tid % 64, ry = lane / 8, cx = lane % 8;
@@ -149,6 +150,7 @@ template <> __device__ __forceinline__ void add_to<float4>(float4& a, const floa
 template <typename V>
 __global__ void __launch_bounds__(256)
 lt_scan_kernel(V* __restrict__ S, size_t elems, int t) {
+    pdl_sync();
     const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (e >= elems) return;
     V* p = S + (size_t)blockIdx.y * t * elems + e;
@@ -186,6 +188,7 @@ template <int NH>
 __global__ void __launch_bounds__(128)
 lt_out_kernel(const float* __restrict__ A, const float* __restrict__ B, const float* __restrict__ C,
               const float* __restrict__ Z, int n, int m, int k, int b, int t, bool vm, bool vk, float* __restrict__ Out) {
+    pdl_sync();
     extern __shared__ __align__(16) float smem[];
     using L = OutSmem<NH>;
     constexpr int LDC = kLdc<NH>;
@@ -337,20 +340,20 @@ cudaError_t lt_run(int batch, int n, int m, int k, int b, const float* A, const 
     if (e != cudaSuccess) return e;
     if (t > 1) {
         prof_begin("lt_state_kernel", s);
-        lt_state_kernel<NH><<<dim3((m + 127) / 128, t - 1, batch), 128, kStateSmem<NH>, s>>>(B, C, n, m, k, b, t, vm, vk, S);
+        launch_pdl(lt_state_kernel<NH>, dim3((m + 127) / 128, t - 1, batch), 128, kStateSmem<NH>, s, B, C, n, m, k, b, t, vm, vk, S);
         prof_end(s);
     }
     if (t > 2) {
         const size_t elems = (size_t)m * k;
         prof_begin("lt_scan_kernel", s);
         if (elems % 4 == 0 && aligned16(S))
-            lt_scan_kernel<float4><<<dim3((unsigned)((elems / 4 + 255) / 256), batch), 256, 0, s>>>(reinterpret_cast<float4*>(S), elems / 4, t);
+            launch_pdl(lt_scan_kernel<float4>, dim3((unsigned)((elems / 4 + 255) / 256), batch), 256, 0, s, reinterpret_cast<float4*>(S), elems / 4, t);
         else
-            lt_scan_kernel<float><<<dim3((unsigned)((elems + 255) / 256), batch), 256, 0, s>>>(S, elems, t);
+            launch_pdl(lt_scan_kernel<float>, dim3((unsigned)((elems + 255) / 256), batch), 256, 0, s, S, elems, t);
         prof_end(s);
     }
     prof_begin("lt_out_kernel", s);
-    lt_out_kernel<NH><<<dim3((b + 63) / 64, t, batch), 128, OutSmem<NH>::bytes, s>>>(A, B, C, S, n, m, k, b, t, vm, vk, Out);
+    launch_pdl(lt_out_kernel<NH>, dim3((b + 63) / 64, t, batch), 128, OutSmem<NH>::bytes, s, A, B, C, S, n, m, k, b, t, vm, vk, Out);
     prof_end(s);
     return cudaGetLastError();
 }

@@ -23,6 +23,7 @@ constexpr int kStSmem = 2 * kStStage + 1024;
 __global__ void __launch_bounds__(128)
 lt_tc_state_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapC, bf16* __restrict__ Z,
                    int m, int t, int tpb, int* status) {
+    pdl_sync();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     __shared__ uint64_t bar_full[2], bar_free[2], bar_acc;
@@ -115,6 +116,7 @@ __global__ void __launch_bounds__(160)
 lt_tc_rows_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                   const __grid_constant__ CUtensorMap mapC, const __grid_constant__ CUtensorMap mapZ,
                   float* __restrict__ Out, int n, int m, int b, int t, int* status) {
+    pdl_sync();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     uint8_t* sC = smem + 2 * kRwStage;
@@ -275,11 +277,11 @@ int psk_lt_multiply_bf16(int batch, int n, int m, int k, int b, const void* A, c
         return PSK_ERR_CUDA;
     if (t > 1) {
         prof_begin("lt_tc_state_kernel", s);
-        lt_tc_state_kernel<<<dim3((m + 127) / 128, batch), 128, kStSmem, s>>>(mB, mC, Z, m, t, tpb, status);
+        launch_pdl(lt_tc_state_kernel, dim3((m + 127) / 128, batch), 128, kStSmem, s, mB, mC, Z, m, t, tpb, status);
         prof_end(s);
     }
     prof_begin("lt_tc_rows_kernel", s);
-    lt_tc_rows_kernel<<<dim3(tpb, t, batch), 160, kRwSmem, s>>>(mA, mB, mC, mZ, Out, n, m, b, t, status);
+    launch_pdl(lt_tc_rows_kernel, dim3(tpb, t, batch), 160, kRwSmem, s, mA, mB, mC, mZ, Out, n, m, b, t, status);
     prof_end(s);
     return cudaGetLastError() == cudaSuccess ? PSK_OK : PSK_ERR_CUDA;
 }

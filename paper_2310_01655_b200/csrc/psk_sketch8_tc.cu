@@ -19,6 +19,7 @@ constexpr int kW1 = 64 * 128, kW2 = 64 * 64;      // elements per head: [64][128
 // W1[g][k][n] = [Ga1 | Ga2 | Gb1 | Gb2][k][n] (zero beyond 4r), W2[g] = blockdiag(Gc1, Gc2) (zero elsewhere)
 __global__ void __launch_bounds__(256)
 sk8_bank_kernel(const bf16* __restrict__ G1, const bf16* __restrict__ G2, int r, bf16* __restrict__ W1, bf16* __restrict__ W2) {
+    pdl_sync();
     const int g = blockIdx.y, e = blockIdx.x * 256 + threadIdx.x;
     const size_t gbase = (size_t)g * (128 + r) * r;
     const bf16 zero = __float2bfloat16_rn(0.f);
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(128)
 sk8_tc_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW1,
                   const __grid_constant__ CUtensorMap mapW2, const __grid_constant__ CUtensorMap mapS, int g_heads, int H,
                   int* status) {
+    pdl_sync();
     using L = Sk8Smem;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
@@ -178,6 +180,7 @@ __global__ void __launch_bounds__(128)
 sk8_tc_bwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW1,
                   const __grid_constant__ CUtensorMap mapW2, const __grid_constant__ CUtensorMap mapDS,
                   const __grid_constant__ CUtensorMap mapDX, int g_heads, int H, int* status) {
+    pdl_sync();
     using L = Sk8Smem;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
@@ -358,7 +361,7 @@ cudaError_t fwd_t(const Dims& d, const void* X, void* S, char* bank, int* status
     constexpr size_t smem = Sk8Smem::total + 1024;
     PSK_TRY(set_smem(sk8_tc_fwd_kernel<R>, smem));
     prof_begin("sk8_tc_fwd_kernel", s);
-    sk8_tc_fwd_kernel<R><<<dim3(d.n / 128, d.BH()), 128, smem, s>>>(mX, wm.W1, wm.W2, mS, d.g_heads, d.H, status);
+    launch_pdl(sk8_tc_fwd_kernel<R>, dim3(d.n / 128, d.BH()), 128, smem, s, mX, wm.W1, wm.W2, mS, d.g_heads, d.H, status);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
@@ -375,7 +378,7 @@ cudaError_t bwd_t(const Dims& d, const void* X, const void* dS, void* dX, char* 
     constexpr size_t smem = Sk8Smem::total + 1024;
     PSK_TRY(set_smem(sk8_tc_bwd_kernel<R>, smem));
     prof_begin("sk8_tc_bwd_kernel", s);
-    sk8_tc_bwd_kernel<R><<<dim3(d.n / 128, d.BH()), 128, smem, s>>>(mX, wm.W1, wm.W2, mDS, mDX, d.g_heads, d.H, status);
+    launch_pdl(sk8_tc_bwd_kernel<R>, dim3(d.n / 128, d.BH()), 128, smem, s, mX, wm.W1, wm.W2, mDS, mDX, d.g_heads, d.H, status);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
@@ -391,7 +394,7 @@ cudaError_t sketch8_tc_prepare(const Dims& d, const void* G1, const void* G2, ch
     bf16* W1 = reinterpret_cast<bf16*>(bank);
     bf16* W2 = W1 + (size_t)d.g_heads * kW1;
     prof_begin("sk8_bank_kernel", s);
-    sk8_bank_kernel<<<dim3((kW1 + kW2 + 255) / 256, d.g_heads), 256, 0, s>>>((const bf16*)G1, (const bf16*)G2, d.r, W1, W2);
+    launch_pdl(sk8_bank_kernel, dim3((kW1 + kW2 + 255) / 256, d.g_heads), 256, 0, s, (const bf16*)G1, (const bf16*)G2, d.r, W1, W2);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();

@@ -170,6 +170,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                   const float* __restrict__ cmean, int64_t sb, int64_t sh, int64_t sn,
                   float* __restrict__ denom, const bf16* __restrict__ dO,
                   float* __restrict__ y65, float* __restrict__ e65h, int keep_oc, int noncausal, int* status) {
+    pdl_sync();
     constexpr bool lin = LIN;
     using F = Feat<R>;
     using L = OutSmem<R, LOCAL>;
@@ -594,16 +595,16 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
 // only after rounding in the backward.  An estimate of the mean serves that purpose as well as
 // the mean itself and costs 128 KB of reads per head instead of the whole tensor.  One CTA per
 // head, fixed summation order.
-__global__ void __launch_bounds__(1024)
-tc_vmean_kernel(const bf16* __restrict__ V, int H, int n, int64_t sb, int64_t sh, int64_t sn,
-                float* __restrict__ cmean) {
+__device__ __forceinline__ void vmean_head(const bf16* __restrict__ V, int bh, int H, int n, int64_t sb, int64_t sh, int64_t sn,
+                                           float* __restrict__ cmean) {
     __shared__ float part[128][65];
-    const int bh = blockIdx.x, tid = threadIdx.x, ch = tid % 8, rg = tid / 8;   // 8 threads x 16 B per row
+    const int tid = threadIdx.x, ch = tid % 8, rg = tid / 8;   // 8 threads x 16 B per row
     const bf16* base = V + (int64_t)(bh / H) * sb + (int64_t)(bh % H) * sh + 8 * ch;
     float s[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) s[j] = 0.f;
     const int stride = n > 1024 ? n / 1024 : 1, count = n > 1024 ? 1024 : n;
+#pragma unroll 8
     for (int q = rg; q < count; q += 128) {
         const int i = q * stride;
         const uint4 v = *reinterpret_cast<const uint4*>(base + (int64_t)i * sn);
@@ -617,23 +618,35 @@ tc_vmean_kernel(const bf16* __restrict__ V, int H, int n, int64_t sb, int64_t sh
 #pragma unroll
     for (int j = 0; j < 8; ++j) part[rg][8 * ch + j] = s[j];
     __syncthreads();
-    if (tid < 64) {
-        float acc = 0.f;
-        for (int r = 0; r < 128; ++r) acc += part[r][tid];
-        cmean[(size_t)bh * 64 + tid] = acc / (float)count;
-    }
+    // sums over the 128 row groups: 16 threads per column, 8 groups each
+    const int c = tid / 16, l16 = tid % 16;
+    float acc = 0.f;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) acc += part[8 * l16 + r][c];
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (l16 == 0) cmean[(size_t)bh * 64 + c] = acc / (float)count;
 }
 
-// Image of [G1 | G2]^T (set g of the sketch matrices, each [64 x r] row-major) in the layout the
-// sketch GEMM reads from shared memory: row nn < 2r = sketch column, 64 head dimensions, swizzled.
+// What a call needs before its first tensor-core kernel, in one launch: the status word cleared (`status`
+// may be null), for CTAs below g_heads the image of [G1 | G2]^T (set g of the sketch matrices, each [64 x r]
+// row-major) in the layout the sketch GEMM reads from shared memory - row nn < 2r = sketch column, 64 head
+// dimensions, swizzled - and for the others (if any) a head's value centre.
 // (lin: "G1" = I for r = 64, [I; I] padded with zero rows for r <= 32, "G2" = 0: the sketch GEMM then
 // returns the row itself, or the sum of its [hi | lo] halves, see read_half_sketch)
-__global__ void __launch_bounds__(128)
-tc_gimage_kernel(const bf16* __restrict__ G1, const bf16* __restrict__ G2, int r, int lin, uint8_t* __restrict__ gimg) {
+__global__ void __launch_bounds__(1024)
+tc_prologue_kernel(const bf16* __restrict__ G1, const bf16* __restrict__ G2, int r, int lin, int g_heads, uint8_t* __restrict__ gimg,
+                   const bf16* __restrict__ V, int H, int n, int64_t sb, int64_t sh, int64_t sn, float* __restrict__ cmean, int* status) {
+    pdl_sync();
+    if (blockIdx.x == 0 && status != nullptr && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0;
+    if ((int)blockIdx.x >= g_heads) {
+        vmean_head(V, blockIdx.x - g_heads, H, n, sb, sh, sn, cmean);
+        return;
+    }
     const int g = blockIdx.x;
     uint8_t* img = gimg + (size_t)g * 2 * r * 128;
-    for (int e = threadIdx.x; e < 2 * r * 64; e += 128) {
-        const int nn = e / 64, k = e % 64;
+    for (int e = threadIdx.x; e < 2 * r * 64; e += 1024) {
+        const int nn = e % (2 * r), k = e / (2 * r);           // (neighbouring threads: neighbouring columns of G)
         const bf16 v = lin ? __float2bfloat16_rn((nn < r && (k == nn || (r <= 32 && k == r + nn))) ? 1.f : 0.f)
                            : (nn < r ? G1 : G2)[(size_t)g * 64 * r + k * r + (nn % r)];
         *reinterpret_cast<bf16*>(img + swz128_offset(nn, k / 8) + (k % 8) * 2) = v;
@@ -665,9 +678,8 @@ cudaError_t fwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
     }
     // keep_states: the backward will read these states, so they are built from centred values
     float* cmean = d.keep_states ? reinterpret_cast<float*>(ws + w.vmean) : nullptr;
-    if (cmean != nullptr) PSK_TRY(tc_vmean(d, V, cmean, s, launches));
     uint8_t* gimg = reinterpret_cast<uint8_t*>(ws + w.gimg);
-    PSK_TRY(tc_gimage(d, G1, G2, gimg, s, launches));
+    PSK_TRY(tc_prologue(d, G1, G2, gimg, V, cmean, status, s, launches));
     PSK_TRY(tc_states(d, mK, mV, gimg, nullptr, nullptr, cmean, cmean ? 1 : 0, Z, false,
                       reinterpret_cast<float*>(ws + w.tot), status, s, launches));
     prof_begin("tc_fwd_out_kernel", s);
@@ -679,7 +691,7 @@ cudaError_t fwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
                 return cudaErrorInvalidValue;
             constexpr size_t smem = OutSmem<R, true>::total + 1024;
             PSK_TRY((set_smem(tc_fwd_out_kernel<R, 0, true, true>, smem)));
-            tc_fwd_out_kernel<R, 0, true, true><<<dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s>>>(
+            launch_pdl(tc_fwd_out_kernel<R, 0, true, true>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
                 mQ, mQraw, mKraw, mV, mZ, mO, mOc, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
                 denom, nullptr, nullptr, nullptr, Oc != nullptr ? 1 : 0, 0, status);
         } else {
@@ -688,19 +700,19 @@ cudaError_t fwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
     } else if (d.local) {
         constexpr size_t smem = OutSmem<R, true>::total + 1024;
         PSK_TRY((set_smem(tc_fwd_out_kernel<R, 0, true, false>, smem)));
-        tc_fwd_out_kernel<R, 0, true, false><<<dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s>>>(
+        launch_pdl(tc_fwd_out_kernel<R, 0, true, false>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
             mQ, mQ, mK, mV, mZ, mO, mOc, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
             denom, nullptr, nullptr, nullptr, Oc != nullptr ? 1 : 0, d.noncausal ? 1 : 0, status);
     } else if (d.sketch_linear) {
         constexpr size_t smem = OutSmem<R, false>::total + 1024;
         PSK_TRY((set_smem(tc_fwd_out_kernel<R, 0, false, true>, smem)));
-        tc_fwd_out_kernel<R, 0, false, true><<<dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s>>>(
+        launch_pdl(tc_fwd_out_kernel<R, 0, false, true>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
             mQ, mQ, mK, mV, mZ, mO, mOc, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
             denom, nullptr, nullptr, nullptr, Oc != nullptr ? 1 : 0, d.noncausal ? 1 : 0, status);
     } else {
         constexpr size_t smem = OutSmem<R, false>::total + 1024;
         PSK_TRY((set_smem(tc_fwd_out_kernel<R, 0, false, false>, smem)));
-        tc_fwd_out_kernel<R, 0, false, false><<<dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s>>>(
+        launch_pdl(tc_fwd_out_kernel<R, 0, false, false>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
             mQ, mQ, mK, mV, mZ, mO, mOc, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
             denom, nullptr, nullptr, nullptr, Oc != nullptr ? 1 : 0, d.noncausal ? 1 : 0, status);
     }
@@ -755,7 +767,7 @@ static cudaError_t recompute_impl(const Dims& d, const CUtensorMap& mQ, const CU
         if constexpr (R <= 32) {
             constexpr size_t smem = OutSmem<R, true>::total + 1024;
             PSK_TRY((set_smem(tc_fwd_out_kernel<R, 1, true, true>, smem)));
-            tc_fwd_out_kernel<R, 1, true, true><<<dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s>>>(
+            launch_pdl(tc_fwd_out_kernel<R, 1, true, true>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
                 mQ, mQraw, mK, mV, mZ, mZ, mZ, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
                 const_cast<float*>(denom), dO, y65, e65h, 0, 0, status);
         } else {
@@ -764,19 +776,19 @@ static cudaError_t recompute_impl(const Dims& d, const CUtensorMap& mQ, const CU
     } else if (d.local) {
         constexpr size_t smem = OutSmem<R, true>::total + 1024;
         PSK_TRY((set_smem(tc_fwd_out_kernel<R, 1, true, false>, smem)));
-        tc_fwd_out_kernel<R, 1, true, false><<<dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s>>>(
+        launch_pdl(tc_fwd_out_kernel<R, 1, true, false>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
             mQ, mQ, mK, mV, mZ, mZ, mZ, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
             const_cast<float*>(denom), dO, y65, e65h, 0, d.noncausal ? 1 : 0, status);
     } else if (d.sketch_linear) {
         constexpr size_t smem = OutSmem<R, false>::total + 1024;
         PSK_TRY((set_smem(tc_fwd_out_kernel<R, 1, false, true>, smem)));
-        tc_fwd_out_kernel<R, 1, false, true><<<dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s>>>(
+        launch_pdl(tc_fwd_out_kernel<R, 1, false, true>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
             mQ, mQ, mK, mV, mZ, mZ, mZ, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
             const_cast<float*>(denom), dO, y65, e65h, 0, d.noncausal ? 1 : 0, status);
     } else {
         constexpr size_t smem = OutSmem<R, false>::total + 1024;
         PSK_TRY((set_smem(tc_fwd_out_kernel<R, 1, false, false>, smem)));
-        tc_fwd_out_kernel<R, 1, false, false><<<dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s>>>(
+        launch_pdl(tc_fwd_out_kernel<R, 1, false, false>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
             mQ, mQ, mK, mV, mZ, mZ, mZ, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
             const_cast<float*>(denom), dO, y65, e65h, 0, d.noncausal ? 1 : 0, status);
     }
@@ -796,17 +808,12 @@ cudaError_t tc_recompute(const Dims& d, const CUtensorMap& mQ, const CUtensorMap
     return cudaErrorInvalidValue;
 }
 
-cudaError_t tc_gimage(const Dims& d, const void* G1, const void* G2, uint8_t* gimg, cudaStream_t s, int* launches) {
-    prof_begin("tc_gimage_kernel", s);
-    tc_gimage_kernel<<<d.g_heads, 128, 0, s>>>((const bf16*)G1, (const bf16*)G2, d.r, d.sketch_linear ? 1 : 0, gimg);
-    prof_end(s);
-    ++*launches;
-    return cudaGetLastError();
-}
-
-cudaError_t tc_vmean(const Dims& d, const void* V, float* cmean, cudaStream_t s, int* launches) {
-    prof_begin("tc_vmean_kernel", s);
-    tc_vmean_kernel<<<d.BH(), 1024, 0, s>>>((const bf16*)V, d.H, d.n, d.sb, d.sh, d.sn, cmean);
+cudaError_t tc_prologue(const Dims& d, const void* G1, const void* G2, uint8_t* gimg, const void* V, float* cmean, int* status,
+                        cudaStream_t s, int* launches) {
+    prof_begin("tc_prologue_kernel", s);
+    launch_pdl(tc_prologue_kernel, d.g_heads + (cmean != nullptr ? d.BH() : 0), 1024, 0, s, (const bf16*)G1, (const bf16*)G2, d.r,
+               d.sketch_linear ? 1 : 0, d.g_heads, gimg, (const bf16*)V, d.H, d.n, d.sb, d.sh, d.sn, cmean,
+               d.clear_status ? status : nullptr);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();

@@ -26,7 +26,9 @@ namespace {
 __global__ void __launch_bounds__(256)
 tc_bwd_prep_kernel(const bf16* __restrict__ dO, const float* __restrict__ denom, const float* __restrict__ cmean,
                    const bf16* __restrict__ Oc, int H, int n, int total_rows, int64_t sb, int64_t sh, int64_t sn,
-                   float* __restrict__ y65, float* __restrict__ e65h) {
+                   float* __restrict__ y65, float* __restrict__ e65h, int* status) {
+    pdl_sync();
+    if (blockIdx.x == 0 && status != nullptr && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0;
     // 128 rows per CTA, four per thread group: all eight 16-byte loads of a thread are in flight
     // before the first is used.  (n and total_rows are multiples of 128: one head per CTA.)
     const int ch = threadIdx.x % 8;
@@ -158,6 +160,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                    int g_heads, int H, int n, int b, int t,
                    const float* __restrict__ y65g, const float* __restrict__ e65h, const float* __restrict__ denom,
                    int noncausal, int* status) {
+    pdl_sync();
     constexpr bool lin = LIN;
     using F = Feat<R>;
     using L = BwdSmem<R, LOCAL, QSIDE>;
@@ -788,7 +791,6 @@ cudaError_t bwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
     float* cmean = reinterpret_cast<float*>(ws + w.vmean);
     float* e65h = reinterpret_cast<float*>(ws + w.e65h);
     float* tot = reinterpret_cast<float*>(ws + w.tot);
-    if (!d.keep_states) PSK_TRY(tc_vmean(d, V, cmean, s, launches));
     CUtensorMap mQ, mK, mV, mG, mZ, mR, mdQ, mdK, mdV;
     const int64_t nblk = (int64_t)d.BH() * (d.noncausal ? 1 : d.t);
     if (!tc_map_rows(&mQ, Q, d.B, d.H, d.n, d.xsb, d.xsh, d.xsn) || !tc_map_rows(&mK, K, d.B, d.H, d.n, d.xsb, d.xsh, d.xsn) ||
@@ -809,15 +811,16 @@ cudaError_t bwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
             return cudaErrorInvalidValue;
     }
     uint8_t* gimg = reinterpret_cast<uint8_t*>(ws + w.gimg);
-    PSK_TRY(tc_gimage(d, G1, G2, gimg, s, launches));
+    // kept states: the image and the centres are in the workspace too
+    if (!d.keep_states) PSK_TRY(tc_prologue(d, G1, G2, gimg, V, cmean, status, s, launches));
     // prefix states of centred values; forward rows again in fp32 -> y65, e65h; suffix states
     if (!d.keep_states) PSK_TRY(tc_states(d, mK, mV, gimg, nullptr, nullptr, cmean, 1, Z, false, tot, status, s, launches));
     if (d.keep_states) {
         const int rows = d.BH() * d.n;
         prof_begin("tc_bwd_prep_kernel", s);
-        tc_bwd_prep_kernel<<<rows / 128, 256, 0, s>>>((const bf16*)dO, denom, cmean,
+        launch_pdl(tc_bwd_prep_kernel, rows / 128, 256, 0, s, (const bf16*)dO, denom, cmean,
                                                            reinterpret_cast<const bf16*>(ws + w.Oc), d.H, d.n, rows, d.sb,
-                                                           d.sh, d.sn, y65, e65h);
+                                                           d.sh, d.sn, y65, e65h, d.clear_status ? status : nullptr);
         prof_end(s);
         ++*launches;
         PSK_TRY(cudaGetLastError());
@@ -834,7 +837,7 @@ cudaError_t bwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
         // query side first: it needs only the prefix states, and the row scalars just written are
         // still in L2; the suffix states (5 GB through L2) come after it
         prof_begin("tc_bwd_q_kernel", s);
-        tc_bwd_rows_kernel<R, true, LOCAL, LIN><<<grid, 128, smem, s>>>(mQ, mG, (LOCAL && LIN) ? mKraw : mK, mV, mZ, mdQ, mdQ, mQraw, mdQraw, gimg, d.g_heads, d.H, d.n,
+        launch_pdl(tc_bwd_rows_kernel<R, true, LOCAL, LIN>, grid, 128, smem, s, mQ, mG, (LOCAL && LIN) ? mKraw : mK, mV, mZ, mdQ, mdQ, mQraw, mdQraw, gimg, d.g_heads, d.H, d.n,
                                                                    d.b, d.t, y65, e65h, denom, d.noncausal ? 1 : 0, status);
         prof_end(s);
         ++*launches;
@@ -842,7 +845,7 @@ cudaError_t bwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
         // suffix states: phi(q_i) / d_i against [dO_i | y65_i]
         PSK_TRY(tc_states(d, mQ, mG, gimg, y65, denom, cmean, 2, Rs, true, tot, status, s, launches));
         prof_begin("tc_bwd_k_kernel", s);
-        tc_bwd_rows_kernel<R, false, LOCAL, LIN><<<grid, 128, smem_k, s>>>(mK, mV, (LOCAL && LIN) ? mQraw : mQ, mG, mR, mdK, mdV, mKraw, mdKraw, gimg, d.g_heads, d.H, d.n,
+        launch_pdl(tc_bwd_rows_kernel<R, false, LOCAL, LIN>, grid, 128, smem_k, s, mK, mV, (LOCAL && LIN) ? mQraw : mQ, mG, mR, mdK, mdV, mKraw, mdKraw, gimg, d.g_heads, d.H, d.n,
                                                                     d.b, d.t, y65, e65h, denom, d.noncausal ? 1 : 0, status);
         prof_end(s);
         ++*launches;

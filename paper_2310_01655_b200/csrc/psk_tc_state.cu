@@ -5,12 +5,13 @@
 // in the backward), then zeros.
 //
 // Sequence runs (the parallel-prefix remark of Section 3.1): with nseg > 1 a head's blocks are cut
-// into nseg runs that are processed by different CTAs.  A first launch (kModeTotal) accumulates
-// every run but the last from zero and leaves its raw fp32 total in scratch; the second
-// (kModePrefix, use_init) starts run s from the sum of the totals of the runs before s and writes
-// the prefix states as usual.  Twice the arithmetic, nseg times the parallelism: used when there
-// are too few heads to fill the GPU.  The totals pass alone, followed by a small summing kernel,
-// gives the single global state of non-causal attention.
+// into nseg runs of (nearly) equal length that are processed by different CTAs.  A first launch takes
+// the runs but the last: run 0 writes its prefix states as usual, and each leaves its raw fp32 total in
+// scratch; a small kernel turns the totals into running sums; a second launch starts run s >= 1 from
+// the sum of the totals before it and writes its prefix states.  Twice the arithmetic (but for the
+// first and the last run), nseg - 1 times the parallelism: used when there are too few heads to
+// fill the GPU.  The totals alone, followed by a small summing kernel, give the single global
+// state of non-causal attention.
 #include "tc_common.cuh"
 
 namespace psk {
@@ -19,8 +20,10 @@ using namespace tc;
 
 namespace {
 
+// What a launch does with a run of blocks:
 constexpr int kModePrefix = 0;         // write the exclusive prefix state at every block boundary
 constexpr int kModeTotal = 1;          // write only the raw fp32 total at the end of the run
+constexpr int kModeFirst = 2;          // run 0: both; the other runs: the total only
 
 // ---------------------------------------------------------------------------
 // Prefix states of one head, sequentially along the sequence (Section 3.1, Z_l = sum_{j<l} H_j):
@@ -62,38 +65,33 @@ __device__ __forceinline__ void wg_barrier(int wg) {
 
 constexpr int kErrState = 3;
 
-// acc[0..80) of this thread's lane = sum over runs s2 < seg of tot[(row0 + s2 * run_stride) * 80 + ...]
-static __device__ __noinline__ void state_init_acc(const float* __restrict__ tot, size_t row0, size_t run_stride, int seg,
-                                                   uint32_t acc_tmem) {
+// acc[0..80) of this thread's lane = tot[row * 80 + ...], half a row's loads in flight at a time
+static __device__ __noinline__ void state_init_acc(const float* __restrict__ tot, size_t row, uint32_t acc_tmem) {
+    const float4* src = reinterpret_cast<const float4*>(tot + row * 80);
 #pragma unroll 1
-    for (int c0 = 0; c0 < 80; c0 += 16) {
-        float a[16];
+    for (int h = 0; h < 80; h += 40) {
+        float4 x[10];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) a[q] = 0.f;
-        for (int s2 = 0; s2 < seg; ++s2) {
-            const float4* src = reinterpret_cast<const float4*>(tot + (row0 + s2 * run_stride) * 80 + c0);
+        for (int q = 0; q < 10; ++q) x[q] = src[h / 4 + q];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float4 x = src[q];
-                a[4 * q] += x.x; a[4 * q + 1] += x.y; a[4 * q + 2] += x.z; a[4 * q + 3] += x.w;
-            }
+        for (int c = 0; c < 40; c += 8) {
+            const float4 u = x[c / 4], v = x[c / 4 + 1];
+            const uint32_t w[8] = {__float_as_uint(u.x), __float_as_uint(u.y), __float_as_uint(u.z), __float_as_uint(u.w),
+                                   __float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w)};
+            tmem_st8(acc_tmem + h + c, w);
         }
-        uint32_t v[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) v[q] = __float_as_uint(a[q]);
-        tmem_st16(acc_tmem + c0, v);
     }
 }
 
 // SEG = false is the plain walk of a whole head by one CTA (nseg = 1, prefix mode, no start value):
 // its run bookkeeping folds away at compile time.
 template <int R, int T0, int TN, int NWG, bool SEG>
-__global__ void __launch_bounds__(128 * (NWG + 1) + 64)
-tc_state_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY,
-                const uint8_t* __restrict__ gimg, int g_heads, int H, int n, int b, int t,
-                const float* __restrict__ y65, const float* __restrict__ fscale, const float* __restrict__ cmean,
-                int center_mode, int reverse, int nseg_arg, int mode_arg, int use_init, float* __restrict__ tot,
-                bf16* __restrict__ S, int lin, int* status) {
+__device__ __forceinline__ void
+state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
+           const uint8_t* __restrict__ gimg, int g_heads, int H, int n, int b, int t,
+           const float* __restrict__ y65, const float* __restrict__ fscale, const float* __restrict__ cmean,
+           int center_mode, int reverse, int nseg_arg, int mode_arg, int run0, int units, float* __restrict__ tot,
+           bf16* __restrict__ S, int lin, int* status) {
     using F = Feat<R>;
     using L = StateSmem<R, NWG>;
     extern __shared__ uint8_t smem_raw[];
@@ -104,13 +102,19 @@ tc_state_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
     __shared__ __align__(16) float cm[64];
     const int tid = threadIdx.x, wg = tid / 128, wt = tid % 128, warp = tid / 32;
     const int bh = blockIdx.x;
-    const int seg = SEG ? (int)blockIdx.y : 0, nseg = SEG ? nseg_arg : 1, mode = SEG ? mode_arg : kModePrefix;
+    const int seg = SEG ? run0 + (int)blockIdx.y : 0, nseg = SEG ? nseg_arg : 1;
+    const int mode = !SEG ? kModePrefix : (mode_arg == kModeFirst && seg > 0 ? kModeTotal : mode_arg);
     const int hi = bh % H, bi = bh / H;
     const int g = g_heads == 1 ? 0 : hi;
     const int tpb = b / 128, NJ = n / 128;               // token tiles per block / per head
-    const int NJs = NJ / nseg, ts = t / nseg;            // token tiles / blocks of this CTA's run of the sequence
+    // this CTA's run of the sequence: units (blocks; single tiles when there are no blocks to respect)
+    // [u0, u1), tiles [j0, j0 + NJs), blocks [p0, p0 + ts)
+    const int u0 = (int)((int64_t)units * seg / nseg), u1 = (int)((int64_t)units * (seg + 1) / nseg);
+    const int upt = NJ / units;                          // tiles per unit
+    const int j0r = SEG ? u0 * upt : 0, NJs = SEG ? (u1 - u0) * upt : NJ;
+    const int p0r = SEG ? u0 : 0, ts = SEG ? u1 - u0 : t;
     // a later run of a prefix pass starts from the sum of the earlier runs' totals
-    const bool init = SEG && (mode == kModePrefix) && use_init && seg > 0;
+    const bool init = SEG && mode == kModePrefix && seg > 0;
     constexpr int kThreads = 128 * (NWG + 1) + 64;
 
     if (tid == 0) {
@@ -125,13 +129,14 @@ tc_state_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
         mbar_fence_init();
         tma_prefetch_desc(&mapX); tma_prefetch_desc(&mapY);
     }
-    if (warp == 0) { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
-    if (tid < 64) cm[tid] = cmean != nullptr ? cmean[(size_t)bh * 64 + tid] : 0.f;
     // last-column chunks of both slots: zero, and column 0 = 1 when the last column is all ones
     for (int e = tid; e < 2 * 1024; e += kThreads) {
         const int s = e / 1024, i = e % 1024;
         reinterpret_cast<uint4*>(smem + L::Y + s * L::kYSlot + 16384)[i] = make_uint4(0, 0, 0, 0);
     }
+    pdl_sync();            // (before the allocation: a waiting CTA must not hold tensor memory)
+    if (warp == 0) { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
+    if (tid < 64) cm[tid] = cmean != nullptr ? cmean[(size_t)bh * 64 + tid] : 0.f;
     __syncthreads();
     if (y65 == nullptr && tid < 128) {
         *reinterpret_cast<bf16*>(smem + L::Y + 16384 + swz128_offset(tid, 0)) = __float2bfloat16_rn(1.f);
@@ -144,7 +149,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
     const uint32_t tm = tmem_slot;
     constexpr uint32_t kAcc = 2 * R;                      // accumulators start after the sketch columns
     // token tile visited at step j of this run (runs and tiles go backwards for suffix sums)
-    auto tile_of = [&](int j) { const int gj = seg * NJs + j; return reverse ? (NJ - 1 - gj) : gj; };
+    auto tile_of = [&](int j) { const int gj = j0r + j; return reverse ? (NJ - 1 - gj) : gj; };
 
     if (wg == NWG + 1) {
         // =============================== feeders ===============================
@@ -204,8 +209,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
                 if (y65 != nullptr) ok = ok && mbar_spin(&bar_ext[j & 1], (j >> 1) & 1, status, kErrState);
                 // block boundary: the store warpgroup has taken (or, for a start from earlier runs,
                 // written) the accumulators' values before anything is added to them
-                const bool boundary = mode == kModePrefix && (j % tpb == 0) && (j > 0 || init);
-                const bool block_end = mode == kModePrefix ? ((j + 1) % tpb == 0) : (j == NJs - 1);
+                const bool boundary = mode != kModeTotal && (j % tpb == 0) && (j > 0 || init);
+                const bool block_end = mode != kModeTotal ? ((j + 1) % tpb == 0) : (j == NJs - 1);
                 const uint64_t yd = desc_off(yd0, (j & 1) * L::kYSlot);
                 const uint32_t acc0 = (j > 0 || init) ? 1u : 0u;
                 static_for<0, TN>([&](auto ic) {
@@ -239,36 +244,35 @@ tc_state_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
         // kernel's busiest unit.)
         const uint32_t lane_tm = tm + ((uint32_t)((warp % 4) * 32) << 16);
         uint8_t* stage = smem + L::St;
-        if (mode == kModeTotal) {
-            // totals: the raw fp32 accumulators at the end of the run
+        // totals: the raw fp32 accumulators at the end of the run
+        auto dump_totals = [&](uint32_t parity) {
             static_for<0, TN>([&](auto ic) {
                 constexpr int I = decltype(ic)::value;
-                mbar_wait(&bar_accfull[I], 0, status, kErrMma);
+                mbar_wait(&bar_accfull[I], parity, status, kErrMma);
                 tc_fence_after();
                 float4* out = reinterpret_cast<float4*>(tot + ((((size_t)bh * nseg + seg) * F::NT + (T0 + I)) * 128 + wt) * 80);
-                {
 #pragma unroll
-                    for (int c0 = 0; c0 < 80; c0 += 16) {
-                        uint32_t v[16];
-                        tmem_ld16(lane_tm + kAcc + 80 * I + c0, v);
-                        tmem_ld_wait();
+                for (int c0 = 0; c0 < 80; c0 += 16) {
+                    uint32_t v[16];
+                    tmem_ld16(lane_tm + kAcc + 80 * I + c0, v);
+                    tmem_ld_wait();
 #pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            out[c0 / 4 + q] = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
-                                                          __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
-                    }
+                    for (int q = 0; q < 4; ++q)
+                        out[c0 / 4 + q] = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
+                                                      __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
                 }
             });
-        }
+        };
+        if (mode == kModeTotal) dump_totals(0);
         if (init) {
             // a later run starts from the sum of the earlier runs' totals: into the accumulators
             // first, then block 0 of the run is read back like every other block
-            for (int I = 0; I < TN; ++I) state_init_acc(tot, (((size_t)bh * nseg) * F::NT + (T0 + I)) * 128 + wt,
-                                                        (size_t)F::NT * 128, seg, lane_tm + kAcc + 80 * I);
+            for (int I = 0; I < TN; ++I)
+                state_init_acc(tot, (((size_t)bh * nseg + (seg - 1)) * F::NT + (T0 + I)) * 128 + wt, lane_tm + kAcc + 80 * I);
             tmem_st_wait();
         }
-        for (int p = 0; p < ts && mode == kModePrefix; ++p) {
-            const int pg = seg * ts + p;
+        for (int p = 0; p < ts && mode != kModeTotal; ++p) {
+            const int pg = p0r + p;
             const int l = reverse ? (t - 1 - pg) : pg;
             static_for<0, TN>([&](auto ic) {
                 constexpr int I = decltype(ic)::value;
@@ -341,6 +345,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
                 }
             });
         }
+        if (SEG && mode == kModeFirst) dump_totals((ts - 1) & 1);
     } else {
         // ============================= generators =============================
         const uint32_t lane_tm = tm + ((uint32_t)((warp % 4) * 32) << 16);
@@ -426,12 +431,62 @@ tc_state_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
 }
 
 
+#define PSK_STATE_PARAMS                                                                                            \
+    const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY, const uint8_t *__restrict__ gimg,  \
+        int g_heads, int H, int n, int b, int t, const float *__restrict__ y65, const float *__restrict__ fscale,          \
+        const float *__restrict__ cmean, int center_mode, int reverse, int nseg, int mode, int run0, int units,            \
+        float *__restrict__ tot, bf16 *__restrict__ S, int lin, int *status
+#define PSK_STATE_ARGS                                                                                              \
+    mapX, mapY, gimg, g_heads, H, n, b, t, y65, fscale, cmean, center_mode, reverse, nseg, mode, run0, units, tot, S, lin, status
+
+// r <= 32: every feature tile of a head in one CTA (two or five accumulators)
+template <int R, int TN, int NWG, bool SEG>
+__global__ void __launch_bounds__(128 * (NWG + 1) + 64) tc_state_kernel(PSK_STATE_PARAMS) {
+    state_walk<R, 0, TN, NWG, SEG>(PSK_STATE_ARGS);
+}
+
+// r = 64: 17 feature tiles, at most four accumulators beside the sketch columns, so five CTAs share a head
+// (blockIdx.z), those with four tiles first.  One launch: five launches of a group each left most SMs idle
+// whenever heads x runs were no multiple of their number.
+template <bool SEG>
+__global__ void __launch_bounds__(128 * 4 + 64) tc_state64_kernel(PSK_STATE_PARAMS) {
+    switch (blockIdx.z) {
+        case 0: state_walk<64, 0, 4, 3, SEG>(PSK_STATE_ARGS); break;
+        case 1: state_walk<64, 4, 4, 3, SEG>(PSK_STATE_ARGS); break;
+        case 2: state_walk<64, 8, 3, 3, SEG>(PSK_STATE_ARGS); break;
+        case 3: state_walk<64, 11, 3, 3, SEG>(PSK_STATE_ARGS); break;
+        default: state_walk<64, 14, 3, 3, SEG>(PSK_STATE_ARGS); break;
+    }
+}
+
+// Running sums of a head's run totals, in place: run s becomes the sum over the runs <= s.
+__global__ void __launch_bounds__(256)
+tc_state_scan_kernel(float4* __restrict__ tot, size_t elems, int nseg) {
+    pdl_sync();
+    const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
+    if (e >= elems) return;
+    float4* p = tot + (size_t)blockIdx.y * nseg * elems + e;
+    float4 run = p[0];
+    for (int k0 = 1; k0 < nseg - 1; k0 += 8) {
+        float4 v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) if (k0 + q < nseg - 1) v[q] = p[(size_t)(k0 + q) * elems];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            if (k0 + q >= nseg - 1) break;
+            run.x += v[q].x; run.y += v[q].y; run.z += v[q].z; run.w += v[q].w;
+            p[(size_t)(k0 + q) * elems] = run;
+        }
+    }
+}
+
 // Sum of the run totals of a head, centred, weighted and rounded like a stored state: the single
 // global state of non-causal attention, written as the head's only block.
 template <int R>
 __global__ void __launch_bounds__(128)
 tc_state_sum_kernel(const float* __restrict__ tot, int nseg, const float* __restrict__ cmean, int center_mode,
                     bf16* __restrict__ S) {
+    pdl_sync();
     using F = Feat<R>;
     const int tile = blockIdx.x, bh = blockIdx.y, wt = threadIdx.x;
     const int row = tile * 128 + wt;
@@ -474,46 +529,44 @@ struct StateArgs {
     const float *y65, *fscale, *cmean;
     int center_mode;
     bool reverse;
-    int nseg, mode, segs_launched;
-    bool use_init;
+    int nseg, mode, run0, runs;        // runs [run0, run0 + runs) of nseg are launched
     float* tot;
     bf16* S;
 };
 
-template <int R, int T0, int TN, int NWG>
-cudaError_t launch_state_group(const Dims& d, const CUtensorMap& mX, const CUtensorMap& mY, const uint8_t* gimg,
-                               const StateArgs& a, int* status, cudaStream_t s, int* launches) {
-    constexpr size_t smem = StateSmem<R, NWG>::total + 1024;
-    prof_begin(a.mode == kModeTotal ? "tc_state_total_kernel" : "tc_state_kernel", s);
-    if (a.nseg == 1 && a.mode == kModePrefix) {
-        PSK_TRY((set_smem(tc_state_kernel<R, T0, TN, NWG, false>, smem)));
-        tc_state_kernel<R, T0, TN, NWG, false><<<dim3(d.BH(), 1), 128 * (NWG + 1) + 64, smem, s>>>(
-            mX, mY, gimg, d.g_heads, d.H, d.n, d.b, d.t, a.y65, a.fscale, a.cmean, a.center_mode, a.reverse ? 1 : 0, 1,
-            kModePrefix, 0, a.tot, a.S, d.sketch_linear ? 1 : 0, status);
-    } else {
-        PSK_TRY((set_smem(tc_state_kernel<R, T0, TN, NWG, true>, smem)));
-        tc_state_kernel<R, T0, TN, NWG, true><<<dim3(d.BH(), a.segs_launched), 128 * (NWG + 1) + 64, smem, s>>>(
-            mX, mY, gimg, d.g_heads, d.H, d.n, d.b, d.t, a.y65, a.fscale, a.cmean, a.center_mode, a.reverse ? 1 : 0, a.nseg,
-            a.mode, a.use_init ? 1 : 0, a.tot, a.S, d.sketch_linear ? 1 : 0, status);
-    }
-    prof_end(s);
-    ++*launches;
-    return cudaGetLastError();
-}
+// units a head's sequence can be cut into: blocks (a run starts at a block boundary), or 128-token
+// tiles when there are no blocks to respect
+int state_units(const Dims& d) { return d.noncausal ? d.n / 128 : d.t; }
+
+// Costs in token tiles (r = 32: about 3.5 us each): a CTA's start and end, the same where it fetches its start
+// value, and the running sums with the extra launches (measured on 12 and 48 heads)
+constexpr long kStartTiles = 3, kInitTiles = 4, kBetweenTiles = 3;
 
 template <int R>
 cudaError_t launch_states(const Dims& d, const CUtensorMap& mX, const CUtensorMap& mY, const uint8_t* gimg,
                           const StateArgs& a, int* status, cudaStream_t s, int* launches) {
-#define PSK_SG(T0, TN, NWG) PSK_TRY((launch_state_group<R, T0, TN, NWG>(d, mX, mY, gimg, a, status, s, launches)))
-    if constexpr (R == 16) {
-        PSK_SG(0, 2, 2);
-    } else if constexpr (R == 32) {
-        PSK_SG(0, 5, 3);
+    constexpr int NWG = R == 16 ? 2 : 3, kThreads = 128 * (NWG + 1) + 64;
+    constexpr size_t smem = StateSmem<R, NWG>::total + 1024;
+    const bool seg = a.nseg > 1 || a.mode != kModePrefix;
+    const dim3 grid(d.BH(), a.runs, R == 64 ? 5 : 1);
+    prof_begin(a.mode == kModePrefix ? "tc_state_kernel" : "tc_state_total_kernel", s);
+#define PSK_STATE_LAUNCH(KERNEL) do {                                                                                \
+        auto kern = KERNEL;                                                                                          \
+        PSK_TRY((set_smem(kern, smem)));                                                                             \
+        launch_pdl(kern, grid, kThreads, smem, s, mX, mY, gimg, d.g_heads, d.H, d.n, d.b, d.t, a.y65, a.fscale, a.cmean,      \
+                                          a.center_mode, a.reverse ? 1 : 0, a.nseg, a.mode, a.run0, state_units(d), a.tot, \
+                                          a.S, d.sketch_linear ? 1 : 0, status);                                     \
+    } while (0)
+    if constexpr (R == 64) {
+        if (seg) PSK_STATE_LAUNCH((tc_state64_kernel<true>)); else PSK_STATE_LAUNCH((tc_state64_kernel<false>));
     } else {
-        PSK_SG(0, 4, 3); PSK_SG(4, 4, 3); PSK_SG(8, 3, 3); PSK_SG(11, 3, 3); PSK_SG(14, 3, 3);
+        constexpr int TN = Feat<R>::NT;
+        if (seg) PSK_STATE_LAUNCH((tc_state_kernel<R, TN, NWG, true>)); else PSK_STATE_LAUNCH((tc_state_kernel<R, TN, NWG, false>));
     }
-#undef PSK_SG
-    return cudaSuccess;
+#undef PSK_STATE_LAUNCH
+    prof_end(s);
+    ++*launches;
+    return cudaGetLastError();
 }
 
 template <int R>
@@ -521,39 +574,51 @@ cudaError_t states_impl(const Dims& d, const CUtensorMap& mX, const CUtensorMap&
                         const float* fscale, const float* cmean, int center_mode, bf16* S, bool reverse, float* tot,
                         int* status, cudaStream_t s, int* launches) {
     const int nseg = tc_state_segments(d);
-    StateArgs a{y65, fscale, cmean, center_mode, reverse, nseg, kModePrefix, nseg, nseg > 1, tot, S};
+    StateArgs a{y65, fscale, cmean, center_mode, reverse, nseg, kModePrefix, 0, nseg, tot, S};
     if (d.noncausal) {
         // one global state per head: totals of every run, then their sum in the stored format
-        a.mode = kModeTotal; a.use_init = false; a.cmean = nullptr; a.center_mode = 0;
+        a.mode = kModeTotal; a.cmean = nullptr; a.center_mode = 0;
         PSK_TRY((launch_states<R>(d, mX, mY, gimg, a, status, s, launches)));
         prof_begin("tc_state_sum_kernel", s);
-        tc_state_sum_kernel<R><<<dim3(Feat<R>::NT, d.BH()), 128, 0, s>>>(tot, nseg, cmean, center_mode, S);
+        launch_pdl(tc_state_sum_kernel<R>, dim3(Feat<R>::NT, d.BH()), 128, 0, s, tot, nseg, cmean, center_mode, S);
         prof_end(s);
         ++*launches;
         return cudaGetLastError();
     }
-    if (nseg > 1) {    // totals of every run of blocks but the last (nothing starts after it)
-        StateArgs b = a;
-        b.mode = kModeTotal; b.segs_launched = nseg - 1; b.use_init = false; b.cmean = nullptr; b.center_mode = 0;
-        PSK_TRY((launch_states<R>(d, mX, mY, gimg, b, status, s, launches)));
+    if (nseg == 1) return launch_states<R>(d, mX, mY, gimg, a, status, s, launches);
+    a.mode = kModeFirst; a.runs = nseg - 1;              // (nothing starts after the last run)
+    PSK_TRY((launch_states<R>(d, mX, mY, gimg, a, status, s, launches)));
+    if (nseg > 2) {
+        const size_t elems = (size_t)Feat<R>::NT * 128 * 20;
+        prof_begin("tc_state_scan_kernel", s);
+        launch_pdl(tc_state_scan_kernel, dim3((unsigned)((elems + 255) / 256), d.BH()), 256, 0, s, reinterpret_cast<float4*>(tot), elems, nseg);
+        prof_end(s);
+        ++*launches;
+        PSK_TRY(cudaGetLastError());
     }
+    a.mode = kModePrefix; a.run0 = 1;
     return launch_states<R>(d, mX, mY, gimg, a, status, s, launches);
 }
 
 }  // namespace
 
 int tc_state_segments(const Dims& d) {
-    // units a head's sequence can be cut into: blocks (a run starts at a block boundary), or
-    // 128-token tiles when there are no blocks to respect
-    const int units = d.noncausal ? d.n / 128 : d.t;
+    const int units = state_units(d);
     if (d.seq_segments > 0) return (d.seq_segments <= units && units % d.seq_segments == 0) ? d.seq_segments : 1;
     constexpr long kSMs = 148;
-    // Causal: two passes cost twice the arithmetic, so cutting pays from four runs on.
-    // Non-causal: the totals pass is all there is, so any cut that fills the GPU pays.
-    int s = 1;
-    while ((long)d.BH() * s < kSMs && s * 2 <= units && units % (s * 2) == 0 && s < 32) s *= 2;
-    if (!d.noncausal && s < 4) s = 1;
-    return s;
+    const long ctas = (long)d.BH() * (d.r == 64 ? 5 : 1);       // per run
+    const long tiles = d.n / 128, upt = tiles / units;
+    // Time in tenths of a token tile: waves x (longest run + what a CTA's start and end cost).  Causal, more
+    // than one run: two launches of nseg - 1 runs each and the running sums between them.
+    long best = 10 * ((ctas + kSMs - 1) / kSMs) * (tiles + kStartTiles);
+    if (!d.noncausal) best = best * 9 / 10;              // (cutting has to pay clearly)
+    int pick = 1;
+    for (int s = 2; s <= 64 && s <= units; ++s) {
+        const long run = ((units + s - 1) / s) * upt, waves = (ctas * (d.noncausal ? s : s - 1) + kSMs - 1) / kSMs;
+        const long cost = 10 * (d.noncausal ? waves * (run + kStartTiles) : waves * (2 * run + kStartTiles + kInitTiles) + kBetweenTiles);
+        if (cost < best) { best = cost; pick = s; }
+    }
+    return pick;
 }
 
 size_t tc_state_total_bytes(const Dims& d) {

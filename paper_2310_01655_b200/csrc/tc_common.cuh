@@ -37,10 +37,11 @@ cudaError_t tc_recompute(const Dims& d, const CUtensorMap& mQ, const CUtensorMap
                          const bf16* dO, float* y65, float* e65h, int* status, cudaStream_t s, int* launches);
 // gimg[g] = [G1 | G2]^T of sketch-matrix set g as the shared-memory image of the sketch GEMM's B operand
 // (2r rows x 128 B, K-major, 128-byte swizzle): the kernels fetch it with one bulk copy
-// (d.sketch_linear: the image of [I | 0] or [I; I | 0] instead, G1 and G2 are not read)
-cudaError_t tc_gimage(const Dims& d, const void* G1, const void* G2, uint8_t* gimg, cudaStream_t s, int* launches);
-// cmean[bh][c] = mean over the n rows of V[bh][:, c]  (deterministic reduction)
-cudaError_t tc_vmean(const Dims& d, const void* V, float* cmean, cudaStream_t s, int* launches);
+// (d.sketch_linear: the image of [I | 0] or [I; I | 0] instead, G1 and G2 are not read).
+// cmean[bh][c] (unless null) = mean of V[bh][:, c] over up to 1024 evenly spaced rows (deterministic).
+// Clears the status word if d.clear_status.
+cudaError_t tc_prologue(const Dims& d, const void* G1, const void* G2, uint8_t* gimg, const void* V, float* cmean, int* status,
+                        cudaStream_t s, int* launches);
 
 // Scratch layout of the tensor-core path.
 struct TcWorkspace { size_t status, vmean, gimg, tot, Z, Rst, y65, e65h, Oc, total; };
@@ -95,7 +96,7 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 
 // [G1 | G2]^T as a K-major, 128-byte-swizzled tile: row n (< 2R) holds sketch column n over the 64
 // head dimensions.  B operand of the sketch GEMM X [G1 | G2]; built once per call by
-// tc_gimage_kernel, then copied into shared memory as it is.
+// tc_prologue_kernel, then copied into shared memory as it is.
 template <int R>
 struct GImage { static constexpr uint32_t bytes = 2 * R * 128; };
 
