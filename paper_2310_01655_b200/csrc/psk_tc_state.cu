@@ -549,11 +549,15 @@ cudaError_t launch_states(const Dims& d, const CUtensorMap& mX, const CUtensorMa
     constexpr size_t smem = StateSmem<R, NWG>::total + 1024;
     const bool seg = a.nseg > 1 || a.mode != kModePrefix;
     const dim3 grid(d.BH(), a.runs, R == 64 ? 5 : 1);
+    // A long walk is better spread over the SMs by an ordinary launch: started early, its CTAs settle on the SMs
+    // that happen to be free first, several to a pair (r = 64, 48 heads of 128 tiles: 6.93 against 7.33 ms a step);
+    // for a short one the launch itself counts more (48 heads of 21 tiles: 374 -> 361 us a step).
+    const bool early = d.n / 128 / a.nseg <= 24;
     prof_begin(a.mode == kModePrefix ? "tc_state_kernel" : "tc_state_total_kernel", s);
 #define PSK_STATE_LAUNCH(KERNEL) do {                                                                                \
         auto kern = KERNEL;                                                                                          \
         PSK_TRY((set_smem(kern, smem)));                                                                             \
-        launch_pdl(kern, grid, kThreads, smem, s, mX, mY, gimg, d.g_heads, d.H, d.n, d.b, d.t, a.y65, a.fscale, a.cmean,      \
+        launch_pdl_if(early, kern, grid, kThreads, smem, s, mX, mY, gimg, d.g_heads, d.H, d.n, d.b, d.t, a.y65, a.fscale, a.cmean,      \
                                           a.center_mode, a.reverse ? 1 : 0, a.nseg, a.mode, a.run0, state_units(d), a.tot, \
                                           a.S, d.sketch_linear ? 1 : 0, status);                                     \
     } while (0)
