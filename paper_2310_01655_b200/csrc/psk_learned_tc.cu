@@ -716,17 +716,27 @@ ltc_wide_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ 
 // ---------------------------------------------------------------------------
 // weight gradients: Gt[256][64] += sum over a slab of rows of P[row][:]^T S[row][:]
 // (P: [rows][256] bf16, S: [rows][64] bf16; both tiles go to the tensor cores as TMA left them:
-// P^T is an MN-major A operand, S an MN-major B operand, the contraction runs over the rows)
+// P^T is an MN-major A operand, S an MN-major B operand, the contraction runs over the rows).
+// The column sums of the delta operand (the bias gradients, and what the folded normalisation gains
+// need) are products with ones on the same tiles: P^T 1 (wide delta) or 1^T S (narrow).
+// One CTA per SM with one slab of tiles.  Bound: the 80 KB a tile takes from memory.  (With the sums
+// added up by four warps from shared memory, two bytes at a time, and twice as many CTAs adding
+// their results in scattered 4-byte atomics, 393 216 rows took 118 us; now 54.)
 // ---------------------------------------------------------------------------
 constexpr int kWgStage = 65536 + 16384;
-constexpr int kWgSmem = 2 * kWgStage + 1024;
+constexpr int kWgSmem = 2 * kWgStage + 32768 + 1024;
 
-__global__ void __launch_bounds__(160)
+__device__ __forceinline__ void red_add4(float* dst, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(__uint_as_float(a)), "f"(__uint_as_float(b)),
+                 "f"(__uint_as_float(c)), "f"(__uint_as_float(d)) : "memory");
+}
+
+__global__ void __launch_bounds__(128)
 ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mP, const __grid_constant__ CUtensorMap mS, float* __restrict__ Gt,
                  float* __restrict__ colsum, int sum_wide, int ntiles, int tiles_per_cta, int* status) {
-    pdl_sync();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
+    uint8_t* ones = smem + 2 * kWgStage;              // two [128 rows x 64 columns] tiles of ones
     __shared__ uint64_t bar_full[2], bar_free[2], bar_done;
     __shared__ uint32_t tm_slot;
     const int tid = threadIdx.x, warp = tid / 32;
@@ -735,15 +745,19 @@ ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mP, const __grid_constant__
     if (tid == 0) {
         cta_giveup_init();
         mbar_init(&bar_full[0], 1); mbar_init(&bar_full[1], 1);
-        mbar_init(&bar_free[0], 5); mbar_init(&bar_free[1], 5);        // the tile's MMAs and the four summing warps
+        mbar_init(&bar_free[0], 1); mbar_init(&bar_free[1], 1);
         mbar_init(&bar_done, 1);
         mbar_fence_init();
     }
-    if (warp == 0) { tmem_alloc(&tm_slot, 128); tmem_relinquish(); }
+    for (int e = tid; e < 2048; e += 128) reinterpret_cast<uint4*>(ones)[e] = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
+    fence_proxy_async_smem();
+    pdl_sync();
+    if (warp == 0) { tmem_alloc(&tm_slot, 256); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tm = tm_slot;
+    constexpr uint32_t kSum = 128;                    // columns of the sums
     if (tid == 0) {
         auto load = [&](int j) {
             const int s = j & 1;
@@ -755,7 +769,8 @@ ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mP, const __grid_constant__
         };
         load(0);
         if (T > 1) load(1);
-        constexpr uint32_t idesc = idesc_bf16(128, 64, true, true);
+        constexpr uint32_t idesc = idesc_bf16(128, 64, true, true), idesc1 = idesc_bf16(128, 16, true, true);
+        const uint64_t oneb = smem_desc(smem_u32(ones), 0, 1024, kSwz128), onea = smem_desc(smem_u32(ones), 16384, 1024, kSwz128);
         bool ok = true;
         for (int j = 0; j < T && ok; ++j) {
             const int s = j & 1;
@@ -770,6 +785,16 @@ ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mP, const __grid_constant__
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
                     umma_ss(tm + half * 64, desc_off(pd, k * 2048), desc_off(sd, k * 2048), idesc, (j > 0 || k > 0) ? 1u : 0u);
+                if (sum_wide) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        umma_ss(tm + kSum + half * 16, desc_off(pd, k * 2048), desc_off(oneb, k * 2048), idesc1, (j > 0 || k > 0) ? 1u : 0u);
+                }
+            }
+            if (!sum_wide) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    umma_ss(tm + kSum, desc_off(onea, k * 2048), desc_off(sd, k * 2048), idesc, (j > 0 || k > 0) ? 1u : 0u);
             }
             umma_commit(&bar_free[s]);
             if (j + 2 < T) {
@@ -778,46 +803,11 @@ ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mP, const __grid_constant__
             }
         }
         if (ok) umma_commit(&bar_done);
-    } else if (warp >= 1) {
-        // Warps 1-4: column sums of the delta operand (the wide one's 256 columns, two per thread,
-        // or the narrow one's 64) from the tiles while they sit in shared memory: the bias
-        // gradients, and what the folded normalisation gains need.
-        const int j0 = tid - 32;
-        float acc0 = 0.f, acc1 = 0.f;
-        bool ok = true;
-        for (int j = 0; j < T; ++j) {
-            const int s = j & 1;
-            if (ok) ok = mbar_wait(&bar_full[s], (j >> 1) & 1, status, kErrTma);
-            if (ok) {
-                const uint8_t* st = smem + s * kWgStage;
-                if (sum_wide) {
-                    const uint8_t* c0p = st + (j0 / 64) * 16384 + (j0 % 8) * 2;
-                    const uint8_t* c1p = c0p + 32768;
-                    const uint32_t ch = (j0 % 64) / 8;
-#pragma unroll 8
-                    for (int row = 0; row < 128; ++row) {
-                        const uint32_t o = swz128_offset(row, ch);
-                        acc0 += __bfloat162float(*reinterpret_cast<const bf16*>(c0p + o));
-                        acc1 += __bfloat162float(*reinterpret_cast<const bf16*>(c1p + o));
-                    }
-                } else if (j0 < 64) {
-                    const uint8_t* cp = st + 65536 + (j0 % 8) * 2;
-                    const uint32_t ch = j0 / 8;
-#pragma unroll 8
-                    for (int row = 0; row < 128; ++row) acc0 += __bfloat162float(*reinterpret_cast<const bf16*>(cp + swz128_offset(row, ch)));
-                }
-            }
-            __syncwarp();
-            if (tid % 32 == 0) mbar_arrive(&bar_free[s]);      // (also after a failed wait: the issuer must not be left waiting)
-        }
-        if (ok && colsum != nullptr) {
-            if (sum_wide) { atomicAdd(colsum + j0, acc0); atomicAdd(colsum + j0 + 128, acc1); }
-            else if (j0 < 64) atomicAdd(colsum + j0, acc0);
-        }
     }
+    __syncwarp();
     const bool ok = mbar_wait(&bar_done, 0, status, kErrMma);
     tc_fence_after();
-    if (ok && warp < 4) {
+    if (ok) {
         const uint32_t lane_tm = tm + ((uint32_t)(warp * 32) << 16);
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
@@ -828,13 +818,31 @@ ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mP, const __grid_constant__
                 tmem_ld_wait();
                 float* dst = Gt + (size_t)(half * 128 + tid) * 64 + c0;
 #pragma unroll
-                for (int j = 0; j < 32; ++j) atomicAdd(dst + j, __uint_as_float(u[j]));
+                for (int j = 0; j < 32; j += 4) red_add4(dst + j, u[j], u[j + 1], u[j + 2], u[j + 3]);
+            }
+        }
+        if (sum_wide) {                               // every column of the product with ones is the sum
+            uint32_t u[32];
+            tmem_ld32(lane_tm + kSum, u);
+            tmem_ld_wait();
+            atomicAdd(colsum + tid, __uint_as_float(u[0]));
+            atomicAdd(colsum + 128 + tid, __uint_as_float(u[16]));
+        } else if (warp == 0) {                       // ... and every row
+#pragma unroll
+            for (int c0 = 0; c0 < 64; c0 += 32) {
+                uint32_t u[32];
+                tmem_ld32(lane_tm + kSum + c0, u);
+                tmem_ld_wait();
+                if (tid == 0) {
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4) red_add4(colsum + c0 + j, u[j], u[j + 1], u[j + 2], u[j + 3]);
+                }
             }
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 128);
+    if (warp == 0) tmem_dealloc(tm, 256);
 }
 
 // ---------------------------------------------------------------------------
@@ -1154,11 +1162,11 @@ cudaError_t narrow(const CUtensorMap& mA, const CUtensorMap& mA2, const CUtensor
 cudaError_t wgrad(const CUtensorMap& mP, const CUtensorMap& mS, float* Gt, float* colsum, bool wide, int tiles, int* status,
                   cudaStream_t s, int* launches) {
     PSK_TRY(set_smem(ltc_wgrad_kernel, kWgSmem));
-    int per = (tiles + 295) / 296;            // about two CTAs per SM, but at least four tiles per result added
+    int per = (tiles + 147) / 148;            // one CTA per SM, but at least four tiles per result added
     if (per < 4) per = tiles < 4 ? tiles : 4;
     const int grid = (tiles + per - 1) / per;
     prof_begin("ltc_wgrad_kernel", s);
-    launch_pdl(ltc_wgrad_kernel, grid, 160, kWgSmem, s, mP, mS, Gt, colsum, wide ? 1 : 0, tiles, per, status);
+    launch_pdl(ltc_wgrad_kernel, grid, 128, kWgSmem, s, mP, mS, Gt, colsum, wide ? 1 : 0, tiles, per, status);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
