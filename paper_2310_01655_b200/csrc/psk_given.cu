@@ -56,11 +56,12 @@ cudaError_t half_sketches(const Dims& d, const void* Q, const void* K, const voi
     const void* X[2] = {Q, K};
     const size_t so[2] = {w.Sq, w.Sk};
     int* status = reinterpret_cast<int*>(ws + w.tc);
-    if (d.learned) PSK_TRY(learned_tc_prepare(d, backward, ws + w.sketch, s, launches));
+    const bool full = backward || d.keep_states;
+    if (d.learned) PSK_TRY(learned_tc_prepare(d, full, backward, ws + w.sketch, s, launches));
     else PSK_TRY(sketch8_tc_prepare(d, G1, G2, ws + w.sketch, s, launches));
     if (kept) return cudaSuccess;
     for (int i = 0; i < 2; ++i) {
-        if (d.learned) PSK_TRY(learned_tc_sketch(d, X[i], ws + so[i], ws + w.sketch, status, s, launches));
+        if (d.learned) PSK_TRY(learned_tc_sketch(d, full, i, X[i], ws + so[i], ws + w.sketch, status, s, launches));
         else PSK_TRY(sketch8_tc_fwd(d, X[i], ws + so[i], ws + w.sketch, status, s, launches));
     }
     return cudaSuccess;
@@ -102,7 +103,7 @@ cudaError_t given_bwd(const Dims& d, const void* Q, const void* K, const void* V
     int* status = reinterpret_cast<int*>(ws + w.tc);
     for (int i = 0; i < 2; ++i) {
         if (d.learned)
-            PSK_TRY(learned_tc_sketch_bwd(d, X[i], ws + go[i], l.local ? ws + xo[i] : nullptr, dX[i], ws + w.sketch, status, s, launches));
+            PSK_TRY(learned_tc_sketch_bwd(d, i, X[i], ws + go[i], l.local ? ws + xo[i] : nullptr, dX[i], ws + w.sketch, status, s, launches));
         else
             PSK_TRY(sketch8_tc_bwd(d, X[i], ws + go[i], dX[i], ws + w.sketch, status, s, launches));
     }

@@ -1,23 +1,37 @@
 // Learnable sketch (Algorithm 2 of the paper's appendix) with its dense layers on the tensor
-// cores: bf16 operands, fp32 accumulation in tensor memory, r <= 32 (8r <= 256), h = 64.
+// cores: bf16 operands, fp32 accumulation in tensor memory, r = 16 or 32 (8r <= 256), h = 64.
 //
 //   f(x) = W4^T gelu(W3^T (W2^T LN1(gelu(W1^T LN0(x) + b1)) + b2) + b3) + b4      (two such networks)
 //   M    = sqrt(r) tanh(f_1(x) * f_2(x) / sqrt(r))
 //
-// Rows are processed in chunks; inside a chunk every layer is one launch (ltc_wide_kernel,
-// ltc_narrow_kernel, ltc_dense_kernel; 128 rows per tile: activations by TMA, the layer's weights
-// as the MN-major B operand, the accumulator read back by thread = row, where bias, gelu and the
-// layer normalisations are plain per-thread loops), with the activations the backward needs
-// kept in the workspace as bf16.
-// The gains of the normalisations are folded into the following layer's weights
-// (z W = n (diag(g) W) + c W), so the normalised activations n are the GEMM operands and
-// their gradients come out of the GEMM with the gain already applied.  Weight gradients are
-// sums over ALL rows of outer products: ltc_wgrad_kernel accumulates P^T S over a slab of rows in
-// tensor memory and adds the result to an fp32 accumulator once per slab, and sums the delta
-// operand's columns from the same tiles; gains, biases and the folded terms are taken from those
-// accumulators and sums by a last small kernel.
-// Every r-wide array is padded to 64 columns and every 8r-wide one to 256 (zeros), so two GEMM
-// shapes, 64 -> 256 and 256 -> 64, serve all sixteen layer passes.
+// The wide activations (8r per row) never leave the SM.  With p1, p3 the pre-activations, n0, n1 the
+// normalised rows, a2 the narrow activations between the halves and a3 = gelu(p3):
+//   ltc_dense_norm_kernel      forward of a 128-row tile in one go, as in attention: groups of 64 columns of p1
+//                              (p3) go from tensor memory through the gelu back into tensor memory as the
+//                              operand of the next layer.  The normalisation between them needs no second
+//                              look at the columns: n1 W2 = rs1 (g W2 - mu1 (1^T W2)).
+//                              Kept for the backward: a2 (hi + lo), mu1, rs1 and f, 264 bytes a row (r = 32).
+//   ltc_wgrad_kernel           layers 4 and 3 backward: p3 again from a2, then da2 and the weight gradients
+//                              a3^T df, dp3^T a2
+//   ltc_dense_bwd_norm_kernel  layers 2 and 1 backward: p1 again from n0, then dn0, n1^T da2, dp1^T n0.  The two
+//                              row sums of the normalisation's backward are inner products of narrow rows:
+//                              sum dn1 = da2 . (1^T W2),  sum dn1 n1 = da2 . (a2 - b2)
+// and small kernels around them.  The gains of the normalisations are folded into the following layer's
+// weights (z W = n (diag(g) W) + c W), so the normalised activations n are the GEMM operands and their
+// gradients come out of the GEMM with the gain already applied.  Weight gradients are sums over ALL rows of
+// outer products: every CTA keeps them in tensor memory for all its tiles and adds them to an fp32
+// accumulator once; gains, biases and the folded terms are taken from those by a last small kernel.
+//
+// Bound: the CUDA cores (the gelu and its derivative, the hi/lo splits), with the tensor pipe second: a
+// tile of 128 rows and one network is 65 536 gelus forward and twice that with derivatives backward.
+// (As sixteen separate layer launches, every activation crossing memory twice, 48 heads x 8192, r = 32,
+// forward + backward took 8.4 ms.)
+//
+// Precision: a half sketch feeds fourth powers of cancelling sums, and single bf16 operands, 2^-9 per entry
+// and four layers deep, would leave percents of error on the attention's output.  The forward multiplies
+// hi + lo pairs of bf16 terms for both activations and weights, A_hi B_hi + A_lo B_hi + A_hi B_lo: 2^-17.  The
+// backward's deltas and weight-gradient operands are single bf16; p1 and p3 are recomputed with the pairs.
+#include "cc_gemm.cuh"
 #include "tc_common.cuh"
 
 #include <cstdlib>
@@ -27,41 +41,62 @@ namespace psk {
 namespace {
 
 using namespace tc;
+using cc::f2;
+using cc::fma2;
+using cc::hi2;
+using cc::lo2;
+using cc::mul2;
+using cc::pack2;
 
 constexpr float kLnEps = 1e-6f;
-constexpr size_t kChunkRows = (size_t)1 << 20;        // rows per pass over the layers
-constexpr int kMat = 64 * 256;                        // elements of one operand matrix
-constexpr int kBank = 12;                             // operand matrices per network
-constexpr int kVec = 256 + 64 + 256 + 64;             // folded biases of one network: b1' | b2' | b3 | b4
+constexpr size_t kChunkRows = (size_t)1 << 20;        // rows per pass over the networks
+constexpr int kMat = 64 * 256;                        // entries of one weight-gradient accumulator [256][64]
+// folded vectors of one network: b1' | b2' | b3 | b4 | column sums of diag(g1) W2
+constexpr int kVb2 = 256, kVb3 = 320, kVb4 = 576, kVcs = 640, kVec = 704;
 constexpr int kSums = 256 + 64 + 256 + 64;            // column sums of one network: dp1 | da2 | dp3 | df
 
-// gelu(x) = x Phi(x) and its derivative Phi(x) + x phi(x).  erfc(z), z = |x| / sqrt(2), by the
-// five-term rational approximation in t = 1 / (1 + 0.3275911 z) (absolute error 1.5e-7); its
-// exponential exp(-z^2) = exp(-x^2 / 2) is the normal density's too.  With E = erfc(z):
-//   gelu(x) = max(x, 0) - |x| E / 2,     Phi(x) = 1/2 + copysign(1/2 - E/2, x).
-__device__ __forceinline__ float rcp_approx(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float ex2_approx(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
-// half of erfc(|x| / sqrt(2)) and exp(-x^2 / 2)
-__device__ __forceinline__ float half_erfc(float ax, float& e) {
-    const float z = ax * 0.70710678118654752f;
-    const float t = rcp_approx(fmaf(0.3275911f, z, 1.f));
-    e = ex2_approx(z * z * -1.4426950408889634f);
-    float poly = fmaf(0.5f * 1.061405429f, t, 0.5f * -1.453152027f);
-    poly = fmaf(poly, t, 0.5f * 1.421413741f);
-    poly = fmaf(poly, t, 0.5f * -0.284496736f);
-    poly = fmaf(poly, t, 0.5f * 0.254829592f);
-    return poly * t * e;
+__device__ __forceinline__ f2 ex2_2(f2 x) { return pack2(ex2_approx(lo2(x)), ex2_approx(hi2(x))); }
+__device__ __forceinline__ f2 both(float x) { return pack2(x, x); }
+
+// gelu(x) = x Phi(x) = max(x, 0) - |x| q,  q = Phi(-|x|) = 2^P(|x|), two entries at a time.  P is this
+// project's own minimax fit of log2 Phi(-t) on [0, 7] (degree 8, P(0) = -1, weighted so that q and t q are
+// off by at most 5e-8; negative leading coefficient, so q goes to 0 beyond).  One special-function
+// operation per entry and packed FMAs; written for -|x|: odd coefficients change sign.
+__device__ __forceinline__ f2 phi_tail(f2 nax) {
+    f2 p = fma2(both(-2.3347236037807306e-06f), nax, both(-3.3734937460394576e-05f));
+    p = fma2(p, nax, both(-0.00016127918206620961f));
+    p = fma2(p, nax, both(0.00019174156477674842f));
+    p = fma2(p, nax, both(0.007126918528228998f));
+    p = fma2(p, nax, both(0.052533652633428574f));
+    p = fma2(p, nax, both(-0.4591982662677765f));
+    p = fma2(p, nax, both(1.1511059999465942f));
+    return ex2_2(fma2(p, nax, both(-1.f)));
 }
-__device__ __forceinline__ float gelu_f(float x) {
-    float e;
-    const float ax = fabsf(x);
-    return fmaf(-ax, half_erfc(ax, e), fmaxf(x, 0.f));
+__device__ __forceinline__ f2 neg_abs(f2 x) { return x | 0x8000000080000000ull; }
+__device__ __forceinline__ f2 relu2(f2 x) { return pack2(fmaxf(lo2(x), 0.f), fmaxf(hi2(x), 0.f)); }
+__device__ __forceinline__ f2 gelu2(f2 x) {
+    const f2 nax = neg_abs(x);
+    return fma2(nax, phi_tail(nax), relu2(x));
 }
-__device__ __forceinline__ float gelu_grad_f(float x) {
-    float e;
-    const float q = half_erfc(fabsf(x), e);
-    return fmaf(x, 0.3989422804014327f * e, 0.5f + copysignf(0.5f - q, x));
+// ... and the derivative Phi(x) + x phi(x), phi the normal density 2^(-x^2 log2(e) / 2 - log2(sqrt(2 pi)))
+__device__ __forceinline__ f2 gelu2_grad(f2 x, f2& grad) {
+    const f2 nax = neg_abs(x);
+    const f2 q = phi_tail(nax);
+    const f2 h = fma2(q, both(-1.f), both(0.5f));
+    const f2 c = (h & 0x7fffffff7fffffffull) | (x & 0x8000000080000000ull);
+    const f2 dens = ex2_2(fma2(mul2(x, x), both(-0.72134752044448170f), both(-1.3257480647361593f)));
+    grad = fma2(x, dens, fma2(c, both(1.f), both(0.5f)));
+    return fma2(nax, q, relu2(x));
 }
+// v = hi + lo as two packed bf16 words
+__device__ __forceinline__ void split2(f2 v, uint32_t& h, uint32_t& l) {
+    h = pack_bf16(lo2(v), hi2(v));
+    const f2 hf = pack2(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u));
+    const f2 r = fma2(hf, both(-1.f), v);
+    l = pack_bf16(lo2(r), hi2(r));
+}
+__device__ __forceinline__ f2 unpack2(uint32_t w) { return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)); }
 
 struct NetLayout {
     int h, r, m;
@@ -79,775 +114,95 @@ struct NetLayout {
 };
 
 // ---------------------------------------------------------------------------
-// operand bank: per network eight bf16 matrices and the folded biases
-//   0: diag(g0) W1  [64][256]     4: W4^T           [64][256]
-//   1: diag(g1) W2  [256][64]     5: W3^T           [256][64]
-//   2: W3           [64][256]     6: (diag(g1) W2)^T [64][256]
-//   3: W4           [256][64]     7: (diag(g0) W1)^T [256][64]
-//   8..11: what rounding 0..3 to bf16 left over (the forward multiplies by hi + lo)
-// (rows / columns beyond r or 8r are zero)
+// Weights as shared-memory images (128-byte swizzle), fetched by plain bulk copies.  Groups of 64 columns j
+// of the wide side (NG of them):
+//   W1h, W1l  [NG][64 k][64 j]   diag(g0) W1 and what rounding it to bf16 left over: MN-major operand of
+//                                p1 = n0 W1, K-major operand of dn0 = dp1 W1^T
+//   W2c, W4c  [8r j][hi r | lo r]  diag(g1) W2, W4: MN-major operand of a2, f (both terms side by side, so that the hi
+//                                term of the activations multiplies them in one instruction), K-major of da3
+//   W3h, W3l  [NG][r c][64 j]    MN-major operand of p3, K-major operand of da2
+//   W2t       [NG][r c][64 j]    (diag(g1) W2)^T: MN-major operand of dn1
 // ---------------------------------------------------------------------------
-__device__ float bank_entry(const NetLayout& nl, const float* P, int which, int row, int col) {
-    const int r = nl.r, m = nl.m;
-    switch (which) {
-        case 0: return col < m ? P[nl.g0 + row] * P[nl.W1 + row * m + col] : 0.f;                  // [k][j]
-        case 1: return (row < m && col < r) ? P[nl.g1 + row] * P[nl.W2 + row * r + col] : 0.f;      // [j][c]
-        case 2: return (row < r && col < m) ? P[nl.W3 + row * m + col] : 0.f;                       // [c][j]
-        case 3: return (row < m && col < r) ? P[nl.W4 + row * r + col] : 0.f;                       // [j][c]
-        case 4: return (col < m && row < r) ? P[nl.W4 + col * r + row] : 0.f;                       // [c][j]
-        case 5: return (row < m && col < r) ? P[nl.W3 + col * m + row] : 0.f;                       // [j][c]
-        case 6: return (col < m && row < r) ? P[nl.g1 + col] * P[nl.W2 + col * r + row] : 0.f;      // [c][j]
-        default: return row < m ? P[nl.g0 + col] * P[nl.W1 + col * m + row] : 0.f;                  // [j][k]
-    }
-}
+template <int R> struct Bank {
+    static constexpr int M = 8 * R, NG = M / 64, NH = NG / 2;
+    static constexpr int kW1 = NG * 8192, kW3 = NG * R * 128, kWc = M * 128;
+    static constexpr int W1h = 0, W1l = kW1, W2c = 2 * kW1, W3h = W2c + kWc, W3l = W3h + kW3, W4c = W3l + kW3, W2t = W4c + kWc;
+    static constexpr int total = W2t + kW3;
+};
+constexpr size_t kBankBytes = Bank<32>::total;        // stride between the networks' banks
 
+template <int R>
 __global__ void __launch_bounds__(256)
-ltc_bank_kernel(int h, int r, const float* __restrict__ params, bf16* __restrict__ bank, float* __restrict__ vec) {
+ltc_bank_kernel(const float* __restrict__ params, uint8_t* __restrict__ bank, float* __restrict__ vec) {
     pdl_sync();
-    const NetLayout nl(h, r);
-    const int net = blockIdx.y;
+    using L = Bank<R>;
+    const NetLayout nl(64, R);
+    const int net = blockIdx.y, m = L::M;
     const float* P = params + (size_t)net * nl.count;
-    const int e = blockIdx.x * 256 + threadIdx.x;
-    if (e < 8 * kMat) {
-        const int which = e / kMat, idx = e % kMat;
-        const int cols = (which % 2 == 0) ? 256 : 64;
-        const float v = bank_entry(nl, P, which, idx / cols, idx % cols);
-        const bf16 hi = __float2bfloat16_rn(v);
-        bank[(size_t)net * kBank * kMat + e] = hi;
-        if (which < 4) bank[(size_t)net * kBank * kMat + 8 * kMat + e] = __float2bfloat16_rn(v - __bfloat162float(hi));
-    } else if (e < 8 * kMat + kVec) {
-        const int v = e - 8 * kMat;
-        float out = 0.f;
-        if (v < 256) {                                   // b1' = c0 W1 + b1
-            if (v < nl.m) { out = P[nl.b1 + v]; for (int k = 0; k < h; ++k) out = fmaf(P[nl.c0 + k], P[nl.W1 + k * nl.m + v], out); }
-        } else if (v < 320) {                            // b2' = c1 W2 + b2
-            const int c = v - 256;
-            if (c < r) { out = P[nl.b2 + c]; for (int j = 0; j < nl.m; ++j) out = fmaf(P[nl.c1 + j], P[nl.W2 + j * r + c], out); }
-        } else if (v < 576) {
-            if (v - 320 < nl.m) out = P[nl.b3 + v - 320];
-        } else {
-            if (v - 576 < r) out = P[nl.b4 + v - 576];
+    uint8_t* B = bank + (size_t)net * kBankBytes;
+    constexpr int n1 = 64 * L::M, n2 = R * L::M;       // weights of W1; of each of the others
+    constexpr int kBlocks = (n1 + 3 * n2) / 256;
+    if ((int)blockIdx.x < kBlocks) {
+        int e = blockIdx.x * 256 + threadIdx.x;
+        auto put = [&](int off, float v) { *reinterpret_cast<bf16*>(B + off) = __float2bfloat16_rn(v); };
+        auto lo_of = [](float v) { return v - __bfloat162float(__float2bfloat16_rn(v)); };
+        auto in_tile = [](int row, int col) { return (int)swz128_offset(row, col / 8) + (col % 8) * 2; };
+        if (e < n1) {
+            const int k = e / m, j = e % m;
+            const float v = P[nl.g0 + k] * P[nl.W1 + e];
+            const int o = (j / 64) * 8192 + in_tile(k, j % 64);
+            put(L::W1h + o, v);
+            put(L::W1l + o, lo_of(v));
+            return;
         }
-        vec[(size_t)net * kVec + v] = out;
+        e -= n1;
+        const int which = e / n2;
+        e -= which * n2;
+        if (which == 1) {                              // W3 [c][j]
+            const int c = e / m, j = e % m;
+            const float v = P[nl.W3 + e];
+            const int o = (j / 64) * (R * 128) + in_tile(c, j % 64);
+            put(L::W3h + o, v);
+            put(L::W3l + o, lo_of(v));
+            return;
+        }
+        const int j = e / R, c = e % R;                // W2, W4 [j][c]
+        const float v = which == 0 ? P[nl.g1 + j] * P[nl.W2 + e] : P[nl.W4 + e];
+        const int base = which == 0 ? L::W2c : L::W4c;
+        put(base + in_tile(j, c), v);
+        put(base + in_tile(j, R + c), lo_of(v));
+        if (which == 0) put(L::W2t + (j / 64) * (R * 128) + in_tile(c, j % 64), v);
+        return;
     }
+    // vectors: one warp per entry
+    const int v = (blockIdx.x - kBlocks) * 8 + threadIdx.x / 32, lane = threadIdx.x % 32;
+    if (v >= kVec) return;
+    float s = 0.f, add = 0.f;
+    if (v < kVb2) {                                    // b1' = c0 W1 + b1
+        if (v < m) {
+            add = P[nl.b1 + v];
+            for (int k = lane; k < 64; k += 32) s = fmaf(P[nl.c0 + k], P[nl.W1 + k * m + v], s);
+        }
+    } else if (v < kVb3) {                             // b2' = c1 W2 + b2
+        const int c = v - kVb2;
+        if (c < R) {
+            add = P[nl.b2 + c];
+            for (int j = lane; j < m; j += 32) s = fmaf(P[nl.c1 + j], P[nl.W2 + j * R + c], s);
+        }
+    } else if (v < kVb4) {
+        if (v - kVb3 < m) add = P[nl.b3 + v - kVb3];
+    } else if (v < kVcs) {
+        if (v - kVb4 < R) add = P[nl.b4 + v - kVb4];
+    } else {                                           // 1^T diag(g1) W2
+        const int c = v - kVcs;
+        if (c < R)
+            for (int j = lane; j < m; j += 32) s = fmaf(P[nl.g1 + j], P[nl.W2 + j * R + c], s);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) vec[(size_t)net * kVec + v] = s + add;
 }
 
-// ---------------------------------------------------------------------------
-// dense layer: Out[128 rows x ND] = epilogue(A[128 x KD] B[KD x ND])
-// ---------------------------------------------------------------------------
-enum { EPI_LN = 0, EPI_B64 = 1, EPI_GELU = 2, EPI_F32 = 3, EPI_DGELU = 4, EPI_LNBWD = 5 };
-
-struct DenseArgs {
-    const float* bias;      // [64] or null
-    bf16* out0;             // EPI_B64: [rows][64] bf16 (the forward's narrow layers: the hi terms)
-    bf16* out1;             //          the lo terms (forward only)
-    float* outf;            // EPI_F32: [rows][ncols]
-    int ncols;              // EPI_F32: columns stored
-    int accumulate;         // EPI_F32: add to what is there (backward only)
-};
-
-__device__ __forceinline__ void store8(bf16* dst, const float* v) {
-    *reinterpret_cast<uint4*>(dst) = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
-}
-// v = hi + lo as two bf16 terms
-__device__ __forceinline__ void store8_split(bf16* hi, bf16* lo, const float* v) {
-    float h[8], l[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) { h[i] = __bfloat162float(__float2bfloat16_rn(v[i])); l[i] = v[i] - h[i]; }
-    store8(hi, h);
-    store8(lo, l);
-}
-// (The forward's layers multiply hi + lo pairs of bf16 arrays for both activations and weights,
-// A_hi B_hi + A_lo B_hi + A_hi B_lo: a half sketch feeds fourth powers of cancelling sums, and
-// single bf16 operands, 2^-9 per entry and four layers deep, would leave percents of error on the
-// attention's output; the pairs leave 2^-17.  The backward's deltas are single bf16.)
-//
-// Narrow layers of the backward (256 -> 64, single operands): one tile per CTA, 128 threads.
-constexpr int kDenseSmem = 128 * 256 * 2 + 256 * 64 * 2 + 1024;
-
-template <int EPI>
-__global__ void __launch_bounds__(128)
-ltc_dense_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB, DenseArgs a, int* status) {
-    pdl_sync();
-    static_assert(EPI == EPI_B64 || EPI == EPI_F32, "the 256 -> 64 layers");
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* sA = align1024(smem_raw);
-    uint8_t* sB = sA + 65536;
-    __shared__ uint64_t bar_ld, bar_mma;
-    __shared__ uint32_t tm_slot;
-    __shared__ float s_bias[64];
-    const int tid = threadIdx.x, warp = tid / 32;
-    const int tile = blockIdx.x;
-    if (tid == 0) {
-        cta_giveup_init();
-        mbar_init(&bar_ld, 1); mbar_init(&bar_mma, 1);
-        mbar_fence_init();
-    }
-    if (warp == 0) { tmem_alloc(&tm_slot, 64); tmem_relinquish(); }
-    if (tid < 64) s_bias[tid] = a.bias != nullptr ? a.bias[tid] : 0.f;
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tm = tm_slot;
-    if (tid == 0) {
-        mbar_expect_tx(&bar_ld, 65536 + 32768);
-#pragma unroll
-        for (int s = 0; s < 4; ++s) tma_load_2d(sA + s * 16384, &mA, s * 64, tile * 128, &bar_ld);
-        tma_load_2d(sB, &mB, 0, 0, &bar_ld);
-        if (mbar_wait(&bar_ld, 0, status, kErrTma)) {
-            tc_fence_after();
-            constexpr uint32_t idesc = idesc_bf16(128, 64, false, true);
-            const uint64_t ad = smem_desc(smem_u32(sA), 0, 1024, kSwz128);
-            const uint64_t bd = smem_desc(smem_u32(sB), 0, 1024, kSwz128);
-#pragma unroll
-            for (int k = 0; k < 16; ++k)
-                umma_ss(tm, desc_off(ad, (k / 4) * 16384 + (k % 4) * 32), desc_off(bd, k * 2048), idesc, k > 0);
-            umma_commit(&bar_mma);
-        }
-    }
-    const bool ok = mbar_wait(&bar_mma, 0, status, kErrMma);
-    tc_fence_after();
-    const uint32_t lane_tm = tm + ((uint32_t)(warp * 32) << 16);
-    const size_t row = (size_t)tile * 128 + tid;
-    if (ok) {
-        if constexpr (EPI == EPI_B64) {
-#pragma unroll
-            for (int c0 = 0; c0 < 64; c0 += 32) {
-                uint32_t u[32];
-                tmem_ld32(lane_tm + c0, u);
-                tmem_ld_wait();
-                float v[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(u[j]) + s_bias[c0 + j];
-#pragma unroll
-                for (int j = 0; j < 32; j += 8) store8(a.out0 + row * 64 + c0 + j, v + j);
-            }
-        } else {
-#pragma unroll
-            for (int c0 = 0; c0 < 64; c0 += 32) {
-                if (c0 < a.ncols) {
-                    uint32_t u[32];
-                    tmem_ld32(lane_tm + c0, u);
-                    tmem_ld_wait();
-                    float* dst = a.outf + row * a.ncols + c0;
-#pragma unroll
-                    for (int j = 0; j < 32; j += 4) {
-                        if (c0 + j < a.ncols) {
-                            float4 o = make_float4(__uint_as_float(u[j]) + s_bias[c0 + j], __uint_as_float(u[j + 1]) + s_bias[c0 + j + 1],
-                                                   __uint_as_float(u[j + 2]) + s_bias[c0 + j + 2], __uint_as_float(u[j + 3]) + s_bias[c0 + j + 3]);
-                            if (a.accumulate) {
-                                const float4 p = *reinterpret_cast<const float4*>(dst + j);
-                                o.x += p.x; o.y += p.y; o.z += p.z; o.w += p.w;
-                            }
-                            *reinterpret_cast<float4*>(dst + j) = o;
-                        }
-                    }
-                }
-            }
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 64);
-}
-
-// ---------------------------------------------------------------------------
-// narrow layers of the forward (256 -> 64, hi + lo pairs): persistent, one CTA per SM.  The layer's
-// weights stay in shared memory; the activation tiles stream through a four-stage ring of
-// 64-column chunks (hi and lo, 32 KB a stage) that the producer thread keeps full across tile
-// boundaries; the accumulator is double-buffered in tensor memory, so the rows' epilogue of one
-// tile runs under the loads and MMAs of the next.  Warps 0-3: epilogue (thread = row); warp 4: TMA
-// producer; warp 5: MMA issuer.
-// ---------------------------------------------------------------------------
-constexpr int kNrStages = 4, kNrStage = 32768;
-constexpr int kNrSmem = 65536 + kNrStages * kNrStage + 1024;
-
-template <int EPI>
-__global__ void __launch_bounds__(192, 1)
-ltc_narrow_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mA2,
-                  const __grid_constant__ CUtensorMap mB, const __grid_constant__ CUtensorMap mB2, DenseArgs a, int tiles,
-                  int* status) {
-    pdl_sync();
-    static_assert(EPI == EPI_B64 || EPI == EPI_F32, "the 256 -> 64 layers");
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* sB = align1024(smem_raw);
-    uint8_t* sR = sB + 65536;
-    __shared__ uint64_t bar_b, bar_full[kNrStages], bar_empty[kNrStages], bar_accfull[2], bar_accfree[2];
-    __shared__ uint32_t tm_slot;
-    __shared__ float s_bias[64];
-    const int tid = threadIdx.x, warp = tid / 32;
-    const int ntl = (tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-    if (tid == 0) {
-        cta_giveup_init();
-        mbar_init(&bar_b, 1);
-        for (int s = 0; s < kNrStages; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&bar_empty[s], 1); }
-        mbar_init(&bar_accfull[0], 1); mbar_init(&bar_accfull[1], 1);
-        mbar_init(&bar_accfree[0], 128); mbar_init(&bar_accfree[1], 128);
-        mbar_fence_init();
-    }
-    if (warp == 0) { tmem_alloc(&tm_slot, 128); tmem_relinquish(); }
-    if (tid < 64) s_bias[tid] = a.bias != nullptr ? a.bias[tid] : 0.f;
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tm = tm_slot;
-    if (tid == 128) {
-        // ---- producer ----
-        mbar_expect_tx(&bar_b, 65536);
-        tma_load_2d(sB, &mB, 0, 0, &bar_b);
-        tma_load_2d(sB + 32768, &mB2, 0, 0, &bar_b);
-        bool ok = true;
-        int it = 0;
-        for (int i = 0; i < ntl && ok; ++i) {
-            const int tile = blockIdx.x + i * gridDim.x;
-            for (int c = 0; c < 4 && ok; ++c, ++it) {
-                const int s = it % kNrStages;
-                if (it >= kNrStages) ok = mbar_spin(&bar_empty[s], ((it / kNrStages) - 1) & 1, status, kErrMma);
-                if (!ok) break;
-                mbar_expect_tx(&bar_full[s], kNrStage);
-                tma_load_2d(sR + s * kNrStage, &mA, c * 64, tile * 128, &bar_full[s]);
-                tma_load_2d(sR + s * kNrStage + 16384, &mA2, c * 64, tile * 128, &bar_full[s]);
-            }
-        }
-    } else if (tid == 160) {
-        // ---- MMA issuer ----
-        constexpr uint32_t idesc = idesc_bf16(128, 64, false, true);
-        bool ok = mbar_spin(&bar_b, 0, status, kErrTma);
-        const uint64_t bhi = smem_desc(smem_u32(sB), 0, 1024, kSwz128);
-        const uint64_t blo = smem_desc(smem_u32(sB) + 32768, 0, 1024, kSwz128);
-        int it = 0;
-        for (int i = 0; i < ntl && ok; ++i) {
-            const int buf = i & 1;
-            if (i >= 2) ok = mbar_spin(&bar_accfree[buf], ((i / 2) - 1) & 1, status, kErrMma);
-            for (int c = 0; c < 4 && ok; ++c, ++it) {
-                const int s = it % kNrStages;
-                ok = mbar_spin(&bar_full[s], (it / kNrStages) & 1, status, kErrTma);
-                if (!ok) break;
-                tc_fence_after();
-                const uint64_t ahi = smem_desc(smem_u32(sR) + s * kNrStage, 0, 1024, kSwz128);
-                const uint64_t alo = smem_desc(smem_u32(sR) + s * kNrStage + 16384, 0, 1024, kSwz128);
-#pragma unroll
-                for (int part = 0; part < 3; ++part) {
-                    const uint64_t ad = part == 1 ? alo : ahi;
-                    const uint64_t bd = part == 2 ? blo : bhi;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        umma_ss(tm + buf * 64, desc_off(ad, k * 32), desc_off(bd, c * 8192 + k * 2048), idesc,
-                                (c > 0 || part > 0 || k > 0) ? 1u : 0u);
-                }
-                umma_commit(&bar_empty[s]);
-            }
-            if (ok) umma_commit(&bar_accfull[buf]);
-        }
-    } else if (warp < 4) {
-        // ---- epilogue ----
-        const uint32_t lane_tm = tm + ((uint32_t)(warp * 32) << 16);
-        bool ok = true;
-        for (int i = 0; i < ntl && ok; ++i) {
-            const int buf = i & 1;
-            const size_t row = (size_t)(blockIdx.x + i * gridDim.x) * 128 + tid;
-            ok = mbar_wait(&bar_accfull[buf], (i / 2) & 1, status, kErrMma);
-            if (!ok) break;
-            tc_fence_after();
-            if constexpr (EPI == EPI_B64) {
-#pragma unroll
-                for (int c0 = 0; c0 < 64; c0 += 32) {
-                    uint32_t u[32];
-                    tmem_ld32(lane_tm + buf * 64 + c0, u);
-                    tmem_ld_wait();
-                    float v[32];
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(u[j]) + s_bias[c0 + j];
-#pragma unroll
-                    for (int j = 0; j < 32; j += 8) store8_split(a.out0 + row * 64 + c0 + j, a.out1 + row * 64 + c0 + j, v + j);
-                }
-            } else {
-#pragma unroll
-                for (int c0 = 0; c0 < 64; c0 += 32) {
-                    if (c0 < a.ncols) {
-                        uint32_t u[32];
-                        tmem_ld32(lane_tm + buf * 64 + c0, u);
-                        tmem_ld_wait();
-                        float* dst = a.outf + row * a.ncols + c0;
-#pragma unroll
-                        for (int j = 0; j < 32; j += 4)
-                            if (c0 + j < a.ncols)
-                                *reinterpret_cast<float4*>(dst + j) =
-                                    make_float4(__uint_as_float(u[j]) + s_bias[c0 + j], __uint_as_float(u[j + 1]) + s_bias[c0 + j + 1],
-                                                __uint_as_float(u[j + 2]) + s_bias[c0 + j + 2], __uint_as_float(u[j + 3]) + s_bias[c0 + j + 3]);
-                    }
-                }
-            }
-            tc_fence_before();
-            mbar_arrive(&bar_accfree[buf]);
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 128);
-}
-
-// ---------------------------------------------------------------------------
-// wide layer: Out[128 rows x 256] = epilogue(A[128 x 64] B[64 x 256]).  256 threads: the two
-// warpgroups share the rows (thread = row) and take two 64-column groups each; every output
-// leaves as TMA stores of [128 x 64] tiles staged in shared memory.  SPLIT (forward): hi + lo
-// operand pairs, the staging tiles lie over the operands (dead once the MMAs have completed).
-// Backward: single operands, side tiles (the forward's activations) by TMA, the output written
-// in place over the side tile it consumed.
-// ---------------------------------------------------------------------------
-struct WideArgs {
-    const float* bias;      // [256] or null
-    float* rs_out;          // EPI_LN: 1 / sigma of every row
-    const float* rs_in;     // EPI_LNBWD
-    int ncols;              // live columns (8r)
-    int keep_pre;           // EPI_LN, EPI_GELU: also store the pre-activation (output 0), which only the backward reads
-};
-
-template <int EPI, bool SPLIT>
-struct WideSmem {
-    static constexpr int kA1 = 16384, kB1 = 32768;
-    static constexpr int kA = kA1 * (SPLIT ? 2 : 1), kB = kB1 * (SPLIT ? 2 : 1);
-    static constexpr int kSides = EPI == EPI_DGELU ? 1 : (EPI == EPI_LNBWD ? 2 : 0);
-    static constexpr int bytes = kA + kB + kSides * 65536 + 1024;
-    static_assert(!SPLIT || kA + kB == 2 * 3 * 16384, "three staging tiles per warpgroup over the operands");
-    static_assert(SPLIT == (kSides == 0), "forward: pairs and no side tiles; backward: the reverse");
-};
-
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* m, const void* src, int c0, int c1) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                 ::"l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(src)), "r"(c0), "r"(c1)
-                 : "memory");
-}
-// 8 consecutive columns of a row of a 128-byte-swizzled [128 x 64] bf16 tile
-__device__ __forceinline__ void tile_put8(uint8_t* tile, int row, int chunk, const float* v) {
-    *reinterpret_cast<uint4*>(tile + swz128_offset(row, chunk)) =
-        make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
-}
-// v = hi + lo: one packed conversion gives two hi terms, whose float values are the halves of that word
-__device__ __forceinline__ void tile_put8_split(uint8_t* hi_tile, uint8_t* lo_tile, int row, int chunk, const float* v) {
-    uint32_t h[4], l[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        h[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
-        l[i] = pack_bf16(v[2 * i] - __uint_as_float(h[i] << 16), v[2 * i + 1] - __uint_as_float(h[i] & 0xffff0000u));
-    }
-    const uint32_t o = swz128_offset(row, chunk);
-    *reinterpret_cast<uint4*>(hi_tile + o) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4*>(lo_tile + o) = make_uint4(l[0], l[1], l[2], l[3]);
-}
-__device__ __forceinline__ void tile_get8(const uint8_t* tile, int row, int chunk, float* v) {
-    const uint4 q = *reinterpret_cast<const uint4*>(tile + swz128_offset(row, chunk));
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        v[2 * i] = __uint_as_float(w[i] << 16);
-        v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-    }
-}
-
-// FULL: all 256 columns are live (8r = 256), no masks
-template <int EPI, bool SPLIT, bool FULL>
-__global__ void __launch_bounds__(256)
-ltc_wide_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mA2,
-                const __grid_constant__ CUtensorMap mB, const __grid_constant__ CUtensorMap mB2,
-                const __grid_constant__ CUtensorMap mS0, const __grid_constant__ CUtensorMap mS1,
-                const __grid_constant__ CUtensorMap mO0, const __grid_constant__ CUtensorMap mO1,
-                const __grid_constant__ CUtensorMap mO2, WideArgs a, int* status) {
-    pdl_sync();
-    using L = WideSmem<EPI, SPLIT>;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* sA = align1024(smem_raw);
-    uint8_t* sB = sA + L::kA;
-    uint8_t* sS = sB + L::kB;
-    __shared__ uint64_t bar_ld, bar_side, bar_mma;
-    __shared__ uint32_t tm_slot;
-    __shared__ __align__(16) float s_bias[256];
-    __shared__ float2 s_part[2][128];
-    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    const int wg = warp / 4, rowt = (warp % 4) * 32 + lane;
-    const int tile = blockIdx.x;
-    if (tid == 0) {
-        cta_giveup_init();
-        mbar_init(&bar_ld, 1); mbar_init(&bar_side, 1); mbar_init(&bar_mma, 1);
-        mbar_fence_init();
-    }
-    if (warp == 0) { tmem_alloc(&tm_slot, 256); tmem_relinquish(); }
-    s_bias[tid] = a.bias != nullptr ? a.bias[tid] : 0.f;
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tm = tm_slot;
-    if (tid == 0) {
-        mbar_expect_tx(&bar_ld, L::kA + L::kB);
-        tma_load_2d(sA, &mA, 0, tile * 128, &bar_ld);
-#pragma unroll
-        for (int g = 0; g < 4; ++g) tma_load_2d(sB + g * 8192, &mB, g * 64, 0, &bar_ld);
-        if constexpr (SPLIT) {
-            tma_load_2d(sA + L::kA1, &mA2, 0, tile * 128, &bar_ld);
-#pragma unroll
-            for (int g = 0; g < 4; ++g) tma_load_2d(sB + L::kB1 + g * 8192, &mB2, g * 64, 0, &bar_ld);
-        }
-        if constexpr (L::kSides > 0) {
-            mbar_expect_tx(&bar_side, L::kSides * 65536);
-#pragma unroll
-            for (int g = 0; g < 4; ++g) tma_load_2d(sS + g * 16384, &mS0, g * 64, tile * 128, &bar_side);
-            if constexpr (L::kSides > 1) {
-#pragma unroll
-                for (int g = 0; g < 4; ++g) tma_load_2d(sS + 65536 + g * 16384, &mS1, g * 64, tile * 128, &bar_side);
-            }
-        }
-        if (mbar_wait(&bar_ld, 0, status, kErrTma)) {
-            tc_fence_after();
-            constexpr uint32_t idesc = idesc_bf16(128, 256, false, true);
-#pragma unroll
-            for (int part = 0; part < (SPLIT ? 3 : 1); ++part) {
-                const uint64_t ad = smem_desc(smem_u32(sA) + (part == 1 ? L::kA1 : 0), 0, 1024, kSwz128);
-                const uint64_t bd = smem_desc(smem_u32(sB) + (part == 2 ? L::kB1 : 0), 8192, 1024, kSwz128);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) umma_ss(tm, desc_off(ad, k * 32), desc_off(bd, k * 2048), idesc, (part > 0 || k > 0) ? 1u : 0u);
-            }
-            umma_commit(&bar_mma);
-        }
-    }
-    bool ok = mbar_wait(&bar_mma, 0, status, kErrMma);
-    if constexpr (L::kSides > 0) ok = ok && mbar_wait(&bar_side, 0, status, kErrTma);
-    ok = __syncthreads_and(ok) != 0;             // one decision for the whole CTA: the epilogue has barriers
-    tc_fence_after();
-    const uint32_t lane_tm = tm + ((uint32_t)((warp % 4) * 32) << 16);
-    const size_t row = (size_t)tile * 128 + rowt;
-    const bool elected = (tid % 128) == 0;
-    auto wg_sync = [&]() {
-        if (wg == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
-        else asm volatile("bar.sync 2, 128;" ::: "memory");
-    };
-    if (ok) {
-        if constexpr (EPI == EPI_GELU) {
-            uint8_t* stg = sA + wg * 3 * 16384;
-#pragma unroll 1
-            for (int i = 0; i < 2; ++i) {
-                const int cg = wg * 2 + i;
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const int c0 = cg * 64 + half * 32;
-                    uint32_t u[32];
-                    tmem_ld32(lane_tm + c0, u);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int j = 0; j < 32; j += 8) {
-                        float pv[8], g[8];
-                        const float4 b0 = *reinterpret_cast<const float4*>(s_bias + c0 + j), b1 = *reinterpret_cast<const float4*>(s_bias + c0 + j + 4);
-                        const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            pv[q] = __uint_as_float(u[j + q]) + bv[q];
-                            g[q] = (FULL || c0 + j + q < a.ncols) ? gelu_f(pv[q]) : 0.f;
-                        }
-                        if (a.keep_pre) tile_put8(stg, rowt, half * 4 + j / 8, pv);
-                        tile_put8_split(stg + 16384, stg + 32768, rowt, half * 4 + j / 8, g);
-                    }
-                }
-                fence_proxy_async_smem();
-                wg_sync();
-                if (elected) {
-                    if (a.keep_pre) tma_store_2d(&mO0, stg, cg * 64, tile * 128);
-                    tma_store_2d(&mO1, stg + 16384, cg * 64, tile * 128);
-                    tma_store_2d(&mO2, stg + 32768, cg * 64, tile * 128);
-                    bulk_commit();
-                    bulk_wait_read();
-                }
-                wg_sync();
-            }
-        } else if constexpr (EPI == EPI_LN) {
-            uint8_t* stg = sA + wg * 3 * 16384;
-            float s = 0.f, ss = 0.f;
-#pragma unroll 1
-            for (int i = 0; i < 2; ++i) {
-                const int cg = wg * 2 + i;
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const int c0 = cg * 64 + half * 32;
-                    uint32_t u[32];
-                    tmem_ld32(lane_tm + c0, u);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int j = 0; j < 32; j += 8) {
-                        float pv[8];
-                        const float4 b0 = *reinterpret_cast<const float4*>(s_bias + c0 + j), b1 = *reinterpret_cast<const float4*>(s_bias + c0 + j + 4);
-                        const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            pv[q] = __uint_as_float(u[j + q]) + bv[q];
-                            const float g = (FULL || c0 + j + q < a.ncols) ? gelu_f(pv[q]) : 0.f;
-                            s += g; ss = fmaf(g, g, ss);
-                            u[j + q] = __float_as_uint(g);
-                        }
-                        if (a.keep_pre) tile_put8(stg, rowt, half * 4 + j / 8, pv);
-                    }
-                    tmem_st32(lane_tm + c0, u);
-                }
-                if (a.keep_pre) {
-                    fence_proxy_async_smem();
-                    wg_sync();
-                    if (elected) {
-                        tma_store_2d(&mO0, stg, cg * 64, tile * 128);
-                        bulk_commit();
-                        bulk_wait_read();
-                    }
-                    wg_sync();
-                }
-            }
-            tmem_st_wait();
-            s_part[wg][rowt] = make_float2(s, ss);
-            __syncthreads();
-            const float2 p0 = s_part[0][rowt], p1 = s_part[1][rowt];
-            const float inv = 1.f / (float)a.ncols;
-            const float mu = (p0.x + p1.x) * inv;
-            const float rs = rsqrtf(fmaxf((p0.y + p1.y) * inv - mu * mu, 0.f) + kLnEps);
-            if (wg == 0) a.rs_out[row] = rs;
-#pragma unroll 1
-            for (int i = 0; i < 2; ++i) {
-                const int cg = wg * 2 + i;
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const int c0 = cg * 64 + half * 32;
-                    uint32_t u[32];
-                    tmem_ld32(lane_tm + c0, u);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int j = 0; j < 32; j += 8) {
-                        float nrm[8];
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) nrm[q] = (FULL || c0 + j + q < a.ncols) ? (__uint_as_float(u[j + q]) - mu) * rs : 0.f;
-                        tile_put8_split(stg + 16384, stg + 32768, rowt, half * 4 + j / 8, nrm);
-                    }
-                }
-                fence_proxy_async_smem();
-                wg_sync();
-                if (elected) {
-                    tma_store_2d(&mO1, stg + 16384, cg * 64, tile * 128);
-                    tma_store_2d(&mO2, stg + 32768, cg * 64, tile * 128);
-                    bulk_commit();
-                    bulk_wait_read();
-                }
-                wg_sync();
-            }
-        } else if constexpr (EPI == EPI_DGELU) {
-#pragma unroll 1
-            for (int i = 0; i < 2; ++i) {
-                const int cg = wg * 2 + i;
-                uint8_t* side = sS + cg * 16384;          // p3's tile, overwritten by dp3
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const int c0 = cg * 64 + half * 32;
-                    uint32_t u[32];
-                    tmem_ld32(lane_tm + c0, u);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int j = 0; j < 32; j += 8) {
-                        float pv[8], o[8];
-                        tile_get8(side, rowt, half * 4 + j / 8, pv);
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) o[q] = (FULL || c0 + j + q < a.ncols) ? __uint_as_float(u[j + q]) * gelu_grad_f(pv[q]) : 0.f;
-                        tile_put8(side, rowt, half * 4 + j / 8, o);
-                    }
-                }
-                fence_proxy_async_smem();
-                wg_sync();
-                if (elected) { tma_store_2d(&mO0, side, cg * 64, tile * 128); bulk_commit(); }
-            }
-            if (elected) bulk_wait_read();
-        } else {   // EPI_LNBWD: back through n = (g - mu) / sigma and g = gelu(p)
-            float s1 = 0.f, s2 = 0.f;
-#pragma unroll 1
-            for (int i = 0; i < 2; ++i) {
-                const int cg = wg * 2 + i;
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    uint32_t u[32];
-                    tmem_ld32(lane_tm + cg * 64 + half * 32, u);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int j = 0; j < 32; j += 8) {
-                        float nrm[8];
-                        tile_get8(sS + cg * 16384, rowt, half * 4 + j / 8, nrm);
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) { const float dn = __uint_as_float(u[j + q]); s1 += dn; s2 = fmaf(dn, nrm[q], s2); }
-                    }
-                }
-            }
-            s_part[wg][rowt] = make_float2(s1, s2);
-            __syncthreads();
-            const float2 p0 = s_part[0][rowt], p1 = s_part[1][rowt];
-            const float inv = 1.f / (float)a.ncols;
-            const float m1 = (p0.x + p1.x) * inv, m2 = (p0.y + p1.y) * inv, rs = a.rs_in[row];
-#pragma unroll 1
-            for (int i = 0; i < 2; ++i) {
-                const int cg = wg * 2 + i;
-                uint8_t* side = sS + 65536 + cg * 16384;  // p1's tile, overwritten by dp1
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const int c0 = cg * 64 + half * 32;
-                    uint32_t u[32];
-                    tmem_ld32(lane_tm + c0, u);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int j = 0; j < 32; j += 8) {
-                        float nrm[8], pv[8], o[8];
-                        tile_get8(sS + cg * 16384, rowt, half * 4 + j / 8, nrm);
-                        tile_get8(side, rowt, half * 4 + j / 8, pv);
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            o[q] = (FULL || c0 + j + q < a.ncols) ? rs * (__uint_as_float(u[j + q]) - m1 - nrm[q] * m2) * gelu_grad_f(pv[q]) : 0.f;
-                        tile_put8(side, rowt, half * 4 + j / 8, o);
-                    }
-                }
-                fence_proxy_async_smem();
-                wg_sync();
-                if (elected) { tma_store_2d(&mO0, side, cg * 64, tile * 128); bulk_commit(); }
-            }
-            if (elected) bulk_wait_read();
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 256);
-}
-
-// ---------------------------------------------------------------------------
-// weight gradients: Gt[256][64] += sum over a slab of rows of P[row][:]^T S[row][:]
-// (P: [rows][256] bf16, S: [rows][64] bf16; both tiles go to the tensor cores as TMA left them:
-// P^T is an MN-major A operand, S an MN-major B operand, the contraction runs over the rows).
-// The column sums of the delta operand (the bias gradients, and what the folded normalisation gains
-// need) are products with ones on the same tiles: P^T 1 (wide delta) or 1^T S (narrow).
-// One CTA per SM with one slab of tiles.  Bound: the 80 KB a tile takes from memory.  (With the sums
-// added up by four warps from shared memory, two bytes at a time, and twice as many CTAs adding
-// their results in scattered 4-byte atomics, 393 216 rows took 118 us; now 54.)
-// ---------------------------------------------------------------------------
-constexpr int kWgStage = 65536 + 16384;
-constexpr int kWgSmem = 2 * kWgStage + 32768 + 1024;
-
-__device__ __forceinline__ void red_add4(float* dst, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(__uint_as_float(a)), "f"(__uint_as_float(b)),
-                 "f"(__uint_as_float(c)), "f"(__uint_as_float(d)) : "memory");
-}
-
-__global__ void __launch_bounds__(128)
-ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mP, const __grid_constant__ CUtensorMap mS, float* __restrict__ Gt,
-                 float* __restrict__ colsum, int sum_wide, int ntiles, int tiles_per_cta, int* status) {
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = align1024(smem_raw);
-    uint8_t* ones = smem + 2 * kWgStage;              // two [128 rows x 64 columns] tiles of ones
-    __shared__ uint64_t bar_full[2], bar_free[2], bar_done;
-    __shared__ uint32_t tm_slot;
-    const int tid = threadIdx.x, warp = tid / 32;
-    const int t0 = blockIdx.x * tiles_per_cta;
-    const int T = min(tiles_per_cta, ntiles - t0);
-    if (tid == 0) {
-        cta_giveup_init();
-        mbar_init(&bar_full[0], 1); mbar_init(&bar_full[1], 1);
-        mbar_init(&bar_free[0], 1); mbar_init(&bar_free[1], 1);
-        mbar_init(&bar_done, 1);
-        mbar_fence_init();
-    }
-    for (int e = tid; e < 2048; e += 128) reinterpret_cast<uint4*>(ones)[e] = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
-    fence_proxy_async_smem();
-    pdl_sync();
-    if (warp == 0) { tmem_alloc(&tm_slot, 256); tmem_relinquish(); }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tm = tm_slot;
-    constexpr uint32_t kSum = 128;                    // columns of the sums
-    if (tid == 0) {
-        auto load = [&](int j) {
-            const int s = j & 1;
-            uint8_t* sP = smem + s * kWgStage;
-            mbar_expect_tx(&bar_full[s], kWgStage);
-#pragma unroll
-            for (int g = 0; g < 4; ++g) tma_load_2d(sP + g * 16384, &mP, g * 64, (t0 + j) * 128, &bar_full[s]);
-            tma_load_2d(sP + 65536, &mS, 0, (t0 + j) * 128, &bar_full[s]);
-        };
-        load(0);
-        if (T > 1) load(1);
-        constexpr uint32_t idesc = idesc_bf16(128, 64, true, true), idesc1 = idesc_bf16(128, 16, true, true);
-        const uint64_t oneb = smem_desc(smem_u32(ones), 0, 1024, kSwz128), onea = smem_desc(smem_u32(ones), 16384, 1024, kSwz128);
-        bool ok = true;
-        for (int j = 0; j < T && ok; ++j) {
-            const int s = j & 1;
-            ok = mbar_spin(&bar_full[s], (j >> 1) & 1, status, kErrTma);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t base = smem_u32(smem + s * kWgStage);
-            const uint64_t sd = smem_desc(base + 65536, 0, 1024, kSwz128);
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                const uint64_t pd = smem_desc(base + half * 32768, 16384, 1024, kSwz128);
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    umma_ss(tm + half * 64, desc_off(pd, k * 2048), desc_off(sd, k * 2048), idesc, (j > 0 || k > 0) ? 1u : 0u);
-                if (sum_wide) {
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        umma_ss(tm + kSum + half * 16, desc_off(pd, k * 2048), desc_off(oneb, k * 2048), idesc1, (j > 0 || k > 0) ? 1u : 0u);
-                }
-            }
-            if (!sum_wide) {
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    umma_ss(tm + kSum, desc_off(onea, k * 2048), desc_off(sd, k * 2048), idesc, (j > 0 || k > 0) ? 1u : 0u);
-            }
-            umma_commit(&bar_free[s]);
-            if (j + 2 < T) {
-                ok = mbar_spin(&bar_free[s], (j >> 1) & 1, status, kErrMma);
-                if (ok) load(j + 2);
-            }
-        }
-        if (ok) umma_commit(&bar_done);
-    }
-    __syncwarp();
-    const bool ok = mbar_wait(&bar_done, 0, status, kErrMma);
-    tc_fence_after();
-    if (ok) {
-        const uint32_t lane_tm = tm + ((uint32_t)(warp * 32) << 16);
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-#pragma unroll
-            for (int c0 = 0; c0 < 64; c0 += 32) {
-                uint32_t u[32];
-                tmem_ld32(lane_tm + half * 64 + c0, u);
-                tmem_ld_wait();
-                float* dst = Gt + (size_t)(half * 128 + tid) * 64 + c0;
-#pragma unroll
-                for (int j = 0; j < 32; j += 4) red_add4(dst + j, u[j], u[j + 1], u[j + 2], u[j + 3]);
-            }
-        }
-        if (sum_wide) {                               // every column of the product with ones is the sum
-            uint32_t u[32];
-            tmem_ld32(lane_tm + kSum, u);
-            tmem_ld_wait();
-            atomicAdd(colsum + tid, __uint_as_float(u[0]));
-            atomicAdd(colsum + 128 + tid, __uint_as_float(u[16]));
-        } else if (warp == 0) {                       // ... and every row
-#pragma unroll
-            for (int c0 = 0; c0 < 64; c0 += 32) {
-                uint32_t u[32];
-                tmem_ld32(lane_tm + kSum + c0, u);
-                tmem_ld_wait();
-                if (tid == 0) {
-#pragma unroll
-                    for (int j = 0; j < 32; j += 4) red_add4(colsum + c0 + j, u[j], u[j + 1], u[j + 2], u[j + 3]);
-                }
-            }
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 256);
-}
-
-// ---------------------------------------------------------------------------
-// CUDA-core helpers around the layers
-// ---------------------------------------------------------------------------
 struct Slice {
     int H, n; int64_t sb, sh, sn;
     __device__ int64_t row(size_t R) const {
@@ -856,12 +211,763 @@ struct Slice {
     }
 };
 
-// n0 = (x - mean) / sigma of every row as hi + lo, 1 / sigma kept.  One warp per row, two columns
-// per lane, eight rows per warp with their loads issued together.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(taddr) : "memory");
+}
+// one arrival per warp, after all its lanes
+__device__ __forceinline__ void warp_arrive(uint64_t* bar) {
+    __syncwarp();
+    if (threadIdx.x % 32 == 0) mbar_arrive(bar);
+}
+// a shared-memory image in pieces of at most 32 KB
+__device__ __forceinline__ void load_image(uint8_t* dst, const uint8_t* src, int bytes, uint64_t* bar) {
+    for (int o = 0; o < bytes; o += 32768) bulk_load(dst + o, src + o, bytes - o < 32768 ? bytes - o : 32768, bar);
+}
+
+// ---------------------------------------------------------------------------
+// Forward of one network (blockIdx.y) for tiles of 128 rows.  Persistent; two tiles (slots) in flight per CTA.
+// Per slot: two warpgroups (thread = row, one half of every 64-column group each) and one issuing thread.
+// Tensor memory of a slot, 256 columns: N 64 (n0, later a2, as hi/lo operand), two 64-column group
+// buffers, O 2r.  A group buffer holds p, then in place gelu(p) as an operand, each warpgroup writing over the
+// 32 columns it has read: 16 columns of hi pairs, 16 of lo.
+// ---------------------------------------------------------------------------
+template <int R> constexpr int kFwdSmem = Bank<R>::W2t + 1024;
+
+template <int R>
+__global__ void __launch_bounds__(576, 1)
+ltc_dense_norm_kernel(Slice sl, const bf16* __restrict__ X, size_t row0, int tiles, const float2* __restrict__ st0,
+                      const uint8_t* __restrict__ bank, const float* __restrict__ vec, bf16* __restrict__ a2, size_t a2_net,
+                      float2* __restrict__ st1, size_t st1_net, float* __restrict__ f, size_t f_net, int* status) {
+    using L = Bank<R>;
+    constexpr int NG = L::NG;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* W = align1024(smem_raw);
+    __shared__ uint64_t bar_w, bar_n[2], bar_s[2][2], bar_p[2][2], bar_f[2][2], bar_o[2];
+    __shared__ uint32_t tm_slot;
+    __shared__ __align__(16) float sv[kVec];
+    __shared__ float2 s_part[2][2][128];
+    const int tid = threadIdx.x, warp = tid / 32, net = blockIdx.y;
+    if (tid == 0) {
+        cta_giveup_init();
+        mbar_init(&bar_w, 1);
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(&bar_n[s], 8); mbar_init(&bar_o[s], 1);
+            for (int b = 0; b < 2; ++b) { mbar_init(&bar_s[s][b], 1); mbar_init(&bar_p[s][b], 8); mbar_init(&bar_f[s][b], 1); }
+        }
+        mbar_fence_init();
+    }
+    pdl_sync();
+    if (warp == 16) { tmem_alloc(&tm_slot, 512); tmem_relinquish(); }
+    for (int e = tid; e < kVec; e += 576) sv[e] = vec[(size_t)net * kVec + e];
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tm = tm_slot;
+    constexpr uint32_t cN = 0, cS = 64, cO = 192;
+    if (warp >= 16) {
+        // ============================ issuing threads ============================
+        const int slot = warp - 16;
+        if (tid % 32 == 0) {
+            if (slot == 0) {
+                mbar_expect_tx(&bar_w, L::W2t);
+                load_image(W, bank + (size_t)net * kBankBytes, L::W2t, &bar_w);
+            }
+            const uint32_t t0 = tm + slot * 256;
+            mbar_spin(&bar_w, 0, status, kErrTma);
+            const uint32_t w = smem_u32(W);
+            constexpr uint32_t id_s = idesc_bf16(128, 64, false, true), id_o = idesc_bf16(128, 2 * R, false, true),
+                               id_l = idesc_bf16(128, R, false, true);
+            uint32_t it = 0, pp[2] = {0, 0}, pf[2] = {0, 0};
+            for (int tile = blockIdx.x * 2 + slot; tile < tiles; tile += 2 * gridDim.x) {
+#pragma unroll
+                for (int layer = 0; layer < 2; ++layer, ++it) {
+                    mbar_spin(&bar_n[slot], it & 1, status, kErrMma);
+                    tc_fence_after();
+                    const uint64_t bh = smem_desc(w + (layer ? L::W3h : L::W1h), 0, 1024, kSwz128);
+                    const uint64_t bl = smem_desc(w + (layer ? L::W3l : L::W1l), 0, 1024, kSwz128);
+                    const uint64_t oc = smem_desc(w + (layer ? L::W4c : L::W2c), 0, 1024, kSwz128);
+                    constexpr uint32_t kG1 = 8192, kG3 = R * 128;
+                    auto groups = [&](int g) {          // columns 64 g of p1 = n0 W1 or p3 = a2 W3
+                        const uint32_t go = g * (layer ? kG3 : kG1);
+                        const int ks = layer ? R / 16 : 4;
+#pragma unroll
+                        for (int part = 0; part < 3; ++part)
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                if (k >= ks) break;
+                                // n0: halves of 32 columns, [hi 16 | lo 16]; a2: 16 entries, [hi 8 | lo 8]
+                                const uint32_t a = layer ? k * 16 + (part == 1 ? 8 : 0) : (k / 2) * 32 + (k % 2) * 8 + (part == 1 ? 16 : 0);
+                                umma_ts(t0 + cS + (g & 1) * 64, t0 + cN + a, desc_off(part == 2 ? bl : bh, go + k * 2048), id_s, (part > 0 || k > 0) ? 1u : 0u);
+                            }
+                        umma_commit(&bar_s[slot][g & 1]);
+                    };
+                    groups(0);
+                    groups(1);
+#pragma unroll
+                    for (int g = 0; g < NG; ++g) {
+                        const int b = g & 1;
+                        mbar_spin(&bar_p[slot][b], pp[b], status, kErrMma);
+                        pp[b] ^= 1;
+                        tc_fence_after();
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const uint32_t a = t0 + cS + b * 64 + (k / 2) * 32 + (k % 2) * 8;
+                            const uint64_t bo = desc_off(oc, g * 8192 + k * 2048);
+                            umma_ts(t0 + cO, a, bo, id_o, (g > 0 || k > 0) ? 1u : 0u);
+                            umma_ts(t0 + cO, a + 16, bo, id_l, 1u);
+                        }
+                        if (g + 2 < NG) {
+                            umma_commit(&bar_f[slot][b]);
+                            mbar_spin(&bar_f[slot][b], pf[b], status, kErrMma);
+                            pf[b] ^= 1;
+                            groups(g + 2);
+                        }
+                    }
+                    umma_commit(&bar_o[slot]);
+                }
+            }
+        }
+    } else {
+        // ============================ rows ============================
+        const int wg = warp / 4, slot = wg & 1, half = wg >> 1, wt = tid % 128;
+        const uint32_t t0 = tm + slot * 256 + ((uint32_t)((warp % 4) * 32) << 16);
+        const bool narrow = half < R / 16;              // this half has 16 of the r narrow columns
+        const int c16 = half * 16;
+        uint32_t ps[2] = {0, 0}, po = 0;
+        uint4 xv[4];
+        float2 s0 = make_float2(0.f, 0.f);
+        auto load_x = [&](int tile) {
+            const uint4* src = reinterpret_cast<const uint4*>(X + sl.row(row0 + (size_t)tile * 128 + wt) + 32 * half);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) xv[q] = src[q];
+            s0 = st0[(size_t)tile * 128 + wt];
+        };
+        int tile = blockIdx.x * 2 + slot;
+        if (tile < tiles) load_x(tile);
+        for (; tile < tiles; tile += 2 * gridDim.x) {
+            const size_t row = (size_t)tile * 128 + wt;
+            {
+                uint32_t h[16], l[16];
+                const f2 mu = both(-s0.x), rs = both(s0.y);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t u[4] = {xv[q].x, xv[q].y, xv[q].z, xv[q].w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) split2(mul2(fma2(unpack2(u[i]), both(1.f), mu), rs), h[4 * q + i], l[4 * q + i]);
+                }
+                tmem_st16(t0 + cN + 32 * half, h);
+                tmem_st16(t0 + cN + 32 * half + 16, l);
+                tmem_st_wait();
+                tc_fence_before();
+                warp_arrive(&bar_n[slot]);
+            }
+            f2 sum = 0ull, sq = 0ull;
+            // p -> gelu(p) of this half of a group, back as an operand
+            auto group = [&](int g, const float* bias, bool stats) {
+                const int b = g & 1;
+                const uint32_t ta = t0 + cS + b * 64 + 32 * half;
+                mbar_wait(&bar_s[slot][b], ps[b], status, kErrMma);
+                ps[b] ^= 1;
+                tc_fence_after();
+                uint32_t u[32];
+                tmem_ld32(ta, u);
+                tmem_ld_wait();
+                uint32_t h[16], l[16];
+                const float* bp = bias + g * 64 + 32 * half;
+#pragma unroll
+                for (int i = 0; i < 16; i += 2) {
+                    const cc::F22 bb = cc::lds22(bp + 2 * i);
+                    const f2 g0 = gelu2(fma2(pack2(__uint_as_float(u[2 * i]), __uint_as_float(u[2 * i + 1])), both(1.f), bb.x));
+                    const f2 g1 = gelu2(fma2(pack2(__uint_as_float(u[2 * i + 2]), __uint_as_float(u[2 * i + 3])), both(1.f), bb.y));
+                    if (stats) {
+                        sum = fma2(g0, both(1.f), sum); sum = fma2(g1, both(1.f), sum);
+                        sq = fma2(g0, g0, sq); sq = fma2(g1, g1, sq);
+                    }
+                    split2(g0, h[i], l[i]);
+                    split2(g1, h[i + 1], l[i + 1]);
+                }
+                tmem_st16(ta, h);
+                tmem_st16(ta + 16, l);
+                tmem_st_wait();
+                tc_fence_before();
+                warp_arrive(&bar_p[slot][b]);
+            };
+#pragma unroll 1
+            for (int g = 0; g < NG; g += 2) { group(g, sv, true); group(g + 1, sv, true); }
+            s_part[slot][half][wt] = make_float2(lo2(sum) + hi2(sum), lo2(sq) + hi2(sq));
+            asm volatile("bar.sync %0, 256;" ::"r"(slot + 1) : "memory");
+            const float2 q0 = s_part[slot][0][wt], q1 = s_part[slot][1][wt];
+            constexpr float inv = 1.f / (float)L::M;
+            const float mu1 = (q0.x + q1.x) * inv;
+            const float rs1 = rsqrtf(fmaxf((q0.y + q1.y) * inv - mu1 * mu1, 0.f) + kLnEps);
+            if (half == 0 && st1 != nullptr) st1[net * st1_net + row] = make_float2(mu1, rs1);
+            // this thread's 16 of the r columns of O: both terms of the weights added up
+            auto read_o = [&](float (&o)[16]) {
+                mbar_wait(&bar_o[slot], po, status, kErrMma);
+                po ^= 1;
+                tc_fence_after();
+                if (narrow) {
+                    uint32_t u[16], v[16];
+                    tmem_ld16(t0 + cO + c16, u);
+                    tmem_ld16(t0 + cO + R + c16, v);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) o[i] = __uint_as_float(u[i]) + __uint_as_float(v[i]);
+                }
+            };
+            {
+                float o[16];
+                read_o(o);
+                if (narrow) {
+                    uint32_t h[8], l[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int c = c16 + 2 * i;
+                        const f2 v = pack2(fmaf(rs1, fmaf(-mu1, sv[kVcs + c], o[2 * i]), sv[kVb2 + c]),
+                                           fmaf(rs1, fmaf(-mu1, sv[kVcs + c + 1], o[2 * i + 1]), sv[kVb2 + c + 1]));
+                        split2(v, h[i], l[i]);
+                    }
+                    tmem_st8(t0 + cN + 16 * half, h);
+                    tmem_st8(t0 + cN + 16 * half + 8, l);
+                    tmem_st_wait();
+                    if (a2 != nullptr) {                // rows of 64: [hi r | lo r]
+                        uint4* dst = reinterpret_cast<uint4*>(a2 + net * a2_net + row * 64 + c16);
+                        dst[0] = make_uint4(h[0], h[1], h[2], h[3]);
+                        dst[1] = make_uint4(h[4], h[5], h[6], h[7]);
+                        dst[R / 8] = make_uint4(l[0], l[1], l[2], l[3]);
+                        dst[R / 8 + 1] = make_uint4(l[4], l[5], l[6], l[7]);
+                    }
+                }
+                tc_fence_before();
+                warp_arrive(&bar_n[slot]);
+            }
+#pragma unroll 1
+            for (int g = 0; g < NG; g += 2) { group(g, sv + kVb3, false); group(g + 1, sv + kVb3, false); }
+            if (tile + 2 * (int)gridDim.x < tiles) load_x(tile + 2 * gridDim.x);      // in flight during the last product
+            {
+                float o[16];
+                read_o(o);
+                if (narrow) {
+                    float4* dst = reinterpret_cast<float4*>(f + net * f_net + row * R + c16);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        dst[i] = make_float4(o[4 * i] + sv[kVb4 + c16 + 4 * i], o[4 * i + 1] + sv[kVb4 + c16 + 4 * i + 1],
+                                             o[4 * i + 2] + sv[kVb4 + c16 + 4 * i + 2], o[4 * i + 3] + sv[kVb4 + c16 + 4 * i + 3]);
+                }
+                tc_fence_before();
+            }
+        }
+    }
+    // (every MMA has completed: the rows waited for the last product of every tile)
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 16) tmem_dealloc(tm, 512);
+}
+
+// ---------------------------------------------------------------------------
+// Layers 4 and 3 backward of one network (blockIdx.y), persistent, one tile of 128 rows at a time:
+//   p3 = a2 W3 + b3,  da3 = df W4^T,  dp3 = da3 gelu'(p3),  a3 = gelu(p3)
+//   da2 = dp3 W3^T,   dW4 += a3^T df,  dW3 += dp3^T a2      and the column sums of dp3 and df.
+// Warps 0-15 (thread = row): warpgroups w and w + 2 take the groups of parity w, a half of 32 columns each; two
+// groups are in tensor memory at a time (p3 and da3, 64 columns each).  Their a3 and dp3 go to shared memory
+// as bf16 tiles, 128 columns (a step) at a time, the operands of the last three products.  Warp 16: one
+// thread loads and issues every MMA; the next step's p3, da3 are formed while the rows work on this one's.
+// Warps 17, 18: column sums, from the same tiles.
+// ---------------------------------------------------------------------------
+constexpr int kBwdThreads = 19 * 32;
+
+// sums of two columns (this lane's) of a [128 x 64] bf16 tile
+__device__ __forceinline__ void tile_column_sums(const uint8_t* t, int lane, float& s0, float& s1) {
+    const uint8_t* p = t + (lane % 4) * 4;
+#pragma unroll 8
+    for (int row = 0; row < 128; ++row) {
+        const uint32_t w = *reinterpret_cast<const uint32_t*>(p + swz128_offset(row, lane / 4));
+        s0 += __uint_as_float(w << 16);
+        s1 += __uint_as_float(w & 0xffff0000u);
+    }
+}
+__device__ __forceinline__ void red_add4(float* dst, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(__uint_as_float(a)), "f"(__uint_as_float(b)),
+                 "f"(__uint_as_float(c)), "f"(__uint_as_float(d)) : "memory");
+}
+// 16 accumulator columns of this thread's row into a gradient row
+__device__ __forceinline__ void add_columns16(uint32_t taddr, float* dst) {
+    uint32_t u[16];
+    tmem_ld16(taddr, u);
+    tmem_ld_wait();
+#pragma unroll
+    for (int j = 0; j < 16; j += 4) red_add4(dst + j, u[j], u[j + 1], u[j + 2], u[j + 3]);
+}
+// 32 columns (16 packed words) of a row into a [128 x 64] tile, half 0 or 1
+__device__ __forceinline__ void tile_put32(uint8_t* tile, int row, int half, const uint32_t (&v)[16]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        *reinterpret_cast<uint4*>(tile + swz128_offset(row, 4 * half + j)) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+}
+
+template <int R> struct Bwd34 {
+    static constexpr int W = Bank<R>::W2t - Bank<R>::W3h;               // W3h | W3l | W4c
+    static constexpr int T = W, In = T + 4 * 16384, kIn = 32768;        // a3, dp3 of a step; three (a2, df) inputs
+    static constexpr int bytes = In + 3 * kIn + 1024;
+};
+
+template <int R>
+__global__ void __launch_bounds__(kBwdThreads, 1)
+ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1, const __grid_constant__ CUtensorMap mD0,
+                 const __grid_constant__ CUtensorMap mD1, size_t row0, int tiles, const uint8_t* __restrict__ bank,
+                 const float* __restrict__ vec, bf16* __restrict__ da2, size_t da2_net, float2* __restrict__ mm, size_t mm_net,
+                 float* __restrict__ G, float* __restrict__ sums, int* status) {
+    using L = Bank<R>;
+    using B = Bwd34<R>;
+    constexpr int NH = L::NH;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = align1024(smem_raw);
+    __shared__ uint64_t bar_w, bar_ld[3], bar_s[2], bar_rd[2], bar_t, bar_free;
+    __shared__ uint32_t tm_slot;
+    __shared__ __align__(16) float sb3[256];
+    __shared__ float scs[R], sb2[R];
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, net = blockIdx.y;
+    const int nt = (tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x, steps = nt * NH;
+    const CUtensorMap* mA = net ? &mA1 : &mA0;
+    const CUtensorMap* mD = net ? &mD1 : &mD0;
+    if (tid == 0) {
+        cta_giveup_init();
+        mbar_init(&bar_w, 1);
+        for (int i = 0; i < 3; ++i) mbar_init(&bar_ld[i], 1);
+        for (int b = 0; b < 2; ++b) { mbar_init(&bar_s[b], 1); mbar_init(&bar_rd[b], 8); }
+        mbar_init(&bar_t, 16);
+        mbar_init(&bar_free, 3);
+        mbar_fence_init();
+    }
+    pdl_sync();
+    if (warp == 16) { tmem_alloc(&tm_slot, 512); tmem_relinquish(); }
+    for (int e = tid; e < 256; e += kBwdThreads) sb3[e] = vec[(size_t)net * kVec + kVb3 + e];
+    if (tid < R) { scs[tid] = vec[(size_t)net * kVec + kVcs + tid]; sb2[tid] = vec[(size_t)net * kVec + kVb2 + tid]; }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tm = tm_slot;
+    constexpr uint32_t cDa2 = 256, cW4 = 256 + 32, cW3 = cW4 + 64;
+    auto tile_at = [&](int i) { return (int)blockIdx.x + i * (int)gridDim.x; };
+    if (warp == 16) {
+        if (lane == 0) {
+            auto load = [&](int i) {
+                uint8_t* dst = smem + B::In + (i % 3) * B::kIn;
+                mbar_expect_tx(&bar_ld[i % 3], B::kIn);
+                tma_load_2d(dst, mA, 0, (int)row0 + tile_at(i) * 128, &bar_ld[i % 3]);
+                tma_load_2d(dst + 16384, mD, 0, tile_at(i) * 128, &bar_ld[i % 3]);
+            };
+            mbar_expect_tx(&bar_w, B::W);
+            load_image(smem, bank + (size_t)net * kBankBytes + L::W3h, B::W, &bar_w);
+            load(0);
+            if (nt > 1) load(1);
+            mbar_spin(&bar_w, 0, status, kErrTma);
+            const uint32_t sw = smem_u32(smem);
+            constexpr uint32_t w3h = 0, w3l = L::W3l - L::W3h, w4c = L::W4c - L::W3h, kG3 = R * 128;
+            constexpr uint32_t id_s = idesc_bf16(128, 64, false, true), id_d = idesc_bf16(128, 64, false, false),
+                               id_a = idesc_bf16(128, R, false, false), id_w = idesc_bf16(128, R, true, true);
+            auto form = [&](int k) {                   // p3 and da3 of step k
+                const int i = k / NH, hf = k % NH;
+                if (hf == 0) mbar_spin(&bar_ld[i % 3], (i / 3) & 1, status, kErrTma);
+                const uint32_t in = sw + B::In + (i % 3) * B::kIn;
+                const uint64_t ad = smem_desc(in, 0, 1024, kSwz128), dd = smem_desc(in + 16384, 0, 1024, kSwz128);
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const int g = 2 * hf + b;
+                    if (k > 0) mbar_spin(&bar_rd[b], (k - 1) & 1, status, kErrMma);
+                    tc_fence_after();
+                    const uint64_t bh = smem_desc(sw + w3h + g * kG3, 0, 1024, kSwz128), bl = smem_desc(sw + w3l + g * kG3, 0, 1024, kSwz128);
+                    const uint64_t w4 = smem_desc(sw + w4c + g * 8192, 0, 1024, kSwz128);
+#pragma unroll
+                    for (int part = 0; part < 3; ++part)
+#pragma unroll
+                        for (int q = 0; q < R / 16; ++q)
+                            umma_ss(tm + b * 128, desc_off(ad, q * 32 + (part == 1 ? 2 * R : 0)), desc_off(part == 2 ? bl : bh, q * 2048), id_s,
+                                    (part > 0 || q > 0) ? 1u : 0u);
+#pragma unroll
+                    for (int q = 0; q < R / 16; ++q)
+                        umma_ss(tm + b * 128 + 64, desc_off(dd, q * 32), desc_off(w4, q * 32), id_d, q > 0 ? 1u : 0u);
+                    umma_commit(&bar_s[b]);
+                }
+            };
+            form(0);
+            for (int k = 0; k < steps; ++k) {
+                const int i = k / NH, hf = k % NH;
+                if (k + 1 < steps) form(k + 1);
+                mbar_spin(&bar_t, k & 1, status, kErrMma);
+                tc_fence_after();
+                // tile i - 1 is done with (its last products have completed, its da2 has been read): its input buffer
+                // takes tile i + 2
+                if (hf == 0 && i + 2 < nt) load(i + 2);
+                const uint32_t in = sw + B::In + (i % 3) * B::kIn, t3 = sw + B::T, td = t3 + 32768;
+                const uint64_t dk = smem_desc(td, 0, 1024, kSwz128);
+                const uint64_t am = smem_desc(t3, 16384, 1024, kSwz128), dm = smem_desc(td, 16384, 1024, kSwz128);
+                const uint64_t a2b = smem_desc(in, 0, 1024, kSwz128), dfb = smem_desc(in + 16384, 0, 1024, kSwz128);
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    umma_ss(tm + cDa2, desc_off(dk, (q / 4) * 16384 + (q % 4) * 32),
+                            desc_off(smem_desc(sw + w3h + (2 * hf + q / 4) * kG3, 0, 1024, kSwz128), (q % 4) * 32), id_a, (hf > 0 || q > 0) ? 1u : 0u);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) umma_ss(tm + cW4 + hf * R, desc_off(am, q * 2048), desc_off(dfb, q * 2048), id_w, (i > 0 || q > 0) ? 1u : 0u);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) umma_ss(tm + cW3 + hf * R, desc_off(dm, q * 2048), desc_off(a2b, q * 2048), id_w, (i > 0 || q > 0) ? 1u : 0u);
+                umma_commit(&bar_free);
+            }
+            if (steps > 0) mbar_spin(&bar_free, (steps - 1) & 1, status, kErrMma);
+        }
+    } else if (warp > 16) {
+        const int j = warp - 17;                       // atom j of dp3; warp 17 also df
+        float s[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, d0 = 0.f, d1 = 0.f;
+        for (int k = 0; k < steps; ++k) {
+            const int i = k / NH, hf = k % NH;
+            mbar_wait(&bar_t, k & 1, status, kErrMma);
+            if (NH > 1 && hf == 1) tile_column_sums(smem + B::T + 32768 + j * 16384, lane, s[1][0], s[1][1]);
+            else tile_column_sums(smem + B::T + 32768 + j * 16384, lane, s[0][0], s[0][1]);
+            if (j == 0 && hf == 0) {
+                mbar_wait(&bar_ld[i % 3], (i / 3) & 1, status, kErrTma);
+                tile_column_sums(smem + B::In + (i % 3) * B::kIn + 16384, lane, d0, d1);
+            }
+            warp_arrive(&bar_free);
+        }
+        float* s_dp3 = sums + (size_t)net * kSums + 320;
+#pragma unroll
+        for (int hf = 0; hf < NH; ++hf) {
+            atomicAdd(s_dp3 + hf * 128 + j * 64 + 2 * lane, s[hf][0]);
+            atomicAdd(s_dp3 + hf * 128 + j * 64 + 2 * lane + 1, s[hf][1]);
+        }
+        if (j == 0 && 2 * lane < R) {
+            atomicAdd(sums + (size_t)net * kSums + 576 + 2 * lane, d0);
+            atomicAdd(sums + (size_t)net * kSums + 576 + 2 * lane + 1, d1);
+        }
+    } else {
+        const int wg = warp / 4, p = wg & 1, half = wg >> 1, wt = tid % 128;
+        const uint32_t lane_tm = tm + ((uint32_t)((warp % 4) * 32) << 16);
+        // da2 of tile i, 16 columns per warpgroup: stored, and this part of the two row sums of the normalisation's
+        // backward, da2 . (1^T W2) and da2 . (a2 - b2), over 8r
+        auto finish_tile = [&](int i) {
+            if (wg >= R / 16) return;
+            const int c0 = 16 * wg;
+            const size_t row = (size_t)tile_at(i) * 128 + wt;
+            uint32_t u[16];
+            tmem_ld16(lane_tm + cDa2 + c0, u);
+            tmem_ld_wait();
+            const uint8_t* ta = smem + B::In + (i % 3) * B::kIn;
+            mbar_wait(&bar_ld[i % 3], (i / 3) & 1, status, kErrTma);
+            float m1 = 0.f, m2 = 0.f;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint4 h = *reinterpret_cast<const uint4*>(ta + swz128_offset(wt, c0 / 8 + q));
+                const uint4 l = *reinterpret_cast<const uint4*>(ta + swz128_offset(wt, (R + c0) / 8 + q));
+                const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, lw[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int c = c0 + 8 * q + e;
+                    const float v = __uint_as_float(u[8 * q + e]);
+                    const float a = __uint_as_float((e & 1) ? (hw[e / 2] & 0xffff0000u) : (hw[e / 2] << 16)) +
+                                    __uint_as_float((e & 1) ? (lw[e / 2] & 0xffff0000u) : (lw[e / 2] << 16));
+                    m1 = fmaf(v, scs[c], m1);
+                    m2 = fmaf(v, a - sb2[c], m2);
+                }
+            }
+            uint32_t pk[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) pk[e] = pack_bf16(__uint_as_float(u[2 * e]), __uint_as_float(u[2 * e + 1]));
+            uint4* dst = reinterpret_cast<uint4*>(da2 + net * da2_net + row * 64 + c0);
+            dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+            constexpr float inv = 1.f / (float)L::M;
+            mm[net * mm_net + row * 2 + wg] = make_float2(m1 * inv, m2 * inv);
+        };
+        for (int k = 0; k < steps; ++k) {
+            const int i = k / NH, hf = k % NH;
+            const uint32_t ta = lane_tm + p * 128 + 32 * half;
+            const float* bp = sb3 + (2 * hf + p) * 64 + 32 * half;
+            mbar_wait(&bar_s[p], k & 1, status, kErrMma);
+            tc_fence_after();
+            uint32_t a3[16], dp[16];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                uint32_t u[16], v[16];
+                tmem_ld16(ta + 16 * q, u);
+                tmem_ld16(ta + 64 + 16 * q, v);
+                tmem_ld_wait();
+                if (q == 1) { tc_fence_before(); warp_arrive(&bar_rd[p]); }
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const f2 bb = *reinterpret_cast<const f2*>(bp + 16 * q + 2 * e);
+                    f2 gr;
+                    const f2 g = gelu2_grad(fma2(pack2(__uint_as_float(u[2 * e]), __uint_as_float(u[2 * e + 1])), both(1.f), bb), gr);
+                    const f2 d = mul2(pack2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1])), gr);
+                    a3[8 * q + e] = pack_bf16(lo2(g), hi2(g));
+                    dp[8 * q + e] = pack_bf16(lo2(d), hi2(d));
+                }
+            }
+            if (k > 0) mbar_wait(&bar_free, (k - 1) & 1, status, kErrMma);
+            tc_fence_after();
+            if (hf == 0 && i > 0) finish_tile(i - 1);
+            tile_put32(smem + B::T + p * 16384, wt, half, a3);
+            tile_put32(smem + B::T + 32768 + p * 16384, wt, half, dp);
+            fence_proxy_async_smem();
+            tc_fence_before();
+            warp_arrive(&bar_t);
+        }
+        if (steps > 0) {
+            mbar_wait(&bar_free, (steps - 1) & 1, status, kErrMma);
+            tc_fence_after();
+            finish_tile(nt - 1);
+            if (wg < 2 * NH) {                         // one of the gradient accumulators each
+                const int hf = wg % NH, which = wg / NH;
+                float* dst = G + ((size_t)net * 4 + (which ? 2 : 3)) * kMat + (size_t)(hf * 128 + wt) * 64;
+#pragma unroll
+                for (int c = 0; c < R; c += 16) add_columns16(lane_tm + (which ? cW3 : cW4) + hf * R + c, dst + c);
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 16) tmem_dealloc(tm, 512);
+}
+
+// ---------------------------------------------------------------------------
+// Layers 2 and 1 backward of one network, in the manner of ltc_wgrad_kernel:
+//   p1 = n0 W1 + b1',  n1 = rs1 (gelu(p1) - mu1),  dn1 = da2 (diag(g1) W2)^T,
+//   dp1 = rs1 (dn1 - m1 - n1 m2) gelu'(p1),   m1, m2 the mean of dn1 and of dn1 n1 (from ltc_wgrad_kernel)
+//   dn0 = dp1 W1^T,   dW2 += n1^T da2,   dW1 += dp1^T n0      and the column sums of dp1 and da2.
+// Inputs by TMA: da2 and the hi terms of n0 in two buffers, the lo terms (needed only for p1) in one.
+// ---------------------------------------------------------------------------
+template <int R> struct Bwd12 {
+    static constexpr int W1 = 0, W2t = 2 * Bank<R>::kW1, T = W2t + Bank<R>::kW3;       // T: n1, dp1 of a step
+    static constexpr int In = T + 4 * 16384, kIn = 32768, Lo = In + 2 * kIn;
+    static constexpr int bytes = Lo + 16384 + 1024;
+};
+
+template <int R>
+__global__ void __launch_bounds__(kBwdThreads, 1)
+ltc_dense_bwd_norm_kernel(const __grid_constant__ CUtensorMap mN, const __grid_constant__ CUtensorMap mNlo,
+                          const __grid_constant__ CUtensorMap mD0, const __grid_constant__ CUtensorMap mD1, size_t row0, int tiles,
+                          const uint8_t* __restrict__ bank, const float* __restrict__ vec, const float2* __restrict__ st1, size_t st1_net,
+                          const float2* __restrict__ mm, size_t mm_net, float* __restrict__ dn0, size_t dn0_net,
+                          float* __restrict__ G, float* __restrict__ sums, int* status) {
+    using L = Bank<R>;
+    using B = Bwd12<R>;
+    constexpr int NH = L::NH;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = align1024(smem_raw);
+    __shared__ uint64_t bar_w, bar_ld[2], bar_lo, bar_s[2], bar_rd[2], bar_t, bar_free;
+    __shared__ uint32_t tm_slot;
+    __shared__ __align__(16) float sb1[256];
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, net = blockIdx.y;
+    const int nt = (tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x, steps = nt * NH;
+    const CUtensorMap* mD = net ? &mD1 : &mD0;
+    if (tid == 0) {
+        cta_giveup_init();
+        mbar_init(&bar_w, 1); mbar_init(&bar_lo, 1);
+        for (int b = 0; b < 2; ++b) { mbar_init(&bar_ld[b], 1); mbar_init(&bar_s[b], 1); mbar_init(&bar_rd[b], 8); }
+        mbar_init(&bar_t, 16);
+        mbar_init(&bar_free, 3);
+        mbar_fence_init();
+    }
+    pdl_sync();
+    if (warp == 16) { tmem_alloc(&tm_slot, 512); tmem_relinquish(); }
+    for (int e = tid; e < 256; e += kBwdThreads) sb1[e] = vec[(size_t)net * kVec + e];
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tm = tm_slot;
+    constexpr uint32_t cN0 = 256, cW2 = cN0 + 64, cW1 = cW2 + 64;
+    auto tile_at = [&](int i) { return (int)blockIdx.x + i * (int)gridDim.x; };
+    if (warp == 16) {
+        if (lane == 0) {
+            auto load = [&](int i) {
+                uint8_t* dst = smem + B::In + (i & 1) * B::kIn;
+                mbar_expect_tx(&bar_ld[i & 1], B::kIn);
+                tma_load_2d(dst, mD, 0, tile_at(i) * 128, &bar_ld[i & 1]);
+                tma_load_2d(dst + 16384, &mN, 0, tile_at(i) * 128, &bar_ld[i & 1]);
+            };
+            auto load_lo = [&](int i) {
+                mbar_expect_tx(&bar_lo, 16384);
+                tma_load_2d(smem + B::Lo, &mNlo, 0, tile_at(i) * 128, &bar_lo);
+            };
+            mbar_expect_tx(&bar_w, B::T);
+            load_image(smem, bank + (size_t)net * kBankBytes + L::W1h, 2 * L::kW1, &bar_w);
+            load_image(smem + B::W2t, bank + (size_t)net * kBankBytes + L::W2t, L::kW3, &bar_w);
+            load(0);
+            load_lo(0);
+            mbar_spin(&bar_w, 0, status, kErrTma);
+            const uint32_t sw = smem_u32(smem);
+            constexpr uint32_t w1l = L::kW1, kG3 = R * 128;
+            constexpr uint32_t id_s = idesc_bf16(128, 64, false, true), id_n = idesc_bf16(128, 64, false, false),
+                               id_w2 = idesc_bf16(128, R, true, true), id_w1 = idesc_bf16(128, 64, true, true);
+            const uint64_t nl = smem_desc(sw + B::Lo, 0, 1024, kSwz128);
+            auto form = [&](int k) {                   // p1 and dn1 of step k
+                const int i = k / NH, hf = k % NH;
+                if (k > 0) { mbar_spin(&bar_rd[0], (k - 1) & 1, status, kErrMma); mbar_spin(&bar_rd[1], (k - 1) & 1, status, kErrMma); }
+                if (hf == 0) {
+                    if (i > 0) load_lo(i);             // (the last products that read it have completed: they were read out)
+                    mbar_spin(&bar_ld[i & 1], (i >> 1) & 1, status, kErrTma);
+                    mbar_spin(&bar_lo, i & 1, status, kErrTma);
+                }
+                tc_fence_after();
+                const uint32_t in = sw + B::In + (i & 1) * B::kIn;
+                const uint64_t dd = smem_desc(in, 0, 1024, kSwz128), nh = smem_desc(in + 16384, 0, 1024, kSwz128);
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const int g = 2 * hf + b;
+                    const uint64_t bh = smem_desc(sw + g * 8192, 0, 1024, kSwz128), bl = smem_desc(sw + w1l + g * 8192, 0, 1024, kSwz128);
+                    const uint64_t w2 = smem_desc(sw + B::W2t + g * kG3, 0, 1024, kSwz128);
+#pragma unroll
+                    for (int part = 0; part < 3; ++part)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            umma_ss(tm + b * 128, desc_off(part == 1 ? nl : nh, q * 32), desc_off(part == 2 ? bl : bh, q * 2048), id_s,
+                                    (part > 0 || q > 0) ? 1u : 0u);
+#pragma unroll
+                    for (int q = 0; q < R / 16; ++q)
+                        umma_ss(tm + b * 128 + 64, desc_off(dd, q * 32), desc_off(w2, q * 2048), id_s, q > 0 ? 1u : 0u);
+                    umma_commit(&bar_s[b]);
+                }
+            };
+            form(0);
+            for (int k = 0; k < steps; ++k) {
+                const int i = k / NH, hf = k % NH;
+                if (hf == 0 && i + 1 < nt) {           // the other input buffer: tile i - 1 is done with
+                    if (k > 0) mbar_spin(&bar_free, (k - 1) & 1, status, kErrMma);
+                    load(i + 1);
+                }
+                if (k + 1 < steps) form(k + 1);
+                mbar_spin(&bar_t, k & 1, status, kErrMma);
+                tc_fence_after();
+                const uint32_t in = sw + B::In + (i & 1) * B::kIn, t1 = sw + B::T, td = t1 + 32768;
+                const uint64_t dk = smem_desc(td, 0, 1024, kSwz128);
+                const uint64_t nm = smem_desc(t1, 16384, 1024, kSwz128), dm = smem_desc(td, 16384, 1024, kSwz128);
+                const uint64_t dab = smem_desc(in, 0, 1024, kSwz128), n0b = smem_desc(in + 16384, 0, 1024, kSwz128);
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    umma_ss(tm + cN0, desc_off(dk, (q / 4) * 16384 + (q % 4) * 32),
+                            desc_off(smem_desc(sw + (2 * hf + q / 4) * 8192, 0, 1024, kSwz128), (q % 4) * 32), id_n, (hf > 0 || q > 0) ? 1u : 0u);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) umma_ss(tm + cW2 + hf * R, desc_off(nm, q * 2048), desc_off(dab, q * 2048), id_w2, (i > 0 || q > 0) ? 1u : 0u);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) umma_ss(tm + cW1 + hf * 64, desc_off(dm, q * 2048), desc_off(n0b, q * 2048), id_w1, (i > 0 || q > 0) ? 1u : 0u);
+                umma_commit(&bar_free);
+            }
+            if (steps > 0) mbar_spin(&bar_free, (steps - 1) & 1, status, kErrMma);
+        }
+    } else if (warp > 16) {
+        const int j = warp - 17;                       // atom j of dp1; warp 17 also da2
+        float s[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, d0 = 0.f, d1 = 0.f;
+        for (int k = 0; k < steps; ++k) {
+            const int i = k / NH, hf = k % NH;
+            mbar_wait(&bar_t, k & 1, status, kErrMma);
+            if (NH > 1 && hf == 1) tile_column_sums(smem + B::T + 32768 + j * 16384, lane, s[1][0], s[1][1]);
+            else tile_column_sums(smem + B::T + 32768 + j * 16384, lane, s[0][0], s[0][1]);
+            if (j == 0 && hf == 0) {
+                mbar_wait(&bar_ld[i & 1], (i >> 1) & 1, status, kErrTma);
+                tile_column_sums(smem + B::In + (i & 1) * B::kIn, lane, d0, d1);
+            }
+            warp_arrive(&bar_free);
+        }
+        float* s_dp1 = sums + (size_t)net * kSums;
+#pragma unroll
+        for (int hf = 0; hf < NH; ++hf) {
+            atomicAdd(s_dp1 + hf * 128 + j * 64 + 2 * lane, s[hf][0]);
+            atomicAdd(s_dp1 + hf * 128 + j * 64 + 2 * lane + 1, s[hf][1]);
+        }
+        if (j == 0 && 2 * lane < R) {
+            atomicAdd(sums + (size_t)net * kSums + 256 + 2 * lane, d0);
+            atomicAdd(sums + (size_t)net * kSums + 256 + 2 * lane + 1, d1);
+        }
+    } else {
+        const int wg = warp / 4, p = wg & 1, half = wg >> 1, wt = tid % 128;
+        const uint32_t lane_tm = tm + ((uint32_t)((warp % 4) * 32) << 16);
+        auto finish_tile = [&](int i) {                // dn0, 16 columns per warpgroup
+            uint32_t u[16];
+            tmem_ld16(lane_tm + cN0 + 16 * wg, u);
+            tmem_ld_wait();
+            uint4* dst = reinterpret_cast<uint4*>(dn0 + net * dn0_net + ((size_t)tile_at(i) * 128 + wt) * 64 + 16 * wg);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) dst[q] = make_uint4(u[4 * q], u[4 * q + 1], u[4 * q + 2], u[4 * q + 3]);
+        };
+        // mu1, rs1, m1, m2 of this thread's row, requested a tile ahead
+        float2 nst = make_float2(0.f, 0.f), nm0 = nst, nm1 = nst;
+        auto load_row = [&](int i) {
+            const size_t row = (size_t)tile_at(i) * 128 + wt;
+            nst = st1[net * st1_net + row0 + row];
+            nm0 = mm[net * mm_net + row * 2];
+            if constexpr (R > 16) nm1 = mm[net * mm_net + row * 2 + 1];
+        };
+        if (nt > 0) load_row(0);
+        float mu1 = 0.f, rs1 = 0.f, m1 = 0.f, m2 = 0.f;
+        for (int k = 0; k < steps; ++k) {
+            const int i = k / NH, hf = k % NH;
+            if (hf == 0) {
+                mu1 = nst.x; rs1 = nst.y; m1 = nm0.x + nm1.x; m2 = nm0.y + nm1.y;
+                if (i + 1 < nt) load_row(i + 1);
+            }
+            const f2 nmu = both(-mu1 * rs1), rs = both(rs1), nm1r = both(-m1 * rs1), nm2r = both(-m2 * rs1);
+            const uint32_t ta = lane_tm + p * 128 + 32 * half;
+            const float* bp = sb1 + (2 * hf + p) * 64 + 32 * half;
+            mbar_wait(&bar_s[p], k & 1, status, kErrMma);
+            tc_fence_after();
+            uint32_t n1[16], dp[16];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                uint32_t u[16], v[16];
+                tmem_ld16(ta + 16 * q, u);
+                tmem_ld16(ta + 64 + 16 * q, v);
+                tmem_ld_wait();
+                if (q == 1) { tc_fence_before(); warp_arrive(&bar_rd[p]); }
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const f2 bb = *reinterpret_cast<const f2*>(bp + 16 * q + 2 * e);
+                    f2 gr;
+                    const f2 g = gelu2_grad(fma2(pack2(__uint_as_float(u[2 * e]), __uint_as_float(u[2 * e + 1])), both(1.f), bb), gr);
+                    const f2 n = fma2(g, rs, nmu);
+                    // rs1 (dn1 - m1 - n1 m2)
+                    const f2 d = fma2(n, nm2r, fma2(pack2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1])), rs, nm1r));
+                    const f2 o = mul2(d, gr);
+                    n1[8 * q + e] = pack_bf16(lo2(n), hi2(n));
+                    dp[8 * q + e] = pack_bf16(lo2(o), hi2(o));
+                }
+            }
+            if (k > 0) mbar_wait(&bar_free, (k - 1) & 1, status, kErrMma);
+            tc_fence_after();
+            if (hf == 0 && i > 0) finish_tile(i - 1);
+            tile_put32(smem + B::T + p * 16384, wt, half, n1);
+            tile_put32(smem + B::T + 32768 + p * 16384, wt, half, dp);
+            fence_proxy_async_smem();
+            tc_fence_before();
+            warp_arrive(&bar_t);
+        }
+        if (steps > 0) {
+            mbar_wait(&bar_free, (steps - 1) & 1, status, kErrMma);
+            tc_fence_after();
+            finish_tile(nt - 1);
+            const int hf = wg % 2, which = wg / 2;     // dW2, dW1; first and second 128 rows
+            if (hf < NH) {
+                float* dst = G + ((size_t)net * 4 + (which ? 0 : 1)) * kMat + (size_t)(hf * 128 + wt) * 64;
+#pragma unroll
+                for (int c = 0; c < 64; c += 16)
+                    if (which || c < R) add_columns16(lane_tm + (which ? cW1 + hf * 64 : cW2 + hf * R) + c, dst + c);
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 16) tmem_dealloc(tm, 512);
+}
+
+// ---------------------------------------------------------------------------
+// CUDA-core helpers
+// ---------------------------------------------------------------------------
+// Mean and 1 / sigma of every row (st0), and (n0 != nullptr: the backward) n0 = (x - mean) / sigma as hi + lo
+// rows.  One warp per row, two columns per lane, eight rows per warp with their loads issued together.
 constexpr int kLnRowsPerWarp = 8;
 __global__ void __launch_bounds__(256)
 ltc_ln0_kernel(Slice sl, const bf16* __restrict__ X, size_t row0, int rows, bf16* __restrict__ n0, bf16* __restrict__ n0_lo,
-               float* __restrict__ rs0) {
+               float2* __restrict__ st0) {
     pdl_sync();
     const int lane = threadIdx.x % 32;
     const int i0 = (blockIdx.x * 8 + threadIdx.x / 32) * kLnRowsPerWarp;
@@ -880,91 +986,114 @@ ltc_ln0_kernel(Slice sl, const bf16* __restrict__ X, size_t row0, int rows, bf16
         float v = (a - mu) * (a - mu) + (b - mu) * (b - mu);
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         const float rs = rsqrtf(v * (1.f / 64.f) + kLnEps);
+        if (lane == 0) st0[i] = make_float2(mu, rs);
+        if (n0 == nullptr) continue;
         const float na = (a - mu) * rs, nb = (b - mu) * rs;
         const uint32_t h = pack_bf16(na, nb);
         *reinterpret_cast<uint32_t*>(n0 + (size_t)i * 64 + 2 * lane) = h;
         *reinterpret_cast<uint32_t*>(n0_lo + (size_t)i * 64 + 2 * lane) =
             pack_bf16(na - __uint_as_float(h << 16), nb - __uint_as_float(h & 0xffff0000u));
-        if (lane == 0) rs0[i] = rs;
     }
 }
 
-// dX = back through the first normalisation of the summed gradient of n0 (+ add)
+// dX = back through the first normalisation of the two networks' gradients of n0 (+ add); one warp per row,
+// four rows' loads in flight
+constexpr int kLnBwdRows = 4;
 __global__ void __launch_bounds__(256)
-ltc_ln0_bwd_kernel(Slice sl, size_t row0, int rows, const float* __restrict__ dn0, const bf16* __restrict__ n0,
-                   const float* __restrict__ rs0, const bf16* __restrict__ add, bf16* __restrict__ dX) {
+ltc_ln0_bwd_kernel(Slice sl, size_t row0, int rows, const float* __restrict__ dn0, size_t dn0_net, const bf16* __restrict__ n0,
+                   const float2* __restrict__ st0, const bf16* __restrict__ add, bf16* __restrict__ dX) {
     pdl_sync();
     const int lane = threadIdx.x % 32;
-    const int i = blockIdx.x * 8 + threadIdx.x / 32;
-    if (i >= rows) return;
-    const float2 d = *reinterpret_cast<const float2*>(dn0 + (size_t)i * 64 + 2 * lane);
-    const __nv_bfloat162 n2 = *reinterpret_cast<const __nv_bfloat162*>(n0 + (size_t)i * 64 + 2 * lane);
-    const float na = __low2float(n2), nb = __high2float(n2);
-    float s1 = d.x + d.y, s2 = d.x * na + d.y * nb;
-    for (int o = 16; o > 0; o >>= 1) { s1 += __shfl_xor_sync(0xffffffffu, s1, o); s2 += __shfl_xor_sync(0xffffffffu, s2, o); }
-    const float m1 = s1 * (1.f / 64.f), m2 = s2 * (1.f / 64.f), rs = rs0[i];
-    float oa = rs * (d.x - m1 - na * m2), ob = rs * (d.y - m1 - nb * m2);
-    if (add != nullptr) {
-        const __nv_bfloat162 q = *reinterpret_cast<const __nv_bfloat162*>(add + (row0 + i) * 64 + 2 * lane);
-        oa += __low2float(q); ob += __high2float(q);
+    const int i0 = (blockIdx.x * 8 + threadIdx.x / 32) * kLnBwdRows;
+    float2 d0[kLnBwdRows], d1[kLnBwdRows];
+    __nv_bfloat162 n2[kLnBwdRows], ad[kLnBwdRows];
+    float rs[kLnBwdRows];
+#pragma unroll
+    for (int q = 0; q < kLnBwdRows; ++q) {
+        const size_t i = i0 + q;
+        if ((int)i >= rows) break;
+        d0[q] = *reinterpret_cast<const float2*>(dn0 + i * 64 + 2 * lane);
+        d1[q] = *reinterpret_cast<const float2*>(dn0 + dn0_net + i * 64 + 2 * lane);
+        n2[q] = *reinterpret_cast<const __nv_bfloat162*>(n0 + i * 64 + 2 * lane);
+        if (add != nullptr) ad[q] = *reinterpret_cast<const __nv_bfloat162*>(add + (row0 + i) * 64 + 2 * lane);
+        rs[q] = st0[i].y;
     }
-    *reinterpret_cast<uint32_t*>(dX + sl.row(row0 + i) + 2 * lane) = pack_bf16(oa, ob);
+#pragma unroll
+    for (int q = 0; q < kLnBwdRows; ++q) {
+        const int i = i0 + q;
+        if (i >= rows) break;
+        const float dx = d0[q].x + d1[q].x, dy = d0[q].y + d1[q].y;
+        const float na = __low2float(n2[q]), nb = __high2float(n2[q]);
+        float s1 = dx + dy, s2 = dx * na + dy * nb;
+        for (int o = 16; o > 0; o >>= 1) { s1 += __shfl_xor_sync(0xffffffffu, s1, o); s2 += __shfl_xor_sync(0xffffffffu, s2, o); }
+        const float m1 = s1 * (1.f / 64.f), m2 = s2 * (1.f / 64.f);
+        float oa = rs[q] * (dx - m1 - na * m2), ob = rs[q] * (dy - m1 - nb * m2);
+        if (add != nullptr) { oa += __low2float(ad[q]); ob += __high2float(ad[q]); }
+        *reinterpret_cast<uint32_t*>(dX + sl.row(row0 + i) + 2 * lane) = pack_bf16(oa, ob);
+    }
 }
 
 // M = sqrt(r) tanh(f1 f2 / sqrt(r)), written as the [hi | lo] rows (64 bf16 columns, zero beyond 2r) the
-// attention kernels read in their linear sketch mode; one thread = 8 consecutive columns of a row
+// attention kernels read in their linear sketch mode; one thread = 8 entries of a row
+__device__ __forceinline__ void load8f(const float* p, float (&v)[8]) {
+    const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+template <int R>
 __global__ void __launch_bounds__(256)
-ltc_combine_kernel(const float* __restrict__ f1, const float* __restrict__ f2, int r, size_t rows, bf16* __restrict__ S) {
+ltc_combine_kernel(const float* __restrict__ f1, const float* __restrict__ f2p, size_t rows, bf16* __restrict__ S) {
     pdl_sync();
     const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (e >= rows * 8) return;
-    const size_t row = e / 8;
-    const int c0 = (int)(e % 8) * 8;
-    const float sr = sqrtf((float)r), isr = rsqrtf((float)r);
-    uint32_t pk[4];
+    if (e >= rows * (R / 8)) return;
+    const size_t row = e / (R / 8);
+    const int c0 = (int)(e % (R / 8)) * 8;
+    const float sr = sqrtf((float)R), isr = rsqrtf((float)R);
+    float a[8], b[8];
+    load8f(f1 + row * R + c0, a);
+    load8f(f2p + row * R + c0, b);
+    uint32_t h[4], l[4];
 #pragma unroll
-    for (int j = 0; j < 8; j += 2) {
-        float x[2];
+    for (int j = 0; j < 4; ++j)
+        split2(pack2(sr * tanhf(a[2 * j] * b[2 * j] * isr), sr * tanhf(a[2 * j + 1] * b[2 * j + 1] * isr)), h[j], l[j]);
+    bf16* dst = S + row * 64 + c0;
+    *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(dst + R) = make_uint4(l[0], l[1], l[2], l[3]);
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int c = c0 + j + q;
-            float v = 0.f;
-            if (c < 2 * r) {
-                const size_t o = row * r + (c % r);
-                const float m = sr * tanhf(f1[o] * f2[o] * isr);
-                const float hi = __bfloat162float(__float2bfloat16_rn(m));
-                v = c < r ? hi : m - hi;
-            }
-            x[q] = v;
-        }
-        pk[j / 2] = pack_bf16(x[0], x[1]);
-    }
-    *reinterpret_cast<uint4*>(S + row * 64 + c0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    for (int z = 2 * R; z < 64; z += R) *reinterpret_cast<uint4*>(dst + z) = make_uint4(0, 0, 0, 0);
 }
 
-// df1 = dM (1 - t^2) f2, df2 = dM (1 - t^2) f1 as bf16 rows of 64 columns (zero beyond r); dM = the
-// first r columns of dS, the gradient of the [hi | lo] rows (M = hi + lo)
+// df1 = dM (1 - t^2) f2, df2 = dM (1 - t^2) f1 as bf16 rows (r of 64 columns); dM = the first r columns of dS, the
+// gradient of the [hi | lo] rows (M = hi + lo)
+template <int R>
 __global__ void __launch_bounds__(256)
-ltc_combine_bwd_kernel(const float* __restrict__ f1, const float* __restrict__ f2, const bf16* __restrict__ dS, int r,
-                       size_t rows, bf16* __restrict__ df1, bf16* __restrict__ df2) {
+ltc_combine_bwd_kernel(const float* __restrict__ f1, const float* __restrict__ f2p, const bf16* __restrict__ dS, size_t rows,
+                       bf16* __restrict__ df1, bf16* __restrict__ df2) {
     pdl_sync();
     const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (e >= rows * 64) return;
-    const size_t row = e / 64;
-    const int c = (int)(e % 64);
-    float o1 = 0.f, o2 = 0.f;
-    if (c < r) {
-        const float a = f1[row * r + c], b = f2[row * r + c];
-        const float t = tanhf(a * b * rsqrtf((float)r));
-        const float du = __bfloat162float(dS[e]) * (1.f - t * t);
-        o1 = du * b; o2 = du * a;
+    if (e >= rows * (R / 8)) return;
+    const size_t row = e / (R / 8);
+    const int c0 = (int)(e % (R / 8)) * 8;
+    const float isr = rsqrtf((float)R);
+    float a[8], b[8];
+    load8f(f1 + row * R + c0, a);
+    load8f(f2p + row * R + c0, b);
+    const uint4 d4 = *reinterpret_cast<const uint4*>(dS + row * 64 + c0);
+    const uint32_t dw[4] = {d4.x, d4.y, d4.z, d4.w};
+    uint32_t o1[4], o2[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float t0 = tanhf(a[2 * j] * b[2 * j] * isr), t1 = tanhf(a[2 * j + 1] * b[2 * j + 1] * isr);
+        const float u0 = __uint_as_float(dw[j] << 16) * (1.f - t0 * t0), u1 = __uint_as_float(dw[j] & 0xffff0000u) * (1.f - t1 * t1);
+        o1[j] = pack_bf16(u0 * b[2 * j], u1 * b[2 * j + 1]);
+        o2[j] = pack_bf16(u0 * a[2 * j], u1 * a[2 * j + 1]);
     }
-    df1[e] = __float2bfloat16_rn(o1);
-    df2[e] = __float2bfloat16_rn(o2);
+    *reinterpret_cast<uint4*>(df1 + row * 64 + c0) = make_uint4(o1[0], o1[1], o1[2], o1[3]);
+    *reinterpret_cast<uint4*>(df2 + row * 64 + c0) = make_uint4(o2[0], o2[1], o2[2], o2[3]);
 }
 
 // parameter gradients of one network from the four accumulators and the column sums
 //   G1t = dp1^T n0, G2 = n1^T da2, G3t = dp3^T a2, G4 = a3^T df   (each [256][64])
+// Entries that are sums over 8r or r products take a warp each, the others a thread.
 __global__ void __launch_bounds__(256)
 ltc_finish_kernel(int h, int r, const float* __restrict__ params, const float* __restrict__ G, const float* __restrict__ sums,
                   float* __restrict__ dparams) {
@@ -981,26 +1110,41 @@ ltc_finish_kernel(int h, int r, const float* __restrict__ params, const float* _
     const float* s_da2 = s_dp1 + 256;
     const float* s_dp3 = s_da2 + 64;
     const float* s_df = s_dp3 + 256;
-    const int e = blockIdx.x * 256 + threadIdx.x;
-    if (e >= nl.count) return;
+    const int nsum = 2 * h + 2 * m, sum_blocks = (nsum + 7) / 8;
+    if ((int)blockIdx.x < sum_blocks) {
+        const int w = blockIdx.x * 8 + threadIdx.x / 32, lane = threadIdx.x % 32;
+        if (w >= nsum) return;
+        float g = 0.f;
+        int e;
+        if (w < h) {                                           // dg0[k] = sum_j W1[k][j] G1t[j][k]
+            e = nl.g0 + w;
+            for (int j = lane; j < m; j += 32) g = fmaf(P[nl.W1 + w * m + j], G1t[j * 64 + w], g);
+        } else if (w < 2 * h) {                                // dc0[k] = sum_j W1[k][j] s_dp1[j]
+            const int k = w - h;
+            e = nl.c0 + k;
+            for (int j = lane; j < m; j += 32) g = fmaf(P[nl.W1 + k * m + j], s_dp1[j], g);
+        } else if (w < 2 * h + m) {                            // dg1[j] = sum_c W2[j][c] G2[j][c]
+            const int j = w - 2 * h;
+            e = nl.g1 + j;
+            for (int c = lane; c < r; c += 32) g = fmaf(P[nl.W2 + j * r + c], G2[j * 64 + c], g);
+        } else {                                               // dc1[j] = sum_c W2[j][c] s_da2[c]
+            const int j = w - 2 * h - m;
+            e = nl.c1 + j;
+            for (int c = lane; c < r; c += 32) g = fmaf(P[nl.W2 + j * r + c], s_da2[c], g);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+        if (lane == 0) dP[e] += g;
+        return;
+    }
+    const int e = (blockIdx.x - sum_blocks) * 256 + threadIdx.x;
+    if (e >= nl.count || e < nl.W1 || (e >= nl.g1 && e < nl.W2)) return;
     float g = 0.f;
-    if (e < nl.c0) {                                           // dg0[k] = sum_j W1[k][j] G1t[j][k]
-        const int k = e - nl.g0;
-        for (int j = 0; j < m; ++j) g = fmaf(P[nl.W1 + k * m + j], G1t[j * 64 + k], g);
-    } else if (e < nl.W1) {                                    // dc0[k] = sum_j W1[k][j] s_dp1[j]
-        const int k = e - nl.c0;
-        for (int j = 0; j < m; ++j) g = fmaf(P[nl.W1 + k * m + j], s_dp1[j], g);
-    } else if (e < nl.b1) {                                    // dW1[k][j] = g0[k] G1t[j][k] + c0[k] s_dp1[j]
+    if (e < nl.b1) {                                           // dW1[k][j] = g0[k] G1t[j][k] + c0[k] s_dp1[j]
         const int k = (e - nl.W1) / m, j = (e - nl.W1) % m;
         g = P[nl.g0 + k] * G1t[j * 64 + k] + P[nl.c0 + k] * s_dp1[j];
     } else if (e < nl.g1) {
         g = s_dp1[e - nl.b1];
-    } else if (e < nl.c1) {                                    // dg1[j] = sum_c W2[j][c] G2[j][c]
-        const int j = e - nl.g1;
-        for (int c = 0; c < r; ++c) g = fmaf(P[nl.W2 + j * r + c], G2[j * 64 + c], g);
-    } else if (e < nl.W2) {                                    // dc1[j] = sum_c W2[j][c] s_da2[c]
-        const int j = e - nl.c1;
-        for (int c = 0; c < r; ++c) g = fmaf(P[nl.W2 + j * r + c], s_da2[c], g);
     } else if (e < nl.b2) {                                    // dW2[j][c] = g1[j] G2[j][c] + c1[j] s_da2[c]
         const int j = (e - nl.W2) / r, c = (e - nl.W2) % r;
         g = P[nl.g1 + j] * G2[j * 64 + c] + P[nl.c1 + j] * s_da2[c];
@@ -1023,11 +1167,10 @@ ltc_finish_kernel(int h, int r, const float* __restrict__ params, const float* _
 // ---------------------------------------------------------------------------
 // host
 // ---------------------------------------------------------------------------
-struct NetBuf { size_t p1, n1, n1_lo, p3, a3, a3_lo, a2, a2_lo, rs1, f; };
 struct LtcWs {
-    size_t bank, vec, G, sums, n0, n0_lo, rs0, df[2], dp3, da2, dp1, dn0, total;
-    NetBuf net[2];
-    size_t C;
+    size_t bank, vec, st0, f, a2, st1, G, sums, n0, n0_lo, df, da2, mm, dn0, total;
+    size_t C, rows;             // rows per pass; rows of one tensor
+    bool full;                  // a2, st1 and f of every row of both tensors are kept (else: f of one pass)
 };
 
 // Rows per pass.  PSK_LEARNED_CHUNK_ROWS in the environment overrides the default (a multiple of
@@ -1042,173 +1185,137 @@ size_t chunk_rows() {
     return kChunkRows;
 }
 
-LtcWs ltc_ws(const Dims& d, bool backward) {
+// `full`: the backward's layout, which a forward call that keeps its states writes into
+LtcWs ltc_ws(const Dims& d, bool full) {
     LtcWs w{};
-    const size_t rows = (size_t)d.BH() * d.n;
-    const size_t chunk = chunk_rows();
-    w.C = rows < chunk ? rows : chunk;
-    const size_t C = w.C;
+    const size_t rows = (size_t)d.BH() * d.n, chunk = chunk_rows();
+    const size_t C = w.C = rows < chunk ? rows : chunk;
+    w.rows = rows;
+    w.full = full;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = off; off += align_up(bytes); return o; };
-    w.bank = take((size_t)2 * kBank * kMat * sizeof(bf16));
+    w.bank = take(2 * kBankBytes);
     w.vec = take((size_t)2 * kVec * sizeof(float));
-    w.G = take((size_t)2 * 4 * kMat * sizeof(float));       // G and sums are zeroed together
-    w.sums = take((size_t)2 * kSums * sizeof(float));
-    w.n0 = take(C * 64 * sizeof(bf16));
-    w.n0_lo = take(C * 64 * sizeof(bf16));
-    w.rs0 = take(C * sizeof(float));
-    for (int t = 0; t < 2; ++t) {
-        w.net[t].p1 = take(C * 256 * sizeof(bf16));
-        w.net[t].n1 = take(C * 256 * sizeof(bf16));
-        w.net[t].n1_lo = take(C * 256 * sizeof(bf16));
-        w.net[t].p3 = take(C * 256 * sizeof(bf16));
-        w.net[t].a3 = take(C * 256 * sizeof(bf16));
-        w.net[t].a3_lo = take(C * 256 * sizeof(bf16));
-        w.net[t].a2 = take(C * 64 * sizeof(bf16));
-        w.net[t].a2_lo = take(C * 64 * sizeof(bf16));
-        w.net[t].rs1 = take(C * sizeof(float));
-        w.net[t].f = take(C * d.r * sizeof(float));
-    }
-    if (backward) {
-        w.df[0] = take(C * 64 * sizeof(bf16));
-        w.df[1] = take(C * 64 * sizeof(bf16));
-        w.dp3 = take(C * 256 * sizeof(bf16));
-        w.da2 = take(C * 64 * sizeof(bf16));
-        w.dp1 = take(C * 256 * sizeof(bf16));
-        w.dn0 = take(C * 64 * sizeof(float));
+    w.st0 = take(C * sizeof(float2));
+    w.f = take((full ? 4 * rows : 2 * C) * d.r * sizeof(float));         // [tensor][net][rows][r]
+    if (full) {
+        w.a2 = take(4 * rows * 64 * sizeof(bf16));                       // [tensor][net][rows][64]
+        w.st1 = take(4 * rows * sizeof(float2));
+        w.G = take((size_t)2 * 4 * kMat * sizeof(float));                // G and sums are zeroed together
+        w.sums = take((size_t)2 * kSums * sizeof(float));
+        w.n0 = take(C * 64 * sizeof(bf16));
+        w.n0_lo = take(C * 64 * sizeof(bf16));
+        w.df = take(2 * C * 64 * sizeof(bf16));
+        w.da2 = take(2 * C * 64 * sizeof(bf16));
+        w.mm = take(4 * C * sizeof(float2));
+        w.dn0 = take(2 * C * 64 * sizeof(float));
     }
     w.total = off;
     return w;
 }
 
-struct Maps {                       // tensor maps over the chunk buffers (built once per call)
-    CUtensorMap bank[2][kBank];
-    CUtensorMap n0, n0_lo, df[2], dp3, da2, dp1;
-    CUtensorMap p1[2], n1[2], n1_lo[2], p3[2], a3[2], a3_lo[2], a2[2], a2_lo[2];
-};
+// CTAs per network: both networks run side by side, one CTA per SM
+inline int net_ctas(int tiles_of_work) { return tiles_of_work < 74 ? tiles_of_work : 74; }
 
-bool build_maps(const LtcWs& w, char* ws, bool backward, Maps* M) {
-    const int64_t C = (int64_t)w.C;
-    bool ok = true;
-    for (int t = 0; t < 2; ++t) {
-        for (int i = 0; i < kBank; ++i) {
-            const bf16* base = reinterpret_cast<const bf16*>(ws + w.bank) + ((size_t)t * kBank + i) * kMat;
-            ok = ok && ((i % 2 == 0) ? tc_map_2d(&M->bank[t][i], base, 256, 64, 64) : tc_map_2d(&M->bank[t][i], base, 64, 256, 256));
-        }
-        ok = ok && tc_map_2d(&M->p1[t], ws + w.net[t].p1, 256, C, 128) && tc_map_2d(&M->n1[t], ws + w.net[t].n1, 256, C, 128) &&
-             tc_map_2d(&M->p3[t], ws + w.net[t].p3, 256, C, 128) && tc_map_2d(&M->a3[t], ws + w.net[t].a3, 256, C, 128) &&
-             tc_map_2d(&M->a2[t], ws + w.net[t].a2, 64, C, 128) && tc_map_2d(&M->n1_lo[t], ws + w.net[t].n1_lo, 256, C, 128) &&
-             tc_map_2d(&M->a3_lo[t], ws + w.net[t].a3_lo, 256, C, 128) && tc_map_2d(&M->a2_lo[t], ws + w.net[t].a2_lo, 64, C, 128);
-    }
-    ok = ok && tc_map_2d(&M->n0, ws + w.n0, 64, C, 128) && tc_map_2d(&M->n0_lo, ws + w.n0_lo, 64, C, 128);
-    if (backward)
-        ok = ok && tc_map_2d(&M->df[0], ws + w.df[0], 64, C, 128) && tc_map_2d(&M->df[1], ws + w.df[1], 64, C, 128) &&
-             tc_map_2d(&M->dp3, ws + w.dp3, 256, C, 128) && tc_map_2d(&M->da2, ws + w.da2, 64, C, 128) &&
-             tc_map_2d(&M->dp1, ws + w.dp1, 256, C, 128);
-    return ok;
-}
-
-// names under which the instances appear in the per-kernel timing records
-const char* const kDenseName[6] = {"", "ltc_dense_bwd_mid_kernel", "", "ltc_dense_bwd_in_kernel", "ltc_dense_bwd_gelu_kernel",
-                                   "ltc_dense_bwd_norm_kernel"};
-const char* const kDenseSplitName[6] = {"ltc_dense_norm_kernel", "ltc_dense_mid_kernel", "ltc_dense_gelu_kernel",
-                                        "ltc_dense_out_kernel", "", ""};
-
-// wide layers (64 -> 256)
-template <int EPI, bool SPLIT>
-cudaError_t wide(const CUtensorMap& mA, const CUtensorMap& mA2, const CUtensorMap& mB, const CUtensorMap& mB2,
-                 const CUtensorMap& mS0, const CUtensorMap& mS1, const CUtensorMap& mO0, const CUtensorMap& mO1,
-                 const CUtensorMap& mO2, const WideArgs& a, int tiles, int* status, cudaStream_t s, int* launches) {
-    constexpr int smem = WideSmem<EPI, SPLIT>::bytes;
-    PSK_TRY(set_smem(ltc_wide_kernel<EPI, SPLIT, true>, smem));
-    PSK_TRY(set_smem(ltc_wide_kernel<EPI, SPLIT, false>, smem));
-    prof_begin(SPLIT ? kDenseSplitName[EPI] : kDenseName[EPI], s);
-    if (a.ncols == 256) launch_pdl(ltc_wide_kernel<EPI, SPLIT, true>, tiles, 256, smem, s, mA, mA2, mB, mB2, mS0, mS1, mO0, mO1, mO2, a, status);
-    else launch_pdl(ltc_wide_kernel<EPI, SPLIT, false>, tiles, 256, smem, s, mA, mA2, mB, mB2, mS0, mS1, mO0, mO1, mO2, a, status);
-    prof_end(s);
-    ++*launches;
-    return cudaGetLastError();
-}
-// narrow layers (256 -> 64) of the backward: single bf16 operands
-template <int EPI>
-cudaError_t dense(const CUtensorMap& mA, const CUtensorMap& mB, const DenseArgs& a, int tiles, int* status, cudaStream_t s,
-                  int* launches) {
-    PSK_TRY(set_smem(ltc_dense_kernel<EPI>, kDenseSmem));
-    prof_begin(kDenseName[EPI], s);
-    launch_pdl(ltc_dense_kernel<EPI>, tiles, 128, kDenseSmem, s, mA, mB, a, status);
-    prof_end(s);
-    ++*launches;
-    return cudaGetLastError();
-}
-// narrow layers of the forward: hi + lo operand pairs, persistent kernel
-template <int EPI>
-cudaError_t narrow(const CUtensorMap& mA, const CUtensorMap& mA2, const CUtensorMap& mB, const CUtensorMap& mB2,
-                   const DenseArgs& a, int tiles, int* status, cudaStream_t s, int* launches) {
-    PSK_TRY(set_smem(ltc_narrow_kernel<EPI>, kNrSmem));
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
-            sms = 148;
-    }
-    prof_begin(kDenseSplitName[EPI], s);
-    launch_pdl(ltc_narrow_kernel<EPI>, tiles < sms ? tiles : sms, 192, kNrSmem, s, mA, mA2, mB, mB2, a, tiles, status);
-    prof_end(s);
-    ++*launches;
-    return cudaGetLastError();
-}
-
-// (colsum: where the column sums of the delta operand are added; wide = that operand is P)
-cudaError_t wgrad(const CUtensorMap& mP, const CUtensorMap& mS, float* Gt, float* colsum, bool wide, int tiles, int* status,
-                  cudaStream_t s, int* launches) {
-    PSK_TRY(set_smem(ltc_wgrad_kernel, kWgSmem));
-    int per = (tiles + 147) / 148;            // one CTA per SM, but at least four tiles per result added
-    if (per < 4) per = tiles < 4 ? tiles : 4;
-    const int grid = (tiles + per - 1) / per;
-    prof_begin("ltc_wgrad_kernel", s);
-    launch_pdl(ltc_wgrad_kernel, grid, 128, kWgSmem, s, mP, mS, Gt, colsum, wide ? 1 : 0, tiles, per, status);
-    prof_end(s);
-    ++*launches;
-    return cudaGetLastError();
-}
-
-// forward of both networks on `c` rows starting at row0: activations and f into the chunk buffers
-// (keep_pre: also the pre-activations p1, p3, which only the backward reads)
-cudaError_t forward_chunk(const Dims& d, const LtcWs& w, const Maps& M, const void* X, size_t row0, int c, bool keep_pre, char* ws,
-                          int* status, cudaStream_t s, int* launches) {
-    const Slice sl{d.H, d.n, d.sb, d.sh, d.sn};
-    const int tiles = c / 128, m = 8 * d.r;
+cudaError_t row_stats(const Dims& d, const LtcWs& w, const void* X, size_t row0, int c, bool n0, char* ws, cudaStream_t s, int* launches) {
     prof_begin("ltc_ln0_kernel", s);
-    launch_pdl(ltc_ln0_kernel, (c + 8 * kLnRowsPerWarp - 1) / (8 * kLnRowsPerWarp), 256, 0, s, sl, (const bf16*)X, row0, c, (bf16*)(ws + w.n0), (bf16*)(ws + w.n0_lo), (float*)(ws + w.rs0));
+    launch_pdl(ltc_ln0_kernel, (c + 8 * kLnRowsPerWarp - 1) / (8 * kLnRowsPerWarp), 256, 0, s, Slice{d.H, d.n, d.sb, d.sh, d.sn}, (const bf16*)X, row0, c,
+               n0 ? (bf16*)(ws + w.n0) : nullptr, n0 ? (bf16*)(ws + w.n0_lo) : nullptr, (float2*)(ws + w.st0));
     prof_end(s);
     ++*launches;
-    PSK_TRY(cudaGetLastError());
-    for (int t = 0; t < 2; ++t) {
-        const NetBuf& nb = w.net[t];
-        const float* vec = (const float*)(ws + w.vec) + (size_t)t * kVec;
-        PSK_TRY((wide<EPI_LN, true>(M.n0, M.n0_lo, M.bank[t][0], M.bank[t][8], M.n0, M.n0, M.p1[t], M.n1[t], M.n1_lo[t],
-                                    WideArgs{vec, (float*)(ws + nb.rs1), nullptr, m, keep_pre ? 1 : 0}, tiles, status, s, launches)));
-        PSK_TRY(narrow<EPI_B64>(M.n1[t], M.n1_lo[t], M.bank[t][1], M.bank[t][9],
-                                DenseArgs{vec + 256, (bf16*)(ws + nb.a2), (bf16*)(ws + nb.a2_lo), nullptr, 0, 0}, tiles, status, s, launches));
-        PSK_TRY((wide<EPI_GELU, true>(M.a2[t], M.a2_lo[t], M.bank[t][2], M.bank[t][10], M.n0, M.n0, M.p3[t], M.a3[t], M.a3_lo[t],
-                                      WideArgs{vec + 320, nullptr, nullptr, m, keep_pre ? 1 : 0}, tiles, status, s, launches)));
-        PSK_TRY(narrow<EPI_F32>(M.a3[t], M.a3_lo[t], M.bank[t][3], M.bank[t][11],
-                                DenseArgs{vec + 576, nullptr, nullptr, (float*)(ws + nb.f), d.r, 0}, tiles, status, s, launches));
+    return cudaGetLastError();
+}
+
+// S = the [hi | lo] rows of the half sketch of X, tensor 0 or 1 (contiguous [rows][64] bf16)
+template <int R>
+cudaError_t sketch_t(const Dims& d, const LtcWs& w, int tensor, const void* X, void* S, char* ws, int* status, cudaStream_t s, int* launches) {
+    const Slice sl{d.H, d.n, d.sb, d.sh, d.sn};
+    PSK_TRY(set_smem(ltc_dense_norm_kernel<R>, kFwdSmem<R>));
+    for (size_t row0 = 0; row0 < w.rows; row0 += w.C) {
+        const int c = (int)(w.rows - row0 < w.C ? w.rows - row0 : w.C), tiles = c / 128;
+        PSK_TRY(row_stats(d, w, X, row0, c, false, ws, s, launches));
+        // strides between the networks' arrays, and where this pass's rows begin in them
+        const size_t net_rows = w.full ? w.rows : w.C, first = w.full ? tensor * 2 * w.rows + row0 : 0;
+        float* f = (float*)(ws + w.f) + first * R;
+        prof_begin("ltc_dense_norm_kernel", s);
+        launch_pdl(ltc_dense_norm_kernel<R>, dim3(net_ctas((tiles + 1) / 2), 2), 576, kFwdSmem<R>, s, sl, (const bf16*)X, row0, tiles,
+                   (const float2*)(ws + w.st0), (const uint8_t*)(ws + w.bank), (const float*)(ws + w.vec),
+                   w.full ? (bf16*)(ws + w.a2) + first * 64 : nullptr, net_rows * 64, w.full ? (float2*)(ws + w.st1) + first : nullptr, net_rows, f,
+                   net_rows * R, status);
+        prof_end(s);
+        ++*launches;
+        PSK_TRY(cudaGetLastError());
+        prof_begin("ltc_combine_kernel", s);
+        launch_pdl(ltc_combine_kernel<R>, (unsigned)(((size_t)c * (R / 8) + 255) / 256), 256, 0, s, (const float*)f, (const float*)(f + net_rows * R), (size_t)c,
+                   (bf16*)S + row0 * 64);
+        prof_end(s);
+        ++*launches;
+        PSK_TRY(cudaGetLastError());
+    }
+    return cudaSuccess;
+}
+
+template <int R>
+cudaError_t sketch_bwd_t(const Dims& d, const LtcWs& w, int tensor, const void* X, const void* dS, const void* add, void* dX, char* ws,
+                         int* status, cudaStream_t s, int* launches) {
+    const Slice sl{d.H, d.n, d.sb, d.sh, d.sn};
+    const size_t C = w.C;
+    bf16* df = (bf16*)(ws + w.df);
+    bf16* da2 = (bf16*)(ws + w.da2);
+    const bf16* a2 = (const bf16*)(ws + w.a2) + (size_t)tensor * 2 * w.rows * 64;
+    const float2* st1 = (const float2*)(ws + w.st1) + (size_t)tensor * 2 * w.rows;
+    const uint8_t* bank = (const uint8_t*)(ws + w.bank);
+    const float* vec = (const float*)(ws + w.vec);
+    float* G = (float*)(ws + w.G);
+    float* sums = (float*)(ws + w.sums);
+    CUtensorMap mA[2], mDf[2], mDa[2], mN, mNlo;
+    bool ok = tc_map_2d(&mN, ws + w.n0, 64, C, 128) && tc_map_2d(&mNlo, ws + w.n0_lo, 64, C, 128);
+    for (int t = 0; t < 2; ++t)
+        ok = ok && tc_map_2d(&mA[t], a2 + t * w.rows * 64, 64, w.rows, 128) && tc_map_2d(&mDf[t], df + t * C * 64, 64, C, 128) &&
+             tc_map_2d(&mDa[t], da2 + t * C * 64, 64, C, 128);
+    if (!ok) return cudaErrorInvalidValue;
+    PSK_TRY(set_smem(ltc_wgrad_kernel<R>, Bwd34<R>::bytes));
+    PSK_TRY(set_smem(ltc_dense_bwd_norm_kernel<R>, Bwd12<R>::bytes));
+    for (size_t row0 = 0; row0 < w.rows; row0 += C) {
+        const int c = (int)(w.rows - row0 < C ? w.rows - row0 : C), tiles = c / 128;
+        const float* f = (const float*)(ws + w.f) + (tensor * 2 * w.rows + row0) * R;
+        PSK_TRY(row_stats(d, w, X, row0, c, true, ws, s, launches));
+        prof_begin("ltc_combine_bwd_kernel", s);
+        launch_pdl(ltc_combine_bwd_kernel<R>, (unsigned)(((size_t)c * (R / 8) + 255) / 256), 256, 0, s, f, f + w.rows * R, (const bf16*)dS + row0 * 64,
+                   (size_t)c, df, df + C * 64);
+        prof_end(s);
+        const dim3 grid(net_ctas(tiles), 2);
+        prof_begin("ltc_wgrad_kernel", s);
+        launch_pdl(ltc_wgrad_kernel<R>, grid, kBwdThreads, Bwd34<R>::bytes, s, mA[0], mA[1], mDf[0], mDf[1], row0, tiles, bank, vec, da2, C * 64,
+                   (float2*)(ws + w.mm), 2 * C, G, sums, status);
+        prof_end(s);
+        prof_begin("ltc_dense_bwd_norm_kernel", s);
+        launch_pdl(ltc_dense_bwd_norm_kernel<R>, grid, kBwdThreads, Bwd12<R>::bytes, s, mN, mNlo, mDa[0], mDa[1], row0, tiles, bank, vec, st1, w.rows,
+                   (const float2*)(ws + w.mm), 2 * C, (float*)(ws + w.dn0), C * 64, G, sums, status);
+        prof_end(s);
+        prof_begin("ltc_ln0_bwd_kernel", s);
+        launch_pdl(ltc_ln0_bwd_kernel, (c + 8 * kLnBwdRows - 1) / (8 * kLnBwdRows), 256, 0, s, sl, row0, c, (const float*)(ws + w.dn0), C * 64,
+                   (const bf16*)(ws + w.n0), (const float2*)(ws + w.st0), (const bf16*)add, (bf16*)dX);
+        prof_end(s);
+        *launches += 4;
+        PSK_TRY(cudaGetLastError());
     }
     return cudaSuccess;
 }
 
 }  // namespace
 
-bool learned_tc_supported(const Dims& d) { return d.bf16 && d.learned && d.h == 64 && d.r <= 32 && d.r % 4 == 0; }
+bool learned_tc_supported(const Dims& d) { return d.bf16 && d.learned && d.h == 64 && (d.r == 16 || d.r == 32); }
 
-size_t learned_tc_workspace_bytes(const Dims& d, bool backward) { return ltc_ws(d, backward).total; }
+size_t learned_tc_workspace_bytes(const Dims& d, bool full) { return ltc_ws(d, full).total; }
 
 // operand bank of both networks; backward: also clears the gradient accumulators
-cudaError_t learned_tc_prepare(const Dims& d, bool backward, char* ws, cudaStream_t s, int* launches) {
-    const LtcWs w = ltc_ws(d, backward);
+cudaError_t learned_tc_prepare(const Dims& d, bool full, bool backward, char* ws, cudaStream_t s, int* launches) {
+    const LtcWs w = ltc_ws(d, full);
+    const int blocks = (64 * 8 * d.r + 3 * 8 * d.r * d.r) / 256 + (kVec + 7) / 8;
     prof_begin("ltc_bank_kernel", s);
-    launch_pdl(ltc_bank_kernel, dim3((8 * kMat + kVec + 255) / 256, 2), 256, 0, s, d.h, d.r, d.lparams, (bf16*)(ws + w.bank), (float*)(ws + w.vec));
+    if (d.r == 16) launch_pdl(ltc_bank_kernel<16>, dim3(blocks, 2), 256, 0, s, d.lparams, (uint8_t*)(ws + w.bank), (float*)(ws + w.vec));
+    else launch_pdl(ltc_bank_kernel<32>, dim3(blocks, 2), 256, 0, s, d.lparams, (uint8_t*)(ws + w.bank), (float*)(ws + w.vec));
     prof_end(s);
     ++*launches;
     PSK_TRY(cudaGetLastError());
@@ -1216,84 +1323,31 @@ cudaError_t learned_tc_prepare(const Dims& d, bool backward, char* ws, cudaStrea
     return cudaSuccess;
 }
 
-// S = the [hi | lo] rows of the half sketch of X (contiguous [rows][64] bf16)
-cudaError_t learned_tc_sketch(const Dims& d, const void* X, void* S, char* ws, int* status, cudaStream_t s, int* launches) {
-    const LtcWs w = ltc_ws(d, false);            // the forward's buffers come first in either layout
-    Maps M;
-    if (!build_maps(w, ws, false, &M)) return cudaErrorInvalidValue;
-    const size_t rows = (size_t)d.BH() * d.n;
-    for (size_t row0 = 0; row0 < rows; row0 += w.C) {
-        const int c = (int)(rows - row0 < w.C ? rows - row0 : w.C);
-        PSK_TRY(forward_chunk(d, w, M, X, row0, c, false, ws, status, s, launches));
-        prof_begin("ltc_combine_kernel", s);
-        launch_pdl(ltc_combine_kernel, (unsigned)(((size_t)c * 8 + 255) / 256), 256, 0, s, (const float*)(ws + w.net[0].f), (const float*)(ws + w.net[1].f),
-                                                                              d.r, (size_t)c, (bf16*)S + row0 * 64);
-        prof_end(s);
-        ++*launches;
-        PSK_TRY(cudaGetLastError());
-    }
-    return cudaSuccess;
+// S = the [hi | lo] rows of the half sketch of X, tensor 0 (Q) or 1 (K); `full`: what the backward reads again
+// (a2, the row statistics, f) stays in the workspace
+cudaError_t learned_tc_sketch(const Dims& d, bool full, int tensor, const void* X, void* S, char* ws, int* status, cudaStream_t s, int* launches) {
+    const LtcWs w = ltc_ws(d, full);
+    return d.r == 16 ? sketch_t<16>(d, w, tensor, X, S, ws, status, s, launches) : sketch_t<32>(d, w, tensor, X, S, ws, status, s, launches);
 }
 
 // dX = chain rule through both networks of the gradient dS of the [hi | lo] rows (+ add, a contiguous [rows][64] bf16 array
 // or null: the part of the gradient that reached X directly); the weight-gradient
 // accumulators in the workspace grow by this tensor's share (learned_tc_finish turns them into
 // parameter gradients)
-cudaError_t learned_tc_sketch_bwd(const Dims& d, const void* X, const void* dS, const void* add, void* dX, char* ws,
+cudaError_t learned_tc_sketch_bwd(const Dims& d, int tensor, const void* X, const void* dS, const void* add, void* dX, char* ws,
                                   int* status, cudaStream_t s, int* launches) {
     const LtcWs w = ltc_ws(d, true);
-    Maps M;
-    if (!build_maps(w, ws, true, &M)) return cudaErrorInvalidValue;
-    const Slice sl{d.H, d.n, d.sb, d.sh, d.sn};
-    const size_t rows = (size_t)d.BH() * d.n;
-    const int m = 8 * d.r;
-    for (size_t row0 = 0; row0 < rows; row0 += w.C) {
-        const int c = (int)(rows - row0 < w.C ? rows - row0 : w.C);
-        const int tiles = c / 128;
-        PSK_TRY(forward_chunk(d, w, M, X, row0, c, true, ws, status, s, launches));
-        prof_begin("ltc_combine_bwd_kernel", s);
-        launch_pdl(ltc_combine_bwd_kernel, (unsigned)(((size_t)c * 64 + 255) / 256), 256, 0, s, 
-            (const float*)(ws + w.net[0].f), (const float*)(ws + w.net[1].f), (const bf16*)dS + row0 * 64, d.r, (size_t)c,
-            (bf16*)(ws + w.df[0]), (bf16*)(ws + w.df[1]));
-        prof_end(s);
-        ++*launches;
-        PSK_TRY(cudaGetLastError());
-        for (int t = 0; t < 2; ++t) {
-            const NetBuf& nb = w.net[t];
-            float* G = (float*)(ws + w.G) + (size_t)t * 4 * kMat;
-            float* sums = (float*)(ws + w.sums) + (size_t)t * kSums;
-            // dp3 = (df W4^T) * gelu'(p3);  dW4 ~ a3^T df
-            PSK_TRY((wide<EPI_DGELU, false>(M.df[t], M.df[t], M.bank[t][4], M.bank[t][4], M.p3[t], M.p3[t], M.dp3, M.dp3, M.dp3,
-                                            WideArgs{nullptr, nullptr, nullptr, m, 0}, tiles, status, s, launches)));
-            PSK_TRY(wgrad(M.a3[t], M.df[t], G + 3 * kMat, sums + 576, false, tiles, status, s, launches));
-            // da2 = dp3 W3^T;  dW3 ~ dp3^T a2
-            PSK_TRY(wgrad(M.dp3, M.a2[t], G + 2 * kMat, sums + 320, true, tiles, status, s, launches));
-            PSK_TRY(dense<EPI_B64>(M.dp3, M.bank[t][5], DenseArgs{nullptr, (bf16*)(ws + w.da2), nullptr, nullptr, 0, 0}, tiles, status, s, launches));
-            // dp1 = LN1 backward(da2 (g1 W2)^T) * gelu'(p1);  dW2 ~ n1^T da2
-            PSK_TRY(wgrad(M.n1[t], M.da2, G + 1 * kMat, sums + 256, false, tiles, status, s, launches));
-            PSK_TRY((wide<EPI_LNBWD, false>(M.da2, M.da2, M.bank[t][6], M.bank[t][6], M.n1[t], M.p1[t], M.dp1, M.dp1, M.dp1,
-                                            WideArgs{nullptr, nullptr, (const float*)(ws + nb.rs1), m, 0}, tiles, status, s, launches)));
-            // dn0 (+)= dp1 (g0 W1)^T;  dW1 ~ dp1^T n0
-            PSK_TRY(wgrad(M.dp1, M.n0, G + 0 * kMat, sums + 0, true, tiles, status, s, launches));
-            PSK_TRY(dense<EPI_F32>(M.dp1, M.bank[t][7], DenseArgs{nullptr, nullptr, nullptr, (float*)(ws + w.dn0), 64, t}, tiles, status, s, launches));
-        }
-        prof_begin("ltc_ln0_bwd_kernel", s);
-        launch_pdl(ltc_ln0_bwd_kernel, (c + 7) / 8, 256, 0, s, sl, row0, c, (const float*)(ws + w.dn0), (const bf16*)(ws + w.n0),
-                                                      (const float*)(ws + w.rs0), (const bf16*)add, (bf16*)dX);
-        prof_end(s);
-        ++*launches;
-        PSK_TRY(cudaGetLastError());
-    }
-    return cudaSuccess;
+    return d.r == 16 ? sketch_bwd_t<16>(d, w, tensor, X, dS, add, dX, ws, status, s, launches)
+                     : sketch_bwd_t<32>(d, w, tensor, X, dS, add, dX, ws, status, s, launches);
 }
 
 // parameter gradients (added to d.dlparams) from everything learned_tc_sketch_bwd accumulated
 cudaError_t learned_tc_finish(const Dims& d, char* ws, cudaStream_t s, int* launches) {
     const LtcWs w = ltc_ws(d, true);
-    const int count = NetLayout(d.h, d.r).count;
+    const NetLayout nl(d.h, d.r);
     prof_begin("ltc_finish_kernel", s);
-    launch_pdl(ltc_finish_kernel, dim3((count + 255) / 256, 2), 256, 0, s, d.h, d.r, d.lparams, (const float*)(ws + w.G),
-                                                                   (const float*)(ws + w.sums), d.dlparams);
+    launch_pdl(ltc_finish_kernel, dim3((2 * nl.h + 2 * nl.m + 7) / 8 + (nl.count + 255) / 256, 2), 256, 0, s, d.h, d.r, d.lparams, (const float*)(ws + w.G),
+               (const float*)(ws + w.sums), d.dlparams);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
