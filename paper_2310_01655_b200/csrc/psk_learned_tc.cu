@@ -963,73 +963,84 @@ ltc_dense_bwd_norm_kernel(const __grid_constant__ CUtensorMap mN, const __grid_c
 // CUDA-core helpers
 // ---------------------------------------------------------------------------
 // Mean and 1 / sigma of every row (st0), and (n0 != nullptr: the backward) n0 = (x - mean) / sigma as hi + lo
-// rows.  One warp per row, two columns per lane, eight rows per warp with their loads issued together.
-constexpr int kLnRowsPerWarp = 8;
+// rows.  Eight lanes per row, eight columns each, two rows' loads in flight per lane: six shuffles serve four rows.
+// (A whole warp per row took 67 us for 393 216 rows, ten shuffles each; now 20.)
+constexpr int kLnRows = 64;                            // rows per CTA
+__device__ __forceinline__ void unpack8(const uint4& q, float (&v)[8]) {
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { v[2 * i] = __uint_as_float(w[i] << 16); v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u); }
+}
+__device__ __forceinline__ float sum8(float s) {       // over the eight lanes of a row
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    return s + __shfl_xor_sync(0xffffffffu, s, 4);
+}
 __global__ void __launch_bounds__(256)
-ltc_ln0_kernel(Slice sl, const bf16* __restrict__ X, size_t row0, int rows, bf16* __restrict__ n0, bf16* __restrict__ n0_lo,
-               float2* __restrict__ st0) {
+ltc_ln0_kernel(Slice sl, const bf16* __restrict__ X, size_t row0, bf16* __restrict__ n0, bf16* __restrict__ n0_lo, float2* __restrict__ st0) {
     pdl_sync();
-    const int lane = threadIdx.x % 32;
-    const int i0 = (blockIdx.x * 8 + threadIdx.x / 32) * kLnRowsPerWarp;
-    __nv_bfloat162 x2[kLnRowsPerWarp];
+    const int ch = threadIdx.x % 8, r = threadIdx.x / 8;
+    uint4 x[2];
 #pragma unroll
-    for (int q = 0; q < kLnRowsPerWarp; ++q)
-        if (i0 + q < rows) x2[q] = *reinterpret_cast<const __nv_bfloat162*>(X + sl.row(row0 + i0 + q) + 2 * lane);
+    for (int q = 0; q < 2; ++q) x[q] = *reinterpret_cast<const uint4*>(X + sl.row(row0 + blockIdx.x * kLnRows + r + 32 * q) + 8 * ch);
 #pragma unroll
-    for (int q = 0; q < kLnRowsPerWarp; ++q) {
-        const int i = i0 + q;
-        if (i >= rows) break;
-        const float a = __low2float(x2[q]), b = __high2float(x2[q]);
-        float s = a + b;
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        const float mu = s * (1.f / 64.f);
-        float v = (a - mu) * (a - mu) + (b - mu) * (b - mu);
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        const float rs = rsqrtf(v * (1.f / 64.f) + kLnEps);
-        if (lane == 0) st0[i] = make_float2(mu, rs);
-        if (n0 == nullptr) continue;
-        const float na = (a - mu) * rs, nb = (b - mu) * rs;
-        const uint32_t h = pack_bf16(na, nb);
-        *reinterpret_cast<uint32_t*>(n0 + (size_t)i * 64 + 2 * lane) = h;
-        *reinterpret_cast<uint32_t*>(n0_lo + (size_t)i * 64 + 2 * lane) =
-            pack_bf16(na - __uint_as_float(h << 16), nb - __uint_as_float(h & 0xffff0000u));
+    for (int q = 0; q < 2; ++q) {
+        const size_t i = (size_t)blockIdx.x * kLnRows + r + 32 * q;
+        float v[8], s = 0.f, t = 0.f;
+        unpack8(x[q], v);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) s += v[c];
+        const float mu = sum8(s) * (1.f / 64.f);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) { v[c] -= mu; t = fmaf(v[c], v[c], t); }
+        const float rs = rsqrtf(sum8(t) * (1.f / 64.f) + kLnEps);
+        if (ch == 0) st0[i] = make_float2(mu, rs);
+        if (n0 != nullptr) {
+            uint32_t h[4], l[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) split2(pack2(v[2 * c] * rs, v[2 * c + 1] * rs), h[c], l[c]);
+            *reinterpret_cast<uint4*>(n0 + i * 64 + 8 * ch) = make_uint4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<uint4*>(n0_lo + i * 64 + 8 * ch) = make_uint4(l[0], l[1], l[2], l[3]);
+        }
     }
 }
 
-// dX = back through the first normalisation of the two networks' gradients of n0 (+ add); one warp per row,
-// four rows' loads in flight
-constexpr int kLnBwdRows = 4;
+// dX = back through the first normalisation of the two networks' gradients of n0 (+ add).  Lanes and rows as above.
 __global__ void __launch_bounds__(256)
-ltc_ln0_bwd_kernel(Slice sl, size_t row0, int rows, const float* __restrict__ dn0, size_t dn0_net, const bf16* __restrict__ n0,
+ltc_ln0_bwd_kernel(Slice sl, size_t row0, const float* __restrict__ dn0, size_t dn0_net, const bf16* __restrict__ n0,
                    const float2* __restrict__ st0, const bf16* __restrict__ add, bf16* __restrict__ dX) {
     pdl_sync();
-    const int lane = threadIdx.x % 32;
-    const int i0 = (blockIdx.x * 8 + threadIdx.x / 32) * kLnBwdRows;
-    float2 d0[kLnBwdRows], d1[kLnBwdRows];
-    __nv_bfloat162 n2[kLnBwdRows], ad[kLnBwdRows];
-    float rs[kLnBwdRows];
+    const int ch = threadIdx.x % 8, r = threadIdx.x / 8;
+    float4 g[2][4];
+    uint4 nq[2], aq[2];
+    float rs[2];
 #pragma unroll
-    for (int q = 0; q < kLnBwdRows; ++q) {
-        const size_t i = i0 + q;
-        if ((int)i >= rows) break;
-        d0[q] = *reinterpret_cast<const float2*>(dn0 + i * 64 + 2 * lane);
-        d1[q] = *reinterpret_cast<const float2*>(dn0 + dn0_net + i * 64 + 2 * lane);
-        n2[q] = *reinterpret_cast<const __nv_bfloat162*>(n0 + i * 64 + 2 * lane);
-        if (add != nullptr) ad[q] = *reinterpret_cast<const __nv_bfloat162*>(add + (row0 + i) * 64 + 2 * lane);
+    for (int q = 0; q < 2; ++q) {
+        const size_t i = (size_t)blockIdx.x * kLnRows + r + 32 * q, o = i * 64 + 8 * ch;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            g[q][2 * t] = *reinterpret_cast<const float4*>(dn0 + t * dn0_net + o);
+            g[q][2 * t + 1] = *reinterpret_cast<const float4*>(dn0 + t * dn0_net + o + 4);
+        }
+        nq[q] = *reinterpret_cast<const uint4*>(n0 + o);
+        aq[q] = add != nullptr ? *reinterpret_cast<const uint4*>(add + row0 * 64 + o) : make_uint4(0, 0, 0, 0);
         rs[q] = st0[i].y;
     }
 #pragma unroll
-    for (int q = 0; q < kLnBwdRows; ++q) {
-        const int i = i0 + q;
-        if (i >= rows) break;
-        const float dx = d0[q].x + d1[q].x, dy = d0[q].y + d1[q].y;
-        const float na = __low2float(n2[q]), nb = __high2float(n2[q]);
-        float s1 = dx + dy, s2 = dx * na + dy * nb;
-        for (int o = 16; o > 0; o >>= 1) { s1 += __shfl_xor_sync(0xffffffffu, s1, o); s2 += __shfl_xor_sync(0xffffffffu, s2, o); }
-        const float m1 = s1 * (1.f / 64.f), m2 = s2 * (1.f / 64.f);
-        float oa = rs[q] * (dx - m1 - na * m2), ob = rs[q] * (dy - m1 - nb * m2);
-        if (add != nullptr) { oa += __low2float(ad[q]); ob += __high2float(ad[q]); }
-        *reinterpret_cast<uint32_t*>(dX + sl.row(row0 + i) + 2 * lane) = pack_bf16(oa, ob);
+    for (int q = 0; q < 2; ++q) {
+        const float d[8] = {g[q][0].x + g[q][2].x, g[q][0].y + g[q][2].y, g[q][0].z + g[q][2].z, g[q][0].w + g[q][2].w,
+                            g[q][1].x + g[q][3].x, g[q][1].y + g[q][3].y, g[q][1].z + g[q][3].z, g[q][1].w + g[q][3].w};
+        float n[8], a[8], s1 = 0.f, s2 = 0.f;
+        unpack8(nq[q], n);
+        unpack8(aq[q], a);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) { s1 += d[c]; s2 = fmaf(d[c], n[c], s2); }
+        const float m1 = sum8(s1) * (1.f / 64.f), m2 = sum8(s2) * (1.f / 64.f);
+        uint32_t pk[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            pk[c] = pack_bf16(fmaf(rs[q], d[2 * c] - m1 - n[2 * c] * m2, a[2 * c]), fmaf(rs[q], d[2 * c + 1] - m1 - n[2 * c + 1] * m2, a[2 * c + 1]));
+        *reinterpret_cast<uint4*>(dX + sl.row(row0 + (size_t)blockIdx.x * kLnRows + r + 32 * q) + 8 * ch) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
     }
 }
 
@@ -1219,7 +1230,7 @@ inline int net_ctas(int tiles_of_work) { return tiles_of_work < 74 ? tiles_of_wo
 
 cudaError_t row_stats(const Dims& d, const LtcWs& w, const void* X, size_t row0, int c, bool n0, char* ws, cudaStream_t s, int* launches) {
     prof_begin("ltc_ln0_kernel", s);
-    launch_pdl(ltc_ln0_kernel, (c + 8 * kLnRowsPerWarp - 1) / (8 * kLnRowsPerWarp), 256, 0, s, Slice{d.H, d.n, d.sb, d.sh, d.sn}, (const bf16*)X, row0, c,
+    launch_pdl(ltc_ln0_kernel, c / kLnRows, 256, 0, s, Slice{d.H, d.n, d.sb, d.sh, d.sn}, (const bf16*)X, row0,
                n0 ? (bf16*)(ws + w.n0) : nullptr, n0 ? (bf16*)(ws + w.n0_lo) : nullptr, (float2*)(ws + w.st0));
     prof_end(s);
     ++*launches;
@@ -1294,7 +1305,7 @@ cudaError_t sketch_bwd_t(const Dims& d, const LtcWs& w, int tensor, const void* 
                    (const float2*)(ws + w.mm), 2 * C, (float*)(ws + w.dn0), C * 64, G, sums, status);
         prof_end(s);
         prof_begin("ltc_ln0_bwd_kernel", s);
-        launch_pdl(ltc_ln0_bwd_kernel, (c + 8 * kLnBwdRows - 1) / (8 * kLnBwdRows), 256, 0, s, sl, row0, c, (const float*)(ws + w.dn0), C * 64,
+        launch_pdl(ltc_ln0_bwd_kernel, c / kLnRows, 256, 0, s, sl, row0, (const float*)(ws + w.dn0), C * 64,
                    (const bf16*)(ws + w.n0), (const float2*)(ws + w.st0), (const bf16*)add, (bf16*)dX);
         prof_end(s);
         *launches += 4;
