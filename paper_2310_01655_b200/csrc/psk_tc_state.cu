@@ -383,9 +383,8 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
             }
             if constexpr (F::kCirc) {
                 // this warpgroup's tiles wg, wg + NWG, ...: the same loop body on a rotated copy of m
-                static_assert(T0 == 0, "circulant order: one launch covers every tile");
                 constexpr int kTileSteps = 128 / (2 * R);
-                for (int i = 0; i < wg; ++i) gen.template skip<kTileSteps>();
+                for (int i = 0; i < T0 + wg; ++i) gen.template skip<kTileSteps>();
 #pragma unroll 1
                 for (int I = wg; I < TN; I += NWG) {
                     if (a_uses > 0) mbar_wait(&bar_afree[wg], (a_uses - 1) & 1, status, kErrMma);
@@ -439,24 +438,23 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
 #define PSK_STATE_ARGS                                                                                              \
     mapX, mapY, gimg, g_heads, H, n, b, t, y65, fscale, cmean, center_mode, reverse, nseg, mode, run0, units, tot, S, lin, status
 
-// r <= 32: every feature tile of a head in one CTA (two or five accumulators)
-template <int R, int TN, int NWG, bool SEG>
-__global__ void __launch_bounds__(128 * (NWG + 1) + 64) tc_state_kernel(PSK_STATE_PARAMS) {
-    state_walk<R, 0, TN, NWG, SEG>(PSK_STATE_ARGS);
-}
+// The feature tiles of a head are dealt to SPLIT CTAs, each of which forms the half sketches anew.  blockIdx.z, the
+// slowest index: CTAs that run at the same time then run the same specialised code (with the shares of a head side by
+// side on neighbouring SMs the kernel took 1.5 times as long, for want of instruction cache).  r = 64 has 17 tiles and tensor memory for four accumulators beside the sketch columns.
+template <int R, int SPLIT> struct StateSplit {
+    static constexpr int NT = Feat<R>::NT, kBase = NT / SPLIT, kMore = NT % SPLIT;
+    __host__ __device__ static constexpr int tiles(int z) { return kBase + (z < kMore ? 1 : 0); }
+    __host__ __device__ static constexpr int first(int z) { return z * kBase + (z < kMore ? z : kMore); }
+    static constexpr int NWG = tiles(0) < 3 ? tiles(0) : 3, kThreads = 128 * (NWG + 1) + 64;
+};
 
-// r = 64: 17 feature tiles, at most four accumulators beside the sketch columns, so five CTAs share a head
-// (blockIdx.z), those with four tiles first.  One launch: five launches of a group each left most SMs idle
-// whenever heads x runs were no multiple of their number.
-template <bool SEG>
-__global__ void __launch_bounds__(128 * 4 + 64) tc_state64_kernel(PSK_STATE_PARAMS) {
-    switch (blockIdx.z) {
-        case 0: state_walk<64, 0, 4, 3, SEG>(PSK_STATE_ARGS); break;
-        case 1: state_walk<64, 4, 4, 3, SEG>(PSK_STATE_ARGS); break;
-        case 2: state_walk<64, 8, 3, 3, SEG>(PSK_STATE_ARGS); break;
-        case 3: state_walk<64, 11, 3, 3, SEG>(PSK_STATE_ARGS); break;
-        default: state_walk<64, 14, 3, 3, SEG>(PSK_STATE_ARGS); break;
-    }
+template <int R, int SPLIT, bool SEG>
+__global__ void __launch_bounds__(StateSplit<R, SPLIT>::kThreads) tc_state_kernel(PSK_STATE_PARAMS) {
+    using P = StateSplit<R, SPLIT>;
+    static_for<0, SPLIT>([&](auto zc) {
+        constexpr int Z = decltype(zc)::value;
+        if (SPLIT == 1 || (int)blockIdx.z == Z) state_walk<R, P::first(Z), P::tiles(Z), P::NWG, SEG>(PSK_STATE_ARGS);
+    });
 }
 
 // Running sums of a head's run totals, in place: run s becomes the sum over the runs <= s.
@@ -538,39 +536,79 @@ struct StateArgs {
 // tiles when there are no blocks to respect
 int state_units(const Dims& d) { return d.noncausal ? d.n / 128 : d.t; }
 
-// Costs in token tiles (r = 32: about 3.5 us each): a CTA's start and end, the same where it fetches its start
-// value, and the running sums with the extra launches (measured on 12 and 48 heads)
-constexpr long kStartTiles = 3, kInitTiles = 4, kBetweenTiles = 3;
+// CTAs per head and run, and runs per head.  Estimated time in nanoseconds: a CTA's walk of its run, times the
+// rounds in which the grid fills the SMs.  `step`, `boundary`: measured time of a 128-token tile and of writing
+// the states out at a block boundary, for the largest share of a split (12 heads, n = 32 768, b = 256 and 4096);
+// `mean`: the average share in percent of the largest.  Where more CTAs than SMs are wanted, the shares of a
+// head get in each other's way for r <= 32 (15 % on 96 heads).  A run's start and end cost about 6 us, its start value
+// 4 us, the launch between the two passes over the runs 8 us.
+struct StatePlan { int split, nseg; };
+struct SplitCost { int split, step, boundary, mean; };
+constexpr SplitCost kCost16[] = {{1, 1350, 600, 100}, {2, 1140, 200, 100}};
+constexpr SplitCost kCost32[] = {{1, 2950, 1300, 100}, {2, 1920, 800, 85}, {3, 1330, 640, 92}, {5, 1220, 220, 100}};
+constexpr SplitCost kCost64[] = {{5, 3190, 2700, 85}, {6, 2110, 1840, 94}, {9, 1460, 540, 94}};
 
-template <int R>
-cudaError_t launch_states(const Dims& d, const CUtensorMap& mX, const CUtensorMap& mY, const uint8_t* gimg,
-                          const StateArgs& a, int* status, cudaStream_t s, int* launches) {
-    constexpr int NWG = R == 16 ? 2 : 3, kThreads = 128 * (NWG + 1) + 64;
-    constexpr size_t smem = StateSmem<R, NWG>::total + 1024;
-    const bool seg = a.nseg > 1 || a.mode != kModePrefix;
-    const dim3 grid(d.BH(), a.runs, R == 64 ? 5 : 1);
+StatePlan state_plan(const Dims& d) {
+    constexpr long kSMs = 148, kStart = 6000, kInit = 4000, kBetween = 8000;
+    const SplitCost* cost = d.r == 16 ? kCost16 : (d.r == 32 ? kCost32 : kCost64);
+    const int ncost = d.r == 16 ? 2 : (d.r == 32 ? 4 : 3), units = state_units(d);
+    const long upt = d.n / 128 / units;
+    auto rounds = [&](long ctas, const SplitCost& c, long walk) {
+        return ctas <= kSMs ? walk : ((ctas + kSMs - 1) / kSMs) * walk * c.mean / 100 * (d.r <= 32 && c.split > 1 ? 115 : 100) / 100;
+    };
+    int lo = 1, hi = units < 64 ? units : 64;
+    if (d.seq_segments > 0) lo = hi = (d.seq_segments <= units && units % d.seq_segments == 0) ? d.seq_segments : 1;
+    StatePlan p{cost[0].split, 1};
+    long best = -1;
+    for (int i = 0; i < ncost; ++i)
+        for (int s = lo; s <= hi; ++s) {
+            const SplitCost& c = cost[i];
+            const long run = (units + s - 1) / s, tiles = run * upt, ctas = (long)d.BH() * c.split;
+            long t;
+            if (d.noncausal) t = rounds(ctas * s, c, tiles * c.step + kStart);
+            else if (s == 1) t = rounds(ctas, c, tiles * c.step + run * c.boundary + kStart);
+            else t = 2 * rounds(ctas * (s - 1), c, tiles * c.step + run * c.boundary + kStart + kInit / 2) + kBetween;
+            if (best < 0 || t < best - best / 20) { best = t; p = StatePlan{c.split, s}; }       // (more CTAs have to pay clearly)
+        }
+    return p;
+}
+
+template <int R, int SPLIT>
+cudaError_t launch_split(const Dims& d, const CUtensorMap& mX, const CUtensorMap& mY, const uint8_t* gimg,
+                         const StateArgs& a, int* status, cudaStream_t s, int* launches) {
+    using P = StateSplit<R, SPLIT>;
+    constexpr size_t smem = StateSmem<R, P::NWG>::total + 1024;
     // A long walk is better spread over the SMs by an ordinary launch: started early, its CTAs settle on the SMs
     // that happen to be free first, several to a pair (r = 64, 48 heads of 128 tiles: 6.93 against 7.33 ms a step);
     // for a short one the launch itself counts more (48 heads of 21 tiles: 374 -> 361 us a step).
     const bool early = d.n / 128 / a.nseg <= 24;
+    auto kern = a.nseg > 1 || a.mode != kModePrefix ? tc_state_kernel<R, SPLIT, true> : tc_state_kernel<R, SPLIT, false>;
+    PSK_TRY((set_smem(kern, smem)));
     prof_begin(a.mode == kModePrefix ? "tc_state_kernel" : "tc_state_total_kernel", s);
-#define PSK_STATE_LAUNCH(KERNEL) do {                                                                                \
-        auto kern = KERNEL;                                                                                          \
-        PSK_TRY((set_smem(kern, smem)));                                                                             \
-        launch_pdl_if(early, kern, grid, kThreads, smem, s, mX, mY, gimg, d.g_heads, d.H, d.n, d.b, d.t, a.y65, a.fscale, a.cmean,      \
-                                          a.center_mode, a.reverse ? 1 : 0, a.nseg, a.mode, a.run0, state_units(d), a.tot, \
-                                          a.S, d.sketch_linear ? 1 : 0, status);                                     \
-    } while (0)
-    if constexpr (R == 64) {
-        if (seg) PSK_STATE_LAUNCH((tc_state64_kernel<true>)); else PSK_STATE_LAUNCH((tc_state64_kernel<false>));
-    } else {
-        constexpr int TN = Feat<R>::NT;
-        if (seg) PSK_STATE_LAUNCH((tc_state_kernel<R, TN, NWG, true>)); else PSK_STATE_LAUNCH((tc_state_kernel<R, TN, NWG, false>));
-    }
-#undef PSK_STATE_LAUNCH
+    launch_pdl_if(early, kern, dim3(d.BH(), a.runs, SPLIT), P::kThreads, smem, s, mX, mY, gimg, d.g_heads, d.H, d.n, d.b, d.t, a.y65, a.fscale,
+                  a.cmean, a.center_mode, a.reverse ? 1 : 0, a.nseg, a.mode, a.run0, state_units(d), a.tot, a.S, d.sketch_linear ? 1 : 0, status);
     prof_end(s);
     ++*launches;
     return cudaGetLastError();
+}
+
+template <int R>
+cudaError_t launch_states(const Dims& d, const CUtensorMap& mX, const CUtensorMap& mY, const uint8_t* gimg,
+                          const StateArgs& a, int* status, cudaStream_t s, int* launches) {
+    const int split = state_plan(d).split;
+    if constexpr (R == 64) {
+        if (split == 9) return launch_split<R, 9>(d, mX, mY, gimg, a, status, s, launches);
+        if (split == 6) return launch_split<R, 6>(d, mX, mY, gimg, a, status, s, launches);
+        return launch_split<R, 5>(d, mX, mY, gimg, a, status, s, launches);
+    } else if constexpr (R == 32) {
+        if (split == 5) return launch_split<R, 5>(d, mX, mY, gimg, a, status, s, launches);
+        if (split == 3) return launch_split<R, 3>(d, mX, mY, gimg, a, status, s, launches);
+        if (split == 2) return launch_split<R, 2>(d, mX, mY, gimg, a, status, s, launches);
+        return launch_split<R, 1>(d, mX, mY, gimg, a, status, s, launches);
+    } else {
+        if (split == 2) return launch_split<R, 2>(d, mX, mY, gimg, a, status, s, launches);
+        return launch_split<R, 1>(d, mX, mY, gimg, a, status, s, launches);
+    }
 }
 
 template <int R>
@@ -606,24 +644,7 @@ cudaError_t states_impl(const Dims& d, const CUtensorMap& mX, const CUtensorMap&
 
 }  // namespace
 
-int tc_state_segments(const Dims& d) {
-    const int units = state_units(d);
-    if (d.seq_segments > 0) return (d.seq_segments <= units && units % d.seq_segments == 0) ? d.seq_segments : 1;
-    constexpr long kSMs = 148;
-    const long ctas = (long)d.BH() * (d.r == 64 ? 5 : 1);       // per run
-    const long tiles = d.n / 128, upt = tiles / units;
-    // Time in tenths of a token tile: waves x (longest run + what a CTA's start and end cost).  Causal, more
-    // than one run: two launches of nseg - 1 runs each and the running sums between them.
-    long best = 10 * ((ctas + kSMs - 1) / kSMs) * (tiles + kStartTiles);
-    if (!d.noncausal) best = best * 9 / 10;              // (cutting has to pay clearly)
-    int pick = 1;
-    for (int s = 2; s <= 64 && s <= units; ++s) {
-        const long run = ((units + s - 1) / s) * upt, waves = (ctas * (d.noncausal ? s : s - 1) + kSMs - 1) / kSMs;
-        const long cost = 10 * (d.noncausal ? waves * (run + kStartTiles) : waves * (2 * run + kStartTiles + kInitTiles) + kBetweenTiles);
-        if (cost < best) { best = cost; pick = s; }
-    }
-    return pick;
-}
+int tc_state_segments(const Dims& d) { return state_plan(d).nseg; }
 
 size_t tc_state_total_bytes(const Dims& d) {
     const int nseg = tc_state_segments(d);
