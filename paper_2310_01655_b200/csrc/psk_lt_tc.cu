@@ -102,129 +102,148 @@ lt_tc_state_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_consta
 }
 
 // ---------------------------------------------------------------------------
-// rows: grid (b/128, t, batch), 160 threads.  Warps 0-3: thread = row (masking, epilogue); warp 4:
-// one thread issues every TMA load and every MMA.  The features are walked once in chunks of 64:
-// each chunk of the own rows multiplies the prefix state's chunk (into O) and the same chunk of
-// every row tile of the block up to the own one (into that tile's scores S); the masked scores then
-// multiply the tiles of C from tensor memory.
+// rows: grid (t, batch), one CTA per block of TPB = b / 128 row tiles.  Warps of the first TPB warpgroups: thread =
+// row (masking, epilogue); the last warp: one thread issues every TMA load and every MMA.  The features are
+// walked once in chunks of 64: a chunk of the block's A rows multiplies the prefix state's chunk (into
+// O) and the same chunk of the block's B rows (into the scores of the tile pairs on and below the diagonal); the
+// masked scores then multiply the tiles of C from tensor memory.  Bound: memory; A, B and Z cross it once.
+// (With a CTA per row tile B's tiles and Z were read again for the second tile: batch 24, n 8192, m 1024,
+// b 256: 234 us.)
 // ---------------------------------------------------------------------------
-constexpr int kRwStage = 16384 + 8192 + 2 * 16384;
-constexpr int kRwSmem = 2 * kRwStage + 2 * 16384 + 1024;
-constexpr uint32_t cO = 0, cS = 128;
+template <int TPB> struct LtRows {
+    static constexpr int A = 0, B = TPB * 16384, Z = 2 * B, kStage = Z + 8192, kStages = 2;
+    static constexpr int C = kStages * kStage, bytes = C + TPB * 16384 + 1024;
+    static constexpr int kThreads = 128 * TPB + 32;
+    static constexpr uint32_t kTmem = TPB == 1 ? 256 : 512;            // O 64 TPB, scores 128 per tile pair
+    static constexpr uint32_t cS = 128;
+};
 
-__global__ void __launch_bounds__(160)
+template <int TPB>
+__global__ void __launch_bounds__(LtRows<TPB>::kThreads)
 lt_tc_rows_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                   const __grid_constant__ CUtensorMap mapC, const __grid_constant__ CUtensorMap mapZ,
-                  float* __restrict__ Out, int n, int m, int b, int t, int* status) {
-    pdl_sync();
+                  float* __restrict__ Out, int n, int m, int t, int* status) {
+    using L = LtRows<TPB>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
-    uint8_t* sC = smem + 2 * kRwStage;
-    __shared__ uint64_t bar_full[2], bar_free[2], bar_c, bar_s, bar_p, bar_o;
+    __shared__ uint64_t bar_full[L::kStages], bar_free[L::kStages], bar_c, bar_s, bar_p[TPB], bar_o[TPB];
     __shared__ uint32_t tm_slot;
     const int tid = threadIdx.x, warp = tid / 32;
-    const int tau = blockIdx.x, l = blockIdx.y, bt = blockIdx.z;
-    const int row0 = l * b + tau * 128, nch = m / 64, ntl = tau + 1;
+    const int l = blockIdx.x, bt = blockIdx.y;
+    const int row0 = l * TPB * 128, nch = m / 64;
     if (tid == 0) {
         cta_giveup_init();
-        mbar_init(&bar_full[0], 1); mbar_init(&bar_full[1], 1);
-        mbar_init(&bar_free[0], 1); mbar_init(&bar_free[1], 1);
-        mbar_init(&bar_c, 1); mbar_init(&bar_s, 1); mbar_init(&bar_o, 1);
-        mbar_init(&bar_p, 128);
+        for (int i = 0; i < L::kStages; ++i) { mbar_init(&bar_full[i], 1); mbar_init(&bar_free[i], 1); }
+        mbar_init(&bar_c, 1); mbar_init(&bar_s, 1);
+        for (int w = 0; w < TPB; ++w) { mbar_init(&bar_p[w], 128); mbar_init(&bar_o[w], 1); }
         mbar_fence_init();
     }
-    if (warp == 4) { tmem_alloc(&tm_slot, 512); tmem_relinquish(); }
+    pdl_sync();
+    if (warp == 4 * TPB) { tmem_alloc(&tm_slot, L::kTmem); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tm = tm_slot;
-    if (tid == 128) {
-        mbar_expect_tx(&bar_c, ntl * 16384);
-        for (int tp = 0; tp < ntl; ++tp) tma_load_3d(sC + tp * 16384, &mapC, 0, l * b + tp * 128, bt, &bar_c);
+    // scores of row tile w against tile tp <= w
+    auto scores = [](int w, int tp) { return L::cS + 128u * (w * (w + 1) / 2 + tp); };
+    if (tid == 128 * TPB) {
         auto load = [&](int c) {
-            const int s = c & 1;
-            uint8_t* st = smem + s * kRwStage;
-            mbar_expect_tx(&bar_full[s], 16384 + (l > 0 ? 8192 : 0) + ntl * 16384);
-            tma_load_3d(st, &mapA, c * 64, row0, bt, &bar_full[s]);
-            if (l > 0) tma_load_3d(st + 16384, &mapZ, 0, c * 64, bt * t + l, &bar_full[s]);
-            for (int tp = 0; tp < ntl; ++tp) tma_load_3d(st + 24576 + tp * 16384, &mapB, c * 64, l * b + tp * 128, bt, &bar_full[s]);
+            const int s = c % L::kStages;
+            uint8_t* st = smem + s * L::kStage;
+            mbar_expect_tx(&bar_full[s], 2 * TPB * 16384 + (l > 0 ? 8192 : 0));
+#pragma unroll
+            for (int w = 0; w < TPB; ++w) {
+                tma_load_3d(st + L::A + w * 16384, &mapA, c * 64, row0 + w * 128, bt, &bar_full[s]);
+                tma_load_3d(st + L::B + w * 16384, &mapB, c * 64, row0 + w * 128, bt, &bar_full[s]);
+            }
+            if (l > 0) tma_load_3d(st + L::Z, &mapZ, 0, c * 64, bt * t + l, &bar_full[s]);
         };
-        load(0);
-        if (nch > 1) load(1);
+        for (int c = 0; c < L::kStages && c < nch; ++c) load(c);
+        mbar_expect_tx(&bar_c, TPB * 16384);
+        for (int w = 0; w < TPB; ++w) tma_load_3d(smem + L::C + w * 16384, &mapC, 0, row0 + w * 128, bt, &bar_c);
         constexpr uint32_t idesc_z = idesc_bf16(128, 64, false, true);
         constexpr uint32_t idesc_s = idesc_bf16(128, 128, false, false);
         bool ok = true;
         for (int c = 0; c < nch && ok; ++c) {
-            const int s = c & 1;
-            ok = mbar_spin(&bar_full[s], (c >> 1) & 1, status, kErrTma);
+            const int s = c % L::kStages;
+            ok = mbar_spin(&bar_full[s], (c / L::kStages) & 1, status, kErrTma);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t base = smem_u32(smem + s * kRwStage);
-            const uint64_t ad = smem_desc(base, 0, 1024, kSwz128);
-            if (l > 0) {
-                const uint64_t zd = smem_desc(base + 16384, 0, 1024, kSwz128);
+            const uint32_t base = smem_u32(smem + s * L::kStage);
+            const uint64_t zd = smem_desc(base + L::Z, 0, 1024, kSwz128);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) umma_ss(tm + cO, desc_off(ad, k * 32), desc_off(zd, k * 2048), idesc_z, (c > 0 || k > 0) ? 1u : 0u);
-            }
-            for (int tp = 0; tp < ntl; ++tp) {
-                const uint64_t bd = smem_desc(base + 24576 + tp * 16384, 0, 1024, kSwz128);
+            for (int w = 0; w < TPB; ++w) {
+                const uint64_t ad = smem_desc(base + L::A + w * 16384, 0, 1024, kSwz128);
+                if (l > 0) {
 #pragma unroll
-                for (int k = 0; k < 4; ++k) umma_ss(tm + cS + tp * 128, desc_off(ad, k * 32), desc_off(bd, k * 32), idesc_s, (c > 0 || k > 0) ? 1u : 0u);
+                    for (int k = 0; k < 4; ++k) umma_ss(tm + w * 64, desc_off(ad, k * 32), desc_off(zd, k * 2048), idesc_z, (c > 0 || k > 0) ? 1u : 0u);
+                }
+#pragma unroll
+                for (int tp = 0; tp <= w; ++tp) {
+                    const uint64_t bd = smem_desc(base + L::B + tp * 16384, 0, 1024, kSwz128);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) umma_ss(tm + scores(w, tp), desc_off(ad, k * 32), desc_off(bd, k * 32), idesc_s, (c > 0 || k > 0) ? 1u : 0u);
+                }
             }
             umma_commit(&bar_free[s]);
-            if (c + 2 < nch) {
-                ok = mbar_spin(&bar_free[s], (c >> 1) & 1, status, kErrMma);
-                if (ok) load(c + 2);
+            if (c + L::kStages < nch) {
+                ok = mbar_spin(&bar_free[s], (c / L::kStages) & 1, status, kErrMma);
+                if (ok) load(c + L::kStages);
             }
         }
-        if (ok) {
-            umma_commit(&bar_s);
-            ok = mbar_spin(&bar_c, 0, status, kErrTma) && mbar_spin(&bar_p, 0, status, kErrMma);
-        }
-        if (ok) {
-            tc_fence_after();
-            for (int tp = 0; tp < ntl; ++tp) {
-                const uint64_t cd = smem_desc(smem_u32(sC + tp * 16384), 0, 1024, kSwz128);
+        if (ok) umma_commit(&bar_s);
+        ok = ok && mbar_spin(&bar_c, 0, status, kErrTma);
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    umma_ts(tm + cO, tm + cS + tp * 128 + k * 8, desc_off(cd, k * 2048), idesc_z, (l > 0 || tp > 0 || k > 0) ? 1u : 0u);
+        for (int w = 0; w < TPB; ++w) {
+            ok = ok && mbar_spin(&bar_p[w], 0, status, kErrMma);
+            if (ok) {
+                tc_fence_after();
+#pragma unroll
+                for (int tp = 0; tp <= w; ++tp) {
+                    const uint64_t cd = smem_desc(smem_u32(smem + L::C + tp * 16384), 0, 1024, kSwz128);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        umma_ts(tm + w * 64, tm + scores(w, tp) + k * 8, desc_off(cd, k * 2048), idesc_z, (l > 0 || tp > 0 || k > 0) ? 1u : 0u);
+                }
+                umma_commit(&bar_o[w]);
             }
-            umma_commit(&bar_o);
         }
-    } else if (warp < 4) {
-        const uint32_t lane_tm = tm + ((uint32_t)(warp * 32) << 16);
+    } else if (warp < 4 * TPB) {
+        const int w = warp / 4, wt = tid % 128;
+        const uint32_t lane_tm = tm + ((uint32_t)((warp % 4) * 32) << 16);
         bool ok = mbar_wait(&bar_s, 0, status, kErrMma);
         tc_fence_after();
         if (ok) {
-            for (int tp = 0; tp < ntl; ++tp) {
-                const bool diag = tp == tau;
+            for (int tp = 0; tp <= w; ++tp) {
+                const bool diag = tp == w;
+                const uint32_t ts = lane_tm + scores(w, tp);
 #pragma unroll
                 for (int c0 = 0; c0 < 128; c0 += 32) {
                     uint32_t u[32], pk[16];
-                    tmem_ld32(lane_tm + cS + tp * 128 + c0, u);
+                    tmem_ld32(ts + c0, u);
                     tmem_ld_wait();
 #pragma unroll
                     for (int j = 0; j < 32; j += 2) {
-                        const float x = (diag && c0 + j > tid) ? 0.f : __uint_as_float(u[j]);
-                        const float y = (diag && c0 + j + 1 > tid) ? 0.f : __uint_as_float(u[j + 1]);
+                        const float x = (diag && c0 + j > wt) ? 0.f : __uint_as_float(u[j]);
+                        const float y = (diag && c0 + j + 1 > wt) ? 0.f : __uint_as_float(u[j + 1]);
                         pk[j / 2] = pack_bf16(x, y);
                     }
                     // the masked scores as the bf16 A operand of the last GEMM, over the columns just read
-                    tmem_st16(lane_tm + cS + tp * 128 + c0 / 2, pk);
+                    tmem_st16(ts + c0 / 2, pk);
                 }
             }
             tmem_st_wait();
         }
         tc_fence_before();
-        mbar_arrive(&bar_p);
-        ok = ok && mbar_wait(&bar_o, 0, status, kErrMma);
+        mbar_arrive(&bar_p[w]);
+        ok = ok && mbar_wait(&bar_o[w], 0, status, kErrMma);
         tc_fence_after();
         if (ok) {
-            float* dst = Out + ((size_t)bt * n + row0 + tid) * 64;
+            float* dst = Out + ((size_t)bt * n + row0 + w * 128 + wt) * 64;
 #pragma unroll
             for (int c0 = 0; c0 < 64; c0 += 32) {
                 uint32_t u[32];
-                tmem_ld32(lane_tm + cO + c0, u);
+                tmem_ld32(lane_tm + w * 64 + c0, u);
                 tmem_ld_wait();
 #pragma unroll
                 for (int j = 0; j < 32; j += 4)
@@ -235,7 +254,18 @@ lt_tc_rows_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constan
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 4) tmem_dealloc(tm, 512);
+    if (warp == 4 * TPB) tmem_dealloc(tm, L::kTmem);
+}
+
+template <int TPB>
+cudaError_t launch_rows(const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mC, const CUtensorMap& mZ, float* Out, int batch, int n, int m,
+                        int t, int* status, cudaStream_t s) {
+    using L = LtRows<TPB>;
+    PSK_TRY(set_smem(lt_tc_rows_kernel<TPB>, L::bytes));
+    prof_begin("lt_tc_rows_kernel", s);
+    launch_pdl(lt_tc_rows_kernel<TPB>, dim3(t, batch), L::kThreads, L::bytes, s, mA, mB, mC, mZ, Out, n, m, t, status);
+    prof_end(s);
+    return cudaGetLastError();
 }
 
 bool lt_tc_args_ok(int batch, int n, int m, int k, int b) {
@@ -272,18 +302,14 @@ int psk_lt_multiply_bf16(int batch, int n, int m, int k, int b, const void* A, c
     if (!tc_map_3d(&mA, A, m, n, batch, 64, 128) || !tc_map_3d(&mB, B, m, n, batch, 64, 128) ||
         !tc_map_3d(&mC, C, 64, n, batch, 64, 128) || !tc_map_3d(&mZ, Z, 64, m, (int64_t)batch * t, 64, 64))
         return PSK_ERR_CUDA;
-    if (cudaFuncSetAttribute(lt_tc_state_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStSmem) != cudaSuccess ||
-        cudaFuncSetAttribute(lt_tc_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRwSmem) != cudaSuccess)
-        return PSK_ERR_CUDA;
+    if (set_smem(lt_tc_state_kernel, kStSmem) != cudaSuccess) return PSK_ERR_CUDA;
     if (t > 1) {
         prof_begin("lt_tc_state_kernel", s);
         launch_pdl(lt_tc_state_kernel, dim3((m + 127) / 128, batch), 128, kStSmem, s, mB, mC, Z, m, t, tpb, status);
         prof_end(s);
     }
-    prof_begin("lt_tc_rows_kernel", s);
-    launch_pdl(lt_tc_rows_kernel, dim3(tpb, t, batch), 160, kRwSmem, s, mA, mB, mC, mZ, Out, n, m, b, t, status);
-    prof_end(s);
-    return cudaGetLastError() == cudaSuccess ? PSK_OK : PSK_ERR_CUDA;
+    const cudaError_t e = tpb == 1 ? launch_rows<1>(mA, mB, mC, mZ, Out, batch, n, m, t, status, s) : launch_rows<2>(mA, mB, mC, mZ, Out, batch, n, m, t, status, s);
+    return e == cudaSuccess ? PSK_OK : PSK_ERR_CUDA;
 }
 
 }  // extern "C"
