@@ -90,6 +90,13 @@ bool tc_map_states(CUtensorMap* m, const void* base, int FP, int64_t nblk) {
 }
 
 
+bool tc_map_hilo(const Dims& d, const void* hl, CUtensorMap (&m)[2]) {
+    const int64_t cols = d.r <= 32 ? 64 : 128, hs = d.n * cols, bs = d.H * hs;
+    if (!tc_map_rows(&m[0], hl, d.B, d.H, d.n, bs, hs, cols)) return false;
+    m[1] = m[0];
+    return d.r <= 32 || tc_map_rows(&m[1], static_cast<const bf16*>(hl) + 64, d.B, d.H, d.n, bs, hs, cols);
+}
+
 namespace {
 
 // ---------------------------------------------------------------------------
@@ -120,33 +127,34 @@ constexpr uint32_t kZStageBytes = 16384;        // two [64 features x 128 B] box
 constexpr int kFeatBufs = kZStages;             // feature staging buffers in tensor memory, 32 columns each:
                                                 // chunk C uses buffer and stage C % 4, both freed by its MMAs
 
-template <int R, bool LOCAL = false>
+template <int R, bool LOCAL, bool LIN>
 struct OutSmem {
-    // The prefix-state stages (first phase), the key/value tiles with the keys' split half
-    // sketches (second phase) and the output staging tiles (epilogue) share one region; small
-    // enough for two CTAs per SM when R <= 32.
-    static constexpr uint32_t Q = 0, G = 16384;
-    static constexpr uint32_t Ones = G + GImage<R>::bytes;           // 4 KB of bf16 1.0: B operand of the row sums
+    // The prefix-state stages (first phase), the same-block key/value tiles (second phase) and the output staging
+    // tiles (epilogue) share one region; small enough for two CTAs per SM.
+    static constexpr int NT = LOCAL ? 1 : OthTiles<R, LIN>::N;
+    static constexpr uint32_t Q = 0;
+    static constexpr uint32_t Ones = 16384;                          // 4 KB of bf16 1.0: B operand of the row sums
+    // the own rows' [hi | lo] half sketches.  (LOCAL: the ring's last stage, because the query tile stays alive for
+    // the exact scores)
     static constexpr uint32_t Mq = Ones + 4096;
-    // split operand: 3R columns.  (LOCAL: no split operands; the region holds the ring's last
-    // stage and then the value tile, because the query tile stays alive for the exact scores.)
-    static constexpr uint32_t kMqBytes = LOCAL ? 16384 : 128 * 3 * R * 2;
-    static constexpr uint32_t U = (Mq + kMqBytes + 1023) / 1024 * 1024;
+    static constexpr uint32_t kMqBytes = NT * 16384;
+    // the sketch matrices' image: needed for the own rows only, dead before their half sketches are stored
+    static constexpr uint32_t G = LOCAL ? Mq + kMqBytes : Mq;
+    static_assert(LOCAL || GImage<R>::bytes <= kMqBytes, "image under the half sketches");
+    static constexpr uint32_t U = G + (LOCAL ? (GImage<R>::bytes + 1023) / 1024 * 1024 : kMqBytes);
     static constexpr uint32_t Z = U;
-    // key tile in ring stage 1, value tile in the query tile's buffer (ring stage 3), split key
-    // sketches over stage 2: the stages the last chunks free first, so the first key/value tile is
-    // fetched while the last chunks are still being multiplied
     static constexpr uint32_t Z3 = LOCAL ? Mq : Q;                   // ring stage 3
-    static constexpr uint32_t K = U + 16384, V = Z3, Mk = U + 32768;
-    static constexpr int kStageK = 1, kStageV = kZStages - 1;
+    // Key and value tiles of the same block, in the ring's stages, in the order in which the last chunks free them: two
+    // tiles are fetched while chunks are still being multiplied.  (r = 64 with two-tile operands: room for one.)
+    static constexpr int kSets = NT == 1 ? 2 : 1;
+    __host__ __device__ static constexpr int stage_k(int p) { return LOCAL ? (p ? 2 : 1) : (p ? 3 : 1); }      // NT = 2: and the next one
+    __host__ __device__ static constexpr int stage_v(int p) { return LOCAL ? (p ? 0 : 3) : (p ? 0 : (NT == 2 ? 3 : 2)); }
     // last chunk that uses ring stage s (-1: none)
     __host__ __device__ static constexpr int last_chunk(int nc, int s) { return nc > s ? s + (nc - 1 - s) / kZStages * kZStages : -1; }
     static constexpr uint32_t So = U, Soc = U + 16384;               // O tile, O - c tile (bf16 each)
-    static constexpr uint32_t kPhase1 = (kZStages - 1) * kZStageBytes, kPhase2 = 32768 + (LOCAL ? 0 : 128 * 3 * R * 2), kEpi = 32768;
-    static constexpr uint32_t kMax12 = kPhase1 > kPhase2 ? kPhase1 : kPhase2;
-    static constexpr uint32_t total = U + (kMax12 > kEpi ? kMax12 : kEpi);
+    static constexpr uint32_t total = U + (kZStages - 1) * kZStageBytes;
     // stage s of the prefix-state ring; the last one is the query tile's buffer, dead after the sketch
-    __device__ static uint32_t zstage(int s) { return s < kZStages - 1 ? Z + s * kZStageBytes : Z3; }
+    __host__ __device__ static constexpr uint32_t zstage(int s) { return s < kZStages - 1 ? Z + s * kZStageBytes : Z3; }
 };
 
 
@@ -158,10 +166,12 @@ struct OutSmem {
 // (bf16 operands, exact products, fp32 sums) in place of m(q_i) . m(k_j); squared like those,
 // they give the exact weights (q_i . k_j)^4.  No key sketches, no split operands.
 // LIN: the rows hold a given half sketch (tc_common.cuh, read_half_sketch).
+// Not LOCAL: mapK holds the keys' half sketches as score operands, [hi | lo] rows (the state kernel's array, or the given
+// rows themselves); r = 64: mapQraw the second 64 columns.
 // LIN and LOCAL: mapQ is the given half sketch, mapQraw the raw query rows (fetched into the query
 // tile's buffer once the sketch GEMM has read it), mapK the raw key rows.
 template <int R, int MODE, bool LOCAL, bool LIN>
-__global__ void __launch_bounds__(kOutThreads, ((R <= 32 || LOCAL) ? 2 : 1))
+__global__ void __launch_bounds__(kOutThreads, 2)
 tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapQraw,
                   const __grid_constant__ CUtensorMap mapK,
                   const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapZ,
@@ -173,10 +183,10 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     pdl_sync();
     constexpr bool lin = LIN;
     using F = Feat<R>;
-    using L = OutSmem<R, LOCAL>;
+    using L = OutSmem<R, LOCAL, LIN>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
-    __shared__ uint64_t bar_q, bar_kv, bar_sk, bar_go, bar_mk, bar_s, bar_p, bar_pv;
+    __shared__ uint64_t bar_q, bar_kv[2], bar_sk, bar_go, bar_s, bar_p, bar_pv;
     __shared__ uint64_t bar_z[kZStages], bar_feat[kFeatBufs], bar_a[kFeatBufs];
     __shared__ uint32_t tmem_slot;
     __shared__ float cm[64];
@@ -197,8 +207,8 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
         mbar_expect_tx(&bar_q, 16384 + GImage<R>::bytes);
         tma_load_4d(smem + L::Q, &mapQ, 0, row0, hi, bi, &bar_q);
         bulk_load(smem + L::G, gimg + (size_t)g * GImage<R>::bytes, GImage<R>::bytes, &bar_q);
-        mbar_init(&bar_kv, 1); mbar_init(&bar_sk, 1); mbar_init(&bar_s, 1); mbar_init(&bar_pv, 1);
-        mbar_init(&bar_mk, 128); mbar_init(&bar_p, 128); mbar_init(&bar_go, 128);
+        mbar_init(&bar_kv[0], 1); mbar_init(&bar_kv[1], 1); mbar_init(&bar_sk, 1); mbar_init(&bar_s, 1); mbar_init(&bar_pv, 1);
+        mbar_init(&bar_p, 128); mbar_init(&bar_go, 128);
         for (int s = 0; s < kZStages; ++s) mbar_init(&bar_z[s], 1);
         for (int s = 0; s < kFeatBufs; ++s) { mbar_init(&bar_feat[s], 128); mbar_init(&bar_a[s], 1); }
         cta_giveup_init();
@@ -212,6 +222,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     if (tid == 32 && !noncausal) {
         for (int tp = 0; tp <= tau; ++tp) {
             tma_prefetch_4d(&mapK, 0, l * b + tp * 128, hi, bi);
+            if constexpr (L::NT == 2) tma_prefetch_4d(&mapQraw, 0, l * b + tp * 128, hi, bi);
             tma_prefetch_4d(&mapV, 0, l * b + tp * 128, hi, bi);
         }
     }
@@ -264,6 +275,13 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     if (warp == 4) {
         // ================================ issuer ================================
         if (tid == 128) {
+            constexpr uint32_t kK0 = L::zstage(L::stage_k(0)), kK1 = L::zstage(L::stage_k(1)), kV0 = L::zstage(L::stage_v(0)), kV1 = L::zstage(L::stage_v(1));
+            auto load_k = [&](int tp, int p) {         // (with the value tile's bytes expected too)
+                mbar_expect_tx(&bar_kv[p], (L::NT + 1) * 16384);
+                tma_load_4d(smem + (p ? kK1 : kK0), &mapK, 0, l * b + tp * 128, hi, bi, &bar_kv[p]);
+                if constexpr (L::NT == 2) tma_load_4d(smem + kK0 + 16384, &mapQraw, 0, l * b + tp * 128, hi, bi, &bar_kv[p]);
+            };
+            auto load_v = [&](int tp, int p) { tma_load_4d(smem + (p ? kV1 : kV0), &mapV, 0, l * b + tp * 128, hi, bi, &bar_kv[p]); };
             // (the first state chunks are requested here, not by the thread that sets the barriers
             // up: everyone waits for that thread, only this one waits for the query tile anyway)
             if (has_prefix) {
@@ -292,64 +310,68 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                 tma_load_3d(smem + L::zstage(kZStages - 1) + 8192, &mapZ, 64, (kZStages - 1) * 64, blk, &bar_z[kZStages - 1]);
             }
             if (has_prefix) issue_chunks(0, PSK_OUT_ISSUERS);     // earlier blocks: features x prefix state chunks
+            const int tp_last = noncausal ? -1 : tau;
             if (has_prefix && !noncausal) {
-                // first key/value tile of the same block, each into its stage as soon as the last
+                // the first key/value tiles of the same block, each into its stage as soon as the last
                 // chunk that used it has been multiplied
-                constexpr int cK = L::last_chunk(F::NC, L::kStageK), cV = L::last_chunk(F::NC, L::kStageV);
-                mbar_expect_tx(&bar_kv, 32768);
-                if (cK >= 0) ok = ok && mbar_spin(&bar_a[L::kStageK], (cK / kZStages) & 1, status, kErrMma);
-                tma_load_4d(smem + L::K, &mapK, 0, l * b, hi, bi, &bar_kv);
-                if (cV >= 0) ok = ok && mbar_spin(&bar_a[L::kStageV], (cV / kZStages) & 1, status, kErrMma);
-                else ok = ok && mbar_spin(&bar_sk, 0, status, kErrMma);     // no chunk used it: the query sketch did
-                tma_load_4d(smem + L::V, &mapV, 0, l * b, hi, bi, &bar_kv);
-                // the sketch reuses the staging columns and the split key sketches the remaining
-                // stage: every MMA of the first phase must have completed
+                auto stage_free = [&](int st) {
+                    const int c = L::last_chunk(F::NC, st);
+                    if (c >= 0) ok = ok && mbar_spin(&bar_a[st], (c / kZStages) & 1, status, kErrMma);
+                    else ok = ok && mbar_spin(&bar_sk, 0, status, kErrMma);     // no chunk used it: the query sketch did
+                };
+                static_for<0, L::kSets>([&](auto pc) {
+                    constexpr int P = decltype(pc)::value;
+                    if (P > tau) return;
+                    stage_free(L::stage_k(P));
+                    if constexpr (L::NT == 2) stage_free(L::stage_k(P) + 1);
+                    load_k(P, P);
+                    stage_free(L::stage_v(P));
+                    load_v(P, P);
+                });
+                // the scores reuse the staging columns: every MMA of the first phase must have completed
                 ok = ok && mbar_spin(&bar_a[(F::NC - 1) % kFeatBufs], ((F::NC - 1) / kFeatBufs) & 1, status, kErrMma);
+            } else if (!noncausal) {
+                // first block: nothing used the stages, only the query sketch its buffer
+                ok = ok && mbar_spin(&bar_sk, 0, status, kErrMma);
+                for (int p = 0; p < L::kSets && p <= tau; ++p) { load_k(p, p); load_v(p, p); }
             }
             // same block: key tiles tp <= tau through squared half-sketch scores; descriptors and
             // addresses are loop invariants, so every issue sequence below is MMA instructions only
-            const uint64_t qd = smem_desc(smem_u32(smem + L::Mq), 2048, 128, kSwzNone);
-            const uint64_t kd = smem_desc(smem_u32(smem + L::Mk), 2048, 128, kSwzNone);
-            const uint64_t vd = smem_desc(smem_u32(smem + L::V), 0, 1024, kSwz128);
             const uint64_t od = smem_desc(smem_u32(smem + L::Ones), 256, 128, kSwzNone);
-            // every row has read the query sketch (the first key sketch overwrites its columns, and
-            // bar_sk must not complete a second time before its slowest waiter has seen the first)
+            // every row has read the query sketch (the scores overwrite its columns) and stored its operand
             ok = ok && mbar_spin(&bar_go, 0, status, kErrMma);
-            const int tp_last = noncausal ? -1 : tau;
 #pragma unroll 1
             for (int tp = 0; tp <= tp_last && ok; ++tp) {
-                if (tp > 0) ok = mbar_spin(&bar_pv, (tp - 1) & 1, status, kErrMma);   // K, V, Mk, weights are free
-                if (tp > 0 || l == 0) {       // (block l > 0: the first tile was requested above)
-                    mbar_expect_tx(&bar_kv, 32768);
-                    tma_load_4d(smem + L::K, &mapK, 0, l * b + tp * 128, hi, bi, &bar_kv);
-                    tma_load_4d(smem + L::V, &mapV, 0, l * b + tp * 128, hi, bi, &bar_kv);
+                const int p = tp % L::kSets;
+                if (tp > 0) {
+                    // the previous tile's K, V and weights are free: the tile after next (or this one) may come
+                    ok = mbar_spin(&bar_pv, (tp - 1) & 1, status, kErrMma);
+                    const int nx = tp - 1 + L::kSets;
+                    if (nx <= tp_last) { load_k(nx, nx % L::kSets); load_v(nx, nx % L::kSets); }
                 }
-                ok = ok && mbar_spin(&bar_kv, tp & 1, status, kErrTma);
+                ok = ok && mbar_spin(&bar_kv[p], (tp / L::kSets) & 1, status, kErrTma);
                 FTR(7, tp);
                 tc_fence_after();
+                constexpr uint32_t idesc_s = idesc_bf16(128, 128, false, false);
+                const uint64_t kr = smem_desc(smem_u32(smem + (p ? kK1 : kK0)), 0, 1024, kSwz128);
+                const uint64_t vd = smem_desc(smem_u32(smem + (p ? kV1 : kV0)), 0, 1024, kSwz128);
                 if constexpr (LOCAL) {
                     // scores = Q_tile K_tile^T over the head dimension
                     if constexpr (LIN) ok = ok && mbar_spin(&bar_q, 1, status, kErrTma);     // the raw query rows
-                    constexpr uint32_t idesc = idesc_bf16(128, 128, false, false);
                     const uint64_t qr = smem_desc(smem_u32(smem + L::Q), 0, 1024, kSwz128);
-                    const uint64_t kr = smem_desc(smem_u32(smem + L::K), 0, 1024, kSwz128);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        umma_ss(tm + cS, desc_off(qr, k * 32), desc_off(kr, k * 32), idesc, k > 0);
-                    umma_commit(&bar_s);
+                    for (int k = 0; k < 4; ++k) umma_ss(tm + cS, desc_off(qr, k * 32), desc_off(kr, k * 32), idesc_s, k > 0);
                 } else {
-                    issue_sketch<R>(tm + cSk, smem + L::K, smem + L::G);
-                    umma_commit(&bar_sk);
-                    FTR(8, tp);
-                    ok = ok && mbar_spin(&bar_mk, tp & 1, status, kErrMma);
-                    FTR(9, tp);
-                    tc_fence_after();
-                    constexpr uint32_t idesc = idesc_bf16(128, 128, false, false);
+                    // hi.hi + lo.hi + hi.lo over the [hi | lo] columns of both operands (no lo where the rows are the half sketch)
+                    const uint64_t qd = smem_desc(smem_u32(smem + L::Mq), 0, 1024, kSwz128);
+                    constexpr int kLo = R == 64 ? 16384 : 2 * R;             // bytes from hi to lo
 #pragma unroll
-                    for (int k = 0; k < 3 * R / 16; ++k)
-                        umma_ss(tm + cS, desc_off(qd, k * 4096), desc_off(kd, k * 4096), idesc, k > 0);
-                    umma_commit(&bar_s);
+                    for (int g = 0; g < ((LIN && R == 64) ? 1 : 3); ++g)
+#pragma unroll
+                        for (int k = 0; k < R / 16; ++k)
+                            umma_ss(tm + cS, desc_off(qd, (g == 1 ? kLo : 0) + k * 32), desc_off(kr, (g == 2 ? kLo : 0) + k * 32), idesc_s, (g > 0 || k > 0) ? 1u : 0u);
                 }
+                umma_commit(&bar_s);
                 FTR(10, tp);
                 ok = ok && mbar_spin(&bar_p, tp & 1, status, kErrMma);
                 FTR(11, tp);
@@ -377,7 +399,10 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
         tc_fence_after();
         float mq[R];
         read_half_sketch<R>(lane_tm + cSk, mq, 1.f, lin != 0);
-        if constexpr (!LOCAL) store_split_rows<R, true>(smem + L::Mq, mq, tid);
+        if constexpr (!LOCAL) {                       // (over the sketch matrices' image: the sketch has completed)
+            store_hilo_tiles<R, L::NT>(smem + L::Mq, mq, tid);
+            fence_proxy_async_smem();
+        }
         tc_fence_before();
         mbar_arrive(&bar_go);
         if (tid == 0) FTR(21, 0);
@@ -437,20 +462,6 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
         const int tp_last = noncausal ? -1 : tau;
 #pragma unroll 1
         for (int tp = 0; tp <= tp_last && ok; ++tp) {
-            if constexpr (!LOCAL) {
-                ok = mbar_wait(&bar_sk, (tp + 1) & 1, status, kErrMma);
-                if (tid == 0) FTR(24, tp);
-                tc_fence_after();
-                {
-                    float mk[R];
-                    read_half_sketch<R>(lane_tm + cSk, mk, 1.f, lin != 0);
-                    store_split_rows<R, false>(smem + L::Mk, mk, tid);
-                }
-                fence_proxy_async_smem();
-                tc_fence_before();
-                mbar_arrive(&bar_mk);
-                if (tid == 0) FTR(25, tp);
-            }
             ok = ok && mbar_wait(&bar_s, tp & 1, status, kErrMma);
             if (tid == 0) FTR(26, tp);
             tc_fence_after();
@@ -680,7 +691,10 @@ cudaError_t fwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
     float* cmean = d.keep_states ? reinterpret_cast<float*>(ws + w.vmean) : nullptr;
     uint8_t* gimg = reinterpret_cast<uint8_t*>(ws + w.gimg);
     PSK_TRY(tc_prologue(d, G1, G2, gimg, V, cmean, status, s, launches));
-    PSK_TRY(tc_states(d, mK, mV, gimg, nullptr, nullptr, cmean, cmean ? 1 : 0, Z, false,
+    bf16* Sk = tc_hilo_rows(d) ? reinterpret_cast<bf16*>(ws + w.Sk) : nullptr;
+    CUtensorMap mKs[2] = {mK, mK};
+    if (Sk != nullptr && !tc_map_hilo(d, Sk, mKs)) return cudaErrorInvalidValue;
+    PSK_TRY(tc_states(d, mK, mV, gimg, nullptr, nullptr, cmean, cmean ? 1 : 0, Z, Sk, false,
                       reinterpret_cast<float*>(ws + w.tot), status, s, launches));
     prof_begin("tc_fwd_out_kernel", s);
     if (d.local && d.sketch_linear) {
@@ -689,7 +703,7 @@ cudaError_t fwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
             if (d.rawQ == nullptr || d.rawK == nullptr || !tc_map_rows(&mQraw, d.rawQ, d.B, d.H, d.n, d.sb, d.sh, d.sn) ||
                 !tc_map_rows(&mKraw, d.rawK, d.B, d.H, d.n, d.sb, d.sh, d.sn))
                 return cudaErrorInvalidValue;
-            constexpr size_t smem = OutSmem<R, true>::total + 1024;
+            constexpr size_t smem = OutSmem<R, true, true>::total + 1024;
             PSK_TRY((set_smem(tc_fwd_out_kernel<R, 0, true, true>, smem)));
             launch_pdl(tc_fwd_out_kernel<R, 0, true, true>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
                 mQ, mQraw, mKraw, mV, mZ, mO, mOc, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
@@ -698,22 +712,22 @@ cudaError_t fwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
             return cudaErrorInvalidValue;
         }
     } else if (d.local) {
-        constexpr size_t smem = OutSmem<R, true>::total + 1024;
+        constexpr size_t smem = OutSmem<R, true, false>::total + 1024;
         PSK_TRY((set_smem(tc_fwd_out_kernel<R, 0, true, false>, smem)));
         launch_pdl(tc_fwd_out_kernel<R, 0, true, false>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
             mQ, mQ, mK, mV, mZ, mO, mOc, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
             denom, nullptr, nullptr, nullptr, Oc != nullptr ? 1 : 0, d.noncausal ? 1 : 0, status);
     } else if (d.sketch_linear) {
-        constexpr size_t smem = OutSmem<R, false>::total + 1024;
+        constexpr size_t smem = OutSmem<R, false, true>::total + 1024;
         PSK_TRY((set_smem(tc_fwd_out_kernel<R, 0, false, true>, smem)));
         launch_pdl(tc_fwd_out_kernel<R, 0, false, true>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
             mQ, mQ, mK, mV, mZ, mO, mOc, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
             denom, nullptr, nullptr, nullptr, Oc != nullptr ? 1 : 0, d.noncausal ? 1 : 0, status);
     } else {
-        constexpr size_t smem = OutSmem<R, false>::total + 1024;
+        constexpr size_t smem = OutSmem<R, false, false>::total + 1024;
         PSK_TRY((set_smem(tc_fwd_out_kernel<R, 0, false, false>, smem)));
-        launch_pdl(tc_fwd_out_kernel<R, 0, false, false>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
-            mQ, mQ, mK, mV, mZ, mO, mOc, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
+        launch_pdl(tc_fwd_out_kernel<R, 0, false, false>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s,
+            mQ, mKs[1], mKs[0], mV, mZ, mO, mOc, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
             denom, nullptr, nullptr, nullptr, Oc != nullptr ? 1 : 0, d.noncausal ? 1 : 0, status);
     }
     prof_end(s);
@@ -765,7 +779,7 @@ static cudaError_t recompute_impl(const Dims& d, const CUtensorMap& mQ, const CU
     prof_begin("tc_bwd_recompute_kernel", s);
     if (d.local && d.sketch_linear) {
         if constexpr (R <= 32) {
-            constexpr size_t smem = OutSmem<R, true>::total + 1024;
+            constexpr size_t smem = OutSmem<R, true, true>::total + 1024;
             PSK_TRY((set_smem(tc_fwd_out_kernel<R, 1, true, true>, smem)));
             launch_pdl(tc_fwd_out_kernel<R, 1, true, true>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
                 mQ, mQraw, mK, mV, mZ, mZ, mZ, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
@@ -774,22 +788,22 @@ static cudaError_t recompute_impl(const Dims& d, const CUtensorMap& mQ, const CU
             return cudaErrorInvalidValue;
         }
     } else if (d.local) {
-        constexpr size_t smem = OutSmem<R, true>::total + 1024;
+        constexpr size_t smem = OutSmem<R, true, false>::total + 1024;
         PSK_TRY((set_smem(tc_fwd_out_kernel<R, 1, true, false>, smem)));
         launch_pdl(tc_fwd_out_kernel<R, 1, true, false>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
             mQ, mQ, mK, mV, mZ, mZ, mZ, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
             const_cast<float*>(denom), dO, y65, e65h, 0, d.noncausal ? 1 : 0, status);
     } else if (d.sketch_linear) {
-        constexpr size_t smem = OutSmem<R, false>::total + 1024;
+        constexpr size_t smem = OutSmem<R, false, true>::total + 1024;
         PSK_TRY((set_smem(tc_fwd_out_kernel<R, 1, false, true>, smem)));
         launch_pdl(tc_fwd_out_kernel<R, 1, false, true>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
             mQ, mQ, mK, mV, mZ, mZ, mZ, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
             const_cast<float*>(denom), dO, y65, e65h, 0, d.noncausal ? 1 : 0, status);
     } else {
-        constexpr size_t smem = OutSmem<R, false>::total + 1024;
+        constexpr size_t smem = OutSmem<R, false, false>::total + 1024;
         PSK_TRY((set_smem(tc_fwd_out_kernel<R, 1, false, false>, smem)));
-        launch_pdl(tc_fwd_out_kernel<R, 1, false, false>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s, 
-            mQ, mQ, mK, mV, mZ, mZ, mZ, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
+        launch_pdl(tc_fwd_out_kernel<R, 1, false, false>, dim3(d.b / 128, d.t, d.BH()), kOutThreads, smem, s,
+            mQ, mQraw, mK, mV, mZ, mZ, mZ, gimg, d.g_heads, d.H, d.n, d.b, d.t, cmean, d.sb, d.sh, d.sn,
             const_cast<float*>(denom), dO, y65, e65h, 0, d.noncausal ? 1 : 0, status);
     }
     prof_end(s);

@@ -76,36 +76,45 @@ tc_bwd_prep_kernel(const bf16* __restrict__ dO, const float* __restrict__ denom,
 
 constexpr uint32_t kBoxBytes = 16384;      // two [64 features x 128 B] boxes: state columns 0..63, 64..79
 
-template <int R, bool LOCAL = false, bool QSIDE = false>
+template <int R, bool LOCAL, bool QSIDE, bool LIN>
 struct BwdSmem {
     // every tile: 128 rows x 128 B, 128-byte swizzle
-    static constexpr uint32_t kM = HiLoTiles<R>::N * 16384;      // [hi | lo] half-sketch operand
-    static constexpr uint32_t Xown = 0, Yown = 16384;
-    static constexpr uint32_t G = 32768;
-    static constexpr uint32_t ExtA = G + GImage<R>::bytes;       // [128 x 16] un-swizzled
+    static constexpr int NT = LOCAL ? 1 : OthTiles<R, LIN>::N;
+    static constexpr uint32_t kM = NT * 16384;           // [hi | lo] half-sketch operand (LOCAL: the raw rows)
+    // r = 64 with two-tile operands, query side: the own rows' operand lies over their raw rows and the sketch matrices'
+    // image, which are fetched again for the last phase; that makes room for two CTAs per SM
+    static constexpr bool kFold = NT == 2 && QSIDE;
+    static constexpr uint32_t Xown = 0, G = 16384;
+    static constexpr uint32_t Yown = G + (GImage<R>::bytes + 1023) / 1024 * 1024;
+    static constexpr uint32_t ExtA = Yown + 16384;       // [128 x 16] un-swizzled
     static constexpr uint32_t Eoth = ExtA + 4096;        // 128 x (1/d, e65h) of the other side's rows
     static constexpr uint32_t U = Eoth + 1024;
     static constexpr uint32_t Box = U;                   // phase B: kSt state boxes
     static constexpr int NC = Feat<R>::NC;
-    // stages of the state-chunk ring: four; three on the query side for r = 64 with exact
-    // same-block weights, which then fits two CTAs per SM (no split-operand tiles in that variant;
-    // the key side, at 255 registers and 225 KB of code, ran slower as two CTAs and keeps four)
-    static constexpr int kSt = (R > 32 && LOCAL && QSIDE) ? 3 : 4;
-    // Phase C tiles.  r <= 32 (two CTAs per SM): they reuse the boxes' memory, each tile in the
-    // stage that the last chunks free first, so the first other-side tile is fetched while the
-    // last chunks are still being processed.  r = 64 (one CTA per SM): memory of their own,
-    // except with exact same-block weights, where X, Y and the second X buffer are all there is.
-    static constexpr bool kAlias = (R <= 32) || LOCAL;
-    static constexpr int sX = NC >= kSt ? (NC - kSt) % kSt : 3, sY = NC >= kSt ? (NC - kSt + 1) % kSt : 0;
-    static constexpr int sMo = NC >= kSt ? (NC - kSt + 2) % kSt : 1, sMn = NC >= kSt ? (NC - 1) % kSt : 2;
+    // stages of the state-chunk ring: four; three on the query side for r = 64, which then fits two CTAs per SM
+    // (the key side, at 255 registers and 225 KB of code, ran slower as two CTAs and keeps four)
+    static constexpr int kSt = (R > 32 && QSIDE) ? 3 : 4;
+    // Phase C tiles: they reuse the boxes' memory, each tile in the stages that the last chunks free first, so
+    // the first other-side tile is fetched while the last chunks are still being processed.  r = 64, key side, two-tile
+    // operands (one CTA per SM): memory of their own.
+    static constexpr bool kAlias = NT == 1 || QSIDE;
+    __host__ __device__ static constexpr int last_chunk(int s) { return NC > s ? s + (NC - 1 - s) / kSt * kSt : -1; }
+    // stages in the order in which they become free
+    __host__ __device__ static constexpr int nth_free(int k) { return NC >= kSt ? (NC - kSt + k) % kSt : (k == 0 ? kSt - 1 : k - 1); }
+    static constexpr int sM = NT == 2 ? 0 : nth_free(0), sY = NT == 2 ? 2 : nth_free(1);       // NT = 2: stages 0 and 1, then 2
+    static_assert(!(NT == 2 && kAlias) || (kSt == 3 && NC % 3 == 0), "two-tile operand in the first two of three stages");
+    static constexpr int cM = NT == 2 ? NC - 2 : last_chunk(sM), cY = NT == 2 ? NC - 1 : last_chunk(sY);      // last chunks there (-1: none)
     static constexpr uint32_t C0 = U + kSt * kBoxBytes;
-    static constexpr uint32_t Xoth = kAlias ? U + sX * kBoxBytes : C0;
-    static constexpr uint32_t Yoth = kAlias ? U + sY * kBoxBytes : C0 + 16384;
-    static constexpr uint32_t Moth = kAlias ? U + sMo * kBoxBytes : C0 + 32768;
-    static constexpr uint32_t Mown = kAlias ? U + sMn * kBoxBytes : C0 + 32768 + kM;
-    static_assert(!kAlias || LOCAL || kM == kBoxBytes, "aliased layout: one tile per stage");
-    static_assert(kSt == 4 || NC >= kSt, "three stages: only with many chunks");
-    static constexpr uint32_t total = kAlias ? C0 : C0 + 32768 + 2 * kM;
+    static constexpr uint32_t Moth = kAlias ? U + sM * kBoxBytes : C0;
+    static constexpr uint32_t Yoth = kAlias ? U + sY * kBoxBytes : C0 + kM;
+    // one-tile operands: a second buffer, the next tile's rows are requested a tile ahead
+    static constexpr bool kTwoM = NT == 1;
+    static constexpr uint32_t Moth2 = kTwoM ? U + nth_free(2) * kBoxBytes : Moth;
+    // the own rows' operand: given rows are it themselves
+    static constexpr uint32_t Mown = (LIN || LOCAL || kFold) ? Xown : (kAlias ? U + nth_free(3) * kBoxBytes : C0 + kM + 16384);
+    static_assert(!kFold || Yown >= kM, "operand over rows and image");
+    static_assert(LIN || LOCAL || kFold || !kAlias || kSt == 4, "a stage of its own");
+    static constexpr uint32_t total = kAlias ? C0 : C0 + kM + 16384 + (LIN ? 0 : kM);
     // output staging (epilogue): dX, dV tiles
     static constexpr uint32_t Sx = U, Sv = U + 16384;
 };
@@ -128,12 +137,13 @@ __device__ __forceinline__ void untensor32(const uint32_t (&x)[32], const float 
 
 // Score GEMM  own rows x 64 other rows over the split half sketches:
 //   hi.hi + lo.hi + hi.lo, the [hi | lo] columns of both operands addressed in place.
-template <int R>
+// (one tile, r = 64: the rows are the half sketch, hi.hi alone)
+template <int R, bool LIN>
 __device__ __forceinline__ void issue_scores(uint32_t d_tmem, uint32_t own, uint32_t oth) {
     constexpr uint32_t idesc = idesc_bf16(128, 64, false, false);
     constexpr int offA[3] = {0, R, 0}, offB[3] = {0, 0, R};
 #pragma unroll
-    for (int g = 0; g < 3; ++g) {
+    for (int g = 0; g < ((LIN && R == 64) ? 1 : 3); ++g) {
 #pragma unroll
         for (int kk = 0; kk < R / 16; ++kk) {
             const int ca = offA[g] + kk * 16, cb = offB[g] + kk * 16;
@@ -151,9 +161,10 @@ __device__ __forceinline__ void issue_scores(uint32_t d_tmem, uint32_t own, uint
 // LIN: the rows hold a given half sketch (tc_common.cuh, read_half_sketch); a template parameter, not
 // an argument: the key side sits at the register limit, and the flag as an argument cost it 4 %.
 template <int R, bool QSIDE, bool LOCAL, bool LIN>
-__global__ void __launch_bounds__(128, ((R <= 32 || (LOCAL && QSIDE)) ? 2 : 1))
+__global__ void __launch_bounds__(128, ((R <= 32 || QSIDE) ? 2 : 1))
 tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_constant__ CUtensorMap mapYown,
-                   const __grid_constant__ CUtensorMap mapXoth, const __grid_constant__ CUtensorMap mapYoth,
+                   const __grid_constant__ CUtensorMap mapXoth, const __grid_constant__ CUtensorMap mapXoth2,
+                   const __grid_constant__ CUtensorMap mapYoth,
                    const __grid_constant__ CUtensorMap mapS, const __grid_constant__ CUtensorMap mapDX,
                    const __grid_constant__ CUtensorMap mapDV, const __grid_constant__ CUtensorMap mapXownRaw,
                    const __grid_constant__ CUtensorMap mapDXraw, const uint8_t* __restrict__ gimg,
@@ -163,7 +174,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     pdl_sync();
     constexpr bool lin = LIN;
     using F = Feat<R>;
-    using L = BwdSmem<R, LOCAL, QSIDE>;
+    using L = BwdSmem<R, LOCAL, QSIDE, LIN>;
     constexpr int kStages = L::kSt;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
@@ -177,6 +188,17 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     const int blk = noncausal ? bh : bh * t + l;
     const int ntiles = b / 128;
     const bool has_state = noncausal || (QSIDE ? (l > 0) : (l < t - 1));
+
+    // the other side's rows of a tile of the block: score operand (raw rows with LOCAL), and values
+    auto load_m = [&](int tp, uint32_t dst) {
+        mbar_expect_tx(&bar_xoth, L::kM);
+        tma_load_4d(smem + dst, &mapXoth, 0, l * b + tp * 128, hi, bi, &bar_xoth);
+        if constexpr (L::NT == 2) tma_load_4d(smem + dst + 16384, &mapXoth2, 0, l * b + tp * 128, hi, bi, &bar_xoth);
+    };
+    auto load_y = [&](int tp) {
+        mbar_expect_tx(&bar_yoth, 16384);
+        tma_load_4d(smem + L::Yoth, &mapYoth, 0, l * b + tp * 128, hi, bi, &bar_yoth);
+    };
 
     if (tid == 0) {
         // the own tiles are what everything waits for: their requests go out before anything else
@@ -200,15 +222,8 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             }
         }
         // first other-side tile: at once where its memory is free from the start
-        const int orow_first = l * b + (QSIDE ? 0 : tau) * 128;
-        if (!noncausal && (!has_state || !L::kAlias || F::NC < kStages)) {
-            mbar_expect_tx(&bar_xoth, 16384);
-            tma_load_4d(smem + L::Xoth, &mapXoth, 0, orow_first, hi, bi, &bar_xoth);
-        }
-        if (!noncausal && (!has_state || !L::kAlias)) {
-            mbar_expect_tx(&bar_yoth, 16384);
-            tma_load_4d(smem + L::Yoth, &mapYoth, 0, orow_first, hi, bi, &bar_yoth);
-        }
+        if (!noncausal && (!has_state || !L::kAlias || L::cM < 0)) load_m(QSIDE ? 0 : tau, L::Moth);
+        if (!noncausal && (!has_state || !L::kAlias || L::cY < 0)) load_y(QSIDE ? 0 : tau);
     }
     if (warp == 0) { tmem_alloc(&tmem_slot, 256); tmem_relinquish(); }
     // Query rows work on the raw dO rows g_i (exact bf16 inputs) and apply 1/d_i in fp32 afterwards:
@@ -336,17 +351,11 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                 mbar_expect_tx(&bar_box[stage], kBoxBytes);
                 tma_load_3d(smem + L::Box + stage * kBoxStride, &mapS, 0, (C + kStages) * 64, blk, &bar_box[stage]);
                 tma_load_3d(smem + L::Box + stage * kBoxStride + 8192, &mapS, 64, (C + kStages) * 64, blk, &bar_box[stage]);
-            } else if (L::kAlias && !noncausal) {
+            }
+            if (L::kAlias && !noncausal) {
                 // the last chunks free the stages that the first other-side tile goes into
-                const int orow_first = l * b + (QSIDE ? 0 : tau) * 128;
-                if (F::NC >= kStages && C == F::NC - kStages) {
-                    mbar_expect_tx(&bar_xoth, 16384);
-                    tma_load_4d(smem + L::Xoth, &mapXoth, 0, orow_first, hi, bi, &bar_xoth);
-                }
-                if (C == (F::NC >= kStages ? F::NC - kStages + 1 : 0)) {
-                    mbar_expect_tx(&bar_yoth, 16384);
-                    tma_load_4d(smem + L::Yoth, &mapYoth, 0, orow_first, hi, bi, &bar_yoth);
-                }
+                if (C == L::cM) load_m(QSIDE ? 0 : tau, L::Moth);
+                if (C == L::cY) load_y(QSIDE ? 0 : tau);
             }
         };
         if constexpr (F::kCirc) {
@@ -466,7 +475,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     }
 
     // ---- phase C: same block, other-side tiles, 64 other rows at a time ----
-    if constexpr (!LOCAL) store_hilo_tiles<R>(smem + L::Mown, m, tid);
+    if constexpr (!LOCAL && !LIN) store_hilo_tiles<R>(smem + L::Mown, m, tid);
     const int tp_begin = QSIDE ? 0 : tau, tp_end = noncausal ? tp_begin : (QSIDE ? tau + 1 : ntiles);
     bool dm_started = false;
     uint32_t oth_uses = 0;
@@ -476,10 +485,9 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
 #pragma unroll 1
     for (int tp = tp_begin; tp < tp_end && ok; ++tp) {
         const int orow0 = l * b + tp * 128;
-        // LOCAL: the other side's raw tiles alternate between two buffers (the second one is the
-        // unused split-operand tile), so the next tile's rows can be requested a tile ahead
-        const uint32_t xo = (LOCAL && ((tp - tp_begin) & 1)) ? L::Moth : L::Xoth;
-        const uint32_t xo_next = (LOCAL && !((tp - tp_begin) & 1)) ? L::Moth : L::Xoth;
+        // one-tile operands alternate between two buffers, so the next tile's rows can be requested a tile ahead
+        const uint32_t xo = (L::kTwoM && ((tp - tp_begin) & 1)) ? L::Moth2 : L::Moth;
+        const uint32_t xo_next = (L::kTwoM && !((tp - tp_begin) & 1)) ? L::Moth2 : L::Moth;
         // (this tile's rows were requested ahead: by the prologue, by phase B's last chunks, or
         // by the previous tile as soon as its own copies had been consumed)
         // Every thread is past its wait for the previous tile's last MMAs before the next commit
@@ -496,23 +504,8 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             }
         }
         ok = mbar_wait(&bar_xoth, oth_uses & 1, status, kErrTma);
-        if constexpr (!LOCAL) {
-            if (tid == 0) {
-                tc_fence_after();
-                issue_sketch<R>(tm + cSk, smem + L::Xoth, smem + L::G);
-                umma_commit(&bar_mma);
-            }
-            ok = ok && mbar_wait(&bar_mma, mma_uses & 1, status, kErrMma);
-            ++mma_uses;
-            tc_fence_after();
-        }
         ok = ok && mbar_wait(&bar_yoth, oth_uses & 1, status, kErrTma);
         ++oth_uses;
-        if constexpr (!LOCAL) {
-            float mo[R];
-            read_half_sketch<R>(lane_tm + cSk, mo, 1.f, lin != 0);
-            store_hilo_tiles<R>(smem + L::Moth, mo, tid);
-        }
         const bool diag = (tp == tau);
 #pragma unroll 1
         for (int hh = 0; hh < 2; ++hh) {
@@ -521,14 +514,9 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             __syncthreads();
             if (tid == 0) {
                 tc_fence_after();
-                // The X tile has been consumed, and every thread is past its wait for it (a
-                // barrier must not complete twice before its slowest waiter has looked): next
-                // tile's rows.
-                // (LOCAL: the raw rows stay operands to the tile's end; the next ones go to the other buffer)
-                if (hh == 0 && tp + 1 < tp_end) {
-                    mbar_expect_tx(&bar_xoth, 16384);
-                    tma_load_4d(smem + xo_next, &mapXoth, 0, orow0 + 128, hi, bi, &bar_xoth);
-                }
+                // Every thread is past its wait for this tile's rows (a barrier must not complete twice
+                // before its slowest waiter has looked): the next tile's, into the other buffer.
+                if (L::kTwoM && hh == 0 && tp + 1 < tp_end) load_m(tp + 1, xo_next);
                 constexpr uint32_t idesc = idesc_bf16(128, 64, false, false);
                 if constexpr (LOCAL) {
 #pragma unroll
@@ -536,7 +524,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                         umma_ss(tm + cS, desc_off(smem_desc(smem_u32(smem + L::Xown), 0, 1024, kSwz128), k * 32),
                                 desc_off(smem_desc(smem_u32(smem + xo) + hh * 8192, 0, 1024, kSwz128), k * 32), idesc, k > 0);
                 } else {
-                    issue_scores<R>(tm + cS, smem_u32(smem + L::Mown), smem_u32(smem + L::Moth) + hh * 8192);
+                    issue_scores<R, LIN>(tm + cS, smem_u32(smem + L::Mown), smem_u32(smem + xo) + hh * 8192);
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {         // dW without its 65th-column term
@@ -608,7 +596,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
 #pragma unroll
                     for (int k = 0; k < 4; ++k)       // dM_own += dS x M_other (its hi columns)
                         umma_ts(tm + cdM, tm + cS + k * 8,
-                                desc_off(smem_desc(smem_u32(smem + L::Moth) + hh * 8192, 0, 1024, kSwz128), k * 2048), idesc_dm,
+                                desc_off(smem_desc(smem_u32(smem + xo) + hh * 8192, 0, 1024, kSwz128), k * 2048), idesc_dm,
                                 (dm_started || k > 0) ? 1u : 0u);
                 }
                 if constexpr (!QSIDE) {
@@ -626,10 +614,22 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             ++mma_uses;
             tc_fence_after();
         }
-        if (tid == 0 && tp + 1 < tp_end) {        // every MMA that read the Y tile has completed
-            mbar_expect_tx(&bar_yoth, 16384);
-            tma_load_4d(smem + L::Yoth, &mapYoth, 0, orow0 + 128, hi, bi, &bar_yoth);
+        if (tid == 0 && tp + 1 < tp_end) {        // every MMA that read this tile's rows has completed
+            load_y(tp + 1);
+            if constexpr (!L::kTwoM) load_m(tp + 1, L::Moth);
         }
+    }
+    if constexpr (L::kFold && !LIN) {             // the own rows and the sketch matrices' image again
+        fence_proxy_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        if (tid == 0) {
+            mbar_expect_tx(&bar_own, 16384 + GImage<R>::bytes);
+            tma_load_4d(smem + L::Xown, &mapXown, 0, row0, hi, bi, &bar_own);
+            bulk_load(smem + L::G, gimg + (size_t)g * GImage<R>::bytes, GImage<R>::bytes, &bar_own);
+        }
+        ok = ok && mbar_wait(&bar_own, 1, status, kErrTma);
+        tc_fence_after();
     }
 
     // ---- phase D: through the sketch, dX = ((dM*A2) G1^T + (dM*A1) G2^T) / sqrt(R) ----
@@ -810,11 +810,16 @@ cudaError_t bwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
             !tc_map_rows(&mdKraw, d.rawdK, d.B, d.H, d.n, bs, hs, 64))
             return cudaErrorInvalidValue;
     }
+    // the other sides' score operands: the state kernels' arrays, or (given half sketches, exact weights) the rows
+    bf16* Sk = tc_hilo_rows(d) ? reinterpret_cast<bf16*>(ws + w.Sk) : nullptr;
+    bf16* Sq = Sk != nullptr ? reinterpret_cast<bf16*>(ws + w.Sq) : nullptr;
+    CUtensorMap mKs[2] = {mK, mK}, mQs[2] = {mQ, mQ};
+    if (Sk != nullptr && (!tc_map_hilo(d, Sk, mKs) || !tc_map_hilo(d, Sq, mQs))) return cudaErrorInvalidValue;
     uint8_t* gimg = reinterpret_cast<uint8_t*>(ws + w.gimg);
     // kept states: the image and the centres are in the workspace too
     if (!d.keep_states) PSK_TRY(tc_prologue(d, G1, G2, gimg, V, cmean, status, s, launches));
     // prefix states of centred values; forward rows again in fp32 -> y65, e65h; suffix states
-    if (!d.keep_states) PSK_TRY(tc_states(d, mK, mV, gimg, nullptr, nullptr, cmean, 1, Z, false, tot, status, s, launches));
+    if (!d.keep_states) PSK_TRY(tc_states(d, mK, mV, gimg, nullptr, nullptr, cmean, 1, Z, Sk, false, tot, status, s, launches));
     if (d.keep_states) {
         const int rows = d.BH() * d.n;
         prof_begin("tc_bwd_prep_kernel", s);
@@ -825,27 +830,27 @@ cudaError_t bwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
         ++*launches;
         PSK_TRY(cudaGetLastError());
     } else {
-        PSK_TRY(tc_recompute(d, mQ, mQraw, linloc ? mKraw : mK, mV, mZ, gimg, cmean, denom, (const bf16*)dO, y65, e65h, status, s, launches));
+        PSK_TRY(tc_recompute(d, mQ, Sk != nullptr ? mKs[1] : mQraw, linloc ? mKraw : mKs[0], mV, mZ, gimg, cmean, denom, (const bf16*)dO, y65, e65h, status, s, launches));
     }
     const dim3 grid(d.b / 128, d.t, d.BH());
     auto rows = [&](auto local_c, auto lin_c) -> cudaError_t {
         constexpr bool LOCAL = decltype(local_c)::value;
         constexpr bool LIN = decltype(lin_c)::value;
-        constexpr size_t smem = BwdSmem<R, LOCAL, true>::total + 1024, smem_k = BwdSmem<R, LOCAL, false>::total + 1024;
+        constexpr size_t smem = BwdSmem<R, LOCAL, true, LIN>::total + 1024, smem_k = BwdSmem<R, LOCAL, false, LIN>::total + 1024;
         PSK_TRY((set_smem(tc_bwd_rows_kernel<R, true, LOCAL, LIN>, smem)));
         PSK_TRY((set_smem(tc_bwd_rows_kernel<R, false, LOCAL, LIN>, smem_k)));
         // query side first: it needs only the prefix states, and the row scalars just written are
         // still in L2; the suffix states (5 GB through L2) come after it
         prof_begin("tc_bwd_q_kernel", s);
-        launch_pdl(tc_bwd_rows_kernel<R, true, LOCAL, LIN>, grid, 128, smem, s, mQ, mG, (LOCAL && LIN) ? mKraw : mK, mV, mZ, mdQ, mdQ, mQraw, mdQraw, gimg, d.g_heads, d.H, d.n,
+        launch_pdl(tc_bwd_rows_kernel<R, true, LOCAL, LIN>, grid, 128, smem, s, mQ, mG, (LOCAL && LIN) ? mKraw : mKs[0], mKs[1], mV, mZ, mdQ, mdQ, mQraw, mdQraw, gimg, d.g_heads, d.H, d.n,
                                                                    d.b, d.t, y65, e65h, denom, d.noncausal ? 1 : 0, status);
         prof_end(s);
         ++*launches;
         PSK_TRY(cudaGetLastError());
         // suffix states: phi(q_i) / d_i against [dO_i | y65_i]
-        PSK_TRY(tc_states(d, mQ, mG, gimg, y65, denom, cmean, 2, Rs, true, tot, status, s, launches));
+        PSK_TRY(tc_states(d, mQ, mG, gimg, y65, denom, cmean, 2, Rs, Sq, true, tot, status, s, launches));
         prof_begin("tc_bwd_k_kernel", s);
-        launch_pdl(tc_bwd_rows_kernel<R, false, LOCAL, LIN>, grid, 128, smem_k, s, mK, mV, (LOCAL && LIN) ? mQraw : mQ, mG, mR, mdK, mdV, mKraw, mdKraw, gimg, d.g_heads, d.H, d.n,
+        launch_pdl(tc_bwd_rows_kernel<R, false, LOCAL, LIN>, grid, 128, smem_k, s, mK, mV, (LOCAL && LIN) ? mQraw : mQs[0], mQs[1], mG, mR, mdK, mdV, mKraw, mdKraw, gimg, d.g_heads, d.H, d.n,
                                                                     d.b, d.t, y65, e65h, denom, d.noncausal ? 1 : 0, status);
         prof_end(s);
         ++*launches;

@@ -35,9 +35,17 @@ constexpr int kModeFirst = 2;          // run 0: both; the other runs: the total
 //   Y: [V] or [dO];  y65: last column (nullptr = all ones);  fscale: per-token d_i, the
 //   features of token i are divided by it (nullptr = not) -- phi(q_i)^T [dO_i | y65_i] / d_i is the
 //   suffix state's phi(q_i)^T E_i without E ever being formed
+//   H, H2: where the tokens' half sketches go as [hi | lo] score operands for the row kernels, which would
+//   otherwise sketch every other-side tile again, once per row tile that meets it.  (Rows of 48 heads x 16384,
+//   r = 64: forward 1050 -> 554 us, query side 1702 -> 1288, key side 2327 -> 2112; of 384 heads x 32768,
+//   r = 32: 4409 -> 3916, 5031 -> 4776, 6249 -> 5867; the walk itself pays 5 to 20 % for it.)
+// What bounds a walk of r = 32: the generators' instructions and their fetch (20 % of the warps wait for an
+// instruction), and at short blocks the store warpgroup, one body for all tiles with a bulk copy out (144 heads x
+// 8192, b = 256: 318 us unrolled and with copies by the lanes, now 234).
 // grid (BH).  Warp roles:
 //   NWG generator warpgroups  thread = token: read the half sketches, write their feature tiles
-//                             (dealt round-robin) as MN-major A operands into shared memory;
+//                             (dealt round-robin) as MN-major A operands into shared memory; the last one also
+//                             puts the half sketches where their rows were;
 //   1 store warpgroup         thread = feature row: at block boundaries reads the accumulators,
 //                             centres, rounds and stores them;
 //   1 feeder warp             one thread issues every TMA load, sketch GEMM and state GEMM.
@@ -45,14 +53,23 @@ constexpr int kModeFirst = 2;          // run 0: both; the other runs: the total
 // ---------------------------------------------------------------------------
 template <int R, int NWG>
 struct StateSmem {
-    static constexpr uint32_t X = 0;                     // 2 x 16 KB: rows to sketch
-    static constexpr uint32_t Y = 32768;                 // 2 x (16 KB values + 16 KB last-column chunk)
+    static constexpr uint32_t kG = 2 * R * 128 < 1024 ? 1024 : 2 * R * 128;
+    // X: 16 KB slots for the rows to sketch, through which their half sketches leave.  A third one where there is room:
+    // with two, a tile's rows can be requested only when the half sketches two tiles earlier have left.
+    static constexpr int kXSlots = 3 * 16384 + 65536 + kG + NWG * 32768 + 128 * 160 + (R == 64 ? 16384 : 0) + 3072 <= 232448 ? 3 : 2;
+    static_assert(R < 64 || kXSlots == 2, "the second half's buffer is single");
+    static constexpr uint32_t X = 0;
+    static constexpr uint32_t Y = kXSlots * 16384;       // 2 x (16 KB values + 16 KB last-column chunk)
     static constexpr uint32_t kYSlot = 32768;
     static constexpr uint32_t G = Y + 2 * kYSlot;
-    static constexpr uint32_t A0 = G + (2 * R * 128 < 1024 ? 1024 : 2 * R * 128);
+    static constexpr uint32_t A0 = G + kG;
     static constexpr uint32_t St = A0 + NWG * 32768;     // one state tile on its way out: 128 rows x 160 B
     static constexpr bool kStaged = St + 128 * 160 + 2048 <= 232448;     // where it fits (r <= 32)
-    static constexpr uint32_t total = St + (kStaged ? 128 * 160 : 0);
+    // r = 64: the second 64 columns of a tile's [hi | lo] half sketches on their way out (the first, and all of
+    // them for r <= 32, leave through the tile's own X buffer)
+    static constexpr uint32_t Hl = St + (kStaged ? 128 * 160 : 0);
+    static constexpr uint32_t total = Hl + (R == 64 ? 16384 : 0);
+    static_assert(total + 2048 <= 232448, "shared memory");
 };
 
 // Barrier among the 128 threads of a warpgroup.  The generator and store roles never leave a
@@ -64,6 +81,32 @@ __device__ __forceinline__ void wg_barrier(int wg) {
 }
 
 constexpr int kErrState = 3;
+
+// Barriers and centres of a CTA: one object for all the shares that a kernel's code covers.
+template <int TN, int NWG>
+struct StateShared {
+    uint64_t fullx[3], fully[2], yfree[2], ext[2], sk, mread, drain[2], hl[2], hlfree;
+    uint64_t aready[NWG], afree[NWG], accfull[TN], accread[TN];
+    uint32_t tmem_slot;
+    alignas(16) float cm[64];
+};
+
+// m as [hi | lo] columns: one tile, or (r = 64) two tiles of 64
+template <int R>
+__device__ __forceinline__ void store_hl_rows(uint8_t* t0, uint8_t* t1, const float (&m)[R], int row) {
+#pragma unroll
+    for (int ch = 0; ch < R / 8; ++ch) {
+        uint32_t h[4], l[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float a = m[8 * ch + 2 * i], b = m[8 * ch + 2 * i + 1];
+            h[i] = pack_bf16(a, b);
+            l[i] = pack_bf16(a - __uint_as_float(h[i] << 16), b - __uint_as_float(h[i] & 0xffff0000u));
+        }
+        *reinterpret_cast<uint4*>(t0 + swz128_offset(row, ch)) = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4*>((R == 64 ? t1 : t0) + swz128_offset(row, R == 64 ? ch : R / 8 + ch)) = make_uint4(l[0], l[1], l[2], l[3]);
+    }
+}
 
 // acc[0..80) of this thread's lane = tot[row * 80 + ...], half a row's loads in flight at a time
 static __device__ __noinline__ void state_init_acc(const float* __restrict__ tot, size_t row, uint32_t acc_tmem) {
@@ -85,9 +128,9 @@ static __device__ __noinline__ void state_init_acc(const float* __restrict__ tot
 
 // SEG = false is the plain walk of a whole head by one CTA (nseg = 1, prefix mode, no start value):
 // its run bookkeeping folds away at compile time.
-template <int R, int T0, int TN, int NWG, bool SEG>
+template <int R, int T0, int TN, int NWG, bool SEG, typename SH>
 __device__ __forceinline__ void
-state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
+state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUtensorMap& mapH, const CUtensorMap& mapH2, int want_hl,
            const uint8_t* __restrict__ gimg, int g_heads, int H, int n, int b, int t,
            const float* __restrict__ y65, const float* __restrict__ fscale, const float* __restrict__ cmean,
            int center_mode, int reverse, int nseg_arg, int mode_arg, int run0, int units, float* __restrict__ tot,
@@ -96,10 +139,6 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
     using L = StateSmem<R, NWG>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
-    __shared__ uint64_t bar_fullx[2], bar_fully[2], bar_yfree[2], bar_ext[2], bar_sk, bar_mread, bar_drain[2];
-    __shared__ uint64_t bar_aready[NWG], bar_afree[NWG], bar_accfull[TN], bar_accread[TN];
-    __shared__ uint32_t tmem_slot;
-    __shared__ __align__(16) float cm[64];
     const int tid = threadIdx.x, wg = tid / 128, wt = tid % 128, warp = tid / 32;
     const int bh = blockIdx.x;
     const int seg = SEG ? run0 + (int)blockIdx.y : 0, nseg = SEG ? nseg_arg : 1;
@@ -113,18 +152,23 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
     const int upt = NJ / units;                          // tiles per unit
     const int j0r = SEG ? u0 * upt : 0, NJs = SEG ? (u1 - u0) * upt : NJ;
     const int p0r = SEG ? u0 : 0, ts = SEG ? u1 - u0 : t;
+    // [hi | lo] half sketches: written by the CTA with a head's last, smallest share of the tiles, in the pass that visits
+    // a run to write its states
+    const bool hl = T0 + TN == F::NT && want_hl != 0 && mode != kModeTotal;
     // a later run of a prefix pass starts from the sum of the earlier runs' totals
     const bool init = SEG && mode == kModePrefix && seg > 0;
     constexpr int kThreads = 128 * (NWG + 1) + 64;
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
-            mbar_init(&bar_fullx[i], 1); mbar_init(&bar_fully[i], 1); mbar_init(&bar_yfree[i], 1);
-            mbar_init(&bar_ext[i], 1);
+            mbar_init(&sh.fully[i], 1); mbar_init(&sh.yfree[i], 1);
+            mbar_init(&sh.ext[i], 1);
         }
-        mbar_init(&bar_sk, 1); mbar_init(&bar_mread, NWG); mbar_init(&bar_drain[0], 1); mbar_init(&bar_drain[1], 1);
-        for (int i = 0; i < NWG; ++i) { mbar_init(&bar_aready[i], 1); mbar_init(&bar_afree[i], 1); }
-        for (int i = 0; i < TN; ++i) { mbar_init(&bar_accread[i], 4); mbar_init(&bar_accfull[i], 1); }
+        for (int i = 0; i < L::kXSlots; ++i) mbar_init(&sh.fullx[i], 1);
+        mbar_init(&sh.hl[0], 1); mbar_init(&sh.hl[1], 1); mbar_init(&sh.hlfree, 1);
+        mbar_init(&sh.sk, 1); mbar_init(&sh.mread, NWG); mbar_init(&sh.drain[0], 1); mbar_init(&sh.drain[1], 1);
+        for (int i = 0; i < NWG; ++i) { mbar_init(&sh.aready[i], 1); mbar_init(&sh.afree[i], 1); }
+        for (int i = 0; i < TN; ++i) { mbar_init(&sh.accread[i], 4); mbar_init(&sh.accfull[i], 1); }
         cta_giveup_init();
         mbar_fence_init();
         tma_prefetch_desc(&mapX); tma_prefetch_desc(&mapY);
@@ -135,8 +179,8 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
         reinterpret_cast<uint4*>(smem + L::Y + s * L::kYSlot + 16384)[i] = make_uint4(0, 0, 0, 0);
     }
     pdl_sync();            // (before the allocation: a waiting CTA must not hold tensor memory)
-    if (warp == 0) { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
-    if (tid < 64) cm[tid] = cmean != nullptr ? cmean[(size_t)bh * 64 + tid] : 0.f;
+    if (warp == 0) { tmem_alloc(&sh.tmem_slot, 512); tmem_relinquish(); }
+    if (tid < 64) sh.cm[tid] = cmean != nullptr ? cmean[(size_t)bh * 64 + tid] : 0.f;
     __syncthreads();
     if (y65 == nullptr && tid < 128) {
         *reinterpret_cast<bf16*>(smem + L::Y + 16384 + swz128_offset(tid, 0)) = __float2bfloat16_rn(1.f);
@@ -146,7 +190,7 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tm = tmem_slot;
+    const uint32_t tm = sh.tmem_slot;
     constexpr uint32_t kAcc = 2 * R;                      // accumulators start after the sketch columns
     // token tile visited at step j of this run (runs and tiles go backwards for suffix sums)
     auto tile_of = [&](int j) { const int gj = j0r + j; return reverse ? (NJ - 1 - gj) : gj; };
@@ -159,40 +203,58 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
         // hundred cycles, during which the tensor pipe would idle).
         if (tid == 128 * (NWG + 1)) {
             bool ok = true;
+            constexpr int NX = L::kXSlots;
             auto load_x = [&](int j) {
                 // the first tile's barrier also covers the sketch matrices' image
-                mbar_expect_tx(&bar_fullx[j & 1], 16384 + (j == 0 ? GImage<R>::bytes : 0u));
-                if (j == 0) bulk_load(smem + L::G, gimg + (size_t)g * GImage<R>::bytes, GImage<R>::bytes, &bar_fullx[0]);
-                tma_load_4d(smem + L::X + (j & 1) * 16384, &mapX, 0, tile_of(j) * 128, hi, bi, &bar_fullx[j & 1]);
+                mbar_expect_tx(&sh.fullx[j % NX], 16384 + (j == 0 ? GImage<R>::bytes : 0u));
+                if (j == 0) bulk_load(smem + L::G, gimg + (size_t)g * GImage<R>::bytes, GImage<R>::bytes, &sh.fullx[0]);
+                tma_load_4d(smem + L::X + (j % NX) * 16384, &mapX, 0, tile_of(j) * 128, hi, bi, &sh.fullx[j % NX]);
             };
             auto load_y = [&](int j) {
-                mbar_expect_tx(&bar_fully[j & 1], 16384);
-                tma_load_4d(smem + L::Y + (j & 1) * L::kYSlot, &mapY, 0, tile_of(j) * 128, hi, bi, &bar_fully[j & 1]);
+                mbar_expect_tx(&sh.fully[j & 1], 16384);
+                tma_load_4d(smem + L::Y + (j & 1) * L::kYSlot, &mapY, 0, tile_of(j) * 128, hi, bi, &sh.fully[j & 1]);
+            };
+            // the tile's half sketches as [hi | lo] rows, once the generators have put them over its X rows
+            auto store_hl = [&](int j) {
+                mbar_wait(&sh.hl[j & 1], (j >> 1) & 1, status, kErrState);
+                tma_store_4d(&mapH, smem + L::X + (j % NX) * 16384, 0, tile_of(j) * 128, hi, bi);
+                if constexpr (R == 64) tma_store_4d(&mapH2, smem + L::Hl, 0, tile_of(j) * 128, hi, bi);
+                bulk_commit();
             };
             load_x(0);
             if (NJs > 1) load_x(1);
             load_y(0);
-            ok = mbar_wait(&bar_fullx[0], 0, status, kErrTma);
+            ok = mbar_wait(&sh.fullx[0], 0, status, kErrTma);
             tc_fence_after();
             issue_sketch<R>(tm, smem + L::X, smem + L::G);
-            umma_commit(&bar_sk);
+            umma_commit(&sh.sk);
             for (int j = 0; j + 1 < NJs && ok; ++j) {
                 // sketch of the next token tile, as soon as this tile's half sketches are read out
-                ok = mbar_wait(&bar_mread, j & 1, status, kErrState);
-                ok = ok && mbar_wait(&bar_fullx[(j + 1) & 1], ((j + 1) >> 1) & 1, status, kErrTma);
+                ok = mbar_wait(&sh.mread, j & 1, status, kErrState);
+                ok = ok && mbar_wait(&sh.fullx[(j + 1) % NX], ((j + 1) / NX) & 1, status, kErrTma);
                 tc_fence_after();
-                issue_sketch<R>(tm, smem + L::X + ((j + 1) & 1) * 16384, smem + L::G);
-                umma_commit(&bar_sk);
-                if (j + 2 < NJs) load_x(j + 2);           // its slot: sketch j has completed (it was read)
+                issue_sketch<R>(tm, smem + L::X + ((j + 1) % NX) * 16384, smem + L::G);
+                umma_commit(&sh.sk);
+                // rows of tile j + 2.  Two slots: sketch j has completed (it was read), but its half sketches leave first;
+                // three: those of tile j - 1 have left
+                if (hl && NX == 3) bulk_wait_read();
+                if ((!hl || NX == 3) && j + 2 < NJs) load_x(j + 2);
                 // values of the next token tile: their slot held tile j-1
-                if (j >= 1) ok = ok && mbar_wait(&bar_yfree[(j + 1) & 1], ((j - 1) >> 1) & 1, status, kErrState);
+                if (j >= 1) ok = ok && mbar_wait(&sh.yfree[(j + 1) & 1], ((j - 1) >> 1) & 1, status, kErrState);
                 load_y(j + 1);
+                if (hl) store_hl(j);
+                if (hl && NX == 2) {
+                    bulk_wait_read();
+                    if constexpr (R == 64) mbar_arrive(&sh.hlfree);
+                    if (j + 2 < NJs) load_x(j + 2);
+                }
             }
+            if (hl) { store_hl(NJs - 1); bulk_wait_read(); }
             // drain: every sketch GEMM has completed before tensor memory is released.  (A barrier
-            // of its own: completing bar_sk once more, right behind the last sketch, could flip it
+            // of its own: completing sh.sk once more, right behind the last sketch, could flip it
             // twice before a generator thread has looked.)
-            umma_commit(&bar_drain[0]);
-            mbar_wait(&bar_drain[0], 0, status, kErrMma);
+            umma_commit(&sh.drain[0]);
+            mbar_wait(&sh.drain[0], 0, status, kErrMma);
         } else if (tid == 128 * (NWG + 1) + 32) {
             constexpr uint32_t idesc_state = idesc_bf16(128, 80, true, true);
             bool ok = true;
@@ -203,10 +265,10 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
 #pragma unroll
             for (int i = 0; i < NWG; ++i) ad[i] = smem_desc(smem_u32(smem + L::A0 + i * 32768), 16384, 1024, kSwz128);
             const uint64_t yd0 = smem_desc(smem_u32(smem + L::Y), 16384, 1024, kSwz128);
-            const int ibase = init ? 0 : 1;               // completions of bar_accread before block 1's
+            const int ibase = init ? 0 : 1;               // completions of sh.accread before block 1's
             for (int j = 0; j < NJs && ok; ++j) {
-                ok = mbar_spin(&bar_fully[j & 1], (j >> 1) & 1, status, kErrTma);
-                if (y65 != nullptr) ok = ok && mbar_spin(&bar_ext[j & 1], (j >> 1) & 1, status, kErrState);
+                ok = mbar_spin(&sh.fully[j & 1], (j >> 1) & 1, status, kErrTma);
+                if (y65 != nullptr) ok = ok && mbar_spin(&sh.ext[j & 1], (j >> 1) & 1, status, kErrState);
                 // block boundary: the store warpgroup has taken (or, for a start from earlier runs,
                 // written) the accumulators' values before anything is added to them
                 const bool boundary = mode != kModeTotal && (j % tpb == 0) && (j > 0 || init);
@@ -217,38 +279,37 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
                     constexpr int I = decltype(ic)::value;
                     constexpr int w = I % NWG;
                     // the store warpgroup has taken this accumulator's values for the boundary
-                    if (boundary) ok = ok && mbar_spin(&bar_accread[I], ((j / tpb) - ibase) & 1, status, kErrState);
-                    ok = ok && mbar_spin(&bar_aready[w], a_cnt[w] & 1, status, kErrState);
+                    if (boundary) ok = ok && mbar_spin(&sh.accread[I], ((j / tpb) - ibase) & 1, status, kErrState);
+                    ok = ok && mbar_spin(&sh.aready[w], a_cnt[w] & 1, status, kErrState);
                     ++a_cnt[w];
                     tc_fence_after();
 #pragma unroll
                     for (int k = 0; k < 8; ++k)
                         umma_ss(tm + kAcc + 80 * I, desc_off(ad[w], k * 2048), desc_off(yd, k * 2048), idesc_state, k > 0 ? 1u : acc0);
-                    umma_commit(&bar_afree[w]);
+                    umma_commit(&sh.afree[w]);
                     // last token tile of a block: this accumulator is complete, and the store
                     // warpgroup may take it while the remaining tiles are still being issued
-                    if (block_end) umma_commit(&bar_accfull[I]);
+                    if (block_end) umma_commit(&sh.accfull[I]);
                 });
-                umma_commit(&bar_yfree[j & 1]);
+                umma_commit(&sh.yfree[j & 1]);
             }
             // drain: every state GEMM has completed before tensor memory is released
-            umma_commit(&bar_drain[1]);
-            mbar_wait(&bar_drain[1], 0, status, kErrMma);
+            umma_commit(&sh.drain[1]);
+            mbar_wait(&sh.drain[1], 0, status, kErrMma);
         }
     } else if (wg == NWG) {
         // ============================ store warpgroup ============================
         // Tiles leave through shared memory: a warp's 32 rows of 160 B are one contiguous 5 KB
-        // piece of the state array, which the warp writes out in ten 512-byte rows of lanes.
-        // (Rows stored by their threads directly would be 10 scattered 16-byte stores each: the L1
-        // data path, which the MMA operands and the generators' tiles also go through, is this
-        // kernel's busiest unit.)
+        // piece of the state array, which goes out as one bulk copy.  (Rows stored by their threads directly would be
+        // 10 scattered 16-byte stores each: the L1 data path, which the MMA operands and the generators' tiles also
+        // go through, is this kernel's busiest unit.)  One body for all tiles: the kernel is short of instruction cache.
         const uint32_t lane_tm = tm + ((uint32_t)((warp % 4) * 32) << 16);
         uint8_t* stage = smem + L::St;
         // totals: the raw fp32 accumulators at the end of the run
         auto dump_totals = [&](uint32_t parity) {
             static_for<0, TN>([&](auto ic) {
                 constexpr int I = decltype(ic)::value;
-                mbar_wait(&bar_accfull[I], parity, status, kErrMma);
+                mbar_wait(&sh.accfull[I], parity, status, kErrMma);
                 tc_fence_after();
                 float4* out = reinterpret_cast<float4*>(tot + ((((size_t)bh * nseg + seg) * F::NT + (T0 + I)) * 128 + wt) * 80);
 #pragma unroll
@@ -274,77 +335,78 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
         for (int p = 0; p < ts && mode != kModeTotal; ++p) {
             const int pg = p0r + p;
             const int l = reverse ? (t - 1 - pg) : pg;
-            static_for<0, TN>([&](auto ic) {
-                constexpr int I = decltype(ic)::value;
+#pragma unroll 1
+            for (int I = 0; I < TN; ++I) {
                 if (p > 0) {
-                    mbar_wait(&bar_accfull[I], (p - 1) & 1, status, kErrMma);
+                    mbar_wait(&sh.accfull[I], (p - 1) & 1, status, kErrMma);
                     tc_fence_after();
                 }
                 const bool live = p > 0 || init;          // the accumulator holds values (else: zeros)
-                // 16 accumulator columns (zeros before the first block of a head)
-                auto fetch = [&](int c0, uint32_t (&v)[16]) {
-                    if (live) {
-                        tmem_ld16(lane_tm + kAcc + 80 * I + c0, v);
-                        tmem_ld_wait();
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < 16; ++q) v[q] = 0u;
-                    }
-                };
-                // centred values, in fp32, without touching the operands (the mode only selects
-                // coefficients):  mode 1: sum phi (y - c)^T = H[:, :64] - H[:, 64] c^T
-                //                 mode 2: last column H[:, 64] - H[:, :64] c
-                float last, corr = 0.f;
-                {
-                    uint32_t v[16];
-                    fetch(64, v);
-                    last = __uint_as_float(v[0]);
-                }
-                const float k1 = center_mode == 1 ? -last : 0.f, k2 = center_mode == 2 ? 1.f : 0.f;
-                // the row's pair weight (tc_features.cuh) goes into the stored state; 0 on padding rows
-                const float wgt = F::weight((T0 + I) * 128 + wt);
+                const uint32_t acc = lane_tm + kAcc + 80 * I;
                 // this thread's feature row: 80 bf16 = ten 16-byte pieces of the staging tile
-                if constexpr (L::kStaged) __syncwarp();       // the previous tile has been read back
+                if constexpr (L::kStaged) {               // the previous tile has left it
+                    if (wt % 32 == 0) bulk_wait_read();
+                    __syncwarp();
+                }
                 uint4* const grow = reinterpret_cast<uint4*>(S + (((size_t)bh * t + l) * F::FP + (size_t)(T0 + I) * 128 + wt) * 80);
                 uint4* dst = L::kStaged ? reinterpret_cast<uint4*>(stage + wt * 160) : grow;
+                if (live) {
+                    // centred values, in fp32, without touching the operands (the mode only selects
+                    // coefficients):  mode 1: sum phi (y - c)^T = H[:, :64] - H[:, 64] c^T
+                    //                 mode 2: last column H[:, 64] - H[:, :64] c
+                    uint32_t v[2][16], last_raw;
+                    tmem_ld1(acc + 64, last_raw);
+                    tmem_ld16(acc, v[0]);
+                    tmem_ld_wait();
+                    const float last = __uint_as_float(last_raw);
+                    float corr = 0.f;
+                    const float k1 = center_mode == 1 ? -last : 0.f, k2 = center_mode == 2 ? 1.f : 0.f;
+                    // the row's pair weight (tc_features.cuh) goes into the stored state; 0 on padding rows
+                    const float wgt = F::weight((T0 + I) * 128 + wt);
 #pragma unroll
-                for (int c0 = 0; c0 < 64; c0 += 16) {
-                    uint32_t v[16];
-                    fetch(c0, v);
-                    if (c0 == 48 && live) {      // last read of this accumulator: hand it (back) to the MMAs
-                        tc_fence_before();
-                        if (wt % 32 == 0) mbar_arrive(&bar_accread[I]);
-                    }
-                    uint32_t pk[8];
-                    float cv[16];
+                    for (int h = 0; h < 4; ++h) {             // 16 columns, the next ones on their way
+                        if (h < 3) tmem_ld16(acc + 16 * (h + 1), v[(h + 1) & 1]);
+                        uint32_t pk[8];
 #pragma unroll
-                    for (int q = 0; q < 16; q += 4) {
-                        const float4 c4 = *reinterpret_cast<const float4*>(&cm[c0 + q]);
-                        cv[q] = c4.x; cv[q + 1] = c4.y; cv[q + 2] = c4.z; cv[q + 3] = c4.w;
-                    }
+                        for (int q = 0; q < 16; q += 4) {
+                            const float4 c4 = *reinterpret_cast<const float4*>(&sh.cm[16 * h + q]);
+                            const float cv[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
-                    for (int q = 0; q < 16; q += 2) {
-                        const float x0 = fmaf(k1, cv[q], __uint_as_float(v[q]));
-                        const float x1 = fmaf(k1, cv[q + 1], __uint_as_float(v[q + 1]));
-                        corr = fmaf(k2 * cv[q], x0, corr);
-                        corr = fmaf(k2 * cv[q + 1], x1, corr);
-                        pk[q / 2] = pack_bf16(x0 * wgt, x1 * wgt);
+                            for (int i = 0; i < 4; i += 2) {
+                                const float x0 = fmaf(k1, cv[i], __uint_as_float(v[h & 1][q + i]));
+                                const float x1 = fmaf(k1, cv[i + 1], __uint_as_float(v[h & 1][q + i + 1]));
+                                corr = fmaf(k2 * cv[i], x0, corr);
+                                corr = fmaf(k2 * cv[i + 1], x1, corr);
+                                pk[(q + i) / 2] = pack_bf16(x0 * wgt, x1 * wgt);
+                            }
+                        }
+                        dst[2 * h] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                        dst[2 * h + 1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                        if (h < 3) {
+                            tmem_ld_wait16(v[(h + 1) & 1]);
+                            if (h == 2) {                     // last read of this accumulator: hand it (back) to the MMAs
+                                tc_fence_before();
+                                if (wt % 32 == 0) mbar_arrive(&sh.accread[I]);
+                            }
+                        }
                     }
-                    dst[c0 / 8] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                    dst[c0 / 8 + 1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                    dst[8] = make_uint4(pack_bf16((last - corr) * wgt, 0.f), 0, 0, 0);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 9; ++q) dst[q] = make_uint4(0, 0, 0, 0);
                 }
-                dst[8] = make_uint4(pack_bf16((last - corr) * wgt, 0.f), 0, 0, 0);
                 dst[9] = make_uint4(0, 0, 0, 0);
                 if constexpr (L::kStaged) {
+                    fence_proxy_async_smem();
                     __syncwarp();
-                    const int w32 = wt & ~31, lane = wt & 31;
-                    const uint4* src = reinterpret_cast<const uint4*>(stage + w32 * 160);
-                    uint4* out = reinterpret_cast<uint4*>(S + (((size_t)bh * t + l) * F::FP + (size_t)(T0 + I) * 128 + w32) * 80);
-#pragma unroll
-                    for (int i = 0; i < 10; ++i) out[i * 32 + lane] = src[i * 32 + lane];
+                    if (wt % 32 == 0) {
+                        bulk_store(grow, dst, 32 * 160);
+                        bulk_commit();
+                    }
                 }
-            });
+            }
         }
+        if constexpr (L::kStaged) if (wt % 32 == 0) bulk_wait_read();
         if (SEG && mode == kModeFirst) dump_totals((ts - 1) & 1);
     } else {
         // ============================= generators =============================
@@ -355,7 +417,7 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
         float y_next = (y65 != nullptr && wg == 0) ? y65[(size_t)bh * n + tile_of(0) * 128 + wt] : 0.f;
         float d_next = fscale != nullptr ? fscale[(size_t)bh * n + tile_of(0) * 128 + wt] : 1.f;
         for (int j = 0; j < NJs; ++j) {
-            mbar_wait(&bar_sk, j & 1, status, kErrMma);
+            mbar_wait(&sh.sk, j & 1, status, kErrMma);
             tc_fence_after();
             PackedM<R> pm;
             CircGen<R> gen;
@@ -364,30 +426,44 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
                 // features m_a m_b / d: both factors carry 1 / sqrt(d) (d requested a token tile ago)
                 const float sc = rsqrtf(d_next);
                 if (fscale != nullptr && j + 1 < NJs) d_next = fscale[(size_t)bh * n + tile_of(j + 1) * 128 + wt];
-                read_half_sketch<R>(lane_tm, m, sc, lin != 0);
+                // (the warpgroup with the fewest tiles also writes the half sketches out, over their dead X rows)
+                const bool out = hl && wg == NWG - 1;
+                read_half_sketch<R>(lane_tm, m, out ? 1.f : sc, lin != 0);
+                tc_fence_before();
+                wg_barrier(wg);
+                if (wt == 0) mbar_arrive(&sh.mread);
+                if (out) {
+                    // (r = 64: the second tile's single buffer has been stored)
+                    if (R == 64 && j > 0) mbar_wait(&sh.hlfree, (j - 1) & 1, status, kErrState);
+                    store_hl_rows<R>(smem + L::X + (j % L::kXSlots) * 16384, smem + L::Hl, m, wt);
+                    fence_proxy_async_smem();
+                    wg_barrier(wg);
+                    if (wt == 0) mbar_arrive(&sh.hl[j & 1]);
+                    if (fscale != nullptr) {
+#pragma unroll
+                        for (int c = 0; c < R; ++c) m[c] *= sc;
+                    }
+                }
                 if constexpr (F::kCirc) gen.init(m); else pack_half_sketch<R>(m, pm);
             }
-            tc_fence_before();
-            wg_barrier(wg);
-            if (wt == 0) mbar_arrive(&bar_mread);
             if (y65 != nullptr && wg == 0) {
                 // last-column chunk of this token tile; its slot is free once tile j-2's MMAs are done
-                if (j >= 2) mbar_wait(&bar_yfree[j & 1], ((j >> 1) - 1) & 1, status, kErrState);
+                if (j >= 2) mbar_wait(&sh.yfree[j & 1], ((j >> 1) - 1) & 1, status, kErrState);
                 const float y = y_next;
                 if (j + 1 < NJs) y_next = y65[(size_t)bh * n + tile_of(j + 1) * 128 + wt];
                 *reinterpret_cast<bf16*>(smem + L::Y + (j & 1) * L::kYSlot + 16384 + swz128_offset(wt, 0)) =
                     __float2bfloat16_rn(y);
                 fence_proxy_async_smem();
                 wg_barrier(0);
-                if (wt == 0) mbar_arrive(&bar_ext[j & 1]);
+                if (wt == 0) mbar_arrive(&sh.ext[j & 1]);
             }
             if constexpr (F::kCirc) {
                 // this warpgroup's tiles wg, wg + NWG, ...: the same loop body on a rotated copy of m
                 constexpr int kTileSteps = 128 / (2 * R);
-                for (int i = 0; i < T0 + wg; ++i) gen.template skip<kTileSteps>();
+                for (int i = 0; i < T0 + wg && wg < TN; ++i) gen.template skip<kTileSteps>();
 #pragma unroll 1
                 for (int I = wg; I < TN; I += NWG) {
-                    if (a_uses > 0) mbar_wait(&bar_afree[wg], (a_uses - 1) & 1, status, kErrMma);
+                    if (a_uses > 0) mbar_wait(&sh.afree[wg], (a_uses - 1) & 1, status, kErrMma);
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
                         uint32_t pk[32];
@@ -399,7 +475,7 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
                     }
                     fence_proxy_async_smem();
                     wg_barrier(wg);
-                    if (wt == 0) mbar_arrive(&bar_aready[wg]);
+                    if (wt == 0) mbar_arrive(&sh.aready[wg]);
                     ++a_uses;
                     gen.template skip<(NWG - 1) * kTileSteps>();
                 }
@@ -407,7 +483,7 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
                 static_for<0, TN>([&](auto ic) {
                     constexpr int I = decltype(ic)::value;
                     if (I % NWG == wg) {
-                        if (a_uses > 0) mbar_wait(&bar_afree[wg], (a_uses - 1) & 1, status, kErrMma);
+                        if (a_uses > 0) mbar_wait(&sh.afree[wg], (a_uses - 1) & 1, status, kErrMma);
                         static_for<0, 16>([&](auto cc) {
                             constexpr int C = decltype(cc)::value;
                             uint32_t pk[4];
@@ -417,7 +493,7 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
                         });
                         fence_proxy_async_smem();
                         wg_barrier(wg);
-                        if (wt == 0) mbar_arrive(&bar_aready[wg]);
+                        if (wt == 0) mbar_arrive(&sh.aready[wg]);
                         ++a_uses;
                     }
                 });
@@ -431,12 +507,13 @@ state_walk(const CUtensorMap& mapX, const CUtensorMap& mapY,
 
 
 #define PSK_STATE_PARAMS                                                                                            \
-    const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY, const uint8_t *__restrict__ gimg,  \
+    const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY,                                    \
+        const __grid_constant__ CUtensorMap mapH, const __grid_constant__ CUtensorMap mapH2, int want_hl, const uint8_t *__restrict__ gimg,  \
         int g_heads, int H, int n, int b, int t, const float *__restrict__ y65, const float *__restrict__ fscale,          \
         const float *__restrict__ cmean, int center_mode, int reverse, int nseg, int mode, int run0, int units,            \
         float *__restrict__ tot, bf16 *__restrict__ S, int lin, int *status
 #define PSK_STATE_ARGS                                                                                              \
-    mapX, mapY, gimg, g_heads, H, n, b, t, y65, fscale, cmean, center_mode, reverse, nseg, mode, run0, units, tot, S, lin, status
+    mapX, mapY, mapH, mapH2, want_hl, gimg, g_heads, H, n, b, t, y65, fscale, cmean, center_mode, reverse, nseg, mode, run0, units, tot, S, lin, status
 
 // The feature tiles of a head are dealt to SPLIT CTAs, each of which forms the half sketches anew.  blockIdx.z, the
 // slowest index: CTAs that run at the same time then run the same specialised code (with the shares of a head side by
@@ -451,9 +528,10 @@ template <int R, int SPLIT> struct StateSplit {
 template <int R, int SPLIT, bool SEG>
 __global__ void __launch_bounds__(StateSplit<R, SPLIT>::kThreads) tc_state_kernel(PSK_STATE_PARAMS) {
     using P = StateSplit<R, SPLIT>;
+    __shared__ StateShared<P::tiles(0), P::NWG> sh;
     static_for<0, SPLIT>([&](auto zc) {
         constexpr int Z = decltype(zc)::value;
-        if (SPLIT == 1 || (int)blockIdx.z == Z) state_walk<R, P::first(Z), P::tiles(Z), P::NWG, SEG>(PSK_STATE_ARGS);
+        if (SPLIT == 1 || (int)blockIdx.z == Z) state_walk<R, P::first(Z), P::tiles(Z), P::NWG, SEG>(sh, PSK_STATE_ARGS);
     });
 }
 
@@ -530,6 +608,8 @@ struct StateArgs {
     int nseg, mode, run0, runs;        // runs [run0, run0 + runs) of nseg are launched
     float* tot;
     bf16* S;
+    CUtensorMap mH[2];                 // where the [hi | lo] half sketches go, if anywhere
+    bool want_hl;
 };
 
 // units a head's sequence can be cut into: blocks (a run starts at a block boundary), or 128-token
@@ -585,7 +665,7 @@ cudaError_t launch_split(const Dims& d, const CUtensorMap& mX, const CUtensorMap
     auto kern = a.nseg > 1 || a.mode != kModePrefix ? tc_state_kernel<R, SPLIT, true> : tc_state_kernel<R, SPLIT, false>;
     PSK_TRY((set_smem(kern, smem)));
     prof_begin(a.mode == kModePrefix ? "tc_state_kernel" : "tc_state_total_kernel", s);
-    launch_pdl_if(early, kern, dim3(d.BH(), a.runs, SPLIT), P::kThreads, smem, s, mX, mY, gimg, d.g_heads, d.H, d.n, d.b, d.t, a.y65, a.fscale,
+    launch_pdl_if(early, kern, dim3(d.BH(), a.runs, SPLIT), P::kThreads, smem, s, mX, mY, a.mH[0], a.mH[1], a.want_hl ? 1 : 0, gimg, d.g_heads, d.H, d.n, d.b, d.t, a.y65, a.fscale,
                   a.cmean, a.center_mode, a.reverse ? 1 : 0, a.nseg, a.mode, a.run0, state_units(d), a.tot, a.S, d.sketch_linear ? 1 : 0, status);
     prof_end(s);
     ++*launches;
@@ -613,10 +693,11 @@ cudaError_t launch_states(const Dims& d, const CUtensorMap& mX, const CUtensorMa
 
 template <int R>
 cudaError_t states_impl(const Dims& d, const CUtensorMap& mX, const CUtensorMap& mY, const uint8_t* gimg, const float* y65,
-                        const float* fscale, const float* cmean, int center_mode, bf16* S, bool reverse, float* tot,
+                        const float* fscale, const float* cmean, int center_mode, bf16* S, bf16* hl, bool reverse, float* tot,
                         int* status, cudaStream_t s, int* launches) {
     const int nseg = tc_state_segments(d);
-    StateArgs a{y65, fscale, cmean, center_mode, reverse, nseg, kModePrefix, 0, nseg, tot, S};
+    StateArgs a{y65, fscale, cmean, center_mode, reverse, nseg, kModePrefix, 0, nseg, tot, S, {mX, mX}, hl != nullptr && !d.noncausal};
+    if (a.want_hl && !tc_map_hilo(d, hl, a.mH)) return cudaErrorInvalidValue;
     if (d.noncausal) {
         // one global state per head: totals of every run, then their sum in the stored format
         a.mode = kModeTotal; a.cmean = nullptr; a.center_mode = 0;
@@ -654,12 +735,12 @@ size_t tc_state_total_bytes(const Dims& d) {
 }
 
 cudaError_t tc_states(const Dims& d, const CUtensorMap& mX, const CUtensorMap& mY, const uint8_t* gimg,
-                      const float* y65, const float* fscale, const float* cmean, int center_mode, bf16* S, bool reverse,
+                      const float* y65, const float* fscale, const float* cmean, int center_mode, bf16* S, bf16* hl, bool reverse,
                       float* tot, int* status, cudaStream_t s, int* launches) {
     switch (d.r) {
-        case 16: return states_impl<16>(d, mX, mY, gimg, y65, fscale, cmean, center_mode, S, reverse, tot, status, s, launches);
-        case 32: return states_impl<32>(d, mX, mY, gimg, y65, fscale, cmean, center_mode, S, reverse, tot, status, s, launches);
-        case 64: return states_impl<64>(d, mX, mY, gimg, y65, fscale, cmean, center_mode, S, reverse, tot, status, s, launches);
+        case 16: return states_impl<16>(d, mX, mY, gimg, y65, fscale, cmean, center_mode, S, hl, reverse, tot, status, s, launches);
+        case 32: return states_impl<32>(d, mX, mY, gimg, y65, fscale, cmean, center_mode, S, hl, reverse, tot, status, s, launches);
+        case 64: return states_impl<64>(d, mX, mY, gimg, y65, fscale, cmean, center_mode, S, hl, reverse, tot, status, s, launches);
     }
     return cudaErrorInvalidValue;
 }

@@ -23,15 +23,20 @@ bool tc_map_3d(CUtensorMap* m, const void* base, int cols, int64_t rows, int64_t
 // center_mode 0: states as they are; 1: values centred by the per-head vector cmean
 // (columns < 64 become H[:, c] - cmean[c] H[:, 64]); 2: last column becomes H[:, 64] - H[:, :64] cmean.
 // `tot`: scratch of tc_state_total_bytes(d) bytes for the segment totals (may be null when that is 0).
+// `hl` (may be null): the half sketches of X's rows as [hi | lo] rows, which the row kernels load as
+// the other side's score operand; contiguous [B][H][n][64 HiLoTiles].
 // Non-causal (d.noncausal): one state per head, the sum over the whole sequence, stored as block 0.
 cudaError_t tc_states(const Dims& d, const CUtensorMap& mX, const CUtensorMap& mY, const uint8_t* gimg,
-                      const float* y65, const float* fscale, const float* cmean, int center_mode, bf16* S, bool reverse,
+                      const float* y65, const float* fscale, const float* cmean, int center_mode, bf16* S, bf16* hl, bool reverse,
                       float* tot, int* status, cudaStream_t s, int* launches);
+// maps of the 64-column tiles of such an array (the second: r = 64 only, else a copy of the first)
+bool tc_map_hilo(const Dims& d, const void* hl, CUtensorMap (&m)[2]);
 // runs a head's blocks are cut into by the state kernel (1 = one CTA group walks the whole head)
 int tc_state_segments(const Dims& d);
 size_t tc_state_total_bytes(const Dims& d);
 // the backward's recomputation of the forward rows: writes y65, e65h (see tc_fwd_out_kernel)
-// (mQraw, and mK = the raw key rows: only with a given half sketch and exact same-block weights)
+// (mK: the keys' [hi | lo] half sketches, with mQraw their second 64 columns for r = 64; the raw key rows with exact
+// same-block weights, and then, with a given half sketch, mQraw the raw query rows)
 cudaError_t tc_recompute(const Dims& d, const CUtensorMap& mQ, const CUtensorMap& mQraw, const CUtensorMap& mK, const CUtensorMap& mV,
                          const CUtensorMap& mZ, const uint8_t* gimg, const float* cmean, const float* denom,
                          const bf16* dO, float* y65, float* e65h, int* status, cudaStream_t s, int* launches);
@@ -44,7 +49,11 @@ cudaError_t tc_prologue(const Dims& d, const void* G1, const void* G2, uint8_t* 
                         cudaStream_t s, int* launches);
 
 // Scratch layout of the tensor-core path.
-struct TcWorkspace { size_t status, vmean, gimg, tot, Z, Rst, y65, e65h, Oc, total; };
+struct TcWorkspace { size_t status, vmean, gimg, tot, Z, Sk, Rst, y65, e65h, Oc, Sq, total; };
+
+// the row kernels read the other side's half sketches from an array of the state kernel's (otherwise: the rows
+// themselves are given half sketches, or the same-block weights come from the raw rows, or there are no blocks)
+inline bool tc_hilo_rows(const Dims& d) { return !d.local && !d.sketch_linear && !d.noncausal; }
 
 template <int R>
 inline TcWorkspace tc_ws(const Dims& d, bool backward) {
@@ -57,7 +66,10 @@ inline TcWorkspace tc_ws(const Dims& d, bool backward) {
     w.gimg = off; off += align_up((size_t)d.g_heads * 2 * R * 128);
     w.tot = off; off += align_up(tc_state_total_bytes(d));
     w.Z = off; off += align_up(st);
+    const size_t hl = tc_hilo_rows(d) ? align_up(rows * (R <= 32 ? 64 : 128) * sizeof(bf16)) : 0;
+    w.Sk = off; off += hl;
     if (backward) {
+        w.Sq = off; off += hl;
         w.Rst = off; off += align_up(st);
         w.y65 = off; off += align_up(rows * sizeof(float));
         w.e65h = off; off += align_up(rows * sizeof(float));
@@ -130,43 +142,23 @@ __device__ __forceinline__ void read_half_sketch(uint32_t lane_tmem, float (&m)[
     }
 }
 
-// Split of an fp32 half-sketch entry into two bf16 terms, m = hi + lo (+ O(2^-17) |m|).  Scores
-// s = m(q).m(k) are formed as hi.hi + hi.lo + lo.hi by one GEMM over 3R columns, the own rows laid
-// out as [hi | hi | lo] and the other rows as [hi | lo | hi]; a score is a cancelling sum, so
-// rounding m to a single bf16 would cost several percent on rows with few keys.
-template <int R, bool OWN>
-__device__ __forceinline__ float split_col(const float (&m)[R], int col) {
-    const int sec = col / R, c = col % R;
-    const float hi = __bfloat162float(__float2bfloat16_rn(m[c]));
-    const bool want_lo = OWN ? (sec == 2) : (sec == 1);
-    return want_lo ? (m[c] - hi) : hi;
-}
-
-// Rows of the 3R-column split operand, K-major and un-swizzled: 8x8 core matrices,
-// [k chunk][row/8][row%8][16 B] (K-direction stride 2048 B, 8-row-group stride 128 B).
-template <int R, bool OWN>
-__device__ __forceinline__ void store_split_rows(uint8_t* dst, const float (&m)[R], int row) {
-#pragma unroll
-    for (int kc = 0; kc < 3 * R / 8; ++kc) {
-        uint4 v;
-        v.x = pack_bf16(split_col<R, OWN>(m, kc * 8 + 0), split_col<R, OWN>(m, kc * 8 + 1));
-        v.y = pack_bf16(split_col<R, OWN>(m, kc * 8 + 2), split_col<R, OWN>(m, kc * 8 + 3));
-        v.z = pack_bf16(split_col<R, OWN>(m, kc * 8 + 4), split_col<R, OWN>(m, kc * 8 + 5));
-        v.w = pack_bf16(split_col<R, OWN>(m, kc * 8 + 6), split_col<R, OWN>(m, kc * 8 + 7));
-        *reinterpret_cast<uint4*>(dst + kc * 2048 + (row / 8) * 128 + (row % 8) * 16) = v;
-    }
-}
-
+// An fp32 half-sketch entry is split into two bf16 terms, m = hi + lo (+ O(2^-17) |m|), and scores s = m(q).m(k) are
+// formed as hi.hi + lo.hi + hi.lo: a score is a cancelling sum, so rounding m to a single bf16 would cost several
+// percent on rows with few keys.
 // The split half sketch as [hi | lo] columns (2R of them) in ceil(2R/64) tiles of
 // [128 rows x 128 B], 128-byte-swizzled, zero beyond 2R.  Tile 0 starts with the R `hi` columns,
 // so it doubles as the MN-major B operand (N = 64, columns >= R ignored) of the dM GEMMs.
 template <int R>
 struct HiLoTiles { static constexpr int N = (2 * R + 63) / 64; };
+// Tiles of 64 columns that a half sketch takes as a score operand: [hi | lo] of r entries each; one of the rows
+// themselves where they are the half sketch (degree 2: r = h, given to the last bit, no lo).
+template <int R, bool LIN> struct OthTiles { static constexpr int N = (LIN && R == 64) ? 1 : HiLoTiles<R>::N; };
 
-template <int R>
+// (TILES: how many of them)
+template <int R, int TILES = HiLoTiles<R>::N>
 __device__ __forceinline__ void store_hilo_tiles(uint8_t* dst, const float (&m)[R], int row) {
 #pragma unroll
-    for (int ch = 0; ch < HiLoTiles<R>::N * 8; ++ch) {
+    for (int ch = 0; ch < TILES * 8; ++ch) {
         uint4 v = make_uint4(0, 0, 0, 0);
         if (ch * 8 < 2 * R) {
             float x[8];
