@@ -44,7 +44,7 @@ constexpr int kModeFirst = 2;          // run 0: both; the other runs: the total
 // 8192, b = 256: 318 us unrolled and with copies by the lanes, now 234).
 // grid (BH).  Warp roles:
 //   NWG generator warpgroups  thread = token: read the half sketches, write their feature tiles
-//                             (dealt round-robin) as MN-major A operands into shared memory; the last one also
+//                             (dealt in turn) as MN-major A operands into shared memory; one of them also
 //                             puts the half sketches where their rows were;
 //   1 store warpgroup         thread = feature row: at block boundaries reads the accumulators,
 //                             centres, rounds and stores them;
@@ -258,12 +258,9 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
         } else if (tid == 128 * (NWG + 1) + 32) {
             constexpr uint32_t idesc_state = idesc_bf16(128, 80, true, true);
             bool ok = true;
-            uint32_t a_cnt[NWG];
-#pragma unroll
-            for (int i = 0; i < NWG; ++i) a_cnt[i] = 0;
-            uint64_t ad[NWG];
-#pragma unroll
-            for (int i = 0; i < NWG; ++i) ad[i] = smem_desc(smem_u32(smem + L::A0 + i * 32768), 16384, 1024, kSwz128);
+            int w = 0;                                    // feature tile number u comes from warpgroup w = u mod NWG, as its
+            uint32_t w_par = 0;                           // tile number u / NWG: parity w_par
+            const uint64_t ad0 = smem_desc(smem_u32(smem + L::A0), 16384, 1024, kSwz128);
             const uint64_t yd0 = smem_desc(smem_u32(smem + L::Y), 16384, 1024, kSwz128);
             const int ibase = init ? 0 : 1;               // completions of sh.accread before block 1's
             for (int j = 0; j < NJs && ok; ++j) {
@@ -277,19 +274,19 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
                 const uint32_t acc0 = (j > 0 || init) ? 1u : 0u;
                 static_for<0, TN>([&](auto ic) {
                     constexpr int I = decltype(ic)::value;
-                    constexpr int w = I % NWG;
                     // the store warpgroup has taken this accumulator's values for the boundary
                     if (boundary) ok = ok && mbar_spin(&sh.accread[I], ((j / tpb) - ibase) & 1, status, kErrState);
-                    ok = ok && mbar_spin(&sh.aready[w], a_cnt[w] & 1, status, kErrState);
-                    ++a_cnt[w];
+                    ok = ok && mbar_spin(&sh.aready[w], w_par, status, kErrState);
+                    const uint64_t ad = desc_off(ad0, w * 32768);
                     tc_fence_after();
 #pragma unroll
                     for (int k = 0; k < 8; ++k)
-                        umma_ss(tm + kAcc + 80 * I, desc_off(ad[w], k * 2048), desc_off(yd, k * 2048), idesc_state, k > 0 ? 1u : acc0);
+                        umma_ss(tm + kAcc + 80 * I, desc_off(ad, k * 2048), desc_off(yd, k * 2048), idesc_state, k > 0 ? 1u : acc0);
                     umma_commit(&sh.afree[w]);
                     // last token tile of a block: this accumulator is complete, and the store
                     // warpgroup may take it while the remaining tiles are still being issued
                     if (block_end) umma_commit(&sh.accfull[I]);
+                    if (++w == NWG) { w = 0; w_par ^= 1; }
                 });
                 umma_commit(&sh.yfree[j & 1]);
             }
@@ -416,7 +413,10 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
         // last-column entry of this thread's token, requested one token tile ahead of its use
         float y_next = (y65 != nullptr && wg == 0) ? y65[(size_t)bh * n + tile_of(0) * 128 + wt] : 0.f;
         float d_next = fscale != nullptr ? fscale[(size_t)bh * n + tile_of(0) * 128 + wt] : 1.f;
-        for (int j = 0; j < NJs; ++j) {
+        // Feature tiles are dealt to the warpgroups in turn, on across the token tiles: with TN not a multiple of NWG each has
+        // its share over a few token tiles, and one with fewer tiles here starts on the next token tile meanwhile.
+        int first = wg;                                   // this warpgroup's first tile of the token tile
+        for (int j = 0; j < NJs; ++j, first = (first + (NWG - TN % NWG)) % NWG) {
             mbar_wait(&sh.sk, j & 1, status, kErrMma);
             tc_fence_after();
             PackedM<R> pm;
@@ -426,8 +426,8 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
                 // features m_a m_b / d: both factors carry 1 / sqrt(d) (d requested a token tile ago)
                 const float sc = rsqrtf(d_next);
                 if (fscale != nullptr && j + 1 < NJs) d_next = fscale[(size_t)bh * n + tile_of(j + 1) * 128 + wt];
-                // (the warpgroup with the fewest tiles also writes the half sketches out, over their dead X rows)
-                const bool out = hl && wg == NWG - 1;
+                // (the warpgroup last in turn, with the fewest tiles, also writes the half sketches out, over their dead X rows)
+                const bool out = hl && first == NWG - 1;
                 read_half_sketch<R>(lane_tm, m, out ? 1.f : sc, lin != 0);
                 tc_fence_before();
                 wg_barrier(wg);
@@ -458,11 +458,11 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
                 if (wt == 0) mbar_arrive(&sh.ext[j & 1]);
             }
             if constexpr (F::kCirc) {
-                // this warpgroup's tiles wg, wg + NWG, ...: the same loop body on a rotated copy of m
+                // this warpgroup's tiles first, first + NWG, ...: the same loop body on a rotated copy of m
                 constexpr int kTileSteps = 128 / (2 * R);
-                for (int i = 0; i < T0 + wg && wg < TN; ++i) gen.template skip<kTileSteps>();
+                for (int i = 0; i < T0 + first && first < TN; ++i) gen.template skip<kTileSteps>();
 #pragma unroll 1
-                for (int I = wg; I < TN; I += NWG) {
+                for (int I = first; I < TN; I += NWG) {
                     if (a_uses > 0) mbar_wait(&sh.afree[wg], (a_uses - 1) & 1, status, kErrMma);
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
@@ -482,7 +482,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
             } else {
                 static_for<0, TN>([&](auto ic) {
                     constexpr int I = decltype(ic)::value;
-                    if (I % NWG == wg) {
+                    if (I % NWG == first) {
                         if (a_uses > 0) mbar_wait(&sh.afree[wg], (a_uses - 1) & 1, status, kErrMma);
                         static_for<0, 16>([&](auto cc) {
                             constexpr int C = decltype(cc)::value;
