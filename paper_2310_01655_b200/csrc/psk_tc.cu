@@ -187,7 +187,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     __shared__ uint64_t bar_q, bar_kv[2], bar_sk, bar_go, bar_s, bar_p, bar_pv;
-    __shared__ uint64_t bar_z[kZStages], bar_feat[kFeatBufs], bar_a[kFeatBufs];
+    __shared__ uint64_t bar_feat[kFeatBufs], bar_a[kFeatBufs];
     __shared__ uint32_t tmem_slot;
     __shared__ float cm[64];
     const int tid = threadIdx.x, warp = tid / 32, tau = blockIdx.x, l = blockIdx.y, bh = blockIdx.z;
@@ -208,9 +208,8 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
         tma_load_4d(smem + L::Q, &mapQ, 0, row0, hi, bi, &bar_q);
         bulk_load(smem + L::G, gimg + (size_t)g * GImage<R>::bytes, GImage<R>::bytes, &bar_q);
         mbar_init(&bar_kv[0], 1); mbar_init(&bar_kv[1], 1); mbar_init(&bar_sk, 1); mbar_init(&bar_s, 1); mbar_init(&bar_pv, 1);
-        mbar_init(&bar_p, 128); mbar_init(&bar_go, 128);
-        for (int s = 0; s < kZStages; ++s) mbar_init(&bar_z[s], 1);
-        for (int s = 0; s < kFeatBufs; ++s) { mbar_init(&bar_feat[s], 128); mbar_init(&bar_a[s], 1); }
+        mbar_init(&bar_p, 4); mbar_init(&bar_go, 4);            // (one arrival per warp)
+        for (int s = 0; s < kFeatBufs; ++s) { mbar_init(&bar_feat[s], 5); mbar_init(&bar_a[s], 1); }
         cta_giveup_init();
         mbar_fence_init();
         tma_prefetch_desc(&mapK); tma_prefetch_desc(&mapV); tma_prefetch_desc(&mapZ);
@@ -246,7 +245,8 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     // B = the chunk's 64 feature rows x 80 columns, MN-major: 16 features per K step, the second
     // 64-column group (columns 64..79) 8192 B further on.  Everything the loop needs is in registers
     // before it waits: between "features staged" and "MMAs issued" lie the four MMA instructions
-    // and nothing else.  (The stages are refilled by the rows' side, which learns first that a
+    // and nothing else, and one barrier says that the features are staged (an arrival per warp) and the state rows there
+    // (144 heads x 8192, r = 32, b = 256: 351 us with two barriers and an arrival per thread, now 335).  (The stages are refilled by the rows' side, which learns first that a
     // buffer is free.)
     auto issue_chunks = [&](int first, int step) {
         constexpr uint32_t idesc = idesc_bf16(128, 80, false, true);
@@ -259,9 +259,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             const int ksteps = (F::FK - C * 64) >= 64 ? 4 : (F::FK - C * 64) / 16;
             const uint64_t zd = s == kZStages - 1 ? zdq : desc_off(zd0, s * kZStageBytes);
             const uint32_t at = tm + cA + s * 32;
-            ok = mbar_spin(&bar_z[s], par, status, kErrTma);
-            FTR(4, C);
-            ok = ok && mbar_spin(&bar_feat[s], par, status, kErrMma);
+            ok = mbar_spin(&bar_feat[s], par, status, kErrTma);          // features staged and state rows there
             FTR(5, C);
             tc_fence_after();
 #pragma unroll
@@ -286,9 +284,9 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             // up: everyone waits for that thread, only this one waits for the query tile anyway)
             if (has_prefix) {
                 for (int c = 0; c < kZStages - 1 && c < F::NC; ++c) {
-                    mbar_expect_tx(&bar_z[c], kZStageBytes);
-                    tma_load_3d(smem + L::zstage(c), &mapZ, 0, c * 64, blk, &bar_z[c]);
-                    tma_load_3d(smem + L::zstage(c) + 8192, &mapZ, 64, c * 64, blk, &bar_z[c]);
+                    mbar_expect_tx(&bar_feat[c], kZStageBytes);
+                    tma_load_3d(smem + L::zstage(c), &mapZ, 0, c * 64, blk, &bar_feat[c]);
+                    tma_load_3d(smem + L::zstage(c) + 8192, &mapZ, 64, c * 64, blk, &bar_feat[c]);
                 }
             }
             ok = mbar_spin(&bar_q, 0, status, kErrTma);
@@ -305,9 +303,9 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             if (has_prefix && kZStages - 1 < F::NC) {
                 // the query tile has been consumed: its buffer becomes the ring's last stage
                 ok = ok && mbar_spin(&bar_sk, 0, status, kErrMma);
-                mbar_expect_tx(&bar_z[kZStages - 1], kZStageBytes);
-                tma_load_3d(smem + L::zstage(kZStages - 1), &mapZ, 0, (kZStages - 1) * 64, blk, &bar_z[kZStages - 1]);
-                tma_load_3d(smem + L::zstage(kZStages - 1) + 8192, &mapZ, 64, (kZStages - 1) * 64, blk, &bar_z[kZStages - 1]);
+                mbar_expect_tx(&bar_feat[kZStages - 1], kZStageBytes);
+                tma_load_3d(smem + L::zstage(kZStages - 1), &mapZ, 0, (kZStages - 1) * 64, blk, &bar_feat[kZStages - 1]);
+                tma_load_3d(smem + L::zstage(kZStages - 1) + 8192, &mapZ, 64, (kZStages - 1) * 64, blk, &bar_feat[kZStages - 1]);
             }
             if (has_prefix) issue_chunks(0, PSK_OUT_ISSUERS);     // earlier blocks: features x prefix state chunks
             const int tp_last = noncausal ? -1 : tau;
@@ -404,7 +402,8 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             fence_proxy_async_smem();
         }
         tc_fence_before();
-        mbar_arrive(&bar_go);
+        __syncwarp();
+        if (tid % 32 == 0) mbar_arrive(&bar_go);
         if (tid == 0) FTR(21, 0);
 
         if (has_prefix) {
@@ -412,15 +411,15 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                 CircGen<R> gen;
                 gen.init(mq);
 #pragma unroll 1
-                for (int C = 0; C < F::NC && ok; ++C) {
+                for (int C = 0; C < F::NC; ++C) {     // (no early exit: a wait that gave up makes the later ones return at once)
                     const int buf = C % kFeatBufs;
                     if (C >= kFeatBufs) {             // the MMAs that read this buffer's previous contents
                         ok = mbar_wait(&bar_a[buf], (C / kFeatBufs - 1) & 1, status, kErrMma);
                         tc_fence_after();
                         if (tid == 0) {               // ... and this stage's: refill it with chunk C's rows
-                            mbar_expect_tx(&bar_z[buf], kZStageBytes);
-                            tma_load_3d(smem + L::zstage(buf), &mapZ, 0, C * 64, blk, &bar_z[buf]);
-                            tma_load_3d(smem + L::zstage(buf) + 8192, &mapZ, 64, C * 64, blk, &bar_z[buf]);
+                            mbar_expect_tx(&bar_feat[buf], kZStageBytes);
+                            tma_load_3d(smem + L::zstage(buf), &mapZ, 0, C * 64, blk, &bar_feat[buf]);
+                            tma_load_3d(smem + L::zstage(buf) + 8192, &mapZ, 64, C * 64, blk, &bar_feat[buf]);
                         }
                     }
                     if (tid == 0) FTR(22, C);
@@ -429,7 +428,8 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                     tmem_st32(lane_tm + cA + buf * 32, pk);
                     tmem_st_wait();
                     tc_fence_before();
-                    mbar_arrive(&bar_feat[buf]);
+                    __syncwarp();
+                    if (tid % 32 == 0) mbar_arrive(&bar_feat[buf]);
                     if (tid == 0) FTR(23, C);
                 }
             } else {
@@ -442,9 +442,9 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                         ok = ok && mbar_wait(&bar_a[buf], (C / kFeatBufs - 1) & 1, status, kErrMma);
                         tc_fence_after();
                         if (tid == 0) {
-                            mbar_expect_tx(&bar_z[buf], kZStageBytes);
-                            tma_load_3d(smem + L::zstage(buf), &mapZ, 0, C * 64, blk, &bar_z[buf]);
-                            tma_load_3d(smem + L::zstage(buf) + 8192, &mapZ, 64, C * 64, blk, &bar_z[buf]);
+                            mbar_expect_tx(&bar_feat[buf], kZStageBytes);
+                            tma_load_3d(smem + L::zstage(buf), &mapZ, 0, C * 64, blk, &bar_feat[buf]);
+                            tma_load_3d(smem + L::zstage(buf) + 8192, &mapZ, 64, C * 64, blk, &bar_feat[buf]);
                         }
                     }
                     uint32_t pk[16];
@@ -454,14 +454,15 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                     tmem_st16(lane_tm + cA + buf * 32 + 16, pk);
                     tmem_st_wait();
                     tc_fence_before();
-                    mbar_arrive(&bar_feat[buf]);
+                    __syncwarp();
+                    if (tid % 32 == 0) mbar_arrive(&bar_feat[buf]);
                 });
             }
         }
 
         const int tp_last = noncausal ? -1 : tau;
 #pragma unroll 1
-        for (int tp = 0; tp <= tp_last && ok; ++tp) {
+        for (int tp = 0; tp <= tp_last; ++tp) {
             ok = ok && mbar_wait(&bar_s, tp & 1, status, kErrMma);
             if (tid == 0) FTR(26, tp);
             tc_fence_after();
@@ -491,7 +492,8 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             }
             tmem_st_wait();
             tc_fence_before();
-            mbar_arrive(&bar_p);
+            __syncwarp();
+            if (tid % 32 == 0) mbar_arrive(&bar_p);
             if (tid == 0) FTR(27, tp);
         }
         if (noncausal)      // the last chunk's MMAs (no same-block tiles follow them)
