@@ -64,14 +64,14 @@ def kernel_flops_per_head_token(name, w, local=False):
     nt = b // 128
     other = (nt + 1) / 2.0              # other-side 128-row tiles met per own tile, averaged
     sk = 2 * h * 2 * r                  # one half-sketch GEMM
-    tile_fwd = sk + 2 * 128 * 3 * r + 2 * 128 * h
-    tile_bwd = sk + 2 * 128 * 3 * r + 2 * 128 * h + 2 * 128 * 64
-    if local:                           # scores over h, no sketch of the other tile; dX product 64 wide
+    tile_fwd = 2 * 128 * 3 * r + 2 * 128 * h        # (the other side's half sketches come from the state kernels)
+    tile_bwd = 2 * 128 * 3 * r + 2 * 128 * h + 2 * 128 * 64
+    if local:                           # scores over h; dX product 64 wide
         tile_fwd = 2 * 128 * h + 2 * 128 * h
         tile_bwd = 2 * 128 * h + 2 * 128 * h + 2 * 128 * 64
     table.update({
-        # (r = 64: the feature tiles are split between five CTAs, which each redo the half sketch)
-        "tc_state_kernel": sk * (1 if r <= 32 else 5) + 2 * FP * 80,
+        # (r = 64, many heads: the feature tiles are dealt to six CTAs, which each redo the half sketch)
+        "tc_state_kernel": sk * (1 if r <= 32 else 6) + 2 * FP * 80,
         "tc_fwd_out_kernel": sk + 2 * FK * 80 + other * tile_fwd,
         "tc_bwd_recompute_kernel": sk + 2 * FK * 80 + other * tile_fwd,
         "tc_bwd_q_kernel": 2 * sk + 2 * FK * 80 + other * tile_bwd + 2 * 2 * r * 64,

@@ -245,9 +245,9 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     // B = the chunk's 64 feature rows x 80 columns, MN-major: 16 features per K step, the second
     // 64-column group (columns 64..79) 8192 B further on.  Everything the loop needs is in registers
     // before it waits: between "features staged" and "MMAs issued" lie the four MMA instructions
-    // and nothing else, and one barrier says that the features are staged (an arrival per warp) and the state rows there
-    // (144 heads x 8192, r = 32, b = 256: 351 us with two barriers and an arrival per thread, now 335).  (The stages are refilled by the rows' side, which learns first that a
-    // buffer is free.)
+    // and nothing else, and one barrier says that the features are staged (an arrival per warp) and the
+    // state rows are there (144 heads x 8192, r = 32, b = 256: 351 us with two barriers and an arrival per
+    // thread, now 335).  (The stages are refilled by the rows' side, which learns first that a buffer is free.)
     auto issue_chunks = [&](int first, int step) {
         constexpr uint32_t idesc = idesc_bf16(128, 80, false, true);
         const uint64_t zd0 = smem_desc(smem_u32(smem + L::Z), 8192, 1024, kSwz128);
