@@ -89,16 +89,15 @@ typedef struct {
                                    are too few heads to fill the GPU); must divide n / b */
 } psk_shape;
 
-/* PSK_FLAG_KEEP_STATES: set on BOTH the
+/* PSK_FLAG_KEEP_STATES (tensor-core path; ignored by the CUDA-core path): set on BOTH the
  * forward and the backward call of one training step.  The forward then leaves in its
  * workspace the prefix states Z_l of Section 3.1, the per-head value centres c they are centred
  * by, and O - c (rounded after the subtraction: the caller's rounded O cannot supply it) - for
  * p = 8 and the learnable sketch also the half sketches of Q and K; the
  * backward, given the SAME workspace memory (not written in between) with the same shape and inputs, reads them instead
- * of rebuilding the states from K and V and recomputing the forward rows.  (CUDA-core path: the half
- * sketches and the prefix states.)  With the flag set psk_workspace_bytes() returns the backward's
- * size for both calls on the tensor-core path; on the CUDA-core path take the backward's.  Without the
- * flag each call is self-contained.
+ * of rebuilding the states from K and V and recomputing the forward rows.  With the flag set
+ * psk_workspace_bytes() returns the backward's size for both calls on the tensor-core path.  Without the
+ * flag, and on the CUDA-core path with it too, each call is self-contained: its workspace is scratch only.
  *
  * PSK_FLAG_LOCAL_EXACT: "applying exact attention locally" (Section 3.2).  Pairs (i, j) of the
  * same block of b rows get the exact polynomial weight (q_i . k_j)^4 instead of the sketched

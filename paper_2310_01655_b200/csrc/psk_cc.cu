@@ -7,14 +7,13 @@
 
 namespace psk {
 
-// The forward's arrays come first and lie the same in both layouts: with PSK_FLAG_KEEP_STATES the
-// backward finds the half sketches and the prefix states where the forward left them.
+// PSK_FLAG_KEEP_STATES means nothing here: every call forms all it reads, from its own arguments.
 CcWorkspace cc_workspace(const Dims& d, bool backward) {
     CcWorkspace w{};
     const size_t rows = (size_t)d.BH() * d.n;
     const size_t chunks = (size_t)(d.r / 8) * (d.r / 8 + 1) / 2;
     const size_t st = (size_t)d.BH() * d.t * chunks * cc::kChunkFloats * sizeof(float);
-        size_t off = 0;
+    size_t off = 0;
     w.status = off; off += kStatusBytes;
     w.Mq = off;  off += align_up(rows * d.r * sizeof(float));
     w.Mk = off;  off += align_up(rows * d.r * sizeof(float));
@@ -351,9 +350,8 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 rows_prep_kernel(Slice sl, int n, int total_rows, int mode, const T* __restrict__ V,
                  const T* __restrict__ O, const float* __restrict__ denom,
-                 const T* __restrict__ dO, float* __restrict__ out, int* status) {
+                 const T* __restrict__ dO, float* __restrict__ out) {
     pdl_sync();
-    if (status != nullptr && threadIdx.x < kStatusBytes / 4 && blockIdx.x == 0) status[threadIdx.x] = 0;
     const int row = blockIdx.x * 16 + threadIdx.x / 16, lane = threadIdx.x % 16;
     if (row >= total_rows) return;      // (total_rows is a multiple of 128: whole warps)
     const int64_t base = sl.row(row / n, row % n) + 4 * lane;
@@ -592,7 +590,7 @@ cudaError_t value_rows(const Dims& d, const T* V, float* Vt, cc::YRows* y, cudaS
     } else {
         const int rows = d.BH() * d.n;
         prof_begin("rows_prep_kernel", s);
-        launch_pdl(rows_prep_kernel<T>, (rows + 15) / 16, 256, 0, s, sl, d.n, rows, 0, V, nullptr, nullptr, nullptr, Vt, nullptr);
+        launch_pdl(rows_prep_kernel<T>, (rows + 15) / 16, 256, 0, s, sl, d.n, rows, 0, V, nullptr, nullptr, nullptr, Vt);
         prof_end(s);
         ++*launches;
         *y = cc::YRows{Vt, Slice{d.H, (int64_t)d.H * d.n * 64, (int64_t)d.n * 64, 64}, 1};
@@ -600,17 +598,11 @@ cudaError_t value_rows(const Dims& d, const T* V, float* Vt, cc::YRows* y, cudaS
     }
 }
 
-// Half sketches, value rows and prefix states: what the forward needs, and the backward again
-// unless the forward left them in this workspace.
+// Half sketches, value rows and prefix states: what the forward needs, and the backward again.
 template <typename T, int R>
 cudaError_t prefix_states(const Dims& d, const T* Q, const T* K, const T* V, const T* G1, const T* G2, char* ws,
-                          const CcWorkspace& w, bool kept, cc::YRows* y, cudaStream_t s, int* launches) {
+                          const CcWorkspace& w, cc::YRows* y, cudaStream_t s, int* launches) {
     float* Mq = (float*)(ws + w.Mq); float* Mk = (float*)(ws + w.Mk);
-    if (kept) {
-        *y = sizeof(T) == 4 ? cc::YRows{(const float*)V, Slice{d.H, d.sb, d.sh, d.sn}, 1}
-                            : cc::YRows{(const float*)(ws + w.Vt), Slice{d.H, (int64_t)d.H * d.n * 64, (int64_t)d.n * 64, 64}, 1};
-        return cudaSuccess;
-    }
     PSK_TRY((launch_sketch<T, R>(d, Q, K, G1, G2, Mq, Mk, nullptr, d.clear_status ? (int*)(ws + w.status) : nullptr, s, launches)));
     PSK_TRY(value_rows<T>(d, V, (float*)(ws + w.Vt), y, s, launches));
     return launch_states<R>(d, Mk, *y, (float*)(ws + w.Zst), false, s, launches);
@@ -621,7 +613,7 @@ cudaError_t fwd_impl(const Dims& d, const T* Q, const T* K, const T* V, const T*
                      T* O, float* denom, char* ws, cudaStream_t s, int* launches) {
     const CcWorkspace w = cc_workspace(d, false);
     cc::YRows y;
-    PSK_TRY((prefix_states<T, R>(d, Q, K, V, G1, G2, ws, w, false, &y, s, launches)));
+    PSK_TRY((prefix_states<T, R>(d, Q, K, V, G1, G2, ws, w, &y, s, launches)));
     return launch_rows<T, R>(d, (float*)(ws + w.Mq), (float*)(ws + w.Mk), y, (float*)(ws + w.Zst), Q, K, false, O, denom, s, launches);
 }
 
@@ -680,10 +672,9 @@ cudaError_t bwd_impl(const Dims& d, const T* Q, const T* K, const T* V, const T*
     float* dXk = d.local ? (float*)(ws + w.dXk) : nullptr;
     const int rows = d.BH() * d.n;
     cc::YRows yv;
-    PSK_TRY((prefix_states<T, R>(d, Q, K, V, G1, G2, ws, w, d.keep_states, &yv, s, launches)));
+    PSK_TRY((prefix_states<T, R>(d, Q, K, V, G1, G2, ws, w, &yv, s, launches)));
     prof_begin("rows_prep_kernel", s);
-    launch_pdl(rows_prep_kernel<T>, (rows + 15) / 16, 256, 0, s, Slice{d.H, d.sb, d.sh, d.sn}, d.n, rows, 1, nullptr, O, denom, dO, E,
-               d.clear_status && d.keep_states ? (int*)(ws + w.status) : nullptr);
+    launch_pdl(rows_prep_kernel<T>, (rows + 15) / 16, 256, 0, s, Slice{d.H, d.sb, d.sh, d.sn}, d.n, rows, 1, nullptr, O, denom, dO, E);
     prof_end(s);
     ++*launches;
     PSK_TRY(cudaGetLastError());
