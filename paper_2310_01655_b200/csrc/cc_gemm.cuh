@@ -96,6 +96,46 @@ __device__ __forceinline__ void load_rows8(f2 (&a)[4], const float* p) {
     a[0] = u.x; a[1] = u.y; a[2] = v.x; a[3] = v.y;
 }
 
+// Token 8 ry + q against the thread's rows 8 ry + 0..7 on the diagonal of a 64 x 64 tile, of which only the pairs
+// with token <= row (UPPER: token >= row) count.  Pairs beyond it are left out or multiplied by zeros on both sides: a
+// weight of zero alone would let an infinity or a NaN of a row that does not count through.  q is a constant
+// after unrolling; c: NQ column pairs, into the accumulators q0, q0 + 1, ...
+template <bool UPPER, int NQ, int NA>
+__device__ __forceinline__ void diagonal_step(f2 (&s)[4][NA], f2 (&x)[4][NA], const f2 (&a)[4], const f2 (&c)[NQ], int q0, int q) {
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const bool lo = UPPER ? q >= 2 * p : q <= 2 * p, hi = UPPER ? q >= 2 * p + 1 : q <= 2 * p + 1;
+        if (!lo && !hi) continue;
+#pragma unroll
+        for (int j = 0; j < NQ; ++j) {
+            const float c0 = lo2(c[j]), c1 = hi2(c[j]);
+            s[p][q0 + j] = fma2(a[p], pack2(lo ? c0 : 0.f, hi ? c1 : 0.f), s[p][q0 + j]);
+            x[p][q0 + j] = fma2(a[p], pack2(lo ? c1 : 0.f, hi ? c0 : 0.f), x[p][q0 + j]);
+        }
+    }
+}
+// acc += At^T B of a diagonal tile, At [64 tokens][kLd] (64 rows), B [64 tokens][ldb] (64 columns); only the
+// pairs that count are visited, half as many as in a whole tile
+template <bool UPPER>
+__device__ __forceinline__ void diagonal_product(Acc& acc, const float* At, const float* B, int ldb, int ry, int cx) {
+    const int k1 = UPPER ? 64 : 8 * ry;
+#pragma unroll 2
+    for (int k = UPPER ? 8 * ry + 8 : 0; k < k1; ++k) {
+        f2 a[4];
+        load_rows8(a, At + k * kLd + 8 * ry);
+        acc.step(a, lds22(B + k * ldb + 4 * cx), lds22(B + k * ldb + 32 + 4 * cx));
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int k = 8 * ry + q;
+        f2 a[4];
+        load_rows8(a, At + k * kLd + 8 * ry);
+        const F22 u = lds22(B + k * ldb + 4 * cx), v = lds22(B + k * ldb + 32 + 4 * cx);
+        const f2 c[4] = {u.x, u.y, v.x, v.y};
+        diagonal_step<UPPER>(acc.s, acc.x, a, c, 0, q);
+    }
+}
+
 // acc += At^T B over k < K: At [K][kLd] (64 rows), B [K][ldb] (64 columns)
 template <int UNROLL = 4>
 __device__ __forceinline__ void outer_product(Acc& acc, const float* At, const float* B, int K, int ldb, int ry, int cx) {

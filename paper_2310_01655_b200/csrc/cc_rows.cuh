@@ -317,7 +317,10 @@ cc_rows_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mown, co
             *reinterpret_cast<float4*>(sW + cj * kLd + 8 * ry + 4) = make_float4(w[4], w[5], w[6], w[7]);
         }
         group_sync(grp);
-        outer_product(acc, sW, sY, 64, kLd, ry, cx);
+        if (!diag) outer_product(acc, sW, sY, 64, kLd, ry, cx);
+        else if (dv) diagonal_product<true>(acc, sW, sY, kLd, ry, cx);
+        else diagonal_product<false>(acc, sW, sY, kLd, ry, cx);
+        // (the last column is all ones, or nobody reads its sum)
         for (int k = cx; k < 64; k += 8) {
             f2 w[4];
             load_rows8(w, sW + k * kLd + 8 * ry);
@@ -481,7 +484,7 @@ cc_dphi_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mown, co
         item -= NC;
     }
     // tiles of the same block
-    f2 gs[4][(NCOL + 1) / 2], gx[4][(NCOL + 1) / 2];
+    f2 gs[4][NCOL / 2], gx[4][NCOL / 2];
 #pragma unroll
     for (int p = 0; p < 4; ++p)
 #pragma unroll
@@ -509,18 +512,19 @@ cc_dphi_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mown, co
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const float s = sum2(d[i][j]);
-                    const int rr = ry + 32 * half + 8 * i, cj = cx + 8 * j;
-                    const bool keep = kside ? cj >= rr : cj <= rr;
-                    const float f = LOCAL ? 4.f * s * s * s : 2.f * s;
-                    ds[4 * half + i][j] = (!diag || keep) ? f : 0.f;
+                    ds[4 * half + i][j] = LOCAL ? 4.f * s * s * s : 2.f * s;
                 }
             dot_half<kLd, kLd>(d, sYo, sY, 16, half, ry, cx);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const float yl = sY[(cx + 8 * j) * kLd + 64];
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    ds[4 * half + i][j] *= fmaf(sYo[(ry + 32 * half + 8 * i) * kLd + 64], yl, sum2(d[i][j]));
+                for (int i = 0; i < 4; ++i) {
+                    const int rr = ry + 32 * half + 8 * i, cj = cx + 8 * j;
+                    const bool keep = kside ? cj >= rr : cj <= rr;
+                    const float g = ds[4 * half + i][j] * fmaf(sYo[rr * kLd + 64], yl, sum2(d[i][j]));
+                    ds[4 * half + i][j] = (!diag || keep) ? g : 0.f;
+                }
             }
         }
         group_sync(grp);
@@ -530,12 +534,9 @@ cc_dphi_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mown, co
             for (int j = 0; j < 8; ++j) sY[(cx + 8 * j) * kLd + ry + 8 * i] = ds[i][j];
         group_sync(grp);
         // same-block gradient += ds (64 own x 64 other) . rows of the other side (64 x 8 NCOL)
-#pragma unroll 2
-        for (int k = 0; k < 64; ++k) {
-            f2 a[4];
+        auto columns = [&](int k, f2 (&a)[4], f2 (&c)[NCOL / 2]) {
             load_rows8(a, sY + k * kLd + 8 * ry);
             const float* o = sO + k * LDS_;
-            f2 c[(NCOL + 1) / 2];
             if constexpr (NCOL == 2) {
                 c[0] = *reinterpret_cast<const f2*>(o + 2 * cx);
             } else {
@@ -543,11 +544,27 @@ cc_dphi_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mown, co
                 c[0] = u.x; c[1] = u.y;
                 if constexpr (NCOL == 8) { const F22 w = lds22(o + 32 + 4 * cx); c[2] = w.x; c[3] = w.y; }
             }
+        };
+        // (diagonal tile: the pairs that count, see diagonal_step)
+        const int k0 = diag && kside ? 8 * ry + 8 : 0, k1 = diag && !kside ? 8 * ry : 64;
+#pragma unroll 2
+        for (int k = k0; k < k1; ++k) {
+            f2 a[4], c[NCOL / 2];
+            columns(k, a, c);
 #pragma unroll
             for (int q = 0; q < NCOL / 2; ++q) {
                 const f2 sw = swap2(c[q]);
 #pragma unroll
                 for (int p = 0; p < 4; ++p) { gs[p][q] = fma2(a[p], c[q], gs[p][q]); gx[p][q] = fma2(a[p], sw, gx[p][q]); }
+            }
+        }
+        if (diag) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                f2 a[4], c[NCOL / 2];
+                columns(8 * ry + q, a, c);
+                if (kside) diagonal_step<true>(gs, gx, a, c, 0, q);
+                else diagonal_step<false>(gs, gx, a, c, 0, q);
             }
         }
         group_sync(grp);

@@ -77,6 +77,15 @@ struct AccN {
             }
         }
     }
+    // token 8 ry + q of the diagonal tile (cc_gemm.cuh, diagonal_step)
+    __device__ __forceinline__ void diagonal(const f2 (&a)[4], const float* b, int q) {
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            const F22 u = lds22(b + 32 * h);
+            const f2 c[2] = {u.x, u.y};
+            diagonal_step<false>(s, x, a, c, 2 * h, q);
+        }
+    }
     __device__ __forceinline__ float at(int i, int h, int j) const {       // row i, column 32 h + 4 cx + j
         const f2 v = ((i ^ j) & 1) ? x[i / 2][2 * h + j / 2] : s[i / 2][2 * h + j / 2];
         return (i & 1) ? hi2(v) : lo2(v);
@@ -260,11 +269,20 @@ lt_out_kernel(const float* __restrict__ A, const float* __restrict__ B, const fl
 #pragma unroll
             for (int j = 0; j < 8; ++j) sG[(cx + 8 * j) * kLd + ry + 8 * i] = w[i][j];
         group_sync(grp);
+        const int j1 = jt < tile ? 64 : 8 * ry;
 #pragma unroll 2
-        for (int j = 0; j < 64; ++j) {
+        for (int j = 0; j < j1; ++j) {
             f2 a[4];
             load_rows8(a, sG + j * kLd + 8 * ry);
             acc.step(a, sG + L::C + j * LDC + 4 * cx);
+        }
+        if (jt == tile) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                f2 a[4];
+                load_rows8(a, sG + (8 * ry + q) * kLd + 8 * ry);
+                acc.diagonal(a, sG + L::C + (8 * ry + q) * LDC + 4 * cx, q);
+            }
         }
         group_sync(grp);
     }
