@@ -172,6 +172,29 @@ __device__ __forceinline__ void dot_half(f2 (&d)[4][8], const float* A, const fl
         }
     }
 }
+// The same with every sum as one chain over k, in the order of outer_product and so to the last bit the value that it
+// forms: for scores whose errors cancel only if the forward and the backward make the same ones.
+template <int LDA, int LDB>
+__device__ __forceinline__ void dot_half_chain(float (&d)[4][8], const float* A, const float* B, int K4, int half, int ry, int cx) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) d[i][j] = 0.f;
+    const float* a0 = A + (ry + 32 * half) * LDA;
+    const float* b0 = B + cx * LDB;
+#pragma unroll 2
+    for (int k = 0; k < 4 * K4; k += 4) {
+        float4 a[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(a0 + 8 * i * LDA + k);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float4 b = *reinterpret_cast<const float4*>(b0 + 8 * j * LDB + k);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) d[i][j] = fmaf(a[i].w, b.w, fmaf(a[i].z, b.z, fmaf(a[i].y, b.y, fmaf(a[i].x, b.x, d[i][j]))));
+        }
+    }
+}
 // all eight rows at once: two thirds of the shared-memory loads per product, for 128 accumulator registers
 template <int LDA, int LDB>
 __device__ __forceinline__ void dot_full(f2 (&d)[8][8], const float* A, const float* B, int K4, int ry, int cx) {

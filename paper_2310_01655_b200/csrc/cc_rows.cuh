@@ -505,15 +505,25 @@ cc_dphi_kernel(Slice sl, int n, int b, int t, const float* __restrict__ Mown, co
         float ds[8][8];
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
+            if constexpr (LOCAL) {
+                // The forward's scores to the last bit.  O and the normaliser carry the error of their score's fourth power, and
+                // the derivative x^3 / (1 + x^4)^2 of a row with few keys nearly cancels it, if the error is the same one.  (With
+                // the two half sums of dot_half: dQ of the first rows of a head off by 2.4 times as much; same time.)
+                float s[4][8];
+                dot_half_chain<kLd, kLd>(s, sX, sO, 16, half, ry, cx);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) ds[4 * half + i][j] = 4.f * s[i][j] * s[i][j] * s[i][j];
+            } else {
+                f2 s[4][8];
+                dot_half<LDM, LDM>(s, sM, sO, R / 4, half, ry, cx);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) ds[4 * half + i][j] = 2.f * sum2(s[i][j]);
+            }
             f2 d[4][8];
-            dot_half<LDS_, LDS_>(d, LOCAL ? sX : sM, sO, LOCAL ? 16 : R / 4, half, ry, cx);
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float s = sum2(d[i][j]);
-                    ds[4 * half + i][j] = LOCAL ? 4.f * s * s * s : 2.f * s;
-                }
             dot_half<kLd, kLd>(d, sYo, sY, 16, half, ry, cx);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
