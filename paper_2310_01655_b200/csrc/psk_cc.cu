@@ -18,7 +18,8 @@ CcWorkspace cc_workspace(const Dims& d, bool backward) {
     w.Mq = off;  off += align_up(rows * d.r * sizeof(float));
     w.Mk = off;  off += align_up(rows * d.r * sizeof(float));
     w.Zst = off; off += align_up(st);
-    if (d.bf16) { w.Vt = off; off += align_up(rows * 64 * sizeof(float)); }      // fp32 values are read where the caller has them
+    // fp32 values are read where the caller has them, unless the forward writes over them
+    if (d.bf16 || !backward) { w.Vt = off; off += align_up(rows * 64 * sizeof(float)); }
     if (backward) {
         w.E = off;   off += align_up(rows * cc::kLd * sizeof(float));
         w.Rst = off; off += align_up(st);
@@ -580,31 +581,35 @@ cudaError_t launch_dphi(const Dims& d, const float* Mown, const float* Moth, con
     return launch_dphi_ng<T, R, false, NG>(d, Mown, Moth, yown, yoth, S, Xown, Xoth, kside, dM, dXl, s, launches);
 }
 
-// [V | 1] rows: the caller's fp32 values as they are, or (bf16 storage) an fp32 copy in scratch.
+// [V | 1] rows: the caller's fp32 values as they are, or an fp32 copy in scratch: for bf16 storage, and where the
+// output O (null: none that is written while V is read) may lie over V, which other rows' CTAs still read.
 template <typename T>
-cudaError_t value_rows(const Dims& d, const T* V, float* Vt, cc::YRows* y, cudaStream_t s, int* launches) {
+cudaError_t value_rows(const Dims& d, const T* V, const T* O, float* Vt, cc::YRows* y, cudaStream_t s, int* launches) {
     Slice sl{d.H, d.sb, d.sh, d.sn};
     if constexpr (sizeof(T) == 4) {
-        *y = cc::YRows{V, sl, 1};
-        return cudaSuccess;
-    } else {
-        const int rows = d.BH() * d.n;
-        prof_begin("rows_prep_kernel", s);
-        launch_pdl(rows_prep_kernel<T>, (rows + 15) / 16, 256, 0, s, sl, d.n, rows, 0, V, nullptr, nullptr, nullptr, Vt);
-        prof_end(s);
-        ++*launches;
-        *y = cc::YRows{Vt, Slice{d.H, (int64_t)d.H * d.n * 64, (int64_t)d.n * 64, 64}, 1};
-        return cudaGetLastError();
+        const uintptr_t v = reinterpret_cast<uintptr_t>(V), o = reinterpret_cast<uintptr_t>(O);
+        const uintptr_t span = ((d.B - 1) * d.sb + (d.H - 1) * d.sh + (d.n - 1) * d.sn + 64) * sizeof(T);
+        if (O == nullptr || v + span <= o || o + span <= v) {
+            *y = cc::YRows{V, sl, 1};
+            return cudaSuccess;
+        }
     }
+    const int rows = d.BH() * d.n;
+    prof_begin("rows_prep_kernel", s);
+    launch_pdl(rows_prep_kernel<T>, (rows + 15) / 16, 256, 0, s, sl, d.n, rows, 0, V, nullptr, nullptr, nullptr, Vt);
+    prof_end(s);
+    ++*launches;
+    *y = cc::YRows{Vt, Slice{d.H, (int64_t)d.H * d.n * 64, (int64_t)d.n * 64, 64}, 1};
+    return cudaGetLastError();
 }
 
 // Half sketches, value rows and prefix states: what the forward needs, and the backward again.
 template <typename T, int R>
-cudaError_t prefix_states(const Dims& d, const T* Q, const T* K, const T* V, const T* G1, const T* G2, char* ws,
+cudaError_t prefix_states(const Dims& d, const T* Q, const T* K, const T* V, const T* G1, const T* G2, const T* O, char* ws,
                           const CcWorkspace& w, cc::YRows* y, cudaStream_t s, int* launches) {
     float* Mq = (float*)(ws + w.Mq); float* Mk = (float*)(ws + w.Mk);
     PSK_TRY((launch_sketch<T, R>(d, Q, K, G1, G2, Mq, Mk, nullptr, d.clear_status ? (int*)(ws + w.status) : nullptr, s, launches)));
-    PSK_TRY(value_rows<T>(d, V, (float*)(ws + w.Vt), y, s, launches));
+    PSK_TRY(value_rows<T>(d, V, O, (float*)(ws + w.Vt), y, s, launches));
     return launch_states<R>(d, Mk, *y, (float*)(ws + w.Zst), false, s, launches);
 }
 
@@ -613,7 +618,7 @@ cudaError_t fwd_impl(const Dims& d, const T* Q, const T* K, const T* V, const T*
                      T* O, float* denom, char* ws, cudaStream_t s, int* launches) {
     const CcWorkspace w = cc_workspace(d, false);
     cc::YRows y;
-    PSK_TRY((prefix_states<T, R>(d, Q, K, V, G1, G2, ws, w, &y, s, launches)));
+    PSK_TRY((prefix_states<T, R>(d, Q, K, V, G1, G2, O, ws, w, &y, s, launches)));
     return launch_rows<T, R>(d, (float*)(ws + w.Mq), (float*)(ws + w.Mk), y, (float*)(ws + w.Zst), Q, K, false, O, denom, s, launches);
 }
 
@@ -672,7 +677,7 @@ cudaError_t bwd_impl(const Dims& d, const T* Q, const T* K, const T* V, const T*
     float* dXk = d.local ? (float*)(ws + w.dXk) : nullptr;
     const int rows = d.BH() * d.n;
     cc::YRows yv;
-    PSK_TRY((prefix_states<T, R>(d, Q, K, V, G1, G2, ws, w, &yv, s, launches)));
+    PSK_TRY((prefix_states<T, R>(d, Q, K, V, G1, G2, nullptr, ws, w, &yv, s, launches)));
     prof_begin("rows_prep_kernel", s);
     launch_pdl(rows_prep_kernel<T>, (rows + 15) / 16, 256, 0, s, Slice{d.H, d.sb, d.sh, d.sn}, d.n, rows, 1, nullptr, O, denom, dO, E);
     prof_end(s);
