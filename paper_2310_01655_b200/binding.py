@@ -2,7 +2,10 @@
 from __future__ import annotations
 
 import ctypes
+import importlib
 import os
+import sysconfig
+import warnings
 from ctypes import c_int, c_int32, c_int64, c_size_t, c_void_p, c_char_p, POINTER, Structure, byref
 
 import torch
@@ -104,6 +107,21 @@ def lib():
     return L
 
 
+def native_tag() -> str:
+    """The Python and torch that the native marshalling module has to be built for: it uses both through C++."""
+    return "%s torch %s cxx11abi %d" % (sysconfig.get_config_var("EXT_SUFFIX"), torch.__version__, torch._C._GLIBCXX_USE_CXX11_ABI)
+
+
+class _NoNative:
+    """In place of the native marshalling module where it cannot be loaded: leaves every call to the checks and the
+    ctypes call below it."""
+
+    def _none(self, *args):
+        return None
+
+    attn_fwd = attn_bwd = learned_fwd = learned_bwd = lt_multiply = decode_step = _none
+
+
 def _native():
     """The native marshalling module: it takes a call's arguments, allocates what the call returns and calls
     the C ABI; for arguments that need a closer look it returns None, and the checks below run."""
@@ -111,11 +129,15 @@ def _native():
     if _fast is None:
         L = lib()
         try:
-            from . import _psk_native
+            mod = importlib.import_module(__package__ + "._psk_native")
+            if mod.BUILT_FOR != native_tag():
+                raise ImportError("built for %s, not %s" % (mod.BUILT_FOR, native_tag()))
+            mod.init(*(ctypes.cast(getattr(L, name), c_void_p).value for name in _FAST_ENTRIES))
         except ImportError as e:
-            raise RuntimeError("_psk_native.so is not built: run `python -m paper_2310_01655_b200.build`") from e
-        _psk_native.init(*(ctypes.cast(getattr(L, name), c_void_p).value for name in _FAST_ENTRIES))
-        _fast = _psk_native
+            warnings.warn("_psk_native.so cannot be used (%s): calls go through ctypes and cost 15-40 us more of host time; "
+                          "`python -m paper_2310_01655_b200.build` rebuilds it" % e, RuntimeWarning, stacklevel=3)
+            mod = _NoNative()
+        _fast = mod
     return _fast
 
 

@@ -15,6 +15,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libpsk.so")
 NATIVE = os.path.join(PKG, "_psk_native.so")
+NATIVE_TAG = os.path.join(PKG, "build", "_psk_native.tag")      # what it was built for (binding.native_tag)
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -33,20 +34,35 @@ def _stale(obj, deps):
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def native_stale():
+    """Is _psk_native.so missing, older than its sources, or built for another Python or torch?"""
+    from . import binding
+    src = os.path.join(CSRC, "psk_binding.cpp")
+    try:
+        with open(NATIVE_TAG) as f:
+            tag = f.read()
+    except OSError:
+        tag = None
+    return tag != binding.native_tag() or _stale(NATIVE, [src, os.path.join(ROOT, "include", "psk.h"), __file__])
+
+
 def build_native(force=False):
     """Compile csrc/psk_binding.cpp against torch's headers; returns the running compiler or None."""
-    src = os.path.join(CSRC, "psk_binding.cpp")
-    if not (force or _stale(NATIVE, [src, os.path.join(ROOT, "include", "psk.h"), __file__])):
+    if not (force or native_stale()):
         return None
     import sysconfig
     import torch
+    from . import binding
     troot = os.path.dirname(torch.__file__)
+    os.makedirs(os.path.dirname(NATIVE_TAG), exist_ok=True)
+    if os.path.exists(NATIVE_TAG):
+        os.remove(NATIVE_TAG)                  # (written again when the compiler has succeeded)
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
-           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), '-DPSK_BUILT_FOR="%s"' % binding.native_tag(),
            "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], "-I", os.path.join(troot, "include"),
            "-I", os.path.join(troot, "include", "torch", "csrc", "api", "include"),
            "-I", os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include"),
-           src, "-o", NATIVE, "-L", os.path.join(troot, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-ltorch",
+           os.path.join(CSRC, "psk_binding.cpp"), "-o", NATIVE, "-L", os.path.join(troot, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-ltorch",
            "-lc10_cuda", "-lc10"]
     return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
 
@@ -74,6 +90,10 @@ def build(force=False, verbose=False):
         out, _ = native.communicate()
         if native.returncode != 0 or verbose:
             sys.stderr.write("== psk_binding.cpp\n%s\n" % out)
+        if native.returncode == 0:
+            from . import binding
+            with open(NATIVE_TAG, "w") as f:
+                f.write(binding.native_tag())
         failed |= native.returncode != 0
     if failed:
         raise RuntimeError("nvcc failed")

@@ -278,4 +278,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_psk_native", nullptr, -1, methods
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__psk_native(void) { return PyModule_Create(&module); }
+// BUILT_FOR: the Python and torch of the build, which binding.py compares with the running ones.
+PyMODINIT_FUNC PyInit__psk_native(void) {
+    PyObject* m = PyModule_Create(&module);
+    if (m != nullptr && PyModule_AddStringConstant(m, "BUILT_FOR", PSK_BUILT_FOR) != 0) { Py_DECREF(m); return nullptr; }
+    return m;
+}
