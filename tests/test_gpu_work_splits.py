@@ -74,3 +74,28 @@ def test_decode_steps_for_few_and_many_heads(r, dtype, B, H):
         O_ref, d_ref = orc.causal_polysketch_attention(q, k, v, g_slice(G1, hi), g_slice(G2, hi))
         check("O", torch.stack([o[bi, hi] for o, _ in rows]), O_ref, TOL[dtype])
         check("denom", torch.stack([d[bi, hi] for _, d in rows]), d_ref, TOL[dtype])
+
+
+@pytest.mark.parametrize("r,b,n,B,H", [
+    (16, 128, 1664, 2, 5), (16, 256, 512, 13, 12), (32, 128, 1408, 1, 1), (32, 256, 2816, 2, 3), (32, 128, 256, 25, 12),
+    (64, 128, 896, 1, 1), (64, 256, 1280, 4, 9), (64, 384, 1152, 8, 12),
+])
+def test_kept_states_however_they_are_dealt(r, b, n, B, H):
+    # Weights of size one instead of 10^4: the first rows' normalisers stay below 10, and what the kept O - c loses in
+    # bf16 stays below the tolerance (see above).
+    w = wl.small_workload(B=B, H=H, n=n, r=r, b=b, dtype="bf16", seed=970 + r + n)
+    inp = wl.make_inputs(w, "cuda")
+    inp["Q"] = 0.3 * inp["Q"]
+    inp["K"] = 0.3 * inp["K"]
+    Q, K, V, G1, G2, dO = (inp[k] for k in ("Q", "K", "V", "G1", "G2", "dO"))
+    shp = psk.binding.make_shape(Q, G1, r, b, flags=psk.FLAG_KEEP_STATES)
+    ws = torch.empty(psk.workspace_bytes(shp, True), dtype=torch.uint8, device="cuda")
+    O, den = psk.causal_attn_fwd(Q, K, V, G1, G2, b, workspace=ws, flags=psk.FLAG_KEEP_STATES)
+    grads = psk.causal_attn_bwd(Q, K, V, G1, G2, O, den, dO, b, workspace=ws, flags=psk.FLAG_KEEP_STATES)
+    assert psk.check(ws) == 0
+    # dV is made of Q, K, dO and the normaliser alone
+    assert torch.equal(grads[2], psk.causal_attn_bwd(Q, K, V, G1, G2, O, den, dO, b)[2])
+    for bi, hi in {(0, 0), (B - 1, H - 1)}:
+        ref = tuple(oracle_forward(inp, bi, hi, b)) + tuple(oracle_backward(inp, bi, hi, b))
+        for name, got, want in zip(("O", "denom", "dQ", "dK", "dV"), (O, den) + tuple(grads), ref):
+            check(name, got[bi, hi], want, TOL["bf16"])
