@@ -108,20 +108,11 @@ namespace {
 // weights, epilogue).  Warp 4: one thread issues every TMA load and every MMA; the two sides meet
 // only at mbarriers, so the rows never wait for an issue sequence and the tensor pipe runs ahead.
 // ---------------------------------------------------------------------------
-#ifdef PSK_FWD_TRACE
-// scratch builds only: clock stamps of one CTA, one slot per (event, index)
-__device__ long long g_ftr[64 * 16];
-#define FTR(ev, idx) do { if (blockIdx.x == 1 && blockIdx.y == 5 && blockIdx.z == 3) g_ftr[(ev) * 16 + (idx)] = clock64(); } while (0)
-#else
-#define FTR(ev, idx)
-#endif
-
 // Warps 0-3: rows.  Warp 4: one thread issues every TMA load and every MMA.  (A second issuing
 // thread in a sixth warp for the odd state chunks was measured: 1 % faster, and the two threads'
 // MMAs reach the accumulator in an order that changes from run to run, so results were no longer
 // bitwise reproducible.  Not kept.)
 constexpr int kOutThreads = 160;
-#define PSK_OUT_ISSUERS 1
 constexpr int kZStages = 4;                     // three in the shared region + the query tile's buffer
 constexpr uint32_t kZStageBytes = 16384;        // two [64 features x 128 B] boxes: columns 0..63, 64..79
 constexpr int kFeatBufs = kZStages;             // feature staging buffers in tensor memory, 32 columns each:
@@ -193,7 +184,6 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     const int tid = threadIdx.x, warp = tid / 32, tau = blockIdx.x, l = blockIdx.y, bh = blockIdx.z;
     const int hi = bh % H, bi = bh / H;
     const int g = g_heads == 1 ? 0 : hi;
-    FTR(0, 0);
     const int row0 = l * b + tau * 128;
     // Non-causal (Section 3, first formula): one state per head, the sum over the whole sequence,
     // multiplies every row tile, and there are no same-block tiles.
@@ -234,7 +224,6 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tm = tmem_slot;
-    if (tid == 0) FTR(1, 0);
     // tensor-memory columns: sketch accumulators, feature staging buffers, scores and packed
     // weights all live in [0, 128), each consumed before the next is produced; then the output
     // accumulator (64 + the prefix normaliser's 16) and the same-block row sums (16)
@@ -248,25 +237,23 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     // and nothing else, and one barrier says that the features are staged (an arrival per warp) and the
     // state rows are there (144 heads x 8192, r = 32, b = 256: 351 us with two barriers and an arrival per
     // thread, now 335).  (The stages are refilled by the rows' side, which learns first that a buffer is free.)
-    auto issue_chunks = [&](int first, int step) {
+    auto issue_chunks = [&]() {
         constexpr uint32_t idesc = idesc_bf16(128, 80, false, true);
         const uint64_t zd0 = smem_desc(smem_u32(smem + L::Z), 8192, 1024, kSwz128);
         const uint64_t zdq = smem_desc(smem_u32(smem + L::Z3), 8192, 1024, kSwz128);
 #pragma unroll 1
-        for (int C = first; C < F::NC && ok; C += step) {
+        for (int C = 0; C < F::NC && ok; ++C) {
             const int s = C % kZStages;
             const uint32_t par = (C / kZStages) & 1;
             const int ksteps = (F::FK - C * 64) >= 64 ? 4 : (F::FK - C * 64) / 16;
             const uint64_t zd = s == kZStages - 1 ? zdq : desc_off(zd0, s * kZStageBytes);
             const uint32_t at = tm + cA + s * 32;
             ok = mbar_spin(&bar_feat[s], par, status, kErrTma);          // features staged and state rows there
-            FTR(5, C);
             tc_fence_after();
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 if (k < ksteps) umma_ts(tm + cO, at + k * 8, desc_off(zd, k * 2048), idesc, (C > 0 || k > 0) ? 1u : 0u);
             umma_commit(&bar_a[s]);
-            FTR(6, C);
         }
     };
 
@@ -290,11 +277,9 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                 }
             }
             ok = mbar_spin(&bar_q, 0, status, kErrTma);
-            FTR(2, 0);
             tc_fence_after();
             issue_sketch<R>(tm + cSk, smem + L::Q, smem + L::G);
             umma_commit(&bar_sk);
-            FTR(3, 0);
             if constexpr (LIN && LOCAL) {
                 ok = ok && mbar_spin(&bar_sk, 0, status, kErrMma);
                 mbar_expect_tx(&bar_q, 16384);
@@ -307,7 +292,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                 tma_load_3d(smem + L::zstage(kZStages - 1), &mapZ, 0, (kZStages - 1) * 64, blk, &bar_feat[kZStages - 1]);
                 tma_load_3d(smem + L::zstage(kZStages - 1) + 8192, &mapZ, 64, (kZStages - 1) * 64, blk, &bar_feat[kZStages - 1]);
             }
-            if (has_prefix) issue_chunks(0, PSK_OUT_ISSUERS);     // earlier blocks: features x prefix state chunks
+            if (has_prefix) issue_chunks();     // earlier blocks: features x prefix state chunks
             const int tp_last = noncausal ? -1 : tau;
             if (has_prefix && !noncausal) {
                 // the first key/value tiles of the same block, each into its stage as soon as the last
@@ -348,7 +333,6 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                     if (nx <= tp_last) { load_k(nx, nx % L::kSets); load_v(nx, nx % L::kSets); }
                 }
                 ok = ok && mbar_spin(&bar_kv[p], (tp / L::kSets) & 1, status, kErrTma);
-                FTR(7, tp);
                 tc_fence_after();
                 constexpr uint32_t idesc_s = idesc_bf16(128, 128, false, false);
                 const uint64_t kr = smem_desc(smem_u32(smem + (p ? kK1 : kK0)), 0, 1024, kSwz128);
@@ -370,9 +354,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                             umma_ss(tm + cS, desc_off(qd, (g == 1 ? kLo : 0) + k * 32), desc_off(kr, (g == 2 ? kLo : 0) + k * 32), idesc_s, (g > 0 || k > 0) ? 1u : 0u);
                 }
                 umma_commit(&bar_s);
-                FTR(10, tp);
                 ok = ok && mbar_spin(&bar_p, tp & 1, status, kErrMma);
-                FTR(11, tp);
                 tc_fence_after();
                 {
                     // numerator += W V; row sums += W 1 (the weights exactly as the value GEMM sees them)
@@ -385,7 +367,6 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                         umma_ts(tm + cN, tm + cW + k * 8, desc_off(od, k * 512), idesc1, k > 0 ? 1u : acc1);
                     }
                     umma_commit(&bar_pv);
-                    FTR(12, tp);
                 }
             }
         }
@@ -393,7 +374,6 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
         // ================================= rows =================================
         const uint32_t lane_tm = tm + ((uint32_t)(warp * 32) << 16);
         ok = mbar_wait(&bar_sk, 0, status, kErrMma);
-        if (tid == 0) FTR(20, 0);
         tc_fence_after();
         float mq[R];
         read_half_sketch<R>(lane_tm + cSk, mq, 1.f, lin != 0);
@@ -404,7 +384,6 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
         tc_fence_before();
         __syncwarp();
         if (tid % 32 == 0) mbar_arrive(&bar_go);
-        if (tid == 0) FTR(21, 0);
 
         if (has_prefix) {
             if constexpr (F::kCirc) {
@@ -422,7 +401,6 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                             tma_load_3d(smem + L::zstage(buf) + 8192, &mapZ, 64, C * 64, blk, &bar_feat[buf]);
                         }
                     }
-                    if (tid == 0) FTR(22, C);
                     uint32_t pk[32];
                     gen.chunk(pk);
                     tmem_st32(lane_tm + cA + buf * 32, pk);
@@ -430,7 +408,6 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                     tc_fence_before();
                     __syncwarp();
                     if (tid % 32 == 0) mbar_arrive(&bar_feat[buf]);
-                    if (tid == 0) FTR(23, C);
                 }
             } else {
                 PackedM<R> pmq;
@@ -464,7 +441,6 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
 #pragma unroll 1
         for (int tp = 0; tp <= tp_last; ++tp) {
             ok = ok && mbar_wait(&bar_s, tp & 1, status, kErrMma);
-            if (tid == 0) FTR(26, tp);
             tc_fence_after();
             // weights = squared scores (lower triangle on the diagonal tile), packed to bf16 over
             // columns whose fp32 contents have already been read
@@ -494,14 +470,12 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             tc_fence_before();
             __syncwarp();
             if (tid % 32 == 0) mbar_arrive(&bar_p);
-            if (tid == 0) FTR(27, tp);
         }
         if (noncausal)      // the last chunk's MMAs (no same-block tiles follow them)
             ok = ok && mbar_wait(&bar_a[(F::NC - 1) % kFeatBufs], ((F::NC - 1) / kFeatBufs) & 1, status, kErrMma);
         else
             ok = ok && mbar_wait(&bar_pv, tau & 1, status, kErrMma);
         tc_fence_after();
-        if (tid == 0) FTR(28, 0);
 
         // ---- epilogue ----
         float acc[64];
@@ -594,11 +568,9 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             e65h[row] = y * inv - ec;
         }
     }
-    if (tid == 0) FTR(29, 0);
     tc_fence_before();
     __syncthreads();
     if (warp == 4) tmem_dealloc(tm, 256);
-    if (tid == 0) FTR(30, 0);
 }
 
 // Centre of the values of a head: cmean[bh][c] = mean of V[bh][i][c] over at most 1024 rows i
@@ -738,14 +710,6 @@ cudaError_t fwd_impl(const Dims& d, const void* Q, const void* K, const void* V,
 }
 
 }  // namespace
-
-#ifdef PSK_FWD_TRACE
-extern "C" int psk_debug_ftrace(long long* host) {
-    cudaDeviceSynchronize();
-    cudaMemcpyFromSymbol(host, g_ftr, sizeof(long long) * 64 * 16);
-    return 64 * 16;
-}
-#endif
 
 bool tc_supported(const Dims& d, bool backward) {
     (void)backward;
