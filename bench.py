@@ -70,8 +70,8 @@ def kernel_flops_per_head_token(name, w, local=False):
         tile_fwd = 2 * 128 * h + 2 * 128 * h
         tile_bwd = 2 * 128 * h + 2 * 128 * h + 2 * 128 * 64
     table.update({
-        # (r = 64, many heads: the feature tiles are dealt to six CTAs, which each redo the half sketch)
-        "tc_state_kernel": sk * (1 if r <= 32 else 6) + 2 * FP * 80,
+        # (with these workloads' heads the feature tiles are dealt to one CTA, r = 64: nine, which each redo the half sketch)
+        "tc_state_kernel": sk * (1 if r <= 32 else 9) + 2 * FP * 80,
         "tc_fwd_out_kernel": sk + 2 * FK * 80 + other * tile_fwd,
         "tc_bwd_recompute_kernel": sk + 2 * FK * 80 + other * tile_fwd,
         "tc_bwd_q_kernel": 2 * sk + 2 * FK * 80 + other * tile_bwd + 2 * 2 * r * 64,

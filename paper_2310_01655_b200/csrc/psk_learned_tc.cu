@@ -964,7 +964,7 @@ ltc_dense_bwd_norm_kernel(const __grid_constant__ CUtensorMap mN, const __grid_c
 // ---------------------------------------------------------------------------
 // Mean and 1 / sigma of every row (st0), and (n0 != nullptr: the backward) n0 = (x - mean) / sigma as hi + lo
 // rows.  Eight lanes per row, eight columns each, two rows' loads in flight per lane: six shuffles serve four rows.
-// (A whole warp per row took 67 us for 393 216 rows, ten shuffles each; now 20.)
+// (A whole warp per row took 67 us for 393 216 rows, ten shuffles each; now 26.)
 constexpr int kLnRows = 64;                            // rows per CTA
 __device__ __forceinline__ void unpack8(const uint4& q, float (&v)[8]) {
     const uint32_t w[4] = {q.x, q.y, q.z, q.w};

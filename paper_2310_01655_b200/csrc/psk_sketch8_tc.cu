@@ -386,7 +386,8 @@ bool sk8_maps(const Dims& d, char* bank, Sk8Maps* m) {
     return tc_map_3d(&m->W1, W1, 128, 64, d.g_heads, 64, 64) && tc_map_3d(&m->W2, W2, 64, 64, d.g_heads, 64, 64);
 }
 
-// CTAs along a head's tiles: about four rounds of the GPU's 296 places in all, four tiles each or more
+// CTAs along a head's tiles: about four rounds of the GPU's 296 places in all, and no more than a quarter of the tiles
+// (rounded up), so that the matrices are loaded for several tiles wherever there are several
 inline dim3 sk8_grid(const Dims& d) {
     const int tiles = d.n / 128, want = (1184 + d.BH() - 1) / d.BH(), most = (tiles + 3) / 4;
     const int c = want < most ? want : most;
