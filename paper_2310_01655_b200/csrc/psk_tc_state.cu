@@ -42,13 +42,13 @@ constexpr int kModeFirst = 2;          // run 0: both; the other runs: the total
 // What bounds a walk of r = 32: the generators' instructions and their fetch (20 % of the warps wait for an
 // instruction), and at short blocks the store warpgroup, one body for all tiles with a bulk copy out (144 heads x
 // 8192, b = 256: 318 us unrolled and with copies by the lanes, now 234).
-// grid (BH).  Warp roles:
+// grid (BH, runs, shares).  Warp roles:
 //   NWG generator warpgroups  thread = token: read the half sketches, write their feature tiles
 //                             (dealt in turn) as MN-major A operands into shared memory; one of them also
 //                             puts the half sketches where their rows were;
 //   1 store warpgroup         thread = feature row: at block boundaries reads the accumulators,
 //                             centres, rounds and stores them;
-//   1 feeder warp             one thread issues every TMA load, sketch GEMM and state GEMM.
+//   2 feeder warps            one thread each: every TMA load and sketch GEMM; every state GEMM.
 // Stored layout S[blk][FP][80]: one row per feature, 64 state columns, the last column, zeros.
 // ---------------------------------------------------------------------------
 template <int R, int NWG>
@@ -658,10 +658,13 @@ cudaError_t launch_split(const Dims& d, const CUtensorMap& mX, const CUtensorMap
                          const StateArgs& a, int* status, cudaStream_t s, int* launches) {
     using P = StateSplit<R, SPLIT>;
     constexpr size_t smem = StateSmem<R, P::NWG>::total + 1024;
-    // A long walk is better spread over the SMs by an ordinary launch: started early, its CTAs settle on the SMs
-    // that happen to be free first, several to a pair (r = 64, 48 heads of 128 tiles: 6.93 against 7.33 ms a step);
-    // for a short one the launch itself counts more (48 heads of 21 tiles: 374 -> 361 us a step).
-    const bool early = d.n / 128 / a.nseg <= 24;
+    // Programmatic dependence saves a short walk 2 to 6 us (forward of 12 heads x 16 512, two passes over 11 runs: 185 -> 180 us;
+    // 12 heads x 1024, training: 88 -> 83).  But CTAs that start early settle on the SMs that happen to be free, shares of a head
+    // side by side, and neighbours that run different code are slow (StateSplit): where the shares fill the GPU that costs a
+    // training step 3 to 25 % (r = 32, 48 heads x 1024, 2048, 2688: 135, 214, 278 us against 149, 250, 308; r = 64, 16 heads
+    // x 2048: 293 against 366; 108 CTAs: 170 against 178; 60 CTAs gain).  Long walks (over 24 tiles; at 64, r = 32, 48 heads: 715
+    // against 776) take longer than the launch either way.
+    const bool early = d.n / 128 / a.nseg <= 24 && (SPLIT == 1 || (long)d.BH() * a.runs * SPLIT <= 74);
     auto kern = a.nseg > 1 || a.mode != kModePrefix ? tc_state_kernel<R, SPLIT, true> : tc_state_kernel<R, SPLIT, false>;
     PSK_TRY((set_smem(kern, smem)));
     prof_begin(a.mode == kModePrefix ? "tc_state_kernel" : "tc_state_total_kernel", s);
