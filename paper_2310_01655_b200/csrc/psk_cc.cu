@@ -533,7 +533,9 @@ cudaError_t launch_states(const Dims& d, const float* M, const cc::YRows& y, flo
 // Groups of 64 threads per CTA of the row kernels: two, so that two CTAs share an SM and one's
 // loads and final sums overlap the other's products, wherever their shared memory allows it (r <= 32,
 // sketched weights) and there are CTAs enough for every SM; else as many as fit one CTA, which also
-// spreads a few rows' work over the most warps.
+// spreads a few rows' work over the most warps.  (Training, four groups against two: r = 16, 128 CTAs 171 and 226 us, 320:
+// 308 and 310, 640: 465 and 445, 1536: 998 and 911; r = 32, 128: 333 and 424, 320: 608 and 633, 640: 967 and 962,
+// 1536: 2084 and 2018.)
 inline bool two_per_sm(const Dims& d) { return (long)d.BH() * (d.n / 64) >= 2 * 148; }
 
 template <typename T, int R, bool LOCAL, int NG>
