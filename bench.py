@@ -554,7 +554,7 @@ def main():
         tensor = name.startswith("tc_")
         peak = pk["bf16_sustained"] if tensor else ALU_PEAK_TFLOPS
         achieved = (fl * w.head_tokens / ((tot / cnt) / 1e3) / 1e12) if fl else None
-        # DRAM bytes per launch: ncu capture on the profiling-sized slice, scaled by head-tokens
+        # DRAM bytes per launch: ncu capture on 96 heads x 8192, scaled by head-tokens
         traffic = None
         tname = "dram_traffic_c2s_local_exact.json" if args.local_exact else "dram_traffic_c2s.json"
         tpath = os.path.join(ROOT, "profiles", tname)
@@ -566,7 +566,7 @@ def main():
                 "unit": "TFLOP/s", "frac": (achieved / peak) if achieved else None,
                 "frac_sustained": (achieved / pk["bf16_sustained"]) if (achieved and tensor) else None,
                 "frac_burst": (achieved / pk["bf16_burst"]) if (achieved and tensor) else None, "traffic": traffic,
-                "traffic_source": ("profiles/%s (ncu on the c2s slice, scaled by head-tokens)" % tname) if traffic else None,
+                "traffic_source": ("profiles/%s (ncu on 786432 head-tokens, scaled)" % tname) if traffic else None,
                 "flops_per_launch": fl * w.head_tokens if fl else None,
                 "peak_source": (pk["source"] + " (sustained bf16)") if tensor else "derived: 148 SM x 128 FMA x 1.965 GHz",
                 "launches": cnt, "avg_ms": tot / cnt, "share_of_kernel_time": tot / total_kernel_ms}

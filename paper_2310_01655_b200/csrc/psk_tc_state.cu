@@ -39,8 +39,9 @@ constexpr int kModeFirst = 2;          // run 0: both; the other runs: the total
 //   otherwise sketch every other-side tile again, once per row tile that meets it.  (Rows of 48 heads x 16384,
 //   r = 64: forward 1050 -> 554 us, query side 1702 -> 1288, key side 2327 -> 2112; of 384 heads x 32768,
 //   r = 32: 4409 -> 3916, 5031 -> 4776, 6249 -> 5867; the walk itself pays 5 to 20 % for it.)
-// What bounds a walk of r = 32: the generators' instructions and their fetch (20 % of the warps wait for an
-// instruction), and at short blocks the store warpgroup, one body for all tiles with a bulk copy out (144 heads x
+// What bounds a walk of r = 32: the shared-memory path, which the generators' tiles, the stores on their way out and the
+// MMAs' operands share (96 heads x 8192, b = 256: 82 % of its cycles on the SMs in use, issue slots 51 %, tensor
+// pipe 27 %), and at short blocks the store warpgroup, one body for all tiles with a bulk copy out (144 heads x
 // 8192, b = 256: 318 us unrolled and with copies by the lanes, now 234).
 // grid (BH, runs, shares).  Warp roles:
 //   NWG generator warpgroups  thread = token: read the half sketches, write their feature tiles
