@@ -248,7 +248,7 @@ ltc_dense_norm_kernel(Slice sl, const bf16* __restrict__ X, size_t row0, int til
     __shared__ uint32_t tm_slot;
     __shared__ __align__(16) float sv[kVec];
     __shared__ float2 s_part[2][2][128];
-    const int tid = threadIdx.x, warp = tid / 32, net = blockIdx.y;
+    const int tid = threadIdx.x, warp = warp_index(), net = blockIdx.y;
     if (tid == 0) {
         cta_giveup_init();
         mbar_init(&bar_w, 1);
@@ -269,7 +269,7 @@ ltc_dense_norm_kernel(Slice sl, const bf16* __restrict__ X, size_t row0, int til
     if (warp >= 16) {
         // ============================ issuing threads ============================
         const int slot = warp - 16;
-        if (tid % 32 == 0) {
+        if (elect_one()) {
             if (slot == 0) {
                 mbar_expect_tx(&bar_w, L::W2t);
                 load_image(W, bank + (size_t)net * kBankBytes, L::W2t, &bar_w);
@@ -528,7 +528,7 @@ ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant_
     __shared__ uint32_t tm_slot;
     __shared__ __align__(16) float sb3[256];
     __shared__ float scs[R], sb2[R];
-    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, net = blockIdx.y;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid % 32, net = blockIdx.y;
     const int nt = (tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x, steps = nt * NH;
     const CUtensorMap* mA = net ? &mA1 : &mA0;
     const CUtensorMap* mD = net ? &mD1 : &mD0;
@@ -552,7 +552,7 @@ ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant_
     constexpr uint32_t cDa2 = 256, cW4 = 256 + 32, cW3 = cW4 + 64;
     auto tile_at = [&](int i) { return (int)blockIdx.x + i * (int)gridDim.x; };
     if (warp == 16) {
-        if (lane == 0) {
+        if (elect_one()) {
             auto load = [&](int i) {
                 uint8_t* dst = smem + B::In + (i % 3) * B::kIn;
                 mbar_expect_tx(&bar_ld[i % 3], B::kIn);
@@ -758,7 +758,7 @@ ltc_dense_bwd_norm_kernel(const __grid_constant__ CUtensorMap mN, const __grid_c
     __shared__ uint64_t bar_w, bar_ld[2], bar_lo, bar_s[2], bar_rd[2], bar_t, bar_free;
     __shared__ uint32_t tm_slot;
     __shared__ __align__(16) float sb1[256];
-    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, net = blockIdx.y;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid % 32, net = blockIdx.y;
     const int nt = (tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x, steps = nt * NH;
     const CUtensorMap* mD = net ? &mD1 : &mD0;
     if (tid == 0) {
@@ -779,7 +779,7 @@ ltc_dense_bwd_norm_kernel(const __grid_constant__ CUtensorMap mN, const __grid_c
     constexpr uint32_t cN0 = 256, cW2 = cN0 + 64, cW1 = cW2 + 64;
     auto tile_at = [&](int i) { return (int)blockIdx.x + i * (int)gridDim.x; };
     if (warp == 16) {
-        if (lane == 0) {
+        if (elect_one()) {
             auto load = [&](int i) {
                 uint8_t* dst = smem + B::In + (i & 1) * B::kIn;
                 mbar_expect_tx(&bar_ld[i & 1], B::kIn);

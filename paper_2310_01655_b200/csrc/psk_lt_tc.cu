@@ -28,7 +28,7 @@ lt_tc_state_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_consta
     uint8_t* smem = align1024(smem_raw);
     __shared__ uint64_t bar_full[2], bar_free[2], bar_acc;
     __shared__ uint32_t tm_slot;
-    const int tid = threadIdx.x, warp = tid / 32;
+    const int tid = threadIdx.x, warp = warp_index();
     const int f0 = blockIdx.x * 128, bt = blockIdx.y;
     const int NT = (t - 1) * tpb;               // the last block's state is never used
     if (tid == 0) {
@@ -54,7 +54,7 @@ lt_tc_state_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_consta
     if (tid == 0 && NT > 0) { load(0); if (NT > 1) load(1); }
     bool ok = true;
     for (int l = 0; l + 1 < t; ++l) {
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             constexpr uint32_t idesc = idesc_bf16(128, 64, true, true);
             for (int tt = 0; tt < tpb && ok; ++tt) {
                 const int j = l * tpb + tt, s = j & 1;
@@ -128,7 +128,7 @@ lt_tc_rows_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constan
     uint8_t* smem = align1024(smem_raw);
     __shared__ uint64_t bar_full[L::kStages], bar_free[L::kStages], bar_c, bar_s, bar_p[TPB], bar_o[TPB];
     __shared__ uint32_t tm_slot;
-    const int tid = threadIdx.x, warp = tid / 32;
+    const int tid = threadIdx.x, warp = warp_index();
     const int l = blockIdx.x, bt = blockIdx.y;
     const int row0 = l * TPB * 128, nch = m / 64;
     if (tid == 0) {
@@ -146,7 +146,7 @@ lt_tc_rows_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constan
     const uint32_t tm = tm_slot;
     // scores of row tile w against tile tp <= w
     auto scores = [](int w, int tp) { return L::cS + 128u * (w * (w + 1) / 2 + tp); };
-    if (tid == 128 * TPB) {
+    if (warp == 4 * TPB && elect_one()) {
         auto load = [&](int c) {
             const int s = c % L::kStages;
             uint8_t* st = smem + s * L::kStage;

@@ -115,7 +115,7 @@ sk8_tc_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     uint8_t* smem = align1024(smem_raw);
     __shared__ uint64_t bar_w, bar_x[2], bar_mma;
     __shared__ uint32_t tm_slot;
-    const int tid = threadIdx.x, warp = tid / 32;
+    const int tid = threadIdx.x, warp = warp_index();
     const int bh = blockIdx.y, hi_ = bh % H, bi = bh / H;
     const int g = g_heads == 1 ? 0 : hi_;
     auto load_x = [&](int tile, int b) {
@@ -144,7 +144,7 @@ sk8_tc_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
         const int b = it & 1;
         const uint32_t x = L::X + b * 16384;
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             // the other buffer: the previous tile's result has left it
             if (it > 0) bulk_wait_read();
             if (tile + (int)gridDim.x < tiles) load_x(tile + gridDim.x, b ^ 1);
@@ -159,7 +159,7 @@ sk8_tc_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
-        if (tid == 0) { tc_fence_after(); issue_second<R>(tm + 128, smem); umma_commit(&bar_mma); }
+        if (warp == 0 && elect_one()) { tc_fence_after(); issue_second<R>(tm + 128, smem); umma_commit(&bar_mma); }
         ok = mbar_wait(&bar_mma, 1, status, kErrMma) && ok;
         tc_fence_after();
         // M = C1 * C2 / sqrt(R), written as the row [hi | lo | 0] over the X tile (dead since GEMM 1)
@@ -178,12 +178,12 @@ sk8_tc_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
-        if (tid == 0 && ok) {
+        if (warp == 0 && elect_one() && ok) {
             tma_store_tile(&mapS, smem + x, tile * 128, hi_, bi);
             bulk_commit();
         }
     }
-    if (tid == 0) bulk_wait_read();
+    if (warp == 0 && elect_one()) bulk_wait_read();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tm, 256);
@@ -201,7 +201,7 @@ sk8_tc_bwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     uint8_t* smem = align1024(smem_raw);
     __shared__ uint64_t bar_w, bar_x[2], bar_d, bar_mma;
     __shared__ uint32_t tm_slot;
-    const int tid = threadIdx.x, warp = tid / 32;
+    const int tid = threadIdx.x, warp = warp_index();
     const int bh = blockIdx.y, hi_ = bh % H, bi = bh / H;
     const int g = g_heads == 1 ? 0 : hi_;
     auto load_x = [&](int tile, int b) {
@@ -237,7 +237,7 @@ sk8_tc_bwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
         const int b = it & 1;
         const uint32_t x = L::X + b * 16384;
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             // the other buffer: the previous tile's result has left it
             if (it > 0) bulk_wait_read();
             if (tile + (int)gridDim.x < tiles) load_x(tile + gridDim.x, b ^ 1);
@@ -252,7 +252,7 @@ sk8_tc_bwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
-        if (tid == 0) { tc_fence_after(); issue_second<R>(tm + cD2, smem); umma_commit(&bar_mma); }
+        if (warp == 0 && elect_one()) { tc_fence_after(); issue_second<R>(tm + cD2, smem); umma_commit(&bar_mma); }
         ok = mbar_wait(&bar_mma, uses++ & 1, status, kErrMma) && ok;
         tc_fence_after();
         {
@@ -291,7 +291,7 @@ sk8_tc_bwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             // [dM1 | dM2] = [dC1 | dC2] W2^T: W2's tile read K-major (its columns are this GEMM's contraction)
             tc_fence_after();
             constexpr uint32_t idesc = idesc_bf16(128, 64, false, false);
@@ -303,7 +303,7 @@ sk8_tc_bwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         }
         ok = mbar_wait(&bar_mma, uses++ & 1, status, kErrMma) && ok;
         tc_fence_after();
-        if (tid == 0 && tile + (int)gridDim.x < tiles) load_d(tile + gridDim.x);      // the product that read this tile's has completed
+        if (warp == 0 && elect_one() && tile + (int)gridDim.x < tiles) load_d(tile + gridDim.x);      // the product that read this tile's has completed
         {
             // [dA1 | dA2 | dB1 | dB2] = [dM1*A2 | dM1*A1 | dM2*B2 | dM2*B1] / sqrt(R) over the hi/lo tiles (dead since GEMM 2)
 #pragma unroll
@@ -334,7 +334,7 @@ sk8_tc_bwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             // dX = [dA1 | dA2 | dB1 | dB2] W1^T: W1's two column groups read K-major
             tc_fence_after();
             constexpr uint32_t idesc = idesc_bf16(128, 64, false, false);
@@ -367,12 +367,12 @@ sk8_tc_bwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
-        if (tid == 0 && ok) {
+        if (warp == 0 && elect_one() && ok) {
             tma_store_tile(&mapDX, smem + x, tile * 128, hi_, bi);
             bulk_commit();
         }
     }
-    if (tid == 0) bulk_wait_read();
+    if (warp == 0 && elect_one()) bulk_wait_read();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tm, 256);

@@ -181,7 +181,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     __shared__ uint64_t bar_feat[kFeatBufs], bar_a[kFeatBufs];
     __shared__ uint32_t tmem_slot;
     __shared__ float cm[64];
-    const int tid = threadIdx.x, warp = tid / 32, tau = blockIdx.x, l = blockIdx.y, bh = blockIdx.z;
+    const int tid = threadIdx.x, warp = warp_index(), tau = blockIdx.x, l = blockIdx.y, bh = blockIdx.z;
     const int hi = bh % H, bi = bh / H;
     const int g = g_heads == 1 ? 0 : hi;
     const int row0 = l * b + tau * 128;
@@ -259,7 +259,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
 
     if (warp == 4) {
         // ================================ issuer ================================
-        if (tid == 128) {
+        if (elect_one()) {
             constexpr uint32_t kK0 = L::zstage(L::stage_k(0)), kK1 = L::zstage(L::stage_k(1)), kV0 = L::zstage(L::stage_v(0)), kV1 = L::zstage(L::stage_v(1));
             auto load_k = [&](int tp, int p) {         // (with the value tile's bytes expected too)
                 mbar_expect_tx(&bar_kv[p], (L::NT + 1) * 16384);

@@ -180,7 +180,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     uint8_t* smem = align1024(smem_raw);
     __shared__ uint64_t bar_own, bar_xoth, bar_yoth, bar_mma, bar_phi[2], bar_box[2];
     __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid / 32, tau = blockIdx.x, l = blockIdx.y, bh = blockIdx.z;
+    const int tid = threadIdx.x, warp = warp_index(), tau = blockIdx.x, l = blockIdx.y, bh = blockIdx.z;
     const int hi = bh % H, bi = bh / H;
     const int g = g_heads == 1 ? 0 : hi;
     const int row0 = l * b + tau * 128;
@@ -275,7 +275,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
 
     // ---- phase A: half sketch of the own rows ----
     ok = mbar_wait(&bar_own, 0, status, kErrTma);
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
         tc_fence_after();
         issue_sketch<R>(tm + cSk, smem + L::Xown, smem + L::G);
         umma_commit(&bar_mma);
@@ -387,18 +387,18 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             ok = ok && mbar_wait(&bar_box[0], 0, status, kErrTma);
             tc_fence_before();
             __syncthreads();
-            if (tid == 0) {
+            if (warp == 0 && elect_one()) {
                 tc_fence_after();
                 issue_chunk(0);
             }
 #pragma unroll 1
-            for (int C = 0; C < F::NC && ok; ++C) {
+            for (int C = 0; C < F::NC; ++C) {          // (no early exit: a wait that gave up makes the later ones return at once)
                 const int buf = C & 1;
                 // Key side: chunk C's MMAs read the one staging buffer, so they must have completed
                 // before chunk C+1's features go in; query side: chunk C+1 is issued first and runs
                 // behind chunk C.
                 if constexpr (!QSIDE) {
-                    ok = mbar_wait(&bar_phi[buf], (C / 2) & 1, status, kErrMma);
+                    ok = ok && mbar_wait(&bar_phi[buf], (C / 2) & 1, status, kErrMma);
                     tc_fence_after();
                 }
                 if (C + 1 < F::NC) {
@@ -406,7 +406,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                     if (C == 0) ok = ok && mbar_wait(&bar_box[1], 0, status, kErrTma);
                     tc_fence_before();
                     __syncthreads();           // chunk C-1's d-phi has been read by every thread
-                    if (tid == 0) {
+                    if (warp == 0 && elect_one()) {
                         tc_fence_after();
                         issue_chunk(C + 1);
                     }
@@ -447,7 +447,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             ok = ok && mbar_wait(&bar_box[0], 0, status, kErrTma);
             tc_fence_before();
             __syncthreads();
-            if (tid == 0) {
+            if (warp == 0 && elect_one()) {
                 tc_fence_after();
                 issue_chunk(0);
             }
@@ -459,7 +459,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                     if (C == 0) ok = ok && mbar_wait(&bar_box[1], 0, status, kErrTma);
                     tc_fence_before();
                     __syncthreads();           // chunk C-1's d-phi has been read by every thread
-                    if (tid == 0) {
+                    if (warp == 0 && elect_one()) {
                         tc_fence_after();
                         issue_chunk(C + 1);
                     }
@@ -495,7 +495,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     const float y65h_inv = y65h * inv_own;
     if constexpr (LIN && LOCAL) ok = ok && mbar_wait(&bar_own, 1, status, kErrTma);      // the raw own rows
 #pragma unroll 1
-    for (int tp = tp_begin; tp < tp_end && ok; ++tp) {
+    for (int tp = tp_begin; tp < tp_end; ++tp) {
         const int orow0 = l * b + tp * 128;
         // one-tile operands alternate between two buffers, so the next tile's rows can be requested a tile ahead
         const uint32_t xo = (L::kTwoM && ((tp - tp_begin) & 1)) ? L::Moth2 : L::Moth;
@@ -515,7 +515,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                 oe_raw = e65h[(size_t)bh * n + orow0 + 128 + tid];
             }
         }
-        ok = mbar_wait(&bar_xoth, oth_uses & 1, status, kErrTma);
+        ok = ok && mbar_wait(&bar_xoth, oth_uses & 1, status, kErrTma);
         ok = ok && mbar_wait(&bar_yoth, oth_uses & 1, status, kErrTma);
         ++oth_uses;
         const bool diag = (tp == tau);
@@ -524,7 +524,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             fence_proxy_async_smem();
             tc_fence_before();
             __syncthreads();
-            if (tid == 0) {
+            if (warp == 0 && elect_one()) {
                 tc_fence_after();
                 // Every thread is past its wait for this tile's rows (a barrier must not complete twice
                 // before its slowest waiter has looked): the next tile's, into the other buffer.
@@ -594,7 +594,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             tmem_st_wait();
             tc_fence_before();
             __syncthreads();
-            if (tid == 0) {
+            if (warp == 0 && elect_one()) {
                 tc_fence_after();
                 constexpr uint32_t idesc = idesc_bf16(128, 64, false, true);
                 constexpr uint32_t idesc_dm = idesc_bf16(128, kNdM, false, true);
@@ -645,7 +645,8 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     }
 
     // ---- phase D: through the sketch, dX = ((dM*A2) G1^T + (dM*A1) G2^T) / sqrt(R) ----
-    if (ok) {
+    // (No `if (ok)` around what follows, and no loop above left early: every lane of warp 0 has to come to elect_one().)
+    {
         // (a given half sketch has no 1/sqrt(R) of its own)
         const float rs = lin ? 1.f : rsqrtf((float)R);
         // dM total = state part (registers) + tile part (tensor memory), scaled by 1/sqrt(R)
@@ -666,17 +667,17 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
         if constexpr (!LIN) {      // (a given half sketch: dX = dM "G1"^T needs neither A1 nor A2)
             tc_fence_before();
             __syncthreads();
-            if (tid == 0) {
+            if (warp == 0 && elect_one()) {
                 tc_fence_after();
                 issue_sketch<R>(tm + cSk, smem + L::Xown, smem + L::G);   // A1, A2 again
                 umma_commit(&bar_mma);
             }
-            ok = mbar_wait(&bar_mma, mma_uses & 1, status, kErrMma);
+            ok = ok && mbar_wait(&bar_mma, mma_uses & 1, status, kErrMma);
             ++mma_uses;
             tc_fence_after();
         }
     }
-    if (ok) {
+    {
         // U = [dM*A2 | dM*A1] as a bf16 A operand in tensor memory (2R values -> R columns at cdM).
         // LOCAL: the dM columns may hold the tiles' dX accumulator, so U goes over the sketch
         // columns this thread has just read (dM*A2 from column 0, dM*A1 from column R), and the
@@ -731,7 +732,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
         tmem_st_wait();
         tc_fence_before();
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             tc_fence_after();
             constexpr uint32_t idesc = idesc_bf16(128, 64, false, true);
 #pragma unroll
@@ -740,7 +741,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                         desc_off(smem_desc(smem_u32(smem + L::G), 0, 1024, kSwz128), k * 2048), idesc, ((LOCAL && !LIN) || k > 0) ? 1u : 0u);
             umma_commit(&bar_mma);
         }
-        ok = mbar_wait(&bar_mma, mma_uses & 1, status, kErrMma);
+        ok = ok && mbar_wait(&bar_mma, mma_uses & 1, status, kErrMma);
         ++mma_uses;
         tc_fence_after();
     }

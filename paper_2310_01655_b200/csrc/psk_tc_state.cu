@@ -140,7 +140,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
     using L = StateSmem<R, NWG>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
-    const int tid = threadIdx.x, wg = tid / 128, wt = tid % 128, warp = tid / 32;
+    const int tid = threadIdx.x, warp = warp_index(), wg = warp / 4, wt = tid % 128;
     const int bh = blockIdx.x;
     const int seg = SEG ? run0 + (int)blockIdx.y : 0, nseg = SEG ? nseg_arg : 1;
     const int mode = !SEG ? kModePrefix : (mode_arg == kModeFirst && seg > 0 ? kModeTotal : mode_arg);
@@ -202,7 +202,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
         // GEMMs, the second issues the state GEMMs: between two of its MMAs lies as little as
         // possible (each satisfied wait, commit or TMA issue costs a single thread about a
         // hundred cycles, during which the tensor pipe would idle).
-        if (tid == 128 * (NWG + 1)) {
+        if (warp == 4 * (NWG + 1) && elect_one()) {
             bool ok = true;
             constexpr int NX = L::kXSlots;
             auto load_x = [&](int j) {
@@ -256,7 +256,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
             // twice before a generator thread has looked.)
             umma_commit(&sh.drain[0]);
             mbar_wait(&sh.drain[0], 0, status, kErrMma);
-        } else if (tid == 128 * (NWG + 1) + 32) {
+        } else if (warp == 4 * (NWG + 1) + 1 && elect_one()) {
             constexpr uint32_t idesc_state = idesc_bf16(128, 80, true, true);
             bool ok = true;
             int w = 0;                                    // feature tile number u comes from warpgroup w = u mod NWG, as its

@@ -14,6 +14,20 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// Which warp this is, as a value the compiler knows to be the same in all 32 lanes.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0); }
+// True in one lane of a converged warp, the same one every time (all 32 have to come here).  Work for a single thread
+// that issues MMAs goes behind `warp_index() == w && elect_one()`, not behind a comparison of threadIdx.x: only then
+// does the compiler keep an MMA's descriptors in uniform registers.  Measured, one thread issuing 32 in a row with A
+// in tensor memory: 48 cycles each up to N = 96 behind a thread index; elected N = 16: 11, 32: 18, 64: 31, 80: 37, 96: 45 (with A in
+// shared memory the operand's way bounds them: 40, 40, 47, 52, 55).  Forward of 12 heads x 16 512, r = 32: 179 -> 155 us;
+// training, 48 heads x 16 384, r = 64: 5362 -> 4650, 384 heads x 32 768, r = 32: 21 789 -> 20 791.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e != 0;
+}
+
 // ---------------------------------------------------------------------------
 // mbarrier
 // ---------------------------------------------------------------------------
