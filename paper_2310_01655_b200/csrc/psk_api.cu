@@ -317,14 +317,8 @@ int feature_table(int* a, int* b, float* w, int cap) {
     using F = psk::tc::Feat<R>;
     if (cap < F::F) return PSK_ERR_WORKSPACE;
     for (int f = 0; f < F::F; ++f) {
-        if (F::kCirc) {
-            const int s = 2 * (f / (2 * R)) + ((f / R) & 1);
-            a[f] = f % R;
-            b[f] = (a[f] + s) % R;
-        } else {
-            a[f] = F::a(f);
-            b[f] = F::b(f);
-        }
+        a[f] = F::a(f);
+        b[f] = F::b(f);
         w[f] = F::weight(f);
     }
     return F::F;

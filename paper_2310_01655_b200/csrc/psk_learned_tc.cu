@@ -41,12 +41,6 @@ namespace psk {
 namespace {
 
 using namespace tc;
-using cc::f2;
-using cc::fma2;
-using cc::hi2;
-using cc::lo2;
-using cc::mul2;
-using cc::pack2;
 
 constexpr float kLnEps = 1e-6f;
 constexpr size_t kChunkRows = (size_t)1 << 20;        // rows per pass over the networks

@@ -386,54 +386,27 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
         if (tid % 32 == 0) mbar_arrive(&bar_go);
 
         if (has_prefix) {
-            if constexpr (F::kCirc) {
-                CircGen<R> gen;
-                gen.init(mq);
+            FeatGen<R> gen;
+            gen.init(mq);
 #pragma unroll 1
-                for (int C = 0; C < F::NC; ++C) {     // (no early exit: a wait that gave up makes the later ones return at once)
-                    const int buf = C % kFeatBufs;
-                    if (C >= kFeatBufs) {             // the MMAs that read this buffer's previous contents
-                        ok = mbar_wait(&bar_a[buf], (C / kFeatBufs - 1) & 1, status, kErrMma);
-                        tc_fence_after();
-                        if (tid == 0) {               // ... and this stage's: refill it with chunk C's rows
-                            mbar_expect_tx(&bar_feat[buf], kZStageBytes);
-                            tma_load_3d(smem + L::zstage(buf), &mapZ, 0, C * 64, blk, &bar_feat[buf]);
-                            tma_load_3d(smem + L::zstage(buf) + 8192, &mapZ, 64, C * 64, blk, &bar_feat[buf]);
-                        }
+            for (int C = 0; C < F::NC; ++C) {         // (no early exit: a wait that gave up makes the later ones return at once)
+                const int buf = C % kFeatBufs;
+                if (C >= kFeatBufs) {                 // the MMAs that read this buffer's previous contents
+                    ok = mbar_wait(&bar_a[buf], (C / kFeatBufs - 1) & 1, status, kErrMma);
+                    tc_fence_after();
+                    if (tid == 0) {                   // ... and this stage's: refill it with chunk C's rows
+                        mbar_expect_tx(&bar_feat[buf], kZStageBytes);
+                        tma_load_3d(smem + L::zstage(buf), &mapZ, 0, C * 64, blk, &bar_feat[buf]);
+                        tma_load_3d(smem + L::zstage(buf) + 8192, &mapZ, 64, C * 64, blk, &bar_feat[buf]);
                     }
-                    uint32_t pk[32];
-                    gen.chunk(pk);
-                    tmem_st32(lane_tm + cA + buf * 32, pk);
-                    tmem_st_wait();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (tid % 32 == 0) mbar_arrive(&bar_feat[buf]);
                 }
-            } else {
-                PackedM<R> pmq;
-                pack_half_sketch<R>(mq, pmq);
-                static_for<0, F::NC>([&](auto cc) {
-                    constexpr int C = decltype(cc)::value;
-                    constexpr int buf = C % kFeatBufs;
-                    if constexpr (C >= kFeatBufs) {
-                        ok = ok && mbar_wait(&bar_a[buf], (C / kFeatBufs - 1) & 1, status, kErrMma);
-                        tc_fence_after();
-                        if (tid == 0) {
-                            mbar_expect_tx(&bar_feat[buf], kZStageBytes);
-                            tma_load_3d(smem + L::zstage(buf), &mapZ, 0, C * 64, blk, &bar_feat[buf]);
-                            tma_load_3d(smem + L::zstage(buf) + 8192, &mapZ, 64, C * 64, blk, &bar_feat[buf]);
-                        }
-                    }
-                    uint32_t pk[16];
-                    gen_features<R, C * 64, 16>(pmq, pk);
-                    tmem_st16(lane_tm + cA + buf * 32, pk);
-                    gen_features<R, C * 64 + 32, 16>(pmq, pk);
-                    tmem_st16(lane_tm + cA + buf * 32 + 16, pk);
-                    tmem_st_wait();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (tid % 32 == 0) mbar_arrive(&bar_feat[buf]);
-                });
+                uint32_t pk[32];
+                switch_chunk<0, F::NC>(C, [&](auto cc) { gen.template words<decltype(cc)::value * 32>(pk); });
+                tmem_st32(lane_tm + cA + buf * 32, pk);
+                tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (tid % 32 == 0) mbar_arrive(&bar_feat[buf]);
             }
         }
 
@@ -460,9 +433,10 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                 }
 #pragma unroll
                 for (int j = 0; j < 32; j += 2) {
-                    float w0 = __uint_as_float(v[j]), w1 = __uint_as_float(v[j + 1]);
-                    if constexpr (LOCAL) { w0 *= w0; w1 *= w1; }          // (q . k)^2, squared once more below
-                    pk[j / 2] = pack_bf16(w0 * w0, w1 * w1);
+                    f2 w = pack2(v[j], v[j + 1]);
+                    if constexpr (LOCAL) w = mul2(w, w);                  // (q . k)^2, squared once more below
+                    w = mul2(w, w);
+                    pk[j / 2] = pack_bf16(lo2(w), hi2(w));
                 }
                 tmem_st16(lane_tm + cW + gq * 16, pk);
             }

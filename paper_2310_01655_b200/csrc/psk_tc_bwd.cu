@@ -87,8 +87,8 @@ struct BwdSmem {
     static constexpr uint32_t Xown = 0, G = 16384;
     static constexpr uint32_t Yown = G + (GImage<R>::bytes + 1023) / 1024 * 1024;
     static constexpr uint32_t ExtA = Yown + 16384;       // [128 x 16] un-swizzled
-    static constexpr uint32_t Eoth = ExtA + 4096;        // 128 x (1/d, e65h) of the other side's rows
-    static constexpr uint32_t U = Eoth + 1024;
+    static constexpr uint32_t Eoth = ExtA + 4096;        // scalars of the other side's rows (key side: three per row)
+    static constexpr uint32_t U = Eoth + 2048;
     static constexpr uint32_t Box = U;                   // phase B: kSt state boxes
     static constexpr int NC = Feat<R>::NC;
     // stages of the state-chunk ring: four; three on the query side for r = 64, which then fits two CTAs per SM
@@ -119,21 +119,6 @@ struct BwdSmem {
     static constexpr uint32_t Sx = U, Sv = U + 16384;
 };
 constexpr uint32_t kBoxStride = kBoxBytes;
-
-// dm += (d feature) * (the other factor) for the 32 features F0 .. F0+31 held in x
-template <int R, int F0>
-__device__ __forceinline__ void untensor32(const uint32_t (&x)[32], const float (&m)[R], float (&dm)[R]) {
-    static_for<0, 32>([&](auto jc) {
-        constexpr int J = decltype(jc)::value;
-        constexpr int f = F0 + J;
-        if constexpr (f < Feat<R>::F) {
-            constexpr int A = Feat<R>::a(f), B = Feat<R>::b(f);
-            const float v = __uint_as_float(x[J]);        // weighted by the state row it came through
-            dm[A] = fmaf(v, m[B], dm[A]);
-            dm[B] = fmaf(v, m[A], dm[B]);
-        }
-    });
-}
 
 // Score GEMM  own rows x 64 other rows over the split half sketches:
 //   hi.hi + lo.hi + hi.lo, the [hi | lo] columns of both operands addressed in place.
@@ -370,114 +355,65 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                 if (C == L::cY) load_y(QSIDE ? 0 : tau);
             }
         };
-        if constexpr (F::kCirc) {
-            // every chunk is the same code on rotated copies of m: a loop
-            CircGen<R> gen;
-            CircUntensor<R> ut;
-            if constexpr (!QSIDE) gen.init(m);
-            ut.init(m);
-            auto stage_features = [&](int C) {    // features of the next chunk -> tensor memory
-                uint32_t pk[32];
-                gen.chunk(pk);
-                (void)C;
-                tmem_st32(lane_tm + cFB, pk);          // one buffer: its previous reader (chunk C-1's MMAs) is done
-                tmem_st_wait();
-            };
-            if constexpr (!QSIDE) stage_features(0);
-            ok = ok && mbar_wait(&bar_box[0], 0, status, kErrTma);
-            tc_fence_before();
-            __syncthreads();
-            if (warp == 0 && elect_one()) {
-                tc_fence_after();
-                issue_chunk(0);
-            }
+        FeatGen<R> gen;
+        Untensor<R> ut;
+        if constexpr (!QSIDE) gen.init(m);
+        ut.init(m);
+        // r <= 32: one staging buffer, free once chunk C's MMAs have completed (the tensor-memory columns beside it hold Y);
+        // r = 64 two.
+        constexpr bool kOneBuf = !QSIDE && kTsA;
+        auto stage_features = [&](int C) {        // features of a chunk -> tensor memory
+            uint32_t pk[32];
+            switch_chunk<0, F::NC>(C, [&](auto cc) { gen.template words<decltype(cc)::value * 32>(pk); });
+            tmem_st32(lane_tm + cFB + (kOneBuf ? 0 : (C & 1) * 32), pk);
+            tmem_st_wait();
+        };
+        if constexpr (!QSIDE) stage_features(0);
+        ok = ok && mbar_wait(&bar_box[0], 0, status, kErrTma);
+        tc_fence_before();
+        __syncthreads();
+        if (warp == 0 && elect_one()) {
+            tc_fence_after();
+            issue_chunk(0);
+        }
 #pragma unroll 1
-            for (int C = 0; C < F::NC; ++C) {          // (no early exit: a wait that gave up makes the later ones return at once)
-                const int buf = C & 1;
-                // Key side: chunk C's MMAs read the one staging buffer, so they must have completed
-                // before chunk C+1's features go in; query side: chunk C+1 is issued first and runs
-                // behind chunk C.
-                if constexpr (!QSIDE) {
-                    ok = ok && mbar_wait(&bar_phi[buf], (C / 2) & 1, status, kErrMma);
-                    tc_fence_after();
-                }
-                if (C + 1 < F::NC) {
-                    if constexpr (!QSIDE) stage_features(C + 1);
-                    if (C == 0) ok = ok && mbar_wait(&bar_box[1], 0, status, kErrTma);
-                    tc_fence_before();
-                    __syncthreads();           // chunk C-1's d-phi has been read by every thread
-                    if (warp == 0 && elect_one()) {
-                        tc_fence_after();
-                        issue_chunk(C + 1);
-                    }
-                }
-                if constexpr (QSIDE) {
-                    ok = ok && mbar_wait(&bar_phi[buf], (C / 2) & 1, status, kErrMma);
-                    tc_fence_after();
-                }
-                if (tid == 32) refill(C);          // (warp 0 issues the MMAs; the loads go out from warp 1)
-                uint32_t x[32];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    tmem_ld32(lane_tm + cPhi + buf * 64 + h * 32, x);
-                    tmem_ld_wait();
-                    if constexpr (R == 32) {
-                        if (h == 0) ut.even(x, m, dm); else { ut.odd(x, m, dm); ut.advance(); }
-                    } else {
-                        ut.even(x, m, dm);
-                        ut.odd(x + 16, m, dm);
-                        ut.advance();
-                    }
-                }
-            }
-            ut.template finish<F::NC * 64 / (2 * R)>(dm);
-        } else {
-            PackedM<R> pm;
-            if constexpr (!QSIDE) pack_half_sketch<R>(m, pm);
-            auto stage_features = [&](auto cc) {
-                constexpr int C = decltype(cc)::value;
-                uint32_t pk[16];
-                gen_features<R, C * 64, 16>(pm, pk);
-                tmem_st16(lane_tm + cFB + (C & 1) * 32, pk);
-                gen_features<R, C * 64 + 32, 16>(pm, pk);
-                tmem_st16(lane_tm + cFB + (C & 1) * 32 + 16, pk);
-                tmem_st_wait();
-            };
-            if constexpr (!QSIDE) stage_features(std::integral_constant<int, 0>{});
-            ok = ok && mbar_wait(&bar_box[0], 0, status, kErrTma);
-            tc_fence_before();
-            __syncthreads();
-            if (warp == 0 && elect_one()) {
-                tc_fence_after();
-                issue_chunk(0);
-            }
-            static_for<0, F::NC>([&](auto cc) {
-                constexpr int C = decltype(cc)::value;
-                constexpr int buf = C & 1;
-                if constexpr (C + 1 < F::NC) {
-                    if constexpr (!QSIDE) stage_features(std::integral_constant<int, C + 1>{});
-                    if (C == 0) ok = ok && mbar_wait(&bar_box[1], 0, status, kErrTma);
-                    tc_fence_before();
-                    __syncthreads();           // chunk C-1's d-phi has been read by every thread
-                    if (warp == 0 && elect_one()) {
-                        tc_fence_after();
-                        issue_chunk(C + 1);
-                    }
-                }
+        for (int C = 0; C < F::NC; ++C) {          // (no early exit: a wait that gave up makes the later ones return at once)
+            const int buf = C & 1;
+            // One staging buffer: chunk C's MMAs read it, so they must have completed before chunk
+            // C+1's features go in; otherwise chunk C+1 is issued first and runs behind chunk C.
+            if constexpr (kOneBuf) {
                 ok = ok && mbar_wait(&bar_phi[buf], (C / 2) & 1, status, kErrMma);
                 tc_fence_after();
-                if (tid == 32) refill(C);          // (warp 0 issues the MMAs; the loads go out from warp 1)
-                {
-                    uint32_t x[32];
-                    tmem_ld32(lane_tm + cPhi + buf * 64, x);
-                    tmem_ld_wait();
-                    untensor32<R, C * 64>(x, m, dm);
+            }
+            if (C + 1 < F::NC) {
+                if constexpr (!QSIDE) stage_features(C + 1);
+                if (C == 0) ok = ok && mbar_wait(&bar_box[1], 0, status, kErrTma);
+                tc_fence_before();
+                __syncthreads();               // chunk C-1's d-phi has been read by every thread
+                if (warp == 0 && elect_one()) {
+                    tc_fence_after();
+                    issue_chunk(C + 1);
+                }
+            }
+            if constexpr (!kOneBuf) {
+                ok = ok && mbar_wait(&bar_phi[buf], (C / 2) & 1, status, kErrMma);
+                tc_fence_after();
+            }
+            if (tid == 32) refill(C);              // (warp 0 issues the MMAs; the loads go out from warp 1)
+            uint32_t x[32];
+            tmem_ld32(lane_tm + cPhi + buf * 64, x);
+            tmem_ld_wait();
+            switch_chunk<0, F::NC>(C, [&](auto cc) {
+                constexpr int F0 = decltype(cc)::value * 64;
+                ut.template add<F0>(x);
+                if constexpr (F0 + 32 < F::F) {
                     tmem_ld32(lane_tm + cPhi + buf * 64 + 32, x);
                     tmem_ld_wait();
-                    untensor32<R, C * 64 + 32>(x, m, dm);
+                    ut.template add<F0 + 32>(x);
                 }
             });
         }
+        ut.finish(dm);
         if constexpr (!QSIDE) dv_started = true;
 #pragma unroll
         for (int c = 0; c < R; ++c) dm[c] *= inv_own;
@@ -491,8 +427,11 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     const int tp_begin = QSIDE ? 0 : tau, tp_end = noncausal ? tp_begin : (QSIDE ? tau + 1 : ntiles);
     bool dm_started = false;
     uint32_t oth_uses = 0;
-    float2* oth_col = reinterpret_cast<float2*>(smem + L::Eoth);   // other rows: (1/d, -(g . O)/d)
+    // ds = 2 s dW, dx = 4 x^3 dW: the factor goes on 1/d and -(g . O)/d, of which dW is a multiple
+    constexpr float kDwScale = LOCAL ? 4.f : 2.f;
+    float* oth_col = reinterpret_cast<float*>(smem + L::Eoth);     // other rows: 1/d, scaled 1/d, scaled -(g . O)/d
     const float y65h_inv = y65h * inv_own;
+    const f2 own_sinv = pack2(kDwScale * inv_own, kDwScale * inv_own), own_syinv = pack2(kDwScale * y65h_inv, kDwScale * y65h_inv);
     if constexpr (LIN && LOCAL) ok = ok && mbar_wait(&bar_own, 1, status, kErrTma);      // the raw own rows
 #pragma unroll 1
     for (int tp = tp_begin; tp < tp_end; ++tp) {
@@ -509,7 +448,8 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
         if constexpr (!QSIDE) {
             // e65h is already -(g . O) / d.  These two were requested a tile (or a phase) ago; the
             // next tile's are requested now.
-            oth_col[tid] = make_float2(1.f / od_raw, oe_raw);
+            const float inv = 1.f / od_raw;
+            oth_col[tid] = inv; oth_col[128 + tid] = kDwScale * inv; oth_col[256 + tid] = kDwScale * oe_raw;
             if (tp + 1 < tp_end) {
                 od_raw = denom[(size_t)bh * n + orow0 + 128 + tid];
                 oe_raw = e65h[(size_t)bh * n + orow0 + 128 + tid];
@@ -560,31 +500,36 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                     tmem_ld32(lane_tm + cDW + c0, wv);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
+                    for (int j = 0; j < 32; j += 4) {
                         const int col = hh * 64 + c0 + j;
-                        float s = __uint_as_float(sv[j]);
-                        if constexpr (DIAG) s = (QSIDE ? (col <= tid) : (col >= tid)) ? s : 0.f;
-                        float inv, yinv;
+                        f2 inv[2], sinv[2], syinv[2];
                         if constexpr (QSIDE) {
-                            inv = inv_own; yinv = y65h_inv;
+                            sinv[0] = sinv[1] = own_sinv; syinv[0] = syinv[1] = own_syinv;
                         } else {
-                            const float2 o = oth_col[col];
-                            inv = o.x; yinv = o.y;
+                            const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(oth_col + col);
+                            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(oth_col + 128 + col);
+                            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(oth_col + 256 + col);
+                            inv[0] = u.x; inv[1] = u.y; sinv[0] = v.x; sinv[1] = v.y; syinv[0] = w.x; syinv[1] = w.y;
                         }
-                        const float dw = fmaf(__uint_as_float(wv[j]), inv, yinv);
-                        if constexpr (LOCAL) {
-                            const float s2 = s * s;                     // s is x_ij here
-                            sv[j] = __float_as_uint(4.f * s * s2 * dw);
-                            wv[j] = __float_as_uint(s2 * (s2 * inv));
-                        } else {
-                            sv[j] = __float_as_uint((s + s) * dw);
-                            wv[j] = __float_as_uint(s * (s * inv));     // weight / d_i: the value side sees g_i / d_i
-                        }
-                    }
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        pds[j] = pack_bf16(__uint_as_float(sv[2 * j]), __uint_as_float(sv[2 * j + 1]));
-                        pw[j] = pack_bf16(__uint_as_float(wv[2 * j]), __uint_as_float(wv[2 * j + 1]));
+                        for (int i = 0; i < 2; ++i) {
+                            float s0 = __uint_as_float(sv[j + 2 * i]), s1 = __uint_as_float(sv[j + 2 * i + 1]);
+                            if constexpr (DIAG) {
+                                s0 = (QSIDE ? (col + 2 * i <= tid) : (col + 2 * i >= tid)) ? s0 : 0.f;
+                                s1 = (QSIDE ? (col + 2 * i + 1 <= tid) : (col + 2 * i + 1 >= tid)) ? s1 : 0.f;
+                            }
+                            const f2 s = pack2(s0, s1);
+                            // 2 dW, or 4 dW with LOCAL (exact: powers of two)
+                            const f2 dw = fma2(pack2(wv[j + 2 * i], wv[j + 2 * i + 1]), sinv[i], syinv[i]);
+                            const f2 s2 = mul2(s, s);
+                            const f2 ds = mul2(LOCAL ? mul2(s, s2) : s, dw);         // (LOCAL: s is x_ij)
+                            pds[j / 2 + i] = pack_bf16(lo2(ds), hi2(ds));
+                            if constexpr (!QSIDE) {
+                                // weight / d_i: the value side sees g_i / d_i
+                                const f2 w = LOCAL ? mul2(s2, mul2(s2, inv[i])) : mul2(s, mul2(s, inv[i]));
+                                pw[j / 2 + i] = pack_bf16(lo2(w), hi2(w));
+                            }
+                        }
                     }
                     tmem_st16(lane_tm + cS + c0 / 2, pds);
                     if constexpr (!QSIDE) tmem_st16(lane_tm + cDW + c0 / 2, pw);

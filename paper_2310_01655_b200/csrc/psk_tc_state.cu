@@ -420,8 +420,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
         for (int j = 0; j < NJs; ++j, first = (first + (NWG - TN % NWG)) % NWG) {
             mbar_wait(&sh.sk, j & 1, status, kErrMma);
             tc_fence_after();
-            PackedM<R> pm;
-            CircGen<R> gen;
+            FeatGen<R> gen;
             {
                 float m[R];
                 // features m_a m_b / d: both factors carry 1 / sqrt(d) (d requested a token tile ago)
@@ -445,7 +444,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
                         for (int c = 0; c < R; ++c) m[c] *= sc;
                     }
                 }
-                if constexpr (F::kCirc) gen.init(m); else pack_half_sketch<R>(m, pm);
+                gen.init(m);
             }
             if (y65 != nullptr && wg == 0) {
                 // last-column chunk of this token tile; its slot is free once tile j-2's MMAs are done
@@ -458,46 +457,23 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
                 wg_barrier(0);
                 if (wt == 0) mbar_arrive(&sh.ext[j & 1]);
             }
-            if constexpr (F::kCirc) {
-                // this warpgroup's tiles first, first + NWG, ...: the same loop body on a rotated copy of m
-                constexpr int kTileSteps = 128 / (2 * R);
-                for (int i = 0; i < T0 + first && first < TN; ++i) gen.template skip<kTileSteps>();
+            // this warpgroup's tiles first, first + NWG, ...
 #pragma unroll 1
-                for (int I = first; I < TN; I += NWG) {
-                    if (a_uses > 0) mbar_wait(&sh.afree[wg], (a_uses - 1) & 1, status, kErrMma);
-#pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        uint32_t pk[32];
-                        gen.chunk(pk);
-#pragma unroll
-                        for (int c = 0; c < 8; ++c)
-                            *reinterpret_cast<uint4*>(sA + half * 16384 + swz128_offset(wt, c)) =
-                                make_uint4(pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
-                    }
-                    fence_proxy_async_smem();
-                    wg_barrier(wg);
-                    if (wt == 0) mbar_arrive(&sh.aready[wg]);
-                    ++a_uses;
-                    gen.template skip<(NWG - 1) * kTileSteps>();
-                }
-            } else {
-                static_for<0, TN>([&](auto ic) {
-                    constexpr int I = decltype(ic)::value;
-                    if (I % NWG == first) {
-                        if (a_uses > 0) mbar_wait(&sh.afree[wg], (a_uses - 1) & 1, status, kErrMma);
-                        static_for<0, 16>([&](auto cc) {
-                            constexpr int C = decltype(cc)::value;
-                            uint32_t pk[4];
-                            gen_features<R, (T0 + I) * 128 + C * 8, 4>(pm, pk);
-                            *reinterpret_cast<uint4*>(sA + (C / 8) * 16384 + swz128_offset(wt, C % 8)) =
-                                make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                        });
-                        fence_proxy_async_smem();
-                        wg_barrier(wg);
-                        if (wt == 0) mbar_arrive(&sh.aready[wg]);
-                        ++a_uses;
-                    }
+            for (int I = first; I < TN; I += NWG) {
+                if (a_uses > 0) mbar_wait(&sh.afree[wg], (a_uses - 1) & 1, status, kErrMma);
+                switch_chunk<0, TN>(I, [&](auto ic) {
+                    constexpr int W0 = (T0 + decltype(ic)::value) * 64;           // the tile's first word
+                    static_for<0, 16>([&](auto cc) {
+                        constexpr int C = decltype(cc)::value;
+                        uint32_t pk[4];
+                        gen.template words<W0 + 4 * C>(pk);
+                        *reinterpret_cast<uint4*>(sA + (C / 8) * 16384 + swz128_offset(wt, C % 8)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                    });
                 });
+                fence_proxy_async_smem();
+                wg_barrier(wg);
+                if (wt == 0) mbar_arrive(&sh.aready[wg]);
+                ++a_uses;
             }
         }
     }

@@ -88,14 +88,6 @@ inline cudaError_t set_smem(Kern k, size_t bytes) {
 
 namespace tc {
 
-template <int I, int N, typename Fn>
-__device__ __forceinline__ void static_for(Fn&& f) {
-    if constexpr (I < N) {
-        f(std::integral_constant<int, I>{});
-        static_for<I + 1, N>(f);
-    }
-}
-
 constexpr int kErrTma = 1, kErrMma = 2;
 
 // barrier among the 128 row threads (warps 0-3) of a kernel whose fifth warp issues the MMAs;

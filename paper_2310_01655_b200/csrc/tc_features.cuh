@@ -10,227 +10,219 @@
 //   dm[a] += d(feature ab) m[b];   dm[b] += d(feature ab) m[a]        for every stored feature,
 // the diagonal included (its two updates coincide, which is the factor 2 of d(m_a^2)).
 //
-// Two feature orders:
+// Two feature orders, both in words of two features (f even: the pair (f, f + 1) is one packed bf16x2 product):
 //
-//  * circulant (r <= 32): feature (s, a) = m[a] m[(a + s) mod r] for shifts s = 0 .. r/2, stored
-//    shift-major in steps of two shifts, f = j * 2r + (s - 2j) * r + a with j = s / 2, for
-//    j = 0 .. r/4.  Shift r/2 lists every pair {a, a + r/2} twice, so its weight is 1; shift
-//    r/2 + 1 only fills the last step and has weight 0.  Every step is the same code on a
-//    rotated copy of m, so generation and its backward are LOOPS over steps: the kernels' code
-//    stays small enough for the instruction cache, which is what bounds them otherwise.
+//  * circulant (r <= 32): feature (s, a) = m[a] m[(a + s) mod r] for shifts s = 0 .. r/2, shift-major,
+//    f = s r + a.  Shift r/2 lists every pair {a, a + r/2} twice, so its weight is 1.  A word is an
+//    even-aligned pair of entries times an even- or odd-aligned one.
 //
-//  * triangular (r = 64): pairs a <= b enumerated so that runs of consecutive features share
-//    `a`; fully unrolled code, one specialised instruction sequence per feature.  (The loop form
-//    needs four r-entry register arrays in the backward, which r = 64 does not have.)
-//      rows p = 0 .. r/2-2, r entries each: first (a = p, b = p+1 .. r-1), then
-//                                           (a = r-2-p, b = r-1-p .. r-1);
-//      then (a = r/2-1, b = r/2 .. r-1), r/2 entries;  then the diagonal (a, a), r entries.
+//  * blocks (r = 64): pairs of entries p = 0 .. 31, coordinates 2p and 2p + 1.  For every p the word (2p, 2p), (2p, 2p + 1),
+//    then for q = p + 1 .. 31 the words (2p, 2q), (2p, 2q + 1) and (2p + 1, 2q), (2p + 1, 2q + 1): one entry times an
+//    even-aligned pair.  Last the diagonal entries that are left, (2p + 1, 2p + 1), p = 0 .. 31.
+//
+// Everything is unrolled: a 64-feature chunk is straight code on registers with fixed indexes, and a kernel's loop over
+// chunks enters the chunk's code through switch_chunk().  So only the products are there once per chunk; waits, MMA
+// issue and loads are there once.  The products in packed pairs (bf16x2, and fp32 pairs in the backward) are 1 (r = 16), 4 (r = 32)
+// and 17 KB (r = 64) of code for the features and 2, 9 and 33 KB for their backward; what a kernel executes has to come
+// from an instruction cache of about 32 KB at full rate, at half rate to about 96 KB, at a tenth beyond 128 KB.
+// (Before, r <= 32 rotated the half sketch through registers in a loop of two shifts, r = 64 had waits and MMA issue once per chunk and
+// scalar FMAs, 130 to 225 KB.  Training, 48 heads x 16 384, r = 64, b = 512: 4647 -> 4030 us; 384 heads x 32 768, r = 32:
+// 20 723 -> 20 615; exact blocks, 48 heads x 2688, r = 32: 259 -> 251; degree 8, 96 heads x 8192: 1673 -> 1619.)
 #pragma once
 
+#include "packed.cuh"
 #include "tc_prims.cuh"
+
+#include <type_traits>
 
 namespace psk {
 namespace tc {
 
+template <int I, int N, typename Fn>
+__device__ __forceinline__ void static_for(Fn&& f) {
+    if constexpr (I < N) {
+        f(std::integral_constant<int, I>{});
+        static_for<I + 1, N>(f);
+    }
+}
+// f(integral_constant<i>) for a run-time i of [LO, HI), the same for the whole warp: a binary search of branches
+template <int LO, int HI, typename Fn>
+__device__ __forceinline__ void switch_chunk(int i, Fn&& f) {
+    if constexpr (HI - LO == 1) {
+        f(std::integral_constant<int, LO>{});
+    } else {
+        constexpr int MID = (LO + HI) / 2;
+        if (i < MID) switch_chunk<LO, MID>(i, f);
+        else switch_chunk<MID, HI>(i, f);
+    }
+}
+
 template <int R>
 struct Feat {
     static constexpr bool kCirc = (R <= 32);
-    static constexpr int kSteps = R / 4 + 1;                         // circulant: steps of two shifts
-    static constexpr int F = kCirc ? kSteps * 2 * R : R * (R + 1) / 2;   // stored features
-    static constexpr int FK = (F + 15) / 16 * 16;    // padded to the MMA K step
+    static constexpr int F = kCirc ? (R / 2 + 1) * R : R * (R + 1) / 2;   // stored features
+    static constexpr int FK = F;                     // a multiple of the MMA K step
     static constexpr int NC = (F + 63) / 64;         // 64-feature chunks (A staging / state TMA boxes)
     static constexpr int NT = (F + 127) / 128;       // 128-feature tiles (state accumulators)
     static constexpr int FP = NT * 128;              // padded feature extent of stored states
-    static constexpr int kPairRows = (R / 2 - 1) * R;
+    static_assert(F % 16 == 0, "whole MMA K steps");
 
-    // triangular order
+    // blocks: first word of pair p (p = r/2: the diagonal entries that are left), and the p of word w
+    __host__ __device__ static constexpr int block_base(int p) { return p * (R - p); }
+    __host__ __device__ static constexpr int block_of(int w) {
+        int p = 0;
+        while (p < R / 2 && w >= block_base(p + 1)) ++p;
+        return p < R / 2 && w < R * R / 4 ? p : R / 2;
+    }
     __host__ __device__ static constexpr int a(int f) {
-        if (f < kPairRows) {
-            const int p = f / R, e = f % R;
-            return (e < R - 1 - p) ? p : (R - 2 - p);
-        }
-        const int g = f - kPairRows;
-        return (g < R / 2) ? (R / 2 - 1) : (g - R / 2);
+        if (kCirc) return f % R;
+        const int w = f / 2, p = block_of(w);
+        if (p == R / 2) return 2 * (f - R * R / 2) + 1;
+        const int k = w - block_base(p);              // 0: the diagonal word; then both words of q = p + 1, ...
+        return k == 0 ? 2 * p : 2 * p + ((k - 1) & 1);
     }
     __host__ __device__ static constexpr int b(int f) {
-        if (f < kPairRows) {
-            const int p = f / R, e = f % R;
-            return (e < R - 1 - p) ? (p + 1 + e) : (R - 2 - p + 1 + (e - (R - 1 - p)));
-        }
-        const int g = f - kPairRows;
-        return (g < R / 2) ? (R / 2 + g) : (g - R / 2);
+        if (kCirc) return (f % R + f / R) % R;
+        const int w = f / 2, p = block_of(w);
+        if (p == R / 2) return 2 * (f - R * R / 2) + 1;
+        const int k = w - block_base(p);
+        return 2 * (p + (k + 1) / 2) + (f & 1);
     }
     // weight of stored state row f (0 for padding rows)
     __host__ __device__ static float weight(int f) {
         if (f >= F) return 0.f;
-        if (kCirc) {
-            const int s = 2 * (f / (2 * R)) + ((f / R) & 1);
-            return (s == 0 || s == R / 2) ? 1.f : (s > R / 2 ? 0.f : 2.f);
-        }
-        return a(f) == b(f) ? 1.f : 2.f;
+        if (kCirc) return (f < R || f >= F - R) ? 1.f : 2.f;
+        if (f >= R * R / 2) return 1.f;
+        // block_base(p) = (r/2)^2 - (r/2 - p)^2: a diagonal word leaves a square
+        const int left = R * R / 4 - f / 2;
+        const int root = (int)(sqrtf((float)left) + 0.5f);
+        return ((f & 1) == 0 && root * root == left) ? 1.f : 2.f;
     }
 };
 
-// The half sketch of one row as packed bf16 pairs, the generators' working set:
-//   e[k] = (m[2k], m[2k+1])   even-aligned pairs,   o[k] = (m[2k+1], m[2k+2])   odd-aligned pairs
-// (o wraps around: its last entry is (m[r-1], m[0]) -- the circulant order needs it, the
-// triangular one never reads that half).  A packed multiply of two such pairs yields two
-// features; the product is rounded to bf16 once more, which the tolerance budget covers
-// (relative 2^-9 each, independent across features).
-template <int R>
-struct PackedM {
-    uint32_t e[R / 2], o[R / 2];
-};
-
-template <int R>
-__device__ __forceinline__ void pack_half_sketch(const float (&m)[R], PackedM<R>& pm) {
-#pragma unroll
-    for (int k = 0; k < R / 2; ++k) {
-        pm.e[k] = pack_bf16(m[2 * k], m[2 * k + 1]);
-        pm.o[k] = pack_bf16(m[2 * k + 1], m[(2 * k + 2) % R]);
-    }
-}
-
+// (volatile, here and below: the products depend on nothing that changes in a loop over chunks, and the compiler would
+// form all of them before it, and spill them)
 __device__ __forceinline__ uint32_t hmul2_bf16(uint32_t x, uint32_t y) {
     uint32_t r;
-    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y));
+    asm volatile("mul.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y));
+    return r;
+}
+// the low (0) or high (1) half of a pair in both halves
+template <int HALF>
+__device__ __forceinline__ uint32_t twice(uint32_t x) {
+    uint32_t r;
+    asm volatile("prmt.b32 %0, %1, %1, %2;" : "=r"(r) : "r"(x), "n"(HALF ? 0x3232 : 0x1010));
     return r;
 }
 
-// ---------------------------------------------------------------------------
-// circulant order: one step = shifts 2j and 2j+1 = 2r features = r packed words
-// ---------------------------------------------------------------------------
-// Holds e (fixed) and the copies of e and o rotated by the current step:
-//   er[k] = e[(k + j) mod r/2] = (m[2k + 2j], m[2k + 2j + 1]),  orr[k] = o[(k + j) mod r/2].
+// The half sketch of one row as packed bf16 pairs, and the features formed from it:
+//   e[k] = (m[2k], m[2k+1]),   circulant order also  o[k] = (m[2k+1], m[(2k+2) mod r]).
+// A packed multiply yields two features; the product is rounded to bf16 once more, which the
+// tolerance budget covers (relative 2^-9 each, independent across features).
 template <int R>
-struct CircGen {
-    static constexpr int H = R / 2;
-    uint32_t e[H], er[H], orr[H];
+struct FeatGen {
+    static constexpr int H = R / 2, HO = Feat<R>::kCirc ? R / 2 : 1;
+    uint32_t e[H], o[HO];
 
     __device__ __forceinline__ void init(const float (&m)[R]) {
 #pragma unroll
         for (int k = 0; k < H; ++k) {
             e[k] = pack_bf16(m[2 * k], m[2 * k + 1]);
-            er[k] = e[k];
-            orr[k] = pack_bf16(m[2 * k + 1], m[(2 * k + 2) % R]);
+            if constexpr (Feat<R>::kCirc) o[k] = pack_bf16(m[2 * k + 1], m[(2 * k + 2) % R]);
         }
     }
-    // advance by K steps without producing anything
-    template <int K>
-    __device__ __forceinline__ void skip() {
-        uint32_t t[H], u[H];
-#pragma unroll
-        for (int k = 0; k < H; ++k) { t[k] = er[(k + K) % H]; u[k] = orr[(k + K) % H]; }
-#pragma unroll
-        for (int k = 0; k < H; ++k) { er[k] = t[k]; orr[k] = u[k]; }
-    }
-    // out[0 .. H) = features of shift 2j (a = 2k, 2k+1), out[H .. R) = shift 2j+1; then advance
-    __device__ __forceinline__ void step(uint32_t* out) {
-#pragma unroll
-        for (int k = 0; k < H; ++k) {
-            out[k] = hmul2_bf16(e[k], er[k]);
-            out[H + k] = hmul2_bf16(e[k], orr[k]);
+    // features 2 W, 2 W + 1
+    template <int W>
+    __device__ __forceinline__ uint32_t word() const {
+        if constexpr (2 * W >= Feat<R>::F) {
+            return 0u;
+        } else if constexpr (Feat<R>::kCirc) {
+            constexpr int S = W / H, K = W % H;
+            if constexpr (S % 2 == 0) return hmul2_bf16(e[K], e[(K + S / 2) % H]);
+            else return hmul2_bf16(e[K], o[(K + S / 2) % H]);
+        } else if constexpr (2 * W >= R * R / 2) {
+            constexpr int A = Feat<R>::a(2 * W) / 2;                        // (m[2A+1], m[2A+3]) squared
+            uint32_t x;
+            asm volatile("prmt.b32 %0, %1, %2, 0x7632;" : "=r"(x) : "r"(e[A]), "r"(e[A + 1]));
+            return hmul2_bf16(x, x);
+        } else {
+            constexpr int A = Feat<R>::a(2 * W), Q = Feat<R>::b(2 * W) / 2;
+            return hmul2_bf16(twice<A % 2>(e[A / 2]), e[Q]);
         }
-        skip<1>();
     }
-    // the next 64 features (32 packed words): 64 / 2r steps
-    __device__ __forceinline__ void chunk(uint32_t (&out)[32]) {
-        static_assert(R == 16 || R == 32, "circulant order: r = 16 or 32");
-#pragma unroll
-        for (int s = 0; s < 32 / R; ++s) step(out + s * R);
+    // words W0 .. W0 + N - 1
+    template <int W0, int N>
+    __device__ __forceinline__ void words(uint32_t (&out)[N]) const {
+        static_for<0, N>([&](auto jc) { out[decltype(jc)::value] = word<W0 + decltype(jc)::value>(); });
     }
 };
 
-// Backward of the circulant features: with x the (weighted) gradients of the features of one
-// step, dm[a] += x m[(a + s) mod r] and dm[(a + s) mod r] += x m[a].  The second term is
-// accumulated in the rotated frame (dr[a] collects dm[(a + 2j) mod r]) and folded back at the end.
+// ---------------------------------------------------------------------------
+// Backward of the features: with x the (weighted) gradients of the features, dm[a] += x m[b], dm[b] += x m[a] for every
+// stored feature, in packed fp32 pairs (two independent IEEE roundings).  On B200 packed and scalar FMAs
+// reach the same rate; the packed ones are half the instructions, and no registers are moved.
+// circulant: m and dm as even- and as odd-aligned pairs.  blocks: even-aligned pairs; the sums over a block row's
+// second factors stay in two pairs (row 2p, row 2p + 1) while the words of p go by.
+// ---------------------------------------------------------------------------
 template <int R>
-struct CircUntensor {
-    float mr[R], dr[R];
+struct Untensor {
+    using F = Feat<R>;
+    static constexpr int H = R / 2, HO = F::kCirc ? R / 2 : 1;
+    f2 me[H], de[H], mo[HO], od[HO];
+    f2 row[2];
 
     __device__ __forceinline__ void init(const float (&m)[R]) {
 #pragma unroll
-        for (int a = 0; a < R; ++a) { mr[a] = m[a]; dr[a] = 0.f; }
+        for (int k = 0; k < H; ++k) {
+            me[k] = pack2(m[2 * k], m[2 * k + 1]);
+            de[k] = 0ull;
+            if constexpr (F::kCirc) { mo[k] = pack2(m[2 * k + 1], m[(2 * k + 2) % R]); od[k] = 0ull; }
+        }
+        row[0] = row[1] = 0ull;
     }
-    // xe / xo: gradients of the features of shifts 2j / 2j+1 (fp32 bit patterns, a = 0 .. r-1)
-    __device__ __forceinline__ void even(const uint32_t* xe, const float (&m)[R], float (&dm)[R]) {
+    // gradients of the features F0 .. F0 + N - 1 (fp32 bit patterns)
+    template <int F0, int N>
+    __device__ __forceinline__ void add(const uint32_t (&x)[N]) {
+        static_for<0, N / 2>([&](auto jc) {
+            constexpr int J = decltype(jc)::value, f = F0 + 2 * J;
+            if constexpr (f < F::F) {
+                const f2 v = pack2(x[2 * J], x[2 * J + 1]);
+                if constexpr (F::kCirc) {
+                    constexpr int S = f / R, K = f % R / 2, Q = (K + S / 2) % H;
+                    if constexpr (S % 2 == 0) {
+                        de[K] = fma2(v, me[Q], de[K]);
+                        de[Q] = fma2(v, me[K], de[Q]);
+                    } else {
+                        de[K] = fma2(v, mo[Q], de[K]);
+                        od[Q] = fma2(v, me[K], od[Q]);
+                    }
+                } else if constexpr (f >= R * R / 2) {
+                    // (2p + 1, 2p + 1), (2p + 3, 2p + 3): both updates of a diagonal entry coincide
+                    constexpr int P = F::a(f) / 2;
+                    de[P] = pack2(lo2(de[P]), fmaf(2.f * lo2(v), hi2(me[P]), hi2(de[P])));
+                    de[P + 1] = pack2(lo2(de[P + 1]), fmaf(2.f * hi2(v), hi2(me[P + 1]), hi2(de[P + 1])));
+                } else {
+                    constexpr int A = F::a(f), P = A / 2, Q = F::b(f) / 2;
+                    const float ma = A % 2 ? hi2(me[P]) : lo2(me[P]);
+                    row[A % 2] = fma2(v, me[Q], row[A % 2]);
+                    de[Q] = fma2(v, pack2(ma, ma), de[Q]);
+                    if constexpr (f + 2 >= R * R / 2 || F::a(f + 2) / 2 != P) {       // last word of this p
+                        de[P] = pack2(lo2(de[P]) + (lo2(row[0]) + hi2(row[0])), hi2(de[P]) + (lo2(row[1]) + hi2(row[1])));
+                        row[0] = row[1] = 0ull;
+                    }
+                }
+            }
+        });
+    }
+    __device__ __forceinline__ void finish(float (&dm)[R]) const {
 #pragma unroll
-        for (int a = 0; a < R; ++a) {
-            const float v = __uint_as_float(xe[a]);
-            dm[a] = fmaf(v, mr[a], dm[a]);
-            dr[a] = fmaf(v, m[a], dr[a]);
+        for (int k = 0; k < H; ++k) {
+            dm[2 * k] = lo2(de[k]);
+            dm[2 * k + 1] = hi2(de[k]);
+            if constexpr (F::kCirc) { dm[2 * k] += hi2(od[(k + H - 1) % H]); dm[2 * k + 1] += lo2(od[k]); }
         }
     }
-    __device__ __forceinline__ void odd(const uint32_t* xo, const float (&m)[R], float (&dm)[R]) {
-#pragma unroll
-        for (int a = 0; a < R; ++a) {
-            const float v = __uint_as_float(xo[a]);
-            dm[a] = fmaf(v, mr[(a + 1) % R], dm[a]);
-            dr[(a + 1) % R] = fmaf(v, m[a], dr[(a + 1) % R]);
-        }
-    }
-    __device__ __forceinline__ void advance() {
-        float t[R], u[R];
-#pragma unroll
-        for (int a = 0; a < R; ++a) { t[a] = mr[(a + 2) % R]; u[a] = dr[(a + 2) % R]; }
-#pragma unroll
-        for (int a = 0; a < R; ++a) { mr[a] = t[a]; dr[a] = u[a]; }
-    }
-    // after TOTAL steps: dr[a] belongs to dm[(a + 2 TOTAL) mod r]
-    template <int TOTAL>
-    __device__ __forceinline__ void finish(float (&dm)[R]) {
-#pragma unroll
-        for (int a = 0; a < R; ++a) dm[(a + 2 * TOTAL) % R] += dr[a];
-    }
 };
-
-// ---------------------------------------------------------------------------
-// triangular order: specialised code per feature pair
-// ---------------------------------------------------------------------------
-// (m_i, m_j) as a packed pair, from the even-aligned registers
-template <int R, int I, int J>
-__device__ __forceinline__ uint32_t pair_of(const PackedM<R>& pm) {
-    constexpr uint32_t sel = (uint32_t)((I % 2) ? 0x32 : 0x10) | ((uint32_t)((J % 2) ? 0x76 : 0x54) << 8);
-    return __byte_perm(pm.e[I / 2], pm.e[J / 2], sel);
-}
-
-// bf16x2 (feature F0, feature F0 + 1); F0 even
-template <int R, int F0>
-__device__ __forceinline__ uint32_t feat_pair(const PackedM<R>& pm) {
-    if constexpr (F0 >= Feat<R>::F) {
-        return 0u;
-    } else {
-        static_assert(Feat<R>::F % 2 == 0 && F0 % 2 == 0, "features are generated in pairs");
-        constexpr int A1 = Feat<R>::a(F0), B1 = Feat<R>::b(F0), A2 = Feat<R>::a(F0 + 1), B2 = Feat<R>::b(F0 + 1);
-        uint32_t x, y;
-        if constexpr (A1 == A2 && B2 == B1 + 1) {
-            x = pair_of<R, A1, A1>(pm);                           // (m_a, m_a): shared by the whole run
-            y = (B1 % 2 == 0) ? pm.e[B1 / 2] : pm.o[B1 / 2];
-        } else {
-            x = pair_of<R, A1, A2>(pm);
-            y = pair_of<R, B1, B2>(pm);
-        }
-        return hmul2_bf16(x, y);
-    }
-}
-
-template <int R, int F0, int J, int N>
-struct FeatPack {
-    static __device__ __forceinline__ void run(const PackedM<R>& pm, uint32_t (&out)[N]) {
-        out[J] = feat_pair<R, F0 + 2 * J>(pm);
-        FeatPack<R, F0, J + 1, N>::run(pm, out);
-    }
-};
-template <int R, int F0, int N>
-struct FeatPack<R, F0, N, N> {
-    static __device__ __forceinline__ void run(const PackedM<R>&, uint32_t (&)[N]) {}
-};
-
-// out[j] = bf16x2(feature F0+2j, feature F0+2j+1), j < N  (2N consecutive features)
-template <int R, int F0, int N>
-__device__ __forceinline__ void gen_features(const PackedM<R>& pm, uint32_t (&out)[N]) {
-    FeatPack<R, F0, 0, N>::run(pm, out);
-}
 
 }  // namespace tc
 }  // namespace psk
