@@ -16,7 +16,8 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 
 // Which warp this is, as a value the compiler knows to be the same in all 32 lanes.
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0); }
-// True in one lane of a converged warp, the same one every time (all 32 have to come here).  Work for a single thread
+// True in one lane of a warp, the same one every time (all 32 have to come here; after a wait on a barrier they need not
+// come together, and two groups of lanes that elect one each would issue everything twice: hence the __syncwarp).  Work for a single thread
 // that issues MMAs goes behind `warp_index() == w && elect_one()`, not behind a comparison of threadIdx.x: only then
 // does the compiler keep an MMA's descriptors in uniform registers.  Measured, one thread issuing 32 in a row with A
 // in tensor memory: 48 cycles each up to N = 96 behind a thread index; elected N = 16: 11, 32: 18, 64: 31, 80: 37, 96: 45 (with A in
@@ -24,6 +25,7 @@ __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (i
 // training, 48 heads x 16 384, r = 64: 5362 -> 4650, 384 heads x 32 768, r = 32: 21 789 -> 20 791.
 __device__ __forceinline__ bool elect_one() {
     uint32_t e;
+    __syncwarp();
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(e));
     return e != 0;
 }
@@ -359,6 +361,19 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     uint32_t r;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
+}
+
+// Before a CTA that has given up a wait frees its tensor memory and ends: the MMAs it has issued must have completed and the
+// copies on their way into its shared memory must have arrived.  The elected lane of the issuing warp waits for a commit
+// of its own (with a limit), then long enough for any copy.  `bar`: a barrier of count 1 that nothing else uses.
+__device__ __forceinline__ void cta_drain(bool issuing_warp, uint64_t* bar, int* status) {
+    if (!__any_sync(0xffffffffu, cta_gave_up())) return;
+    if (issuing_warp && elect_one()) {
+        umma_commit(bar);
+        for (int i = 0; i < 1000 && !mbar_test(bar, 0); ++i) __nanosleep(1000);
+        for (int i = 0; i < 200; ++i) __nanosleep(1000);
+    }
+    (void)status;
 }
 
 // Byte offset of 16-byte chunk `chunk` (0..7) of row `row` inside a [rows x 128 B] tile held in
