@@ -163,7 +163,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     constexpr int kStages = L::kSt;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
-    __shared__ uint64_t bar_own, bar_xoth, bar_yoth, bar_mma, bar_phi[2], bar_box[2];
+    __shared__ uint64_t bar_own, bar_again, bar_xoth, bar_yoth, bar_mma, bar_phi[2], bar_box[2], bar_drain;
     __shared__ uint32_t tmem_slot;
     const int tid = threadIdx.x, warp = warp_index(), tau = blockIdx.x, l = blockIdx.y, bh = blockIdx.z;
     const int hi = bh % H, bi = bh / H;
@@ -185,6 +185,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
         tma_load_4d(smem + L::Yoth, &mapYoth, 0, l * b + tp * 128, hi, bi, &bar_yoth);
     };
 
+    // Set-up by two threads side by side (everyone waits for the slower): the own rows' loads and the tiles' barriers; the state rows.
     if (tid == 0) {
         // the own tiles are what everything waits for: their requests go out before anything else
         mbar_init(&bar_own, 1);
@@ -193,12 +194,18 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
         tma_load_4d(smem + L::Xown, &mapXown, 0, row0, hi, bi, &bar_own);
         tma_load_4d(smem + L::Yown, &mapYown, 0, row0, hi, bi, &bar_own);
         bulk_load(smem + L::G, gimg + (size_t)g * GImage<R>::bytes, GImage<R>::bytes, &bar_own);
-        mbar_init(&bar_xoth, 1); mbar_init(&bar_yoth, 1); mbar_init(&bar_mma, 1);
-        // (a chunk's d-phi barrier: its MMAs, and the state rows of the chunk after next)
-        mbar_init(&bar_phi[0], 2); mbar_init(&bar_phi[1], 2); mbar_init(&bar_box[0], 1); mbar_init(&bar_box[1], 1);
+        mbar_init(&bar_again, 1); mbar_init(&bar_xoth, 1); mbar_init(&bar_yoth, 1); mbar_init(&bar_mma, 1); mbar_init(&bar_drain, 1);
         cta_giveup_init();
         mbar_fence_init();
-        tma_prefetch_desc(&mapXoth); tma_prefetch_desc(&mapYoth); tma_prefetch_desc(&mapS);
+        tma_prefetch_desc(&mapXoth); tma_prefetch_desc(&mapYoth);
+        // first other-side tile: at once where its memory is free from the start
+        if (!noncausal && (!has_state || !L::kAlias || L::cM < 0)) load_m(QSIDE ? 0 : tau, L::Moth);
+        if (!noncausal && (!has_state || !L::kAlias || L::cY < 0)) load_y(QSIDE ? 0 : tau);
+    }
+    if (tid == 32) {
+        // (a chunk's d-phi barrier: its MMAs, and the state rows of the chunk after next)
+        mbar_init(&bar_phi[0], 2); mbar_init(&bar_phi[1], 2); mbar_init(&bar_box[0], 1); mbar_init(&bar_box[1], 1);
+        mbar_fence_init();
         if (has_state) {
             for (int c = 0; c < kStages; ++c) {
                 uint64_t* bar = c < 2 ? &bar_box[c] : &bar_phi[c - 2];
@@ -211,11 +218,8 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                 }
             }
         }
-        // first other-side tile: at once where its memory is free from the start
-        if (!noncausal && (!has_state || !L::kAlias || L::cM < 0)) load_m(QSIDE ? 0 : tau, L::Moth);
-        if (!noncausal && (!has_state || !L::kAlias || L::cY < 0)) load_y(QSIDE ? 0 : tau);
     }
-    if (warp == 0) { tmem_alloc(&tmem_slot, 256); tmem_relinquish(); }
+    if (warp == 2) { tmem_alloc(&tmem_slot, 256); tmem_relinquish(); }
     // Query rows work on the raw dO rows g_i (exact bf16 inputs) and apply 1/d_i in fp32 afterwards:
     // dL/dW_ij = (g_i . v_j - g_i . O_i) / d_i cancels heavily when one key dominates a row, and a
     // rounded g_i / d_i would not survive it.  y65 = -(g_i . (O_i - c)) pairs with the centred
@@ -274,8 +278,8 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
         // The own tile held the given half sketch; the exact same-block scores need the raw rows.
         // The sketch GEMM has completed: fetch them into the same buffer (phase C waits for them).
         if (tid == 0) {
-            mbar_expect_tx(&bar_own, 16384);
-            tma_load_4d(smem + L::Xown, &mapXownRaw, 0, row0, hi, bi, &bar_own);
+            mbar_expect_tx(&bar_again, 16384);
+            tma_load_4d(smem + L::Xown, &mapXownRaw, 0, row0, hi, bi, &bar_again);
         }
     }
 #pragma unroll
@@ -307,7 +311,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
         // generate chunk C+1's features; while those of chunk C+1 run, they un-tensor chunk C.
         // d-phi is double-buffered in [0,128); during this phase the feature staging buffers sit
         // in the dM accumulator's columns, which only phase C uses.
-        constexpr uint32_t cFB = cdM;
+        constexpr uint32_t cFB = R <= 32 ? 64 : cdM;          // (staging is for the key side only)
         // descriptors are loop invariants: an issue sequence is its MMA instructions and little else
         const uint64_t yd = smem_desc(smem_u32(smem + L::Yown), 0, 1024, kSwz128);
         const uint64_t ed = smem_desc(smem_u32(smem + L::ExtA), 2048, 128, kSwzNone);
@@ -316,7 +320,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             const int buf = C & 1, stage = C % kStages;
             const int ksteps = (F::FK - C * 64) >= 64 ? 4 : (F::FK - C * 64) / 16;
             const uint64_t bd = desc_off(bd0, stage * kBoxStride);
-            const uint32_t dphi = tm + cPhi + buf * 64;
+            const uint32_t dphi = tm + cPhi + (R <= 32 && !QSIDE ? 0 : buf * 64);
             // d-phi chunk = [Yown | y65] x box^T: the box's feature rows are a K-major B operand,
             // contraction over the 64 state columns, then the last column (second box)
 #pragma unroll
@@ -328,7 +332,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             if constexpr (!QSIDE) {
                 // dV += phi(k) chunk x box (MN-major B: 16 features per K step)
                 constexpr uint32_t idesc = idesc_bf16(128, 64, false, true);
-                const uint32_t fb = tm + cFB + (kTsA ? 0 : buf * 32);   // r <= 32: one staging buffer
+                const uint32_t fb = tm + cFB + buf * 32;
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
                     if (k < ksteps) umma_ts(tm + cdV, fb + k * 8, desc_off(bd, k * 2048), idesc, (C > 0 || k > 0) ? 1u : 0u);
@@ -359,59 +363,94 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
         Untensor<R> ut;
         if constexpr (!QSIDE) gen.init(m);
         ut.init(m);
-        // r <= 32: one staging buffer, free once chunk C's MMAs have completed (the tensor-memory columns beside it hold Y);
-        // r = 64 two.
-        constexpr bool kOneBuf = !QSIDE && kTsA;
-        auto stage_features = [&](int C) {        // features of a chunk -> tensor memory
-            uint32_t pk[32];
-            switch_chunk<0, F::NC>(C, [&](auto cc) { gen.template words<decltype(cc)::value * 32>(pk); });
-            tmem_st32(lane_tm + cFB + (kOneBuf ? 0 : (C & 1) * 32), pk);
-            tmem_st_wait();
-        };
-        if constexpr (!QSIDE) stage_features(0);
-        ok = ok && mbar_wait(&bar_box[0], 0, status, kErrTma);
-        tc_fence_before();
-        __syncthreads();
-        if (warp == 0 && elect_one()) {
-            tc_fence_after();
-            issue_chunk(0);
-        }
+        if constexpr (!QSIDE && R <= 32) {
+            // One d-phi buffer and two staging buffers: a chunk's d-phi goes into registers whole, the next chunk's MMAs go out
+            // and run behind the arithmetic and the staging of the chunk after that.  (With two d-phi buffers and one for the
+            // features these had to be staged between one chunk's MMAs and the next: key side, 48 heads x 16 384, r = 32: 375 us,
+            // now 340.  The query side in this manner: 265 -> 306.  Warps that drift apart, each at barriers of its own, fetch the
+            // unrolled code one after the other: a chunk's arithmetic 890 cycles instead of 660.)
+            auto stage_features = [&](int C) {             // features of a chunk -> tensor memory
+                uint32_t pk[32];
+                switch_chunk<0, F::NC>(C, [&](auto cc) { gen.template words<decltype(cc)::value * 32>(pk); });
+                tmem_st32(lane_tm + cFB + (C & 1) * 32, pk);
+                tmem_st_wait();
+            };
+            stage_features(0);
+            stage_features(1);
+            ok = ok && mbar_wait(&bar_box[0], 0, status, kErrTma) && mbar_wait(&bar_box[1], 0, status, kErrTma);
 #pragma unroll 1
-        for (int C = 0; C < F::NC; ++C) {          // (no early exit: a wait that gave up makes the later ones return at once)
-            const int buf = C & 1;
-            // One staging buffer: chunk C's MMAs read it, so they must have completed before chunk
-            // C+1's features go in; otherwise chunk C+1 is issued first and runs behind chunk C.
-            if constexpr (kOneBuf) {
-                ok = ok && mbar_wait(&bar_phi[buf], (C / 2) & 1, status, kErrMma);
-                tc_fence_after();
-            }
-            if (C + 1 < F::NC) {
-                if constexpr (!QSIDE) stage_features(C + 1);
-                if (C == 0) ok = ok && mbar_wait(&bar_box[1], 0, status, kErrTma);
+            for (int C = -1; C < F::NC; ++C) {        // (no early exit: a wait that gave up makes the later ones return at once)
+                uint32_t x0[32], x1[32];
+                if (C >= 0) {
+                    ok = ok && mbar_wait(&bar_phi[C & 1], (C / 2) & 1, status, kErrMma);
+                    tc_fence_after();
+                    if (tid == 32) refill(C);              // (warp 0 issues the MMAs; the loads go out from warp 1)
+                    const uint32_t dphi = lane_tm + cPhi;
+                    tmem_ld32(dphi, x0);
+                    tmem_ld32(dphi + 32, x1);
+                    tmem_ld_wait();
+                }
+                // every thread has read this chunk's d-phi and staged the features of the one to be issued
                 tc_fence_before();
-                __syncthreads();               // chunk C-1's d-phi has been read by every thread
-                if (warp == 0 && elect_one()) {
+                __syncthreads();
+                if (C + 1 < F::NC && warp == 0 && elect_one()) {
                     tc_fence_after();
                     issue_chunk(C + 1);
                 }
+                if (C >= 0) {
+                    switch_chunk<0, F::NC>(C, [&](auto cc) {
+                        constexpr int F0 = decltype(cc)::value * 64;
+                        ut.template add<F0>(x0);
+                        ut.template add<F0 + 32>(x1);
+                    });
+                    // (chunk C's MMAs, the last readers of this staging buffer, have completed)
+                    if (C + 2 < F::NC) stage_features(C + 2);
+                }
             }
-            if constexpr (!kOneBuf) {
+        } else {
+            auto stage_features = [&](int C) {        // features of a chunk -> tensor memory
+                uint32_t pk[32];
+                switch_chunk<0, F::NC>(C, [&](auto cc) { gen.template words<decltype(cc)::value * 32>(pk); });
+                tmem_st32(lane_tm + cFB + (C & 1) * 32, pk);
+                tmem_st_wait();
+            };
+            if constexpr (!QSIDE) stage_features(0);
+            ok = ok && mbar_wait(&bar_box[0], 0, status, kErrTma);
+            tc_fence_before();
+            __syncthreads();
+            if (warp == 0 && elect_one()) {
+                tc_fence_after();
+                issue_chunk(0);
+            }
+#pragma unroll 1
+            for (int C = 0; C < F::NC; ++C) {          // (no early exit: a wait that gave up makes the later ones return at once)
+                const int buf = C & 1;
+                if (C + 1 < F::NC) {
+                    if constexpr (!QSIDE) stage_features(C + 1);
+                    if (C == 0) ok = ok && mbar_wait(&bar_box[1], 0, status, kErrTma);
+                    tc_fence_before();
+                    __syncthreads();               // chunk C-1's d-phi has been read by every thread
+                    if (warp == 0 && elect_one()) {
+                        tc_fence_after();
+                        issue_chunk(C + 1);
+                    }
+                }
                 ok = ok && mbar_wait(&bar_phi[buf], (C / 2) & 1, status, kErrMma);
                 tc_fence_after();
+                if (tid == 32) refill(C);              // (warp 0 issues the MMAs; the loads go out from warp 1)
+                uint32_t x[32];
+                tmem_ld32(lane_tm + cPhi + buf * 64, x);
+                tmem_ld_wait();
+                switch_chunk<0, F::NC>(C, [&](auto cc) {
+                    constexpr int F0 = decltype(cc)::value * 64;
+                    ut.template add<F0>(x);
+                    if constexpr (F0 + 32 < F::F) {
+                        tmem_ld32(lane_tm + cPhi + buf * 64 + 32, x);
+                        tmem_ld_wait();
+                        ut.template add<F0 + 32>(x);
+                    }
+                });
             }
-            if (tid == 32) refill(C);              // (warp 0 issues the MMAs; the loads go out from warp 1)
-            uint32_t x[32];
-            tmem_ld32(lane_tm + cPhi + buf * 64, x);
-            tmem_ld_wait();
-            switch_chunk<0, F::NC>(C, [&](auto cc) {
-                constexpr int F0 = decltype(cc)::value * 64;
-                ut.template add<F0>(x);
-                if constexpr (F0 + 32 < F::F) {
-                    tmem_ld32(lane_tm + cPhi + buf * 64 + 32, x);
-                    tmem_ld_wait();
-                    ut.template add<F0 + 32>(x);
-                }
-            });
         }
         ut.finish(dm);
         if constexpr (!QSIDE) dv_started = true;
@@ -432,7 +471,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     float* oth_col = reinterpret_cast<float*>(smem + L::Eoth);     // other rows: 1/d, scaled 1/d, scaled -(g . O)/d
     const float y65h_inv = y65h * inv_own;
     const f2 own_sinv = pack2(kDwScale * inv_own, kDwScale * inv_own), own_syinv = pack2(kDwScale * y65h_inv, kDwScale * y65h_inv);
-    if constexpr (LIN && LOCAL) ok = ok && mbar_wait(&bar_own, 1, status, kErrTma);      // the raw own rows
+    if constexpr (LIN && LOCAL) ok = ok && mbar_wait(&bar_again, 0, status, kErrTma);    // the raw own rows
 #pragma unroll 1
     for (int tp = tp_begin; tp < tp_end; ++tp) {
         const int orow0 = l * b + tp * 128;
@@ -491,6 +530,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             tc_fence_after();
             // dW = (own . other + y) / d_i,  ds = 2 s dW,  W / d_i = s^2 / d_i, masked on the diagonal
             // tile; packed to bf16 over columns whose fp32 contents have already been read
+            // (key side: one copy of the code, the mask in front of it; query side: a copy for the diagonal tile)
             auto tile_math = [&](auto diag_c) {
                 constexpr bool DIAG = decltype(diag_c)::value;
 #pragma unroll
@@ -499,6 +539,11 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                     tmem_ld32(lane_tm + cS + c0, sv);
                     tmem_ld32(lane_tm + cDW + c0, wv);
                     tmem_ld_wait();
+                    if (!QSIDE && diag) {
+                        const int own = tid - hh * 64 - c0;           // the own row among these 32 others
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) sv[j] = j >= own ? sv[j] : 0u;
+                    }
 #pragma unroll
                     for (int j = 0; j < 32; j += 4) {
                         const int col = hh * 64 + c0 + j;
@@ -515,8 +560,8 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                         for (int i = 0; i < 2; ++i) {
                             float s0 = __uint_as_float(sv[j + 2 * i]), s1 = __uint_as_float(sv[j + 2 * i + 1]);
                             if constexpr (DIAG) {
-                                s0 = (QSIDE ? (col + 2 * i <= tid) : (col + 2 * i >= tid)) ? s0 : 0.f;
-                                s1 = (QSIDE ? (col + 2 * i + 1 <= tid) : (col + 2 * i + 1 >= tid)) ? s1 : 0.f;
+                                s0 = col + 2 * i <= tid ? s0 : 0.f;
+                                s1 = col + 2 * i + 1 <= tid ? s1 : 0.f;
                             }
                             const f2 s = pack2(s0, s1);
                             // 2 dW, or 4 dW with LOCAL (exact: powers of two)
@@ -535,7 +580,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                     if constexpr (!QSIDE) tmem_st16(lane_tm + cDW + c0 / 2, pw);
                 }
             };
-            if (diag) tile_math(std::true_type{}); else tile_math(std::false_type{});
+            if (QSIDE && diag) tile_math(std::true_type{}); else tile_math(std::false_type{});
             tmem_st_wait();
             tc_fence_before();
             __syncthreads();
@@ -581,11 +626,11 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
         tc_fence_before();
         __syncthreads();
         if (tid == 0) {
-            mbar_expect_tx(&bar_own, 16384 + GImage<R>::bytes);
-            tma_load_4d(smem + L::Xown, &mapXown, 0, row0, hi, bi, &bar_own);
-            bulk_load(smem + L::G, gimg + (size_t)g * GImage<R>::bytes, GImage<R>::bytes, &bar_own);
+            mbar_expect_tx(&bar_again, 16384 + GImage<R>::bytes);
+            tma_load_4d(smem + L::Xown, &mapXown, 0, row0, hi, bi, &bar_again);
+            bulk_load(smem + L::G, gimg + (size_t)g * GImage<R>::bytes, GImage<R>::bytes, &bar_again);
         }
-        ok = ok && mbar_wait(&bar_own, 1, status, kErrTma);
+        ok = ok && mbar_wait(&bar_again, 0, status, kErrTma);
         tc_fence_after();
     }
 
@@ -732,9 +777,10 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
         bulk_commit();
         bulk_wait_read();
     }
+    cta_drain(warp == 0, &bar_drain);
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 256);
+    if (warp == 2) tmem_dealloc(tm, 256);
 }
 
 template <int R>

@@ -146,25 +146,24 @@ struct HiLoTiles { static constexpr int N = (2 * R + 63) / 64; };
 // themselves where they are the half sketch (degree 2: r = h, given to the last bit, no lo).
 template <int R, bool LIN> struct OthTiles { static constexpr int N = (LIN && R == 64) ? 1 : HiLoTiles<R>::N; };
 
-// (TILES: how many of them)
+// (TILES: how many of them are wanted)
 template <int R, int TILES = HiLoTiles<R>::N>
 __device__ __forceinline__ void store_hilo_tiles(uint8_t* dst, const float (&m)[R], int row) {
+    auto chunk = [&](int c) { return reinterpret_cast<uint4*>(dst + (c / 8) * 16384 + swz128_offset(row, c % 8)); };
 #pragma unroll
-    for (int ch = 0; ch < TILES * 8; ++ch) {
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (ch * 8 < 2 * R) {
-            float x[8];
+    for (int ch = 0; ch < R / 8; ++ch) {
+        uint32_t h[4], l[4];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int col = ch * 8 + j, c = col % R;
-                const float hi = __bfloat162float(__float2bfloat16_rn(m[c]));
-                x[j] = col < R ? hi : (m[c] - hi);
-            }
-            v.x = pack_bf16(x[0], x[1]); v.y = pack_bf16(x[2], x[3]);
-            v.z = pack_bf16(x[4], x[5]); v.w = pack_bf16(x[6], x[7]);
+        for (int i = 0; i < 4; ++i) {
+            const float a = m[8 * ch + 2 * i], b = m[8 * ch + 2 * i + 1];
+            h[i] = pack_bf16(a, b);
+            l[i] = pack_bf16(a - __uint_as_float(h[i] << 16), b - __uint_as_float(h[i] & 0xffff0000u));
         }
-        *reinterpret_cast<uint4*>(dst + (ch / 8) * 16384 + swz128_offset(row, ch % 8)) = v;
+        *chunk(ch) = make_uint4(h[0], h[1], h[2], h[3]);
+        if (R / 8 + ch < TILES * 8) *chunk(R / 8 + ch) = make_uint4(l[0], l[1], l[2], l[3]);
     }
+#pragma unroll
+    for (int ch = R / 4; ch < TILES * 8; ++ch) *chunk(ch) = make_uint4(0, 0, 0, 0);
 }
 
 }  // namespace tc

@@ -366,14 +366,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // Before a CTA that has given up a wait frees its tensor memory and ends: the MMAs it has issued must have completed and the
 // copies on their way into its shared memory must have arrived.  The elected lane of the issuing warp waits for a commit
 // of its own (with a limit), then long enough for any copy.  `bar`: a barrier of count 1 that nothing else uses.
-__device__ __forceinline__ void cta_drain(bool issuing_warp, uint64_t* bar, int* status) {
+__device__ __forceinline__ void cta_drain(bool issuing_warp, uint64_t* bar) {
     if (!__any_sync(0xffffffffu, cta_gave_up())) return;
     if (issuing_warp && elect_one()) {
         umma_commit(bar);
         for (int i = 0; i < 1000 && !mbar_test(bar, 0); ++i) __nanosleep(1000);
         for (int i = 0; i < 200; ++i) __nanosleep(1000);
     }
-    (void)status;
 }
 
 // Byte offset of 16-byte chunk `chunk` (0..7) of row `row` inside a [rows x 128 B] tile held in
