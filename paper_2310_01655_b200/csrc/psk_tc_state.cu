@@ -47,28 +47,31 @@ constexpr int kModeFirst = 2;          // run 0: both; the other runs: the total
 //   NWG generator warpgroups  thread = token: read the half sketches, write their feature tiles
 //                             (dealt in turn) as MN-major A operands into shared memory; one of them also
 //                             puts the half sketches where their rows were;
-//   1 store warpgroup         thread = feature row: at block boundaries reads the accumulators,
+//   NSW store warpgroups      thread = feature row: at block boundaries reads the accumulators,
 //                             centres, rounds and stores them;
 //   2 feeder warps            one thread each: every TMA load and sketch GEMM; every state GEMM.
 // Stored layout S[blk][FP][80]: one row per feature, 64 state columns, the last column, zeros.
 // ---------------------------------------------------------------------------
-template <int R, int NWG>
+template <int R, int NWG, int NSW>
 struct StateSmem {
     static constexpr uint32_t kG = 2 * R * 128 < 1024 ? 1024 : 2 * R * 128;
     // X: 16 KB slots for the rows to sketch, through which their half sketches leave.  A third one where there is room:
     // with two, a tile's rows can be requested only when the half sketches two tiles earlier have left.
-    static constexpr int kXSlots = 3 * 16384 + 65536 + kG + NWG * 32768 + 128 * 160 + (R == 64 ? 16384 : 0) + 3072 <= 232448 ? 3 : 2;
+    static constexpr int kXSlots = R < 64 && 3 * 16384 + 49152 + kG + NWG * 32768 + NSW * 128 * 160 + 3072 <= 232448 ? 3 : 2;
     static_assert(R < 64 || kXSlots == 2, "the second half's buffer is single");
     static constexpr uint32_t X = 0;
-    static constexpr uint32_t Y = kXSlots * 16384;       // 2 x (16 KB values + 16 KB last-column chunk)
-    static constexpr uint32_t kYSlot = 32768;
-    static constexpr uint32_t G = Y + 2 * kYSlot;
+    static constexpr uint32_t Y = kXSlots * 16384;       // two slots of 16 KB values
+    // The operand's columns 64..79 (the last column, zeros) of both slots: 32 of the 128 bytes of a row each, so one chunk of the
+    // same layout holds both, slot 1's two 16-byte pieces further on
+    static constexpr uint32_t kYSlot = 16384, Ext = Y + 2 * kYSlot;
+    static constexpr uint32_t G = Ext + 16384;
     static constexpr uint32_t A0 = G + kG;
-    static constexpr uint32_t St = A0 + NWG * 32768;     // one state tile on its way out: 128 rows x 160 B
-    static constexpr bool kStaged = St + 128 * 160 + 2048 <= 232448;     // where it fits (r <= 32)
+    static constexpr uint32_t St = A0 + NWG * 32768;     // a state tile on its way out per store warpgroup: 128 rows x 160 B
+    static constexpr uint32_t kSt = NSW * 128 * 160;
+    static constexpr bool kStaged = St + kSt + (R == 64 ? 16384 : 0) + 2048 <= 232448;     // where it fits
     // r = 64: the second 64 columns of a tile's [hi | lo] half sketches on their way out (the first, and all of
     // them for r <= 32, leave through the tile's own X buffer)
-    static constexpr uint32_t Hl = St + (kStaged ? 128 * 160 : 0);
+    static constexpr uint32_t Hl = St + (kStaged ? kSt : 0);
     static constexpr uint32_t total = Hl + (R == 64 ? 16384 : 0);
     static_assert(total + 2048 <= 232448, "shared memory");
 };
@@ -129,7 +132,7 @@ static __device__ __noinline__ void state_init_acc(const float* __restrict__ tot
 
 // SEG = false is the plain walk of a whole head by one CTA (nseg = 1, prefix mode, no start value):
 // its run bookkeeping folds away at compile time.
-template <int R, int T0, int TN, int NWG, bool SEG, typename SH>
+template <int R, int T0, int TN, int NWG, int NSW, bool SEG, typename SH>
 __device__ __forceinline__ void
 state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUtensorMap& mapH, const CUtensorMap& mapH2, int want_hl,
            const uint8_t* __restrict__ gimg, int g_heads, int H, int n, int b, int t,
@@ -137,7 +140,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
            int center_mode, int reverse, int nseg_arg, int mode_arg, int run0, int units, float* __restrict__ tot,
            bf16* __restrict__ S, int lin, int* status) {
     using F = Feat<R>;
-    using L = StateSmem<R, NWG>;
+    using L = StateSmem<R, NWG, NSW>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     const int tid = threadIdx.x, warp = warp_index(), wg = warp / 4, wt = tid % 128;
@@ -158,7 +161,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
     const bool hl = T0 + TN == F::NT && want_hl != 0 && mode != kModeTotal;
     // a later run of a prefix pass starts from the sum of the earlier runs' totals
     const bool init = SEG && mode == kModePrefix && seg > 0;
-    constexpr int kThreads = 128 * (NWG + 1) + 64;
+    constexpr int kThreads = 128 * (NWG + NSW) + 64;
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -174,18 +177,15 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
         mbar_fence_init();
         tma_prefetch_desc(&mapX); tma_prefetch_desc(&mapY);
     }
-    // last-column chunks of both slots: zero, and column 0 = 1 when the last column is all ones
-    for (int e = tid; e < 2 * 1024; e += kThreads) {
-        const int s = e / 1024, i = e % 1024;
-        reinterpret_cast<uint4*>(smem + L::Y + s * L::kYSlot + 16384)[i] = make_uint4(0, 0, 0, 0);
-    }
+    // last-column chunk of both slots: zero, and each slot's column 0 = 1 when the last column is all ones
+    for (int e = tid; e < 1024; e += kThreads) reinterpret_cast<uint4*>(smem + L::Ext)[e] = make_uint4(0, 0, 0, 0);
     pdl_sync();            // (before the allocation: a waiting CTA must not hold tensor memory)
     if (warp == 0) { tmem_alloc(&sh.tmem_slot, 512); tmem_relinquish(); }
     if (tid < 64) sh.cm[tid] = cmean != nullptr ? cmean[(size_t)bh * 64 + tid] : 0.f;
     __syncthreads();
     if (y65 == nullptr && tid < 128) {
-        *reinterpret_cast<bf16*>(smem + L::Y + 16384 + swz128_offset(tid, 0)) = __float2bfloat16_rn(1.f);
-        *reinterpret_cast<bf16*>(smem + L::Y + L::kYSlot + 16384 + swz128_offset(tid, 0)) = __float2bfloat16_rn(1.f);
+        *reinterpret_cast<bf16*>(smem + L::Ext + swz128_offset(tid, 0)) = __float2bfloat16_rn(1.f);
+        *reinterpret_cast<bf16*>(smem + L::Ext + swz128_offset(tid, 2)) = __float2bfloat16_rn(1.f);
     }
     fence_proxy_async_smem();
     tc_fence_before();
@@ -196,13 +196,13 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
     // token tile visited at step j of this run (runs and tiles go backwards for suffix sums)
     auto tile_of = [&](int j) { const int gj = j0r + j; return reverse ? (NJ - 1 - gj) : gj; };
 
-    if (wg == NWG + 1) {
+    if (wg == NWG + NSW) {
         // =============================== feeders ===============================
         // Two issuing threads in two warps.  The first loads the tiles and issues the sketch
         // GEMMs, the second issues the state GEMMs: between two of its MMAs lies as little as
         // possible (each satisfied wait, commit or TMA issue costs a single thread about a
         // hundred cycles, during which the tensor pipe would idle).
-        if (warp == 4 * (NWG + 1) && elect_one()) {
+        if (warp == 4 * (NWG + NSW) && elect_one()) {
             bool ok = true;
             constexpr int NX = L::kXSlots;
             auto load_x = [&](int j) {
@@ -256,13 +256,14 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
             // twice before a generator thread has looked.)
             umma_commit(&sh.drain[0]);
             mbar_wait(&sh.drain[0], 0, status, kErrMma);
-        } else if (warp == 4 * (NWG + 1) + 1 && elect_one()) {
+        } else if (warp == 4 * (NWG + NSW) + 1 && elect_one()) {
             constexpr uint32_t idesc_state = idesc_bf16(128, 80, true, true);
             bool ok = true;
             int w = 0;                                    // feature tile number u comes from warpgroup w = u mod NWG, as its
             uint32_t w_par = 0;                           // tile number u / NWG: parity w_par
             const uint64_t ad0 = smem_desc(smem_u32(smem + L::A0), 16384, 1024, kSwz128);
-            const uint64_t yd0 = smem_desc(smem_u32(smem + L::Y), 16384, 1024, kSwz128);
+            const uint64_t yd0 = smem_desc(smem_u32(smem + L::Y), L::Ext - L::Y, 1024, kSwz128);
+            const uint64_t yd1 = smem_desc(smem_u32(smem + L::Y) + L::kYSlot, L::Ext + 32 - L::Y - L::kYSlot, 1024, kSwz128);
             const int ibase = init ? 0 : 1;               // completions of sh.accread before block 1's
             for (int j = 0; j < NJs && ok; ++j) {
                 ok = mbar_spin(&sh.fully[j & 1], (j >> 1) & 1, status, kErrTma);
@@ -271,7 +272,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
                 // written) the accumulators' values before anything is added to them
                 const bool boundary = mode != kModeTotal && (j % tpb == 0) && (j > 0 || init);
                 const bool block_end = mode != kModeTotal ? ((j + 1) % tpb == 0) : (j == NJs - 1);
-                const uint64_t yd = desc_off(yd0, (j & 1) * L::kYSlot);
+                const uint64_t yd = (j & 1) ? yd1 : yd0;
                 const uint32_t acc0 = (j > 0 || init) ? 1u : 0u;
                 static_for<0, TN>([&](auto ic) {
                     constexpr int I = decltype(ic)::value;
@@ -295,18 +296,21 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
             umma_commit(&sh.drain[1]);
             mbar_wait(&sh.drain[1], 0, status, kErrMma);
         }
-    } else if (wg == NWG) {
-        // ============================ store warpgroup ============================
+    } else if (wg >= NWG) {
+        // ============================ store warpgroups ============================
+        // (the tiles are dealt to them in turn)
         // Tiles leave through shared memory: a warp's 32 rows of 160 B are one contiguous 5 KB
         // piece of the state array, which goes out as one bulk copy.  (Rows stored by their threads directly would be
         // 10 scattered 16-byte stores each: the L1 data path, which the MMA operands and the generators' tiles also
         // go through, is this kernel's busiest unit.)  One body for all tiles: the kernel is short of instruction cache.
         const uint32_t lane_tm = tm + ((uint32_t)((warp % 4) * 32) << 16);
-        uint8_t* stage = smem + L::St;
+        const int sw = wg - NWG;
+        uint8_t* stage = smem + L::St + sw * (128 * 160);
         // totals: the raw fp32 accumulators at the end of the run
         auto dump_totals = [&](uint32_t parity) {
             static_for<0, TN>([&](auto ic) {
                 constexpr int I = decltype(ic)::value;
+                if (NSW > 1 && I % NSW != sw) return;
                 mbar_wait(&sh.accfull[I], parity, status, kErrMma);
                 tc_fence_after();
                 float4* out = reinterpret_cast<float4*>(tot + ((((size_t)bh * nseg + seg) * F::NT + (T0 + I)) * 128 + wt) * 80);
@@ -326,7 +330,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
         if (init) {
             // a later run starts from the sum of the earlier runs' totals: into the accumulators
             // first, then block 0 of the run is read back like every other block
-            for (int I = 0; I < TN; ++I)
+            for (int I = sw; I < TN; I += NSW)
                 state_init_acc(tot, (((size_t)bh * nseg + (seg - 1)) * F::NT + (T0 + I)) * 128 + wt, lane_tm + kAcc + 80 * I);
             tmem_st_wait();
         }
@@ -334,7 +338,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
             const int pg = p0r + p;
             const int l = reverse ? (t - 1 - pg) : pg;
 #pragma unroll 1
-            for (int I = 0; I < TN; ++I) {
+            for (int I = sw; I < TN; I += NSW) {
                 if (p > 0) {
                     mbar_wait(&sh.accfull[I], (p - 1) & 1, status, kErrMma);
                     tc_fence_after();
@@ -342,57 +346,75 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
                 const bool live = p > 0 || init;          // the accumulator holds values (else: zeros)
                 const uint32_t acc = lane_tm + kAcc + 80 * I;
                 // this thread's feature row: 80 bf16 = ten 16-byte pieces of the staging tile
-                if constexpr (L::kStaged) {               // the previous tile has left it
-                    if (wt % 32 == 0) bulk_wait_read();
-                    __syncwarp();
-                }
                 uint4* const grow = reinterpret_cast<uint4*>(S + (((size_t)bh * t + l) * F::FP + (size_t)(T0 + I) * 128 + wt) * 80);
                 uint4* dst = L::kStaged ? reinterpret_cast<uint4*>(stage + wt * 160) : grow;
-                if (live) {
+                uint32_t pk[33];                          // the row's 64 columns and the last one, formed before the staging tile is waited for
+                if (live && (T0 + I) * 128 + wt / 32 * 32 < F::F) {       // (a warp's rows beyond the last feature: zeros)
                     // centred values, in fp32, without touching the operands (the mode only selects
                     // coefficients):  mode 1: sum phi (y - c)^T = H[:, :64] - H[:, 64] c^T
                     //                 mode 2: last column H[:, 64] - H[:, :64] c
-                    uint32_t v[2][16], last_raw;
+                    // One store warpgroup, staged: all columns in one trip to tensor memory, the accumulator handed back before
+                    // they are worked on.  Two (fewer registers), or rows stored directly: 16 columns at a time, the next on their way.
+                    constexpr bool kAtOnce = NSW == 1 && L::kStaged;
+                    uint32_t v[kAtOnce ? 4 : 2][16], last_raw;
                     tmem_ld1(acc + 64, last_raw);
-                    tmem_ld16(acc, v[0]);
-                    tmem_ld_wait();
-                    const float last = __uint_as_float(last_raw);
-                    float corr = 0.f;
-                    const float k1 = center_mode == 1 ? -last : 0.f, k2 = center_mode == 2 ? 1.f : 0.f;
-                    // the row's pair weight (tc_features.cuh) goes into the stored state; 0 on padding rows
-                    const float wgt = F::weight((T0 + I) * 128 + wt);
 #pragma unroll
-                    for (int h = 0; h < 4; ++h) {             // 16 columns, the next ones on their way
-                        if (h < 3) tmem_ld16(acc + 16 * (h + 1), v[(h + 1) & 1]);
-                        uint32_t pk[8];
+                    for (int h = 0; h < (kAtOnce ? 4 : 1); ++h) tmem_ld16(acc + 16 * h, v[h]);
+                    tmem_ld_wait();
+                    auto handed_back = [&]() {
+                        tc_fence_before();
+                        if (wt % 32 == 0) mbar_arrive(&sh.accread[I]);
+                    };
+                    if (kAtOnce) handed_back();
+                    const float last = __uint_as_float(last_raw);
+                    const float k1s = center_mode == 1 ? -last : 0.f;
+                    const f2 k1 = pack2(k1s, k1s);
+                    f2 corr = 0ull;
+                    // the row's pair weight (tc_features.cuh) goes into the stored state
+                    const float wgt = F::weight((T0 + I) * 128 + wt);
+                    const f2 w2 = pack2(wgt, wgt);
+                    const bool pad = F::F % 32 != 0 && (T0 + I) * 128 + wt >= F::F;        // (such a row's sums may be anything)
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        if (!kAtOnce && h < 3) tmem_ld16(acc + 16 * (h + 1), v[(h + 1) & 1]);
+                        const uint32_t (&u)[16] = v[kAtOnce ? h : h & 1];
 #pragma unroll
                         for (int q = 0; q < 16; q += 4) {
-                            const float4 c4 = *reinterpret_cast<const float4*>(&sh.cm[16 * h + q]);
-                            const float cv[4] = {c4.x, c4.y, c4.z, c4.w};
-#pragma unroll
-                            for (int i = 0; i < 4; i += 2) {
-                                const float x0 = fmaf(k1, cv[i], __uint_as_float(v[h & 1][q + i]));
-                                const float x1 = fmaf(k1, cv[i + 1], __uint_as_float(v[h & 1][q + i + 1]));
-                                corr = fmaf(k2 * cv[i], x0, corr);
-                                corr = fmaf(k2 * cv[i + 1], x1, corr);
-                                pk[(q + i) / 2] = pack_bf16(x0 * wgt, x1 * wgt);
-                            }
+                            const ulonglong2 c4 = *reinterpret_cast<const ulonglong2*>(&sh.cm[16 * h + q]);
+                            const f2 x0 = fma2(k1, c4.x, pack2(u[q], u[q + 1])), x1 = fma2(k1, c4.y, pack2(u[q + 2], u[q + 3]));
+                            if (center_mode == 2) corr = fma2(c4.y, x1, fma2(c4.x, x0, corr));
+                            const f2 y0 = mul2(x0, w2), y1 = mul2(x1, w2);
+                            pk[8 * h + q / 2] = pad ? 0u : pack_bf16(lo2(y0), hi2(y0));
+                            pk[8 * h + q / 2 + 1] = pad ? 0u : pack_bf16(lo2(y1), hi2(y1));
                         }
-                        dst[2 * h] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                        dst[2 * h + 1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-                        if (h < 3) {
+                        if constexpr (!L::kStaged) {
+                            dst[2 * h] = make_uint4(pk[8 * h], pk[8 * h + 1], pk[8 * h + 2], pk[8 * h + 3]);
+                            dst[2 * h + 1] = make_uint4(pk[8 * h + 4], pk[8 * h + 5], pk[8 * h + 6], pk[8 * h + 7]);
+                        }
+                        if (!kAtOnce && h < 3) {
                             tmem_ld_wait16(v[(h + 1) & 1]);
-                            if (h == 2) {                     // last read of this accumulator: hand it (back) to the MMAs
-                                tc_fence_before();
-                                if (wt % 32 == 0) mbar_arrive(&sh.accread[I]);
-                            }
+                            if (h == 2) handed_back();        // last read of this accumulator
                         }
                     }
-                    dst[8] = make_uint4(pack_bf16((last - corr) * wgt, 0.f), 0, 0, 0);
+                    pk[32] = pad ? 0u : pack_bf16((last - (lo2(corr) + hi2(corr))) * wgt, 0.f);
                 } else {
 #pragma unroll
-                    for (int q = 0; q < 9; ++q) dst[q] = make_uint4(0, 0, 0, 0);
+                    for (int q = 0; q < 33; ++q) pk[q] = 0u;
+                    if constexpr (!L::kStaged) {
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) dst[q] = make_uint4(0, 0, 0, 0);
+                    }
+                    if (live) { __syncwarp(); if (wt % 32 == 0) mbar_arrive(&sh.accread[I]); }
                 }
+                if constexpr (L::kStaged) {                   // the previous tile has left it
+                    if (wt % 32 == 0) bulk_wait_read();
+                    __syncwarp();
+                }
+                if constexpr (L::kStaged) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) dst[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+                }
+                dst[8] = make_uint4(pk[32], 0, 0, 0);
                 dst[9] = make_uint4(0, 0, 0, 0);
                 if constexpr (L::kStaged) {
                     fence_proxy_async_smem();
@@ -451,7 +473,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
                 if (j >= 2) mbar_wait(&sh.yfree[j & 1], ((j >> 1) - 1) & 1, status, kErrState);
                 const float y = y_next;
                 if (j + 1 < NJs) y_next = y65[(size_t)bh * n + tile_of(j + 1) * 128 + wt];
-                *reinterpret_cast<bf16*>(smem + L::Y + (j & 1) * L::kYSlot + 16384 + swz128_offset(wt, 0)) =
+                *reinterpret_cast<bf16*>(smem + L::Ext + swz128_offset(wt, 2 * (j & 1))) =
                     __float2bfloat16_rn(y);
                 fence_proxy_async_smem();
                 wg_barrier(0);
@@ -465,9 +487,12 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
                     constexpr int W0 = (T0 + decltype(ic)::value) * 64;           // the tile's first word
                     static_for<0, 16>([&](auto cc) {
                         constexpr int C = decltype(cc)::value;
-                        uint32_t pk[4];
-                        gen.template words<W0 + 4 * C>(pk);
-                        *reinterpret_cast<uint4*>(sA + (C / 8) * 16384 + swz128_offset(wt, C % 8)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                        // (rows beyond the last feature keep what an earlier tile left: their sums are never used)
+                        if constexpr (2 * (W0 + 4 * C) < F::F) {
+                            uint32_t pk[4];
+                            gen.template words<W0 + 4 * C>(pk);
+                            *reinterpret_cast<uint4*>(sA + (C / 8) * 16384 + swz128_offset(wt, C % 8)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                        }
                     });
                 });
                 fence_proxy_async_smem();
@@ -495,11 +520,15 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
 // The feature tiles of a head are dealt to SPLIT CTAs, each of which forms the half sketches anew.  blockIdx.z, the
 // slowest index: CTAs that run at the same time then run the same specialised code (with the shares of a head side by
 // side on neighbouring SMs the kernel took 1.5 times as long, for want of instruction cache).  r = 64 has 17 tiles and tensor memory for four accumulators beside the sketch columns.
+// Store warpgroups: the walk stalls at a block boundary until the accumulators have been read, one tile after the other.  Two help
+// where a share has two tiles and registers for them (r = 32 in three shares: 48 heads x 16 384, b = 256: 402 us per training step for both
+// walks, one warpgroup that reads all columns at once 382, two 374); with five tiles a CTA (one share, 96 heads x 8192) the generators
+// bound it (400, 394, 402), r = 16 has 212, 204, 212, and r = 64 no registers (1276, 1237, spills).
 template <int R, int SPLIT> struct StateSplit {
     static constexpr int NT = Feat<R>::NT, kBase = NT / SPLIT, kMore = NT % SPLIT;
     __host__ __device__ static constexpr int tiles(int z) { return kBase + (z < kMore ? 1 : 0); }
     __host__ __device__ static constexpr int first(int z) { return z * kBase + (z < kMore ? z : kMore); }
-    static constexpr int NWG = tiles(0) < 3 ? tiles(0) : 3, kThreads = 128 * (NWG + 1) + 64;
+    static constexpr int NWG = tiles(0) < 3 ? tiles(0) : 3, NSW = R == 32 && SPLIT == 3 ? 2 : 1, kThreads = 128 * (NWG + NSW) + 64;
 };
 
 template <int R, int SPLIT, bool SEG>
@@ -508,7 +537,7 @@ __global__ void __launch_bounds__(StateSplit<R, SPLIT>::kThreads) tc_state_kerne
     __shared__ StateShared<P::tiles(0), P::NWG> sh;
     static_for<0, SPLIT>([&](auto zc) {
         constexpr int Z = decltype(zc)::value;
-        if (SPLIT == 1 || (int)blockIdx.z == Z) state_walk<R, P::first(Z), P::tiles(Z), P::NWG, SEG>(sh, PSK_STATE_ARGS);
+        if (SPLIT == 1 || (int)blockIdx.z == Z) state_walk<R, P::first(Z), P::tiles(Z), P::NWG, P::NSW, SEG>(sh, PSK_STATE_ARGS);
     });
 }
 
@@ -565,9 +594,9 @@ tc_state_sum_kernel(const float* __restrict__ tot, int nseg, const float* __rest
         const float x0 = center_mode == 1 ? v[c] - last * c0 : v[c];
         const float x1 = center_mode == 1 ? v[c + 1] - last * c1 : v[c + 1];
         if (center_mode == 2) corr += c0 * x0 + c1 * x1;
-        pk[c / 2] = pack_bf16(x0 * wgt, x1 * wgt);
+        pk[c / 2] = row < F::F ? pack_bf16(x0 * wgt, x1 * wgt) : 0u;       // (rows beyond the last feature may hold anything)
     }
-    pk[32] = pack_bf16((last - corr) * wgt, 0.f);
+    pk[32] = row < F::F ? pack_bf16((last - corr) * wgt, 0.f) : 0u;
 #pragma unroll
     for (int c = 33; c < 40; ++c) pk[c] = 0u;
     uint4* out = reinterpret_cast<uint4*>(S + ((size_t)bh * F::FP + row) * 80);
@@ -634,7 +663,7 @@ template <int R, int SPLIT>
 cudaError_t launch_split(const Dims& d, const CUtensorMap& mX, const CUtensorMap& mY, const uint8_t* gimg,
                          const StateArgs& a, int* status, cudaStream_t s, int* launches) {
     using P = StateSplit<R, SPLIT>;
-    constexpr size_t smem = StateSmem<R, P::NWG>::total + 1024;
+    constexpr size_t smem = StateSmem<R, P::NWG, P::NSW>::total + 1024;
     // Programmatic dependence saves a short walk 2 to 6 us (forward of 12 heads x 16 512, two passes over 11 runs: 185 -> 180 us;
     // 12 heads x 1024, training: 88 -> 83).  But CTAs that start early settle on the SMs that happen to be free, shares of a head
     // side by side, and neighbours that run different code are slow (StateSplit): where the shares fill the GPU that costs a
