@@ -138,6 +138,20 @@ __device__ __forceinline__ void issue_scores(uint32_t d_tmem, uint32_t own, uint
     }
 }
 
+// The same with the own rows' [hi | lo] half sketches in tensor memory (a_tmem; r <= 32: R words a row).
+// (An operand read from shared memory makes an MMA of N = 64 take 47 cycles instead of 31 and takes the path from the other CTA;
+// query side, 384 heads x 8192, r = 32: 1014 -> 996 us, 96 heads x 8192, r = 16: 181 -> 177.)
+template <int R>
+__device__ __forceinline__ void issue_scores_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t oth) {
+    constexpr uint32_t idesc = idesc_bf16(128, 64, false, false);
+    constexpr int offA[3] = {0, R, 0}, offB[3] = {0, 0, R};
+#pragma unroll
+    for (int g = 0; g < 3; ++g)
+#pragma unroll
+        for (int kk = 0; kk < R / 16; ++kk)
+            umma_ts(d_tmem, a_tmem + (offA[g] + kk * 16) / 2, desc_off(smem_desc(oth, 0, 1024, kSwz128), (offB[g] + kk * 16) * 2), idesc, (g > 0 || kk > 0) ? 1u : 0u);
+}
+
 // LOCAL (Section 3.2): same-block pairs carry the exact weights x_ij^4, x_ij = q_i . k_j.  The
 // tile scores are then X_own X_other^T over the head dimension (raw bf16 rows: exact products),
 // dL/dx_ij = 4 x_ij^3 dW_ij replaces ds_ij, and it multiplies the other side's raw rows straight
@@ -259,6 +273,9 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     // which phase C then reads from shared memory instead.
     constexpr bool kTsC = kTsA && !(LOCAL && !QSIDE);
     constexpr uint32_t cXl = (kTsA && QSIDE) ? cdV : cdM;
+    // Query side, r <= 32, sketched weights: the own rows' [hi | lo] half sketches take the unused dV columns, as the scores' A
+    // operand.  (The key side has no columns left, given half sketches are operands where TMA put them.)
+    constexpr bool kTsM = QSIDE && kTsA && !LOCAL && !LIN;
     uint32_t mma_uses = 0;
     bool ok = true;
 
@@ -462,7 +479,18 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     }
 
     // ---- phase C: same block, other-side tiles, 64 other rows at a time ----
-    if constexpr (!LOCAL && !LIN) store_hilo_tiles<R>(smem + L::Mown, m, tid);
+    if constexpr (kTsM) {
+        uint32_t hl[R];
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i) {
+            hl[i] = pack_bf16(m[2 * i], m[2 * i + 1]);
+            hl[R / 2 + i] = pack_bf16(m[2 * i] - __uint_as_float(hl[i] << 16), m[2 * i + 1] - __uint_as_float(hl[i] & 0xffff0000u));
+        }
+        if constexpr (R == 32) tmem_st32(lane_tm + cdV, hl); else tmem_st16(lane_tm + cdV, hl);
+        tmem_st_wait();
+    } else if constexpr (!LOCAL && !LIN) {
+        store_hilo_tiles<R>(smem + L::Mown, m, tid);
+    }
     const int tp_begin = QSIDE ? 0 : tau, tp_end = noncausal ? tp_begin : (QSIDE ? tau + 1 : ntiles);
     bool dm_started = false;
     uint32_t oth_uses = 0;
@@ -514,6 +542,8 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                     for (int k = 0; k < 4; ++k)       // x = own rows . other rows, over the head dimension
                         umma_ss(tm + cS, desc_off(smem_desc(smem_u32(smem + L::Xown), 0, 1024, kSwz128), k * 32),
                                 desc_off(smem_desc(smem_u32(smem + xo) + hh * 8192, 0, 1024, kSwz128), k * 32), idesc, k > 0);
+                } else if constexpr (kTsM) {
+                    issue_scores_ts<R>(tm + cS, tm + cdV, smem_u32(smem + xo) + hh * 8192);
                 } else {
                     issue_scores<R, LIN>(tm + cS, smem_u32(smem + L::Mown), smem_u32(smem + xo) + hh * 8192);
                 }
