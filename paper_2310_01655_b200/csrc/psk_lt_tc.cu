@@ -14,19 +14,23 @@ using namespace tc;
 
 // ---------------------------------------------------------------------------
 // prefix states, bf16 [batch][t][m][64] (entry l: the sum over the blocks before l; l = 0 unused).
-// grid (ceil(m/128), batch), 128 threads: a CTA walks the whole sequence for 128 features, the
-// running sum stays in tensor memory and is copied out at every block boundary.
+// grid (ceil(m/128), batch): a CTA walks the whole sequence for 128 features, the running sum stays in tensor
+// memory and is copied out at every block boundary by the first four warps; the fifth issues the MMAs, the sixth the loads.
+// Bound with few CTAs: the latency of a load, with two stages.  (With loads and MMAs issued by one elected lane of a row warp, whose
+// other lanes wait for it and read the sum late: batch 1, n 8192, m 64, b 256: 65 us, now 42; batch 24, m 320: 76 and 60; batch 12,
+// n 4096, m 1024, b 128: 54 and 44.  Behind a thread index instead of an election: 57, 62, 46.)
 // ---------------------------------------------------------------------------
+constexpr int kStThreads = 192;
 constexpr int kStStage = 32768 + 16384;     // two 64-feature groups of the B tile, the C tile
 constexpr int kStSmem = 2 * kStStage + 1024;
 
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kStThreads)
 lt_tc_state_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapC, bf16* __restrict__ Z,
                    int m, int t, int tpb, int* status) {
     pdl_sync();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
-    __shared__ uint64_t bar_full[2], bar_free[2], bar_acc;
+    __shared__ uint64_t bar_full[2], bar_free[2], bar_acc, bar_read;
     __shared__ uint32_t tm_slot;
     const int tid = threadIdx.x, warp = warp_index();
     const int f0 = blockIdx.x * 128, bt = blockIdx.y;
@@ -35,7 +39,7 @@ lt_tc_state_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_consta
         cta_giveup_init();
         mbar_init(&bar_full[0], 1); mbar_init(&bar_full[1], 1);
         mbar_init(&bar_free[0], 1); mbar_init(&bar_free[1], 1);
-        mbar_init(&bar_acc, 1);
+        mbar_init(&bar_acc, 1); mbar_init(&bar_read, 4);
         mbar_fence_init();
     }
     if (warp == 0) { tmem_alloc(&tm_slot, 64); tmem_relinquish(); }
@@ -43,58 +47,64 @@ lt_tc_state_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tm = tm_slot;
-    auto load = [&](int j) {
-        const int s = j & 1;
-        uint8_t* st = smem + s * kStStage;
-        mbar_expect_tx(&bar_full[s], kStStage);
-        tma_load_3d(st, &mapB, f0, j * 128, bt, &bar_full[s]);
-        tma_load_3d(st + 16384, &mapB, f0 + 64, j * 128, bt, &bar_full[s]);     // beyond m: zeros
-        tma_load_3d(st + 32768, &mapC, 0, j * 128, bt, &bar_full[s]);
-    };
-    if (tid == 0 && NT > 0) { load(0); if (NT > 1) load(1); }
     bool ok = true;
-    for (int l = 0; l + 1 < t; ++l) {
-        if (warp == 0 && elect_one()) {
-            constexpr uint32_t idesc = idesc_bf16(128, 64, true, true);
-            for (int tt = 0; tt < tpb && ok; ++tt) {
-                const int j = l * tpb + tt, s = j & 1;
-                ok = mbar_spin(&bar_full[s], (j >> 1) & 1, status, kErrTma);
+    if (warp == 5) {
+        if (elect_one()) {
+            for (int j = 0; j < NT; ++j) {
+                const int s = j & 1;
+                if (j >= 2) ok = mbar_spin(&bar_free[s], ((j - 2) >> 1) & 1, status, kErrMma);
                 if (!ok) break;
-                tc_fence_after();
-                const uint32_t base = smem_u32(smem + s * kStStage);
-                const uint64_t ad = smem_desc(base, 16384, 1024, kSwz128);
-                const uint64_t bd = smem_desc(base + 32768, 0, 1024, kSwz128);
+                uint8_t* st = smem + s * kStStage;
+                mbar_expect_tx(&bar_full[s], kStStage);
+                tma_load_3d(st, &mapB, f0, j * 128, bt, &bar_full[s]);
+                tma_load_3d(st + 16384, &mapB, f0 + 64, j * 128, bt, &bar_full[s]);     // beyond m: zeros
+                tma_load_3d(st + 32768, &mapC, 0, j * 128, bt, &bar_full[s]);
+            }
+        }
+    } else if (warp == 4) {
+        if (elect_one()) {
+            constexpr uint32_t idesc = idesc_bf16(128, 64, true, true);
+            for (int l = 0; l + 1 < t && ok; ++l) {
+                // this block's MMAs add to the accumulator only after everyone has read it
+                if (l > 0) ok = mbar_spin(&bar_read, (l - 1) & 1, status, kErrMma);
+                for (int tt = 0; tt < tpb && ok; ++tt) {
+                    const int j = l * tpb + tt, s = j & 1;
+                    ok = mbar_spin(&bar_full[s], (j >> 1) & 1, status, kErrTma);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t base = smem_u32(smem + s * kStStage);
+                    const uint64_t ad = smem_desc(base, 16384, 1024, kSwz128);
+                    const uint64_t bd = smem_desc(base + 32768, 0, 1024, kSwz128);
 #pragma unroll
-                for (int k = 0; k < 8; ++k) umma_ss(tm, desc_off(ad, k * 2048), desc_off(bd, k * 2048), idesc, (j > 0 || k > 0) ? 1u : 0u);
-                umma_commit(&bar_free[s]);
-                if (j + 2 < NT) {
-                    ok = mbar_spin(&bar_free[s], (j >> 1) & 1, status, kErrMma);
-                    if (ok) load(j + 2);
+                    for (int k = 0; k < 8; ++k) umma_ss(tm, desc_off(ad, k * 2048), desc_off(bd, k * 2048), idesc, (j > 0 || k > 0) ? 1u : 0u);
+                    umma_commit(&bar_free[s]);
+                    if (tt + 1 == tpb) umma_commit(&bar_acc);
                 }
             }
-            if (ok) umma_commit(&bar_acc);
         }
-        ok = mbar_wait(&bar_acc, l & 1, status, kErrMma) && ok;
-        tc_fence_after();
-        if (ok && f0 + tid < m) {
-            bf16* dst = Z + (((size_t)bt * t + l + 1) * m + f0 + tid) * 64;
-            const uint32_t lane_tm = tm + ((uint32_t)(warp * 32) << 16);
+    } else {
+        const uint32_t lane_tm = tm + ((uint32_t)(warp * 32) << 16);
+        for (int l = 0; l + 1 < t; ++l) {
+            ok = mbar_wait(&bar_acc, l & 1, status, kErrMma) && ok;
+            tc_fence_after();
+            if (ok && f0 + tid < m) {
+                bf16* dst = Z + (((size_t)bt * t + l + 1) * m + f0 + tid) * 64;
 #pragma unroll
-            for (int c0 = 0; c0 < 64; c0 += 32) {
-                uint32_t u[32];
-                tmem_ld32(lane_tm + c0, u);
-                tmem_ld_wait();
+                for (int c0 = 0; c0 < 64; c0 += 32) {
+                    uint32_t u[32];
+                    tmem_ld32(lane_tm + c0, u);
+                    tmem_ld_wait();
 #pragma unroll
-                for (int j = 0; j < 32; j += 8)
-                    *reinterpret_cast<uint4*>(dst + c0 + j) =
-                        make_uint4(pack_bf16(__uint_as_float(u[j]), __uint_as_float(u[j + 1])), pack_bf16(__uint_as_float(u[j + 2]), __uint_as_float(u[j + 3])),
-                                   pack_bf16(__uint_as_float(u[j + 4]), __uint_as_float(u[j + 5])), pack_bf16(__uint_as_float(u[j + 6]), __uint_as_float(u[j + 7])));
+                    for (int j = 0; j < 32; j += 8)
+                        *reinterpret_cast<uint4*>(dst + c0 + j) =
+                            make_uint4(pack_bf16(__uint_as_float(u[j]), __uint_as_float(u[j + 1])), pack_bf16(__uint_as_float(u[j + 2]), __uint_as_float(u[j + 3])),
+                                       pack_bf16(__uint_as_float(u[j + 4]), __uint_as_float(u[j + 5])), pack_bf16(__uint_as_float(u[j + 6]), __uint_as_float(u[j + 7])));
+                }
             }
+            tc_fence_before();
+            __syncwarp();
+            if (tid % 32 == 0) mbar_arrive(&bar_read);
         }
-        // the next block's MMAs add to the accumulator only after everyone has read it
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
     }
     tc_fence_before();
     __syncthreads();
@@ -305,7 +315,7 @@ int psk_lt_multiply_bf16(int batch, int n, int m, int k, int b, const void* A, c
     if (set_smem(lt_tc_state_kernel, kStSmem) != cudaSuccess) return PSK_ERR_CUDA;
     if (t > 1) {
         prof_begin("lt_tc_state_kernel", s);
-        launch_pdl(lt_tc_state_kernel, dim3((m + 127) / 128, batch), 128, kStSmem, s, mB, mC, Z, m, t, tpb, status);
+        launch_pdl(lt_tc_state_kernel, dim3((m + 127) / 128, batch), kStThreads, kStSmem, s, mB, mC, Z, m, t, tpb, status);
         prof_end(s);
     }
     const cudaError_t e = tpb == 1 ? launch_rows<1>(mA, mB, mC, mZ, Out, batch, n, m, t, status, s) : launch_rows<2>(mA, mB, mC, mZ, Out, batch, n, m, t, status, s);

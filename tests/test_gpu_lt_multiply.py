@@ -76,6 +76,26 @@ def test_tensor_core_instance_matches_oracle(batch, n, m, b):
             assert np.allclose(out[i][row], ref[row], rtol=3e-2, atol=3e-2 * np.abs(ref[row]).max() + 1e-6)
 
 
+@pytest.mark.parametrize("batch,n,m,b", [(1, 1152, 320, 128), (3, 1280, 64, 256), (1, 2048, 192, 256), (2, 384, 128, 128)])
+def test_tensor_core_states_over_several_blocks(batch, n, m, b):
+    # odd and even numbers of blocks and of tiles, a last CTA with 64 of its 128 features
+    g = torch.Generator(device="cpu").manual_seed(2100 + n + m)
+    A, B = ((torch.randn(batch, n, m, generator=g) / m ** 0.5).bfloat16() for _ in range(2))
+    C = torch.randn(batch, n, 64, generator=g).bfloat16()
+    out, ws = psk.lt_multiply_bf16(A.cuda(), B.cuda(), C.cuda(), b)
+    assert psk.check(ws) == 0
+    again, _ = psk.lt_multiply_bf16(A.cuda(), B.cuda(), C.cuda(), b, torch.full_like(ws, 0xFF))
+    assert torch.equal(out, again)
+    for i in range(batch):
+        a, bb, c = (x[i].double().numpy() for x in (A, B, C))
+        ref = orc.lt_multiply_blocked(a, bb, c, b)
+        # one bf16 rounding (2^-9) of the states and of the masked scores
+        assert orc.rel_l2(out[i].cpu().double().numpy(), ref) < 1e-2
+        for l in range(n // b):
+            rows = slice(l * b, (l + 1) * b)
+            assert orc.rel_l2(out[i][rows].cpu().double().numpy(), ref[rows]) < 1e-2
+
+
 def test_tensor_core_instance_bad_arguments():
     A = torch.zeros(1, 256, 64, device="cuda", dtype=torch.bfloat16)
     C = torch.zeros(1, 256, 64, device="cuda", dtype=torch.bfloat16)
