@@ -563,45 +563,72 @@ tc_state_scan_kernel(float4* __restrict__ tot, size_t elems, int nseg) {
 }
 
 // Sum of the run totals of a head, centred, weighted and rounded like a stored state: the single
-// global state of non-causal attention, written as the head's only block.
+// global state of non-causal attention, written as the head's only block.  A CTA takes 32 of the state's rows; its threads
+// share the 10 KB of a run's total and finish the rows, one lane each, in shared memory.  (A thread per row that read its
+// own 320 bytes of every total lived on the L1 cache, of which the row kernels' CTAs, waiting for this kernel on the same SMs
+// with up to 227 KB of shared memory each SM, leave next to nothing: 24 heads x 4096, r = 16: 15 us alone and 48 to 85 in front of them.)
+constexpr int kSumRows = 32, kSumPitch = 84;              // (floats; 16-byte steps of an odd number: no bank conflicts)
 template <int R>
 __global__ void __launch_bounds__(128)
 tc_state_sum_kernel(const float* __restrict__ tot, int nseg, const float* __restrict__ cmean, int center_mode,
                     bf16* __restrict__ S) {
     pdl_sync();
     using F = Feat<R>;
-    const int tile = blockIdx.x, bh = blockIdx.y, wt = threadIdx.x;
-    const int row = tile * 128 + wt;
-    float v[80];
+    __shared__ __align__(16) float rows[kSumRows * kSumPitch];
+    __shared__ float cm[64];
+    const int row0 = blockIdx.x * kSumRows, bh = blockIdx.y, tid = threadIdx.x;
+    constexpr int kVec = kSumRows * 20 / 128;             // 16-byte pieces of the CTA's rows per thread
+    if (tid < 64) cm[tid] = cmean != nullptr ? cmean[(size_t)bh * 64 + tid] : 0.f;
+    if (row0 < F::F) {                                    // (rows beyond the last feature may hold anything: zeros are stored)
+        float4 v[kVec];
 #pragma unroll
-    for (int c = 0; c < 80; ++c) v[c] = 0.f;
-    for (int s = 0; s < nseg; ++s) {
-        const float4* src = reinterpret_cast<const float4*>(tot + ((((size_t)bh * nseg + s) * F::NT + tile) * 128 + wt) * 80);
+        for (int q = 0; q < kVec; ++q) v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4* src = reinterpret_cast<const float4*>(tot + ((size_t)bh * nseg * F::FP + row0) * 80) + tid;
+#pragma unroll 2
+        for (int s = 0; s < nseg; ++s) {
 #pragma unroll
-        for (int c = 0; c < 20; ++c) {
-            const float4 x = src[c];
-            v[4 * c] += x.x; v[4 * c + 1] += x.y; v[4 * c + 2] += x.z; v[4 * c + 3] += x.w;
+            for (int q = 0; q < kVec; ++q) {
+                const float4 x = src[(size_t)s * (F::FP * 20) + 128 * q];
+                v[q].x += x.x; v[q].y += x.y; v[q].z += x.z; v[q].w += x.w;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kVec; ++q) {
+            const int e = tid + 128 * q;
+            *reinterpret_cast<float4*>(rows + (e / 20) * kSumPitch + 4 * (e % 20)) = v[q];
         }
     }
-    const float wgt = F::weight(row);
-    const float last = v[64];
-    float corr = 0.f;
-    uint32_t pk[40];
+    __syncthreads();
+    if (tid < kSumRows) {
+        const int row = row0 + tid;
+        float* const mine = rows + tid * kSumPitch;
+        uint32_t pk[40];
 #pragma unroll
-    for (int c = 0; c < 64; c += 2) {
-        const float c0 = cmean != nullptr ? cmean[(size_t)bh * 64 + c] : 0.f;
-        const float c1 = cmean != nullptr ? cmean[(size_t)bh * 64 + c + 1] : 0.f;
-        const float x0 = center_mode == 1 ? v[c] - last * c0 : v[c];
-        const float x1 = center_mode == 1 ? v[c + 1] - last * c1 : v[c + 1];
-        if (center_mode == 2) corr += c0 * x0 + c1 * x1;
-        pk[c / 2] = row < F::F ? pack_bf16(x0 * wgt, x1 * wgt) : 0u;       // (rows beyond the last feature may hold anything)
+        for (int c = 0; c < 40; ++c) pk[c] = 0u;
+        if (row < F::F) {
+            const float wgt = F::weight(row), last = mine[64];
+            float corr = 0.f;
+#pragma unroll
+            for (int c = 0; c < 64; c += 4) {
+                const float4 u = *reinterpret_cast<const float4*>(mine + c);
+                const float x0 = center_mode == 1 ? u.x - last * cm[c] : u.x, x1 = center_mode == 1 ? u.y - last * cm[c + 1] : u.y;
+                const float x2 = center_mode == 1 ? u.z - last * cm[c + 2] : u.z, x3 = center_mode == 1 ? u.w - last * cm[c + 3] : u.w;
+                if (center_mode == 2) {
+                    corr += cm[c] * x0 + cm[c + 1] * x1;
+                    corr += cm[c + 2] * x2 + cm[c + 3] * x3;
+                }
+                pk[c / 2] = pack_bf16(x0 * wgt, x1 * wgt);
+                pk[c / 2 + 1] = pack_bf16(x2 * wgt, x3 * wgt);
+            }
+            pk[32] = pack_bf16((last - corr) * wgt, 0.f);
+        }
+#pragma unroll
+        for (int c = 0; c < 10; ++c) reinterpret_cast<uint4*>(mine)[c] = make_uint4(pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
     }
-    pk[32] = row < F::F ? pack_bf16((last - corr) * wgt, 0.f) : 0u;
-#pragma unroll
-    for (int c = 33; c < 40; ++c) pk[c] = 0u;
-    uint4* out = reinterpret_cast<uint4*>(S + ((size_t)bh * F::FP + row) * 80);
-#pragma unroll
-    for (int c = 0; c < 10; ++c) out[c] = make_uint4(pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
+    __syncthreads();
+    uint4* out = reinterpret_cast<uint4*>(S + ((size_t)bh * F::FP + row0) * 80);
+    for (int e = tid; e < kSumRows * 10; e += 128)
+        out[e] = *reinterpret_cast<const uint4*>(rows + (e / 10) * kSumPitch + 4 * (e % 10));
 }
 
 // ---------------------------------------------------------------------------
@@ -712,7 +739,7 @@ cudaError_t states_impl(const Dims& d, const CUtensorMap& mX, const CUtensorMap&
         a.mode = kModeTotal; a.cmean = nullptr; a.center_mode = 0;
         PSK_TRY((launch_states<R>(d, mX, mY, gimg, a, status, s, launches)));
         prof_begin("tc_state_sum_kernel", s);
-        launch_pdl(tc_state_sum_kernel<R>, dim3(Feat<R>::NT, d.BH()), 128, 0, s, tot, nseg, cmean, center_mode, S);
+        launch_pdl(tc_state_sum_kernel<R>, dim3(Feat<R>::FP / kSumRows, d.BH()), 128, 0, s, tot, nseg, cmean, center_mode, S);
         prof_end(s);
         ++*launches;
         return cudaGetLastError();
