@@ -392,7 +392,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             for (int C = 0; C < F::NC; ++C) {         // (no early exit: a wait that gave up makes the later ones return at once)
                 const int buf = C % kFeatBufs;
                 if (C >= kFeatBufs) {                 // the MMAs that read this buffer's previous contents
-                    ok = mbar_wait(&bar_a[buf], (C / kFeatBufs - 1) & 1, status, kErrMma);
+                    ok = mbar_wait(&bar_a[buf], (C / kFeatBufs - 1) & 1, status, kErrMma) && ok;
                     tc_fence_after();
                     if (tid == 0) {                   // ... and this stage's: refill it with chunk C's rows
                         mbar_expect_tx(&bar_feat[buf], kZStageBytes);
@@ -509,7 +509,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             if (denom != nullptr && ok) denom[(size_t)bh * n + row0 + tid] = d;
             fence_proxy_async_smem();
             consumer_barrier();
-            if (tid == 0 && ok) {
+            if (tid == 0 && ok && !cta_gave_up()) {       // (a row of another thread's that gave up is not stored either)
                 tma_store_4d(&mapO, smem + L::So, 0, row0, hi, bi);
                 if (keep_oc) tma_store_4d(&mapOc, smem + L::Soc, 0, bh * n + row0, 0, 0);
                 bulk_commit();

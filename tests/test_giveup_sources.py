@@ -1,0 +1,37 @@
+"""What a kernel does after a bounded wait has given up, read from its source (no GPU: no test makes a real kernel
+lose a signal)."""
+import os
+import re
+
+import pytest
+
+import paper_2310_01655_b200 as psk
+
+CSRC = os.path.join(os.path.dirname(psk.__file__), "csrc")
+
+
+def source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def loops(text):
+    """(header, body) of every for loop with a braced body."""
+    for m in re.finditer(r"\bfor \(([^{}]*?)\) \{", text):
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(text[i], 0)
+            i += 1
+        yield m.group(1), text[m.end():i]
+
+
+@pytest.mark.parametrize("name", ["psk_tc.cu", "psk_tc_bwd.cu", "psk_tc_state.cu", "psk_lt_tc.cu", "psk_sketch8_tc.cu"])
+def test_a_later_wait_does_not_hide_one_that_gave_up(name):
+    """In a loop that runs on after a wait gave up, `ok` keeps that: it is only ever and-ed."""
+    for header, body in loops(source(name)):
+        if re.search(r"&& ok\b", header):            # (such a loop ends instead)
+            continue
+        for stmt in re.findall(r"\bok = mbar_(?:wait|spin)\([^;]*;", body):
+            inner = next((h for h, b in loops(body) if stmt in b and re.search(r"&& ok\b", h)), None)
+            follows = body[body.index(stmt) + len(stmt):].lstrip()
+            assert inner or "&& ok;" in stmt or follows.startswith("if (!ok) break;"), (header, stmt)
