@@ -188,6 +188,8 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     const int ntiles = b / 128;
     const bool has_state = noncausal || (QSIDE ? (l > 0) : (l < t - 1));
 
+    // A thread whose wait gave up asks for no more copies (`ok` in front of every one behind a wait): the barrier's phase may still be
+    // open, an arrival too many would complete it or worse, and the buffer may still be some copy's or MMA's.
     // the other side's rows of a tile of the block: score operand (raw rows with LOCAL), and values
     auto load_m = [&](int tp, uint32_t dst) {
         mbar_expect_tx(&bar_xoth, L::kM);
@@ -294,7 +296,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     if constexpr (LIN && LOCAL) {
         // The own tile held the given half sketch; the exact same-block scores need the raw rows.
         // The sketch GEMM has completed: fetch them into the same buffer (phase C waits for them).
-        if (tid == 0) {
+        if (tid == 0 && ok) {
             mbar_expect_tx(&bar_again, 16384);
             tma_load_4d(smem + L::Xown, &mapXownRaw, 0, row0, hi, bi, &bar_again);
         }
@@ -401,7 +403,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                 if (C >= 0) {
                     ok = ok && mbar_wait(&bar_phi[C & 1], (C / 2) & 1, status, kErrMma);
                     tc_fence_after();
-                    if (tid == 32) refill(C);              // (warp 0 issues the MMAs; the loads go out from warp 1)
+                    if (tid == 32 && ok) refill(C);              // (warp 0 issues the MMAs; the loads go out from warp 1)
                     const uint32_t dphi = lane_tm + cPhi;
                     tmem_ld32(dphi, x0);
                     tmem_ld32(dphi + 32, x1);
@@ -454,7 +456,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                 }
                 ok = ok && mbar_wait(&bar_phi[buf], (C / 2) & 1, status, kErrMma);
                 tc_fence_after();
-                if (tid == 32) refill(C);              // (warp 0 issues the MMAs; the loads go out from warp 1)
+                if (tid == 32 && ok) refill(C);              // (warp 0 issues the MMAs; the loads go out from warp 1)
                 uint32_t x[32];
                 tmem_ld32(lane_tm + cPhi + buf * 64, x);
                 tmem_ld_wait();
@@ -535,7 +537,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
                 tc_fence_after();
                 // Every thread is past its wait for this tile's rows (a barrier must not complete twice
                 // before its slowest waiter has looked): the next tile's, into the other buffer.
-                if (L::kTwoM && hh == 0 && tp + 1 < tp_end) load_m(tp + 1, xo_next);
+                if (L::kTwoM && ok && hh == 0 && tp + 1 < tp_end) load_m(tp + 1, xo_next);
                 constexpr uint32_t idesc = idesc_bf16(128, 64, false, false);
                 if constexpr (LOCAL) {
 #pragma unroll
@@ -646,7 +648,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             ++mma_uses;
             tc_fence_after();
         }
-        if (tid == 0 && tp + 1 < tp_end) {        // every MMA that read this tile's rows has completed
+        if (tid == 0 && ok && tp + 1 < tp_end) {  // every MMA that read this tile's rows has completed
             load_y(tp + 1);
             if constexpr (!L::kTwoM) load_m(tp + 1, L::Moth);
         }
@@ -654,8 +656,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     if constexpr (L::kFold && !LIN) {             // the own rows and the sketch matrices' image again
         fence_proxy_async_smem();
         tc_fence_before();
-        __syncthreads();
-        if (tid == 0) {
+        if (__syncthreads_and(ok) && tid == 0) {
             mbar_expect_tx(&bar_again, 16384 + GImage<R>::bytes);
             tma_load_4d(smem + L::Xown, &mapXown, 0, row0, hi, bi, &bar_again);
             bulk_load(smem + L::G, gimg + (size_t)g * GImage<R>::bytes, GImage<R>::bytes, &bar_again);
@@ -723,8 +724,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
             }
             fence_proxy_async_smem();
             tc_fence_before();
-            __syncthreads();
-            if (tid == 0) {
+            if (__syncthreads_and(ok) && tid == 0) {
                 tma_store_4d(&mapDXraw, smem + L::Sx, 0, row0, hi, bi);
                 bulk_commit();
                 bulk_wait_read();
@@ -800,8 +800,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     }
     fence_proxy_async_smem();
     tc_fence_before();
-    __syncthreads();
-    if (tid == 0 && ok) {
+    if (__syncthreads_and(ok) && tid == 0) {           // (nothing is stored if any row's thread gave up)
         tma_store_4d(&mapDX, smem + L::Sx, 0, row0, hi, bi);
         if constexpr (!QSIDE) tma_store_4d(&mapDV, smem + L::Sv, 0, row0, hi, bi);
         bulk_commit();

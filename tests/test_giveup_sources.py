@@ -35,3 +35,20 @@ def test_a_later_wait_does_not_hide_one_that_gave_up(name):
             inner = next((h for h, b in loops(body) if stmt in b and re.search(r"&& ok\b", h)), None)
             follows = body[body.index(stmt) + len(stmt):].lstrip()
             assert inner or "&& ok;" in stmt or follows.startswith("if (!ok) break;"), (header, stmt)
+
+
+@pytest.mark.parametrize("name,calls", [
+    ("psk_tc_bwd.cu", [r"refill\(C\);", r"load_m\(tp \+ 1,", r"load_y\(tp \+ 1\);", r"mbar_expect_tx\(&bar_again,"]),
+])
+def test_no_copy_is_asked_for_after_a_wait_gave_up(name, calls):
+    """Every copy that is asked for behind a wait has `ok` in the condition in front of it.  (Its barrier's phase may still be
+    open: one more arrival with bytes outstanding, and a second copy into the buffer.)"""
+    text = source(name)
+    for call in calls:
+        found = [m.start() for m in re.finditer(call, text)]
+        assert found, call
+        for at in found:
+            # the nearest `if (...)` before the call
+            conditions = re.findall(r"\bif (?:constexpr )?\((.*)\)", text[:at][-400:])
+            conditions = [c for c in conditions if "L::" not in c or "ok" in c]
+            assert conditions and re.search(r"\bok\b", conditions[-1]), (name, call, conditions[-1:])
