@@ -273,10 +273,12 @@ int psk_check(const void* workspace, void* stream);
  * signal costs about a second and can never hang the GPU.  This call exercises exactly that path:
  * it enqueues one small kernel whose 128 threads wait, through the same code with the limit
  * `limit_ns` (1 .. 100 000 000), on a barrier that nobody completes.  Afterwards
- * psk_check(workspace, stream) returns PSK_ERR_TIMEOUT, and four uint64 values at byte offset 64
+ * psk_check(workspace, stream) returns PSK_ERR_TIMEOUT, and seven uint64 values at byte offset 64
  * of the workspace (DEVICE) report: nanoseconds the first wait took, nanoseconds a second wait on
- * the same barrier took (it must return at once), and the number of threads whose first / second
- * wait reported failure (128 each).  The next regular call on the workspace clears the status
+ * the same barrier took (it must return at once), the number of threads whose first / second
+ * wait reported failure (128 each); then, of the teardown that follows in such a thread block (before it gives its
+ * tensor memory back, MMAs still running and copies still on their way are waited for, with limits of a few milliseconds):
+ * the nanoseconds it took, and 1 each if an MMA and a copy that nobody had waited for had completed after it.  The next regular call on the workspace clears the status
  * word.  `workspace`: DEVICE, at least 256 bytes, 256-byte aligned. */
 int psk_selftest_wait_timeout(void* workspace, size_t workspace_bytes, uint64_t limit_ns, void* stream);
 

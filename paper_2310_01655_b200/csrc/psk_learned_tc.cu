@@ -457,6 +457,7 @@ ltc_dense_norm_kernel(Slice sl, const bf16* __restrict__ X, size_t row0, int til
     // (every MMA has completed: the rows waited for the last product of every tile)
     tc_fence_before();
     __syncthreads();
+    cta_teardown(warp >= 16, warp - 16);
     if (warp == 16) tmem_dealloc(tm, 512);
 }
 
@@ -721,6 +722,7 @@ ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant_
     }
     tc_fence_before();
     __syncthreads();
+    cta_teardown(warp == 16);
     if (warp == 16) tmem_dealloc(tm, 512);
 }
 
@@ -950,6 +952,7 @@ ltc_dense_bwd_norm_kernel(const __grid_constant__ CUtensorMap mN, const __grid_c
     }
     tc_fence_before();
     __syncthreads();
+    cta_teardown(warp == 16);
     if (warp == 16) tmem_dealloc(tm, 512);
 }
 

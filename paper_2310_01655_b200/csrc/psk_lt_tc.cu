@@ -108,6 +108,7 @@ lt_tc_state_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_consta
     }
     tc_fence_before();
     __syncthreads();
+    cta_teardown(warp == 4);
     if (warp == 0) tmem_dealloc(tm, 64);
 }
 
@@ -264,6 +265,7 @@ lt_tc_rows_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constan
     }
     tc_fence_before();
     __syncthreads();
+    cta_teardown(warp == 4 * TPB);
     if (warp == 4 * TPB) tmem_dealloc(tm, L::kTmem);
 }
 

@@ -186,6 +186,7 @@ sk8_tc_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     if (warp == 0 && elect_one()) bulk_wait_read();
     tc_fence_before();
     __syncthreads();
+    cta_teardown(warp == 0);
     if (warp == 0) tmem_dealloc(tm, 256);
 }
 
@@ -375,6 +376,7 @@ sk8_tc_bwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     if (warp == 0 && elect_one()) bulk_wait_read();
     tc_fence_before();
     __syncthreads();
+    cta_teardown(warp == 0);
     if (warp == 0) tmem_dealloc(tm, 256);
 }
 

@@ -177,7 +177,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     constexpr int kStages = L::kSt;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
-    __shared__ uint64_t bar_own, bar_again, bar_xoth, bar_yoth, bar_mma, bar_phi[2], bar_box[2], bar_drain;
+    __shared__ uint64_t bar_own, bar_again, bar_xoth, bar_yoth, bar_mma, bar_phi[2], bar_box[2];
     __shared__ uint32_t tmem_slot;
     const int tid = threadIdx.x, warp = warp_index(), tau = blockIdx.x, l = blockIdx.y, bh = blockIdx.z;
     const int hi = bh % H, bi = bh / H;
@@ -210,7 +210,7 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
         tma_load_4d(smem + L::Xown, &mapXown, 0, row0, hi, bi, &bar_own);
         tma_load_4d(smem + L::Yown, &mapYown, 0, row0, hi, bi, &bar_own);
         bulk_load(smem + L::G, gimg + (size_t)g * GImage<R>::bytes, GImage<R>::bytes, &bar_own);
-        mbar_init(&bar_again, 1); mbar_init(&bar_xoth, 1); mbar_init(&bar_yoth, 1); mbar_init(&bar_mma, 1); mbar_init(&bar_drain, 1);
+        mbar_init(&bar_again, 1); mbar_init(&bar_xoth, 1); mbar_init(&bar_yoth, 1); mbar_init(&bar_mma, 1);
         cta_giveup_init();
         mbar_fence_init();
         tma_prefetch_desc(&mapXoth); tma_prefetch_desc(&mapYoth);
@@ -806,9 +806,9 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
         bulk_commit();
         bulk_wait_read();
     }
-    cta_drain(warp == 0, &bar_drain);
     tc_fence_before();
     __syncthreads();
+    cta_teardown(warp == 0);
     if (warp == 2) tmem_dealloc(tm, 256);
 }
 

@@ -504,6 +504,7 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
     }
     tc_fence_before();
     __syncthreads();
+    cta_teardown(warp >= 4 * (NWG + NSW), warp - 4 * (NWG + NSW));
     if (warp == 0) tmem_dealloc(tm, 512);
 }
 

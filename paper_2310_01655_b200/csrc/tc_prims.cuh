@@ -71,7 +71,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // it costs anything.  Kernels therefore never have to leave a loop early because a wait failed --
 // which matters wherever a loop contains a barrier that counts its participants.
 // Every kernel that waits calls cta_giveup_init() from one thread before its first block-wide
-// barrier, and may read cta_gave_up() after its last one to skip its global stores.
+// barrier, may read cta_gave_up() after its last one to skip its global stores, and calls cta_teardown() after that one,
+// before it gives tensor memory back.
 constexpr uint64_t kWaitLimitNs = 1000000000ull;
 __device__ __forceinline__ uint64_t globaltimer_ns() {
     uint64_t t;
@@ -84,19 +85,21 @@ __device__ __forceinline__ volatile int* cta_giveup_flag() {
 }
 __device__ __forceinline__ void cta_giveup_init() { *cta_giveup_flag() = 0; }
 __device__ __forceinline__ bool cta_gave_up() { return *cta_giveup_flag() != 0; }
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_test_addr(uint32_t bar_addr, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.b32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
+        : "r"(bar_addr), "r"(parity)
         : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ bool wait_failed(int* status, int code) {
-    *cta_giveup_flag() = 1;
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) { return mbar_test_addr(smem_u32(bar), parity); }
+// (the flag of the first to give up also says which barrier it was and which phase)
+__device__ __forceinline__ bool wait_failed(int* status, int code, uint32_t bar_addr, uint32_t parity) {
+    atomicCAS(const_cast<int*>(cta_giveup_flag()), 0, (int)(bar_addr << 2 | (parity & 1) << 1 | 1));
     if (status != nullptr) atomicCAS(status, 0, code);
     return false;
 }
@@ -119,7 +122,7 @@ static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar_addr, uint32_t p
         if (t0 == 0) t0 = now;
         else if (now - t0 > limit_ns) break;
     }
-    return wait_failed(status, code);
+    return wait_failed(status, code, bar_addr, parity);
 }
 // Bounded wait by polling only (no suspension): for a lone issuing thread, whose wake-up latency
 // is on the critical path of everything it feeds and whose polling costs no one else issue slots.
@@ -133,13 +136,7 @@ static __device__ __noinline__ bool mbar_spin_slow(uint32_t bar_addr, uint32_t p
         for (int g = 0; g < 64; ++g) {
 #pragma unroll 1
             for (int i = 0; i < 64; ++i) {
-                uint32_t ok;
-                asm volatile(
-                    "{\n\t.reg .pred p;\n\t"
-                    "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                    "selp.b32 %0, 1, 0, p;\n\t}"
-                    : "=r"(ok) : "r"(bar_addr), "r"(parity) : "memory");
-                if (ok) return true;
+                if (mbar_test_addr(bar_addr, parity)) return true;
             }
             if (cta_gave_up()) return false;
         }
@@ -147,7 +144,7 @@ static __device__ __noinline__ bool mbar_spin_slow(uint32_t bar_addr, uint32_t p
         if (t0 == 0) t0 = now;
         else if (now - t0 > limit_ns) break;
     }
-    return wait_failed(status, code);
+    return wait_failed(status, code, bar_addr, parity);
 }
 __device__ __forceinline__ bool mbar_spin(uint64_t* bar, uint32_t parity, int* status, int code) {
     if (mbar_test(bar, parity)) return true;
@@ -363,16 +360,46 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return r;
 }
 
-// Before a CTA that has given up a wait frees its tensor memory and ends: the MMAs it has issued must have completed and the
-// copies on their way into its shared memory must have arrived.  The elected lane of the issuing warp waits for a commit
-// of its own (with a limit), then long enough for any copy.  `bar`: a barrier of count 1 that nothing else uses.
-__device__ __forceinline__ void cta_drain(bool issuing_warp, uint64_t* bar) {
-    if (!__any_sync(0xffffffffu, cta_gave_up())) return;
-    if (issuing_warp && elect_one()) {
+// Teardown.  A CTA that has given up a wait must not give its tensor memory back, nor end, with MMAs of its own still running or
+// copies into its shared memory still on their way.  Called by all threads after the last block-wide barrier, when nobody waits
+// any more and the flag is final; `issuing`: the warp whose elected lane issued MMAs (slot: which of the two such warps).
+// Every poll has a limit of its own and takes no notice of the flag:
+//  * MMAs: a commit of the lane that issued them, polled;
+//  * the barrier that ran out first, polled again: if it waited for a copy, that copy may have come meanwhile;
+//  * other copies: a pause.  Those asked for before that wait began have had its second; those after it (nothing is asked for by a
+//    thread whose own wait gave up) come within microseconds unless the memory system is lost.  This part is best effort: a copy
+//    that has not come within a second has no bound.
+constexpr uint64_t kDrainLimitNs = 10000000ull, kDrainPauseNs = 1000000ull;
+__device__ __forceinline__ uint64_t* cta_drain_bars() {       // one for each such warp; set up only when needed
+    __shared__ uint64_t bars[2];
+    return bars;
+}
+static __device__ __noinline__ bool mbar_drain(uint32_t bar_addr, uint32_t parity) {
+    const uint64_t t0 = globaltimer_ns();
+#pragma unroll 1
+    do {
+        if (mbar_test_addr(bar_addr, parity)) return true;
+        __nanosleep(1000);
+    } while (globaltimer_ns() - t0 < kDrainLimitNs);
+    return false;
+}
+static __device__ __noinline__ void cta_drain(bool issuing, int slot) {
+    if (issuing && elect_one()) {
+        uint64_t* bar = cta_drain_bars() + slot;
+        mbar_init(bar, 1);
+        mbar_fence_init();
         umma_commit(bar);
-        for (int i = 0; i < 1000 && !mbar_test(bar, 0); ++i) __nanosleep(1000);
-        for (int i = 0; i < 200; ++i) __nanosleep(1000);
+        mbar_drain(smem_u32(bar), 0);
+        const uint32_t what = (uint32_t)*cta_giveup_flag();
+        mbar_drain(what >> 2, what >> 1 & 1);
+        const uint64_t t0 = globaltimer_ns();
+#pragma unroll 1
+        while (globaltimer_ns() - t0 < kDrainPauseNs) __nanosleep(1000);
     }
+    __syncthreads();
+}
+__device__ __forceinline__ void cta_teardown(bool issuing, int slot = 0) {
+    if (cta_gave_up()) cta_drain(issuing, slot);
 }
 
 // Byte offset of 16-byte chunk `chunk` (0..7) of row `row` inside a [rows x 128 B] tile held in

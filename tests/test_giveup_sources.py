@@ -52,3 +52,18 @@ def test_no_copy_is_asked_for_after_a_wait_gave_up(name, calls):
             conditions = re.findall(r"\bif (?:constexpr )?\((.*)\)", text[:at][-400:])
             conditions = [c for c in conditions if "L::" not in c or "ok" in c]
             assert conditions and re.search(r"\bok\b", conditions[-1]), (name, call, conditions[-1:])
+
+
+def test_tensor_memory_is_given_back_after_the_teardown():
+    """Every kernel that issues MMAs goes through cta_teardown() between its last block-wide barrier and the release of its
+    tensor memory: MMAs and copies of a CTA that gave up a wait must not outlive it."""
+    kernels = 0
+    for name in sorted(os.listdir(CSRC)):
+        if not name.endswith(".cu"):
+            continue
+        text = source(name)
+        for m in re.finditer(r"\btmem_dealloc\(", text):
+            kernels += 1
+            before = text[:m.start()]
+            assert before.rfind("cta_teardown(") > before.rfind("__syncthreads"), name
+    assert kernels >= 10

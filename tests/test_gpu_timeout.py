@@ -33,6 +33,19 @@ def test_wait_runs_out_and_is_reported():
     assert torch.equal(O1, O2) and torch.equal(den1, den2)
 
 
+def test_teardown_waits_for_what_is_still_running():
+    """What the CTA of a wait that ran out leaves behind: its MMA and its copy have completed before it gives its tensor memory
+    back, within the teardown's own limits (10 ms for each of two barriers, a pause of 1 ms), time after time."""
+    ws = torch.zeros(4096, dtype=torch.uint8, device="cuda")
+    for _ in range(40):                                        # (512 columns in pieces of 32: a leak would show in 16)
+        first_ns = psk.binding.selftest_wait_timeout(ws, 1_000_000)[0]
+        teardown_ns, mma_done, copy_done = ws[96:120].view(torch.int64).cpu().tolist()
+        assert first_ns >= 1_000_000
+        assert (mma_done, copy_done) == (1, 1)
+        assert 1_000_000 <= teardown_ns < 60_000_000
+        assert psk.check(ws) == ERR_TIMEOUT
+
+
 def test_selftest_rejects_bad_arguments():
     ws = torch.empty(4096, dtype=torch.uint8, device="cuda")
     with pytest.raises(psk.binding.PskError):
