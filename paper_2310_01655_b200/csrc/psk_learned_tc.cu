@@ -722,8 +722,7 @@ ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant_
     }
     tc_fence_before();
     __syncthreads();
-    cta_teardown(warp == 16);
-    if (warp == 16) tmem_dealloc(tm, 512);
+    if (warp == 16) { cta_teardown_warp(); tmem_dealloc(tm, 512); }
 }
 
 // ---------------------------------------------------------------------------
@@ -952,8 +951,7 @@ ltc_dense_bwd_norm_kernel(const __grid_constant__ CUtensorMap mN, const __grid_c
     }
     tc_fence_before();
     __syncthreads();
-    cta_teardown(warp == 16);
-    if (warp == 16) tmem_dealloc(tm, 512);
+    if (warp == 16) { cta_teardown_warp(); tmem_dealloc(tm, 512); }
 }
 
 // ---------------------------------------------------------------------------

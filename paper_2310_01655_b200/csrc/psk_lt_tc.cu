@@ -42,7 +42,7 @@ lt_tc_state_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_consta
         mbar_init(&bar_acc, 1); mbar_init(&bar_read, 4);
         mbar_fence_init();
     }
-    if (warp == 0) { tmem_alloc(&tm_slot, 64); tmem_relinquish(); }
+    if (warp == 4) { tmem_alloc(&tm_slot, 64); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -108,8 +108,7 @@ lt_tc_state_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_consta
     }
     tc_fence_before();
     __syncthreads();
-    cta_teardown(warp == 4);
-    if (warp == 0) tmem_dealloc(tm, 64);
+    if (warp == 4) { cta_teardown_warp(); tmem_dealloc(tm, 64); }
 }
 
 // ---------------------------------------------------------------------------
@@ -265,8 +264,7 @@ lt_tc_rows_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constan
     }
     tc_fence_before();
     __syncthreads();
-    cta_teardown(warp == 4 * TPB);
-    if (warp == 4 * TPB) tmem_dealloc(tm, L::kTmem);
+    if (warp == 4 * TPB) { cta_teardown_warp(); tmem_dealloc(tm, L::kTmem); }
 }
 
 template <int TPB>

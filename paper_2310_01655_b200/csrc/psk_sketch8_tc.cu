@@ -186,8 +186,7 @@ sk8_tc_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     if (warp == 0 && elect_one()) bulk_wait_read();
     tc_fence_before();
     __syncthreads();
-    cta_teardown(warp == 0);
-    if (warp == 0) tmem_dealloc(tm, 256);
+    if (warp == 0) { cta_teardown_warp(); tmem_dealloc(tm, 256); }
 }
 
 // dX from the gradient of the [hi | lo] rows (its first R columns are dL/dM)
@@ -376,8 +375,7 @@ sk8_tc_bwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     if (warp == 0 && elect_one()) bulk_wait_read();
     tc_fence_before();
     __syncthreads();
-    cta_teardown(warp == 0);
-    if (warp == 0) tmem_dealloc(tm, 256);
+    if (warp == 0) { cta_teardown_warp(); tmem_dealloc(tm, 256); }
 }
 
 struct Sk8Maps { CUtensorMap W1, W2; };

@@ -544,8 +544,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     }
     tc_fence_before();
     __syncthreads();
-    cta_teardown(warp == 4);
-    if (warp == 4) tmem_dealloc(tm, 256);
+    if (warp == 4) { cta_teardown_warp(); tmem_dealloc(tm, 256); }
 }
 
 // Centre of the values of a head: cmean[bh][c] = mean of V[bh][i][c] over at most 1024 rows i

@@ -361,8 +361,9 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 }
 
 // Teardown.  A CTA that has given up a wait must not give its tensor memory back, nor end, with MMAs of its own still running or
-// copies into its shared memory still on their way.  Called by all threads after the last block-wide barrier, when nobody waits
-// any more and the flag is final; `issuing`: the warp whose elected lane issued MMAs (slot: which of the two such warps).
+// copies into its shared memory still on their way.  Called after the last block-wide barrier, when nobody waits
+// any more and the flag is final, by the one warp whose elected lane issues MMAs and which also gives the tensor memory back
+// (cta_teardown_warp), or else by all threads (cta_teardown; `issuing`: such a warp, `slot`: which of two).
 // Every poll has a limit of its own and takes no notice of the flag:
 //  * MMAs: a commit of the lane that issued them, polled;
 //  * the barrier that ran out first, polled again: if it waited for a copy, that copy may have come meanwhile;
@@ -383,8 +384,8 @@ static __device__ __noinline__ bool mbar_drain(uint32_t bar_addr, uint32_t parit
     } while (globaltimer_ns() - t0 < kDrainLimitNs);
     return false;
 }
-static __device__ __noinline__ void cta_drain(bool issuing, int slot) {
-    if (issuing && elect_one()) {
+static __device__ __noinline__ void cta_drain_warp(int slot) {
+    if (elect_one()) {
         uint64_t* bar = cta_drain_bars() + slot;
         mbar_init(bar, 1);
         mbar_fence_init();
@@ -396,10 +397,16 @@ static __device__ __noinline__ void cta_drain(bool issuing, int slot) {
 #pragma unroll 1
         while (globaltimer_ns() - t0 < kDrainPauseNs) __nanosleep(1000);
     }
-    __syncthreads();
+    __syncwarp();
+}
+__device__ __forceinline__ void cta_teardown_warp() {
+    if (cta_gave_up()) cta_drain_warp(0);
 }
 __device__ __forceinline__ void cta_teardown(bool issuing, int slot = 0) {
-    if (cta_gave_up()) cta_drain(issuing, slot);
+    if (cta_gave_up()) {
+        if (issuing) cta_drain_warp(slot);
+        __syncthreads();
+    }
 }
 
 // Byte offset of 16-byte chunk `chunk` (0..7) of row `row` inside a [rows x 128 B] tile held in

@@ -65,5 +65,5 @@ def test_tensor_memory_is_given_back_after_the_teardown():
         for m in re.finditer(r"\btmem_dealloc\(", text):
             kernels += 1
             before = text[:m.start()]
-            assert before.rfind("cta_teardown(") > before.rfind("__syncthreads"), name
+            assert before.rfind("cta_teardown") > before.rfind("__syncthreads"), name
     assert kernels >= 10
