@@ -591,7 +591,7 @@ ltc_wgrad_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant_
             for (int k = 0; k < steps; ++k) {
                 const int i = k / NH, hf = k % NH;
                 if (k + 1 < steps) form(k + 1);
-                mbar_spin(&bar_t, k & 1, status, kErrMma);
+                if (!mbar_spin(&bar_t, k & 1, status, kErrMma)) break;       // (gave up: no more copies are asked for)
                 tc_fence_after();
                 // tile i - 1 is done with (its last products have completed, its da2 has been read): its input buffer
                 // takes tile i + 2
@@ -798,7 +798,8 @@ ltc_dense_bwd_norm_kernel(const __grid_constant__ CUtensorMap mN, const __grid_c
             const uint64_t nl = smem_desc(sw + B::Lo, 0, 1024, kSwz128);
             auto form = [&](int k) {                   // p1 and dn1 of step k
                 const int i = k / NH, hf = k % NH;
-                if (k > 0) { mbar_spin(&bar_rd[0], (k - 1) & 1, status, kErrMma); mbar_spin(&bar_rd[1], (k - 1) & 1, status, kErrMma); }
+                // (a wait in front of a copy that gave up: no more copies are asked for)
+                if (k > 0 && (!mbar_spin(&bar_rd[0], (k - 1) & 1, status, kErrMma) || !mbar_spin(&bar_rd[1], (k - 1) & 1, status, kErrMma))) return false;
                 if (hf == 0) {
                     if (i > 0) load_lo(i);             // (the last products that read it have completed: they were read out)
                     mbar_spin(&bar_ld[i & 1], (i >> 1) & 1, status, kErrTma);
@@ -823,15 +824,16 @@ ltc_dense_bwd_norm_kernel(const __grid_constant__ CUtensorMap mN, const __grid_c
                         umma_ss(tm + b * 128 + 64, desc_off(dd, q * 32), desc_off(w2, q * 2048), id_s, q > 0 ? 1u : 0u);
                     umma_commit(&bar_s[b]);
                 }
+                return true;
             };
             form(0);
             for (int k = 0; k < steps; ++k) {
                 const int i = k / NH, hf = k % NH;
                 if (hf == 0 && i + 1 < nt) {           // the other input buffer: tile i - 1 is done with
-                    if (k > 0) mbar_spin(&bar_free, (k - 1) & 1, status, kErrMma);
+                    if (k > 0 && !mbar_spin(&bar_free, (k - 1) & 1, status, kErrMma)) break;
                     load(i + 1);
                 }
-                if (k + 1 < steps) form(k + 1);
+                if (k + 1 < steps && !form(k + 1)) break;
                 mbar_spin(&bar_t, k & 1, status, kErrMma);
                 tc_fence_after();
                 const uint32_t in = sw + B::In + (i & 1) * B::kIn, t1 = sw + B::T, td = t1 + 32768;

@@ -147,8 +147,8 @@ sk8_tc_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         if (warp == 0 && elect_one()) {
             // the other buffer: the previous tile's result has left it
             if (it > 0) bulk_wait_read();
-            if (tile + (int)gridDim.x < tiles) load_x(tile + gridDim.x, b ^ 1);
-            mbar_wait(&bar_x[b], (it >> 1) & 1, status, kErrTma);
+            if (ok && tile + (int)gridDim.x < tiles) load_x(tile + gridDim.x, b ^ 1);
+            ok = mbar_wait(&bar_x[b], (it >> 1) & 1, status, kErrTma) && ok;      // (this lane also stores the result)
             tc_fence_after();
             issue_first<R>(tm, smem, x);
             umma_commit(&bar_mma);
@@ -240,8 +240,8 @@ sk8_tc_bwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         if (warp == 0 && elect_one()) {
             // the other buffer: the previous tile's result has left it
             if (it > 0) bulk_wait_read();
-            if (tile + (int)gridDim.x < tiles) load_x(tile + gridDim.x, b ^ 1);
-            mbar_wait(&bar_x[b], (it >> 1) & 1, status, kErrTma);
+            if (ok && tile + (int)gridDim.x < tiles) load_x(tile + gridDim.x, b ^ 1);
+            ok = mbar_wait(&bar_x[b], (it >> 1) & 1, status, kErrTma) && ok;      // (this lane also stores the result)
             tc_fence_after();
             issue_first<R>(tm + cD1, smem, x);
             umma_commit(&bar_mma);
@@ -303,7 +303,7 @@ sk8_tc_bwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         }
         ok = mbar_wait(&bar_mma, uses++ & 1, status, kErrMma) && ok;
         tc_fence_after();
-        if (warp == 0 && elect_one() && tile + (int)gridDim.x < tiles) load_d(tile + gridDim.x);      // the product that read this tile's has completed
+        if (warp == 0 && elect_one() && ok && tile + (int)gridDim.x < tiles) load_d(tile + gridDim.x);      // the product that read this tile's has completed
         {
             // [dA1 | dA2 | dB1 | dB2] = [dM1*A2 | dM1*A1 | dM2*B2 | dM2*B1] / sqrt(R) over the hi/lo tiles (dead since GEMM 2)
 #pragma unroll

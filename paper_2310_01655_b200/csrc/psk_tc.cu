@@ -230,6 +230,8 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     constexpr uint32_t cSk = 0, cS = 0, cW = 0, cA = 0, cO = 128, cN = cO + 80;
     bool ok = true;
 
+    // (A thread whose wait gave up asks for no more copies, and does not arrive where one is counted: see the barrier's phase,
+    // which may still be open.)
     // First phase, issuing side: the chunks `first`, `first + step`, ... of the prefix state.
     // B = the chunk's 64 feature rows x 80 columns, MN-major: 16 features per K step, the second
     // 64-column group (columns 64..79) 8192 B further on.  Everything the loop needs is in registers
@@ -282,15 +284,19 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
             umma_commit(&bar_sk);
             if constexpr (LIN && LOCAL) {
                 ok = ok && mbar_spin(&bar_sk, 0, status, kErrMma);
-                mbar_expect_tx(&bar_q, 16384);
-                tma_load_4d(smem + L::Q, &mapQraw, 0, row0, hi, bi, &bar_q);
+                if (ok) {
+                    mbar_expect_tx(&bar_q, 16384);
+                    tma_load_4d(smem + L::Q, &mapQraw, 0, row0, hi, bi, &bar_q);
+                }
             }
             if (has_prefix && kZStages - 1 < F::NC) {
                 // the query tile has been consumed: its buffer becomes the ring's last stage
                 ok = ok && mbar_spin(&bar_sk, 0, status, kErrMma);
-                mbar_expect_tx(&bar_feat[kZStages - 1], kZStageBytes);
-                tma_load_3d(smem + L::zstage(kZStages - 1), &mapZ, 0, (kZStages - 1) * 64, blk, &bar_feat[kZStages - 1]);
-                tma_load_3d(smem + L::zstage(kZStages - 1) + 8192, &mapZ, 64, (kZStages - 1) * 64, blk, &bar_feat[kZStages - 1]);
+                if (ok) {
+                    mbar_expect_tx(&bar_feat[kZStages - 1], kZStageBytes);
+                    tma_load_3d(smem + L::zstage(kZStages - 1), &mapZ, 0, (kZStages - 1) * 64, blk, &bar_feat[kZStages - 1]);
+                    tma_load_3d(smem + L::zstage(kZStages - 1) + 8192, &mapZ, 64, (kZStages - 1) * 64, blk, &bar_feat[kZStages - 1]);
+                }
             }
             if (has_prefix) issue_chunks();     // earlier blocks: features x prefix state chunks
             const int tp_last = noncausal ? -1 : tau;
@@ -307,16 +313,16 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                     if (P > tau) return;
                     stage_free(L::stage_k(P));
                     if constexpr (L::NT == 2) stage_free(L::stage_k(P) + 1);
-                    load_k(P, P);
+                    if (ok) load_k(P, P);
                     stage_free(L::stage_v(P));
-                    load_v(P, P);
+                    if (ok) load_v(P, P);
                 });
                 // the scores reuse the staging columns: every MMA of the first phase must have completed
                 ok = ok && mbar_spin(&bar_a[(F::NC - 1) % kFeatBufs], ((F::NC - 1) / kFeatBufs) & 1, status, kErrMma);
             } else if (!noncausal) {
                 // first block: nothing used the stages, only the query sketch its buffer
                 ok = ok && mbar_spin(&bar_sk, 0, status, kErrMma);
-                for (int p = 0; p < L::kSets && p <= tau; ++p) { load_k(p, p); load_v(p, p); }
+                for (int p = 0; ok && p < L::kSets && p <= tau; ++p) { load_k(p, p); load_v(p, p); }
             }
             // same block: key tiles tp <= tau through squared half-sketch scores; descriptors and
             // addresses are loop invariants, so every issue sequence below is MMA instructions only
@@ -330,7 +336,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                     // the previous tile's K, V and weights are free: the tile after next (or this one) may come
                     ok = mbar_spin(&bar_pv, (tp - 1) & 1, status, kErrMma);
                     const int nx = tp - 1 + L::kSets;
-                    if (nx <= tp_last) { load_k(nx, nx % L::kSets); load_v(nx, nx % L::kSets); }
+                    if (ok && nx <= tp_last) { load_k(nx, nx % L::kSets); load_v(nx, nx % L::kSets); }
                 }
                 ok = ok && mbar_spin(&bar_kv[p], (tp / L::kSets) & 1, status, kErrTma);
                 tc_fence_after();
@@ -394,7 +400,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                 if (C >= kFeatBufs) {                 // the MMAs that read this buffer's previous contents
                     ok = mbar_wait(&bar_a[buf], (C / kFeatBufs - 1) & 1, status, kErrMma) && ok;
                     tc_fence_after();
-                    if (tid == 0) {                   // ... and this stage's: refill it with chunk C's rows
+                    if (tid == 0 && ok) {             // ... and this stage's: refill it with chunk C's rows
                         mbar_expect_tx(&bar_feat[buf], kZStageBytes);
                         tma_load_3d(smem + L::zstage(buf), &mapZ, 0, C * 64, blk, &bar_feat[buf]);
                         tma_load_3d(smem + L::zstage(buf) + 8192, &mapZ, 64, C * 64, blk, &bar_feat[buf]);
@@ -406,7 +412,7 @@ tc_fwd_out_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
                 tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (tid % 32 == 0) mbar_arrive(&bar_feat[buf]);
+                if (tid % 32 == 0 && ok) mbar_arrive(&bar_feat[buf]);
             }
         }
 

@@ -217,7 +217,8 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
             };
             // the tile's half sketches as [hi | lo] rows, once the generators have put them over its X rows
             auto store_hl = [&](int j) {
-                mbar_wait(&sh.hl[j & 1], (j >> 1) & 1, status, kErrState);
+                ok = ok && mbar_wait(&sh.hl[j & 1], (j >> 1) & 1, status, kErrState);
+                if (!ok) return;
                 tma_store_4d(&mapH, smem + L::X + (j % NX) * 16384, 0, tile_of(j) * 128, hi, bi);
                 if constexpr (R == 64) tma_store_4d(&mapH2, smem + L::Hl, 0, tile_of(j) * 128, hi, bi);
                 bulk_commit();
@@ -239,15 +240,15 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
                 // rows of tile j + 2.  Two slots: sketch j has completed (it was read), but its half sketches leave first;
                 // three: those of tile j - 1 have left
                 if (hl && NX == 3) bulk_wait_read();
-                if ((!hl || NX == 3) && j + 2 < NJs) load_x(j + 2);
+                if (ok && (!hl || NX == 3) && j + 2 < NJs) load_x(j + 2);
                 // values of the next token tile: their slot held tile j-1
                 if (j >= 1) ok = ok && mbar_wait(&sh.yfree[(j + 1) & 1], ((j - 1) >> 1) & 1, status, kErrState);
-                load_y(j + 1);
+                if (ok) load_y(j + 1);            // (a wait that gave up: nothing more is asked for or stored)
                 if (hl) store_hl(j);
                 if (hl && NX == 2) {
                     bulk_wait_read();
                     if constexpr (R == 64) mbar_arrive(&sh.hlfree);
-                    if (j + 2 < NJs) load_x(j + 2);
+                    if (ok && j + 2 < NJs) load_x(j + 2);
                 }
             }
             if (hl) { store_hl(NJs - 1); bulk_wait_read(); }

@@ -39,6 +39,10 @@ def test_a_later_wait_does_not_hide_one_that_gave_up(name):
 
 @pytest.mark.parametrize("name,calls", [
     ("psk_tc_bwd.cu", [r"refill\(C\);", r"load_m\(tp \+ 1,", r"load_y\(tp \+ 1\);", r"mbar_expect_tx\(&bar_again,"]),
+    ("psk_tc.cu", [r"mbar_expect_tx\(&bar_q, 16384\);", r"mbar_expect_tx\(&bar_feat\[kZStages", r"load_k\(P, P\);", r"load_v\(P, P\);",
+                   r"load_k\(nx,", r"mbar_expect_tx\(&bar_feat\[buf\]", r"mbar_arrive\(&bar_feat\[buf\]\);"]),
+    ("psk_tc_state.cu", [r"load_x\(j \+ 2\);", r"load_y\(j \+ 1\);", r"tma_store_4d\(&mapH,"]),
+    ("psk_sketch8_tc.cu", [r"load_x\(tile \+", r"load_d\(tile \+", r"tma_store_tile\(&map"]),
 ])
 def test_no_copy_is_asked_for_after_a_wait_gave_up(name, calls):
     """Every copy that is asked for behind a wait has `ok` in the condition in front of it.  (Its barrier's phase may still be
@@ -52,6 +56,14 @@ def test_no_copy_is_asked_for_after_a_wait_gave_up(name, calls):
             conditions = re.findall(r"\bif (?:constexpr )?\((.*)\)", text[:at][-400:])
             conditions = [c for c in conditions if "L::" not in c or "ok" in c]
             assert conditions and re.search(r"\bok\b", conditions[-1]), (name, call, conditions[-1:])
+
+
+def test_the_networks_feeders_stop_asking_for_copies():
+    """The learnable sketch's issuing lanes leave their loop where a wait in front of a copy gave up."""
+    text = source("psk_learned_tc.cu")
+    for wait, copy, leave in ((r"bar_t, k & 1", r"load\(i \+ 2\);", "break;"), (r"bar_free, \(k - 1\) & 1", r"load\(i \+ 1\);", "break;"),
+                              (r"bar_rd\[1\], \(k - 1\) & 1", r"load_lo\(i\);", "return false;")):
+        assert re.search(r"!mbar_spin\(&" + wait + r", status, kErrMma\)+ " + leave + r".{0,200}?" + copy, text, re.S), copy
 
 
 def test_tensor_memory_is_given_back_after_the_teardown():
