@@ -91,8 +91,9 @@ struct BwdSmem {
     static constexpr uint32_t U = Eoth + 2048;
     static constexpr uint32_t Box = U;                   // phase B: kSt state boxes
     static constexpr int NC = Feat<R>::NC;
-    // stages of the state-chunk ring: four; three on the query side for r = 64, which then fits two CTAs per SM
-    // (the key side, at 255 registers and 225 KB of code, ran slower as two CTAs and keeps four)
+    // stages of the state-chunk ring: four; three on the query side for r = 64, which then fits two CTAs per SM.  (The key side
+    // keeps four and one CTA: as two it was slower, 32.9 against 30.8 ms, when it took 255 registers, spilled and was 225 KB of
+    // code.  It now takes 236 without spills and half the code; two CTAs have not been timed since.)
     static constexpr int kSt = (R > 32 && QSIDE) ? 3 : 4;
     // Phase C tiles: they reuse the boxes' memory, each tile in the stages that the last chunks free first, so
     // the first other-side tile is fetched while the last chunks are still being processed.  r = 64, key side, two-tile
@@ -158,7 +159,7 @@ __device__ __forceinline__ void issue_scores_ts(uint32_t d_tmem, uint32_t a_tmem
 // into a dX accumulator that the sketch's backward (phase D) adds to: no half sketch of the other
 // tile, no split operands, no dM from the tiles.
 // LIN: the rows hold a given half sketch (tc_common.cuh, read_half_sketch); a template parameter, not
-// an argument: the key side sits at the register limit, and the flag as an argument cost it 4 %.
+// an argument: it decides the layout, and as an argument it cost the key side 4 % (when that was at the register limit).
 template <int R, bool QSIDE, bool LOCAL, bool LIN>
 __global__ void __launch_bounds__(128, ((R <= 32 || QSIDE) ? 2 : 1))
 tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_constant__ CUtensorMap mapYown,
@@ -326,10 +327,10 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     // ---- phase B: other blocks through the state ----
     if (has_state) {
         constexpr uint32_t idesc_phi = idesc_bf16(128, 64, false, false);
-        // Software pipeline over the 64-feature chunks: while the MMAs of chunk C run, the threads
-        // generate chunk C+1's features; while those of chunk C+1 run, they un-tensor chunk C.
-        // d-phi is double-buffered in [0,128); during this phase the feature staging buffers sit
-        // in the dM accumulator's columns, which only phase C uses.
+        // Software pipeline over the 64-feature chunks.  Tensor memory: key side, r <= 32: one d-phi buffer in [0,64), two feature
+        // staging buffers in [64,128) (first branch below).  Otherwise d-phi is double-buffered in [0,128): while the MMAs of
+        // chunk C+1 run, the threads un-tensor chunk C; the key side (r = 64) forms chunk C+1's features before those go out,
+        // in two staging buffers in the dM accumulator's columns, which only phase C uses.
         constexpr uint32_t cFB = R <= 32 ? 64 : cdM;          // (staging is for the key side only)
         // descriptors are loop invariants: an issue sequence is its MMA instructions and little else
         const uint64_t yd = smem_desc(smem_u32(smem + L::Yown), 0, 1024, kSwz128);

@@ -40,8 +40,8 @@ constexpr int kModeFirst = 2;          // run 0: both; the other runs: the total
 //   r = 64: forward 1050 -> 554 us, query side 1702 -> 1288, key side 2327 -> 2112; of 384 heads x 32768,
 //   r = 32: 4409 -> 3916, 5031 -> 4776, 6249 -> 5867; the walk itself pays 5 to 20 % for it.)
 // What bounds a walk of r = 32: the shared-memory path, which the generators' tiles, the stores on their way out and the
-// MMAs' operands share (96 heads x 8192, b = 256: 82 % of its cycles on the SMs in use, issue slots 51 %, tensor
-// pipe 27 %), and at short blocks the store warpgroup, one body for all tiles with a bulk copy out (144 heads x
+// MMAs' operands share (96 heads x 8192, b = 256, before elected issue and unrolled features: 82 % of its cycles on the SMs in
+// use, issue slots 51 %, tensor pipe 27 %), and at short blocks the store warpgroup, one body for all tiles with a bulk copy out (144 heads x
 // 8192, b = 256: 318 us unrolled and with copies by the lanes, now 234).
 // grid (BH, runs, shares).  Warp roles:
 //   NWG generator warpgroups  thread = token: read the half sketches, write their feature tiles
@@ -525,7 +525,8 @@ state_walk(SH& sh, const CUtensorMap& mapX, const CUtensorMap& mapY, const CUten
 // Store warpgroups: the walk stalls at a block boundary until the accumulators have been read, one tile after the other.  Two help
 // where a share has two tiles and registers for them (r = 32 in three shares: 48 heads x 16 384, b = 256: 402 us per training step for both
 // walks, one warpgroup that reads all columns at once 382, two 374); with five tiles a CTA (one share, 96 heads x 8192) the generators
-// bound it (400, 394, 402), r = 16 has 212, 204, 212, and r = 64 no registers (1276, 1237, spills).
+// bound it (400, 394, 402), r = 16 has 212, 204, 212, and r = 64 no registers (1276, 1237, spills).  (Two shares at r = 32, with
+// columns at once and 44 bytes of spill stores: 48 to 72 heads, training, 0.84 to 0.96 of before; the rule is the same for them.)
 template <int R, int SPLIT> struct StateSplit {
     static constexpr int NT = Feat<R>::NT, kBase = NT / SPLIT, kMore = NT % SPLIT;
     __host__ __device__ static constexpr int tiles(int z) { return kBase + (z < kMore ? 1 : 0); }
@@ -653,7 +654,9 @@ int state_units(const Dims& d) { return d.noncausal ? d.n / 128 : d.t; }
 
 // CTAs per head and run, and runs per head.  Estimated time in nanoseconds: a CTA's walk of its run, times the
 // rounds in which the grid fills the SMs.  `step`, `boundary`: measured time of a 128-token tile and of writing
-// the states out at a block boundary, for the largest share of a split (12 heads, n = 32 768, b = 256 and 4096);
+// the states out at a block boundary, for the largest share of a split (12 heads, n = 32 768, b = 256 and 4096; taken before elected
+// MMA issue, unrolled features and the second store warpgroup, which made all of them shorter, and not again: none of 270
+// sketched shapes tried got slower with the plans they choose);
 // `mean`: the average share in percent of the largest.  Where more CTAs than SMs are wanted, the shares of a
 // head get in each other's way for r <= 32 (15 % on 96 heads).  A run's start and end cost about 6 us, its start value
 // 4 us, the launch between the two passes over the runs 8 us.
