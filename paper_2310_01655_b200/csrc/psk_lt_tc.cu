@@ -87,7 +87,7 @@ lt_tc_state_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_consta
         for (int l = 0; l + 1 < t; ++l) {
             ok = mbar_wait(&bar_acc, l & 1, status, kErrMma) && ok;
             tc_fence_after();
-            if (ok && f0 + tid < m) {
+            if (f0 + tid < m) {                       // (the same for a whole warp, as tensor-memory loads need it; `ok` may not be)
                 bf16* dst = Z + (((size_t)bt * t + l + 1) * m + f0 + tid) * 64;
 #pragma unroll
                 for (int c0 = 0; c0 < 64; c0 += 32) {
@@ -96,7 +96,7 @@ lt_tc_state_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_consta
                     tmem_ld_wait();
 #pragma unroll
                     for (int j = 0; j < 32; j += 8)
-                        *reinterpret_cast<uint4*>(dst + c0 + j) =
+                        if (ok) *reinterpret_cast<uint4*>(dst + c0 + j) =
                             make_uint4(pack_bf16(__uint_as_float(u[j]), __uint_as_float(u[j + 1])), pack_bf16(__uint_as_float(u[j + 2]), __uint_as_float(u[j + 3])),
                                        pack_bf16(__uint_as_float(u[j + 4]), __uint_as_float(u[j + 5])), pack_bf16(__uint_as_float(u[j + 6]), __uint_as_float(u[j + 7])));
                 }
@@ -223,7 +223,7 @@ lt_tc_rows_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constan
         const uint32_t lane_tm = tm + ((uint32_t)((warp % 4) * 32) << 16);
         bool ok = mbar_wait(&bar_s, 0, status, kErrMma);
         tc_fence_after();
-        if (ok) {
+        {                                             // (not behind `ok`: all lanes of a warp read and write tensor memory)
             for (int tp = 0; tp <= w; ++tp) {
                 const bool diag = tp == w;
                 const uint32_t ts = lane_tm + scores(w, tp);
@@ -248,7 +248,7 @@ lt_tc_rows_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constan
         mbar_arrive(&bar_p[w]);
         ok = ok && mbar_wait(&bar_o[w], 0, status, kErrMma);
         tc_fence_after();
-        if (ok) {
+        {
             float* dst = Out + ((size_t)bt * n + row0 + w * 128 + wt) * 64;
 #pragma unroll
             for (int c0 = 0; c0 < 64; c0 += 32) {
@@ -257,7 +257,7 @@ lt_tc_rows_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constan
                 tmem_ld_wait();
 #pragma unroll
                 for (int j = 0; j < 32; j += 4)
-                    *reinterpret_cast<float4*>(dst + c0 + j) = make_float4(__uint_as_float(u[j]), __uint_as_float(u[j + 1]),
+                    if (ok) *reinterpret_cast<float4*>(dst + c0 + j) = make_float4(__uint_as_float(u[j]), __uint_as_float(u[j + 1]),
                                                                            __uint_as_float(u[j + 2]), __uint_as_float(u[j + 3]));
             }
         }

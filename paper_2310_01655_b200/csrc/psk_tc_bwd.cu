@@ -768,8 +768,8 @@ tc_bwd_rows_kernel(const __grid_constant__ CUtensorMap mapXown, const __grid_con
     }
     // rows go out through shared memory and tiled stores (every MMA has completed: the other-side
     // tiles' memory is free); a thread-per-row store pattern would keep the load/store unit busy
-    // for thousands of cycles
-    if (ok) {
+    // for thousands of cycles.  (Not behind `ok`, which lanes of a warp may differ in: tensor memory is read by all of them.)
+    {
 #pragma unroll
         for (int c0 = 0; c0 < 64; c0 += 32) {
             uint32_t v[32];

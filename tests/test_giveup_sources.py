@@ -58,6 +58,18 @@ def test_no_copy_is_asked_for_after_a_wait_gave_up(name, calls):
             assert conditions and re.search(r"\bok\b", conditions[-1]), (name, call, conditions[-1:])
 
 
+@pytest.mark.parametrize("name", ["psk_tc.cu", "psk_tc_bwd.cu", "psk_tc_state.cu", "psk_lt_tc.cu", "psk_sketch8_tc.cu"])
+def test_tensor_memory_is_read_by_whole_warps(name):
+    """Loads and stores of tensor memory need every lane of a warp; after a wait gave up in some lanes only, `ok` differs."""
+    text = source(name)
+    for m in re.finditer(r"\bif \((?:[^{};]*\W)?ok\b[^{};]*\) \{", text):
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(text[i], 0)
+            i += 1
+        assert not re.search(r"\btmem_(?:ld|st)", text[m.end():i]), (name, m.group(0))
+
+
 def test_the_networks_feeders_stop_asking_for_copies():
     """The learnable sketch's issuing lanes leave their loop where a wait in front of a copy gave up."""
     text = source("psk_learned_tc.cu")
